@@ -195,8 +195,8 @@ ef21_status ef21_topk(const float* v_dev, int32_t batch, int64_t d, int32_t k,
  *
  * Limits: batch <= 64 and batch * ceil(d / 4096) <= 16384 (e.g. 64 vectors of 2^20 entries, or
  * one of 2^26); beyond that the call returns EF21_ERR_UNSUPPORTED and does nothing.  Vectors
- * of up to 8,192 entries take the one-launch kernel (which needs no scratch), longer ones the
- * multi-pass radix select.
+ * that fit into a cluster's shared memory take the one-launch kernel (which needs no scratch), longer
+ * ones the multi-pass radix select.
  * The first call on a device looks up the device address of the scratch array
  * (cudaGetSymbolAddress, with that device current) and caches it; make that first call outside
  * of any stream capture.
@@ -270,13 +270,14 @@ ef21_status ef21_set_variant(ef21_ctx* ctx, int32_t variant);
  * synchronises. */
 ef21_status ef21_get_plus_choice(ef21_ctx* ctx, int32_t* choice_host);
 
-/* Top-k algorithm used inside the EF21 rounds of the launch path: 0 = automatic (long vectors,
- * d >= 2^18 and k <= 6144, take the one-pass path: sampled threshold, single streaming pass,
- * exact selection among the candidates; everything else takes the multi-pass radix select),
- * 1 = always the multi-pass radix select.  Both give the same bits. */
+/* Top-k algorithm used inside the EF21 rounds of the launch path: 0 = automatic (a vector that fits into the
+ * shared memory of a thread-block cluster is selected there in one launch; longer ones, and large batches of
+ * long ones, take the one-pass path: bracket from a sample, single streaming pass, exact selection among the
+ * candidates; messages of more than half of a long vector take the multi-pass radix select), 1 = no one-pass
+ * path.  All give the same bits. */
 ef21_status ef21_set_topk_algorithm(ef21_ctx* ctx, int32_t algorithm);
-/* Number of vectors, since creation, for which the one-pass Top-k had to fall back to the exact
- * selection over the whole vector (threshold missed or too many ties); synchronises. */
+/* Number of vectors of d >= 2^18 entries, since creation, whose selection had to be repeated over the whole
+ * vector (the sampled bracket missed, or too many ties); synchronises. */
 ef21_status ef21_fallback_count(ef21_ctx* ctx, int64_t* count);
 
 /* Clears the device status word (after an error has been read with ef21_poll). */

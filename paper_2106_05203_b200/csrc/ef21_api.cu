@@ -6,6 +6,8 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <set>
+#include <utility>
 #include <vector>
 
 #include "apply.cuh"
@@ -15,14 +17,28 @@
 #include "persistent.cuh"
 #include "wait_selftest.cuh"
 #include "plus.cuh"
-#include "stress.cuh"
 #include "topk.cuh"
+#include "topk_cluster.cuh"
+#include "topk_stream.cuh"
 
 using namespace ef21;
+
+#define CU(call)                                         \
+    do {                                                 \
+        cudaError_t e__ = (call);                        \
+        if (e__ != cudaSuccess) return EF21_ERR_CUDA;    \
+    } while (0)
+#define EF(call)                                         \
+    do {                                                 \
+        ef21_status s__ = (call);                        \
+        if (s__ != EF21_OK) return s__;                  \
+    } while (0)
+
 
 namespace {
 
 constexpr size_t ALIGN = 256;
+constexpr i64 GRAPH_MAX_D = 8192;      // launch-path iterations up to this dimension are replayed as a CUDA graph
 inline size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 inline i64 ceil_div(i64 a, i64 b) { return (a + b - 1) / b; }
 
@@ -30,16 +46,51 @@ inline i64 ceil_div(i64 a, i64 b) { return (a + b - 1) / b; }
 // Workspace layouts
 // ---------------------------------------------------------------------------------------------
 
+// Kernel launch as a programmatic dependent of whatever precedes it in the stream (see pdl_wait), with clusters of C blocks.
+template <typename... Params, typename... Args>
+cudaError_t launch(void (*kern)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, unsigned C, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = C > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
+// Opt-in of a kernel to more dynamic shared memory than the default 48 KB (and to clusters of more than eight blocks): an
+// attribute per device, set once.
+ef21_status allow_smem(const void* kern, size_t bytes, bool big_cluster = false) {
+    static std::mutex mu;
+    static std::set<std::pair<int, const void*>> done;
+    int dev = -1;
+    CU(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({dev, kern})) return EF21_OK;
+    CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    if (big_cluster) CU(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    done.insert({dev, kern});
+    return EF21_OK;
+}
+
 struct TopkLayout {
     size_t state, hist, chunks, total;
     int nchunks;
-    // one-pass path for long vectors (stress.cuh); fast == false: sections absent
+    // one-pass path for long vectors (topk_stream.cuh); fast == false: sections absent
     bool fast;
-    int nreg;
-    size_t thr, flags, done, slow_count, region_cnt, cand;
+    int nreg, nreg_pitch, region_log, cap;   // regions per vector (and rounded up to 8), log2 of their entries, candidate records per region
+    i64 open_cap;                        // open entries per vector
+    i64 samples;                         // per vector
+    size_t ctl, open_hist, open_list, reg_cand, reg_base, slow_count, cand;
 };
 
-bool fast_topk_eligible(i64 d, i64 k) { return d >= ST_MIN_D && k <= ST_MAX_K; }
+// From half of the entries on the bracket saves nothing: such messages take the multi-pass select.
+bool fast_topk_eligible(i64 d, i64 k) { return d >= ST_MIN_D && 2 * k <= d; }
+
+// Distance of the bracket's ends from the expected rank in the sample: 4.5 standard deviations of that rank.
+double st_margin(double rank) { return 4.5 * std::sqrt(rank) + 4.0; }
 
 // The three sections every Top-k call needs (selection state, histogram, per-chunk counts); the
 // one-pass sections are absent.
@@ -51,7 +102,6 @@ TopkLayout topk_layout_general(i64 batch, i64 d) {
     L.hist = o; o += align_up((size_t)batch * TK_BINS * sizeof(unsigned));
     L.chunks = o; o += align_up((size_t)batch * (size_t)L.nchunks * sizeof(uint2));
     L.fast = false;
-    L.nreg = (int)ceil_div(d, ST_SUB);
     L.total = o;
     return L;
 }
@@ -61,12 +111,30 @@ TopkLayout topk_layout(i64 batch, i64 d, i64 k) {
     size_t o = L.total;
     L.fast = fast_topk_eligible(d, k);
     if (L.fast) {
-        L.thr = o; o += align_up((size_t)batch * 4);
-        L.flags = o; o += align_up((size_t)batch * 4);
-        L.done = o; o += align_up((size_t)batch * 4);
+        L.region_log = batch * d >= ST_LARGE_TOTAL ? ST_REGION_LOG_LARGE : ST_REGION_LOG_SMALL;
+        const i64 region = (i64)1 << L.region_log;
+        L.nreg = (int)ceil_div(d, region);
+        L.nreg_pitch = (L.nreg + 7) / 8 * 8;
+        // Sample size: 512 sampled entries above the cut give a bracket of about +-20 %; at least 64 K, at most 256 K
+        // entries, 4 M over the whole batch, a quarter of the vector.
+        L.samples = std::max<i64>(512 * d / k, d / 64);
+        L.samples = std::min<i64>(std::max<i64>(L.samples, 65536), std::max<i64>(65536, std::min<i64>(262144, 4194304 / batch)));
+        L.samples = std::min<i64>(L.samples, d / 4);
+        L.samples = L.samples >= 262144 ? 262144 : (L.samples >= 131072 ? 131072 : 65536);
+        // Records per region: the expected candidates (the message plus the bracket's upper half) and six standard deviations
+        // of a region's count; where more than a tenth of the entries are wanted a region is cheaper to read again.
+        const double rank = (double)k * (double)L.samples / (double)d;
+        const double expect = (double)region * (double)k / (double)d * (1.0 + st_margin(rank) / rank);
+        const i64 cap = (i64)(expect + 6.0 * std::sqrt(expect)) + 16;
+        L.cap = 10 * expect > (double)region ? 0 : (int)((cap + 7) / 8 * 8);
+        L.open_cap = std::min<i64>(d, k <= 65536 ? 2 * k + 16384 : k / 2 + 131072);
+        L.ctl = o; o += align_up((size_t)batch * sizeof(StCtl));
+        L.open_hist = o; o += align_up((size_t)batch * ST_OPEN_BINS * 4);
+        L.open_list = o; o += align_up((size_t)batch * L.open_cap * 8);
+        L.reg_cand = o; o += align_up((size_t)batch * L.nreg_pitch * 4);
+        L.reg_base = o; o += align_up((size_t)batch * L.nreg_pitch * 4);
         L.slow_count = o; o += align_up(4);
-        L.region_cnt = o; o += align_up((size_t)batch * L.nreg * 4);
-        L.cand = o; o += align_up((size_t)batch * L.nreg * ST_REGION_CAP * sizeof(int4));
+        L.cand = o; o += align_up((size_t)batch * L.nreg * L.cap * sizeof(int4));
     }
     L.total = o;
     return L;
@@ -212,23 +280,11 @@ struct ef21_ctx {
     unsigned* status() const { return at<unsigned>(L.status); }
 };
 
-#define CU(call)                                         \
-    do {                                                 \
-        cudaError_t e__ = (call);                        \
-        if (e__ != cudaSuccess) return EF21_ERR_CUDA;    \
-    } while (0)
-#define EF(call)                                         \
-    do {                                                 \
-        ef21_status s__ = (call);                        \
-        if (s__ != EF21_OK) return s__;                  \
-    } while (0)
-
 namespace {
 
 struct TopkBuffers {
     TkState* state; unsigned* hist; uint2* chunks; int nchunks;
-    bool fast; int nreg;
-    unsigned* thr; unsigned* flags; unsigned* done; unsigned* slow_count; int* region_cnt; int4* cand;
+    TopkLayout L; char* base;            // sections of the one-pass path
 };
 
 TopkBuffers topk_buffers(char* base, const TopkLayout& L) {
@@ -237,78 +293,153 @@ TopkBuffers topk_buffers(char* base, const TopkLayout& L) {
     B.hist = reinterpret_cast<unsigned*>(base + L.hist);
     B.chunks = reinterpret_cast<uint2*>(base + L.chunks);
     B.nchunks = L.nchunks;
-    B.fast = L.fast; B.nreg = L.nreg;
-    B.thr = reinterpret_cast<unsigned*>(base + L.thr);
-    B.flags = reinterpret_cast<unsigned*>(base + L.flags);
-    B.done = reinterpret_cast<unsigned*>(base + L.done);
-    B.slow_count = reinterpret_cast<unsigned*>(base + L.slow_count);
-    B.region_cnt = reinterpret_cast<int*>(base + L.region_cnt);
-    B.cand = reinterpret_cast<int4*>(base + L.cand);
+    B.L = L; B.base = base;
     return B;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Threshold estimate of the one-pass Top-k (first of its three kernels).
-ef21_status enqueue_topk_fast_sample(cudaStream_t st, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
-                                     int batch, i64 d, int k, const TopkBuffers& B, i64* launches) {
-    const i64 target = std::max<i64>(2 * (i64)k, (i64)k + 2048);
-    i64 rank = ceil_div(target * (i64)(ST_SAMPLE_BLOCKS * ST_SAMPLE_LEN), d);
-    rank = std::min<i64>(std::max<i64>(rank, 32), ST_SAMPLE_BLOCKS * ST_SAMPLE_LEN / 2);
-    st_sample_kernel<<<batch, ST_THREADS, 0, st>>>(a, pitch_a, b, pitch_b, d, (unsigned)rank, B.thr, B.flags);
-    if (launches) *launches += 1;
-    CU(cudaGetLastError());
-    return EF21_OK;
+// ---- Top-k by one cluster per vector (topk_cluster.cuh) ----
+struct TcShape { int C, slice, threads; };
+
+// Blocks per vector: as few as hold the vector in shared memory, then more while all clusters still run at once and a
+// block keeps at least 8,192 entries (a shorter sweep per block; below that the two cluster barriers cost more than they
+// save).  False where the vector is too long, or so long and the batch so large that the clusters would run in several
+// waves of one-block-per-SM: the streaming kernels read such a batch at HBM speed.
+bool tc_shape(i64 batch, i64 d, TcShape& S) {
+    constexpr i64 SMS = 148;
+    i64 C = 1;
+    while (C <= TC_MAX_CLUSTER && ceil_div(d, C) > TC_MAX_SLICE) C *= 2;
+    if (C > TC_MAX_CLUSTER || (d >= ST_MIN_D && batch * C > SMS)) return false;
+    while (C < 8 && batch * C * 2 <= SMS && d / (2 * C) >= 8192) C *= 2;
+    S.C = (int)C;
+    S.slice = (int)((ceil_div(d, C) + 127) / 128 * 128);
+    S.threads = C == 1 && d <= 2048 ? 256 : (C == 1 && d <= 8192 ? 512 : 1024);
+    return true;
 }
 
-// Exact Top-k of v = a - b for long vectors in one pass over a and b (see stress.cuh).  If gi_rows
-// is given, g_i += c_i is applied by the same kernel that writes the messages.
-ef21_status enqueue_topk_fast(cudaStream_t st, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
-                              int batch, i64 d, int k, int* idx_out, float* val_out, float* gi_rows, i64 ld,
-                              const TopkBuffers& B, i64* launches, unsigned* status, bool sampled = false,
-                              int* tile_off = nullptr, int ntiles = 0) {
-    const size_t finish_smem = (size_t)ST_CAND_CAP * 12 + 2048 * 4;
-    {
-        // the shared-memory opt-in is a per-device attribute of the kernel: set once per device ordinal
-        constexpr int MAX_DEVICES = 64;
-        static std::mutex mu;
-        static bool smem_set[MAX_DEVICES] = {};
-        int dev = -1;
-        CU(cudaGetDevice(&dev));
-        std::lock_guard<std::mutex> lock(mu);
-        if (dev < 0 || dev >= MAX_DEVICES || !smem_set[dev]) {
-            CU(cudaFuncSetAttribute(st_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)finish_smem));
-            if (dev >= 0 && dev < MAX_DEVICES) smem_set[dev] = true;
-        }
+typedef void (*TcKernel)(const TcArgs);
+template <int MODE>
+TcKernel tc_lookup(const TcShape& S) {
+    if (S.threads == 256) return tc_topk_kernel<MODE, 1, 256>;
+    if (S.threads == 512) return tc_topk_kernel<MODE, 1, 512>;
+    switch (S.C) {
+        case 1: return tc_topk_kernel<MODE, 1, 1024>;
+        case 2: return tc_topk_kernel<MODE, 2, 1024>;
+        case 4: return tc_topk_kernel<MODE, 4, 1024>;
+        case 8: return tc_topk_kernel<MODE, 8, 1024>;
+        default: return tc_topk_kernel<MODE, 16, 1024>;
     }
-    if (!sampled) EF(enqueue_topk_fast_sample(st, a, pitch_a, b, pitch_b, batch, d, k, B, launches));
-    dim3 grid((unsigned)ceil_div(B.nreg, ST_COLLECT_WARPS), (unsigned)batch);
-    const bool vec = aligned16(a) && pitch_a % 4 == 0 && (!b || (aligned16(b) && pitch_b % 4 == 0));
-    auto collect = vec ? st_collect_kernel<true> : st_collect_kernel<false>;
-    collect<<<grid, ST_COLLECT_WARPS * 32, 0, st>>>(a, pitch_a, b, pitch_b, d, B.nreg, B.thr, B.cand, B.region_cnt, B.flags);
-    st_finish_kernel<<<batch, ST_THREADS, finish_smem, st>>>(a, pitch_a, b, pitch_b, d, B.nreg, k, B.cand, B.region_cnt,
-                                                             B.flags, idx_out, val_out, gi_rows, ld, B.slow_count, tile_off,
-                                                             ntiles, AGG_TILE, status);
-    if (launches) *launches += 2;
-    CU(cudaGetLastError());
+}
+
+ef21_status enqueue_topk_cluster(cudaStream_t st, int mode, const TcShape& S, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
+                                 float gamma, int batch, i64 d, int k, int* idx_out, float* val_out, float* apply, i64 pitch_apply,
+                                 i64* launches, unsigned* status, unsigned* slow_count = nullptr) {
+    const TcKernel kern = mode == TC_PLAIN ? tc_lookup<TC_PLAIN>(S) : (mode == TC_DIFF ? tc_lookup<TC_DIFF>(S) : tc_lookup<TC_EF>(S));
+    const size_t smem = tc_smem_bytes(S.C, S.slice);
+    EF(allow_smem(reinterpret_cast<const void*>(kern), tc_smem_bytes(S.C, S.C == 1 && S.threads < 1024 ? 8192 : TC_MAX_SLICE), S.C > 8));
+    TcArgs p = {};
+    p.a = a; p.pitch_a = pitch_a; p.b = const_cast<float*>(b); p.pitch_b = pitch_b;
+    p.d = (int)d; p.k = k; p.slice = S.slice; p.gamma = gamma;
+    p.idx_out = idx_out; p.val_out = val_out; p.apply = apply; p.pitch_apply = pitch_apply; p.status = status; p.slow_count = slow_count;
+    CU(launch(kern, dim3((unsigned)batch * (unsigned)S.C), (unsigned)S.threads, smem, st, (unsigned)S.C, p));
+    if (launches) *launches += 1;
     return EF21_OK;
 }
 
-// Exact Top-k of v = a - b for `batch` vectors (b may be null); general multi-block path.
+// ---- Top-k of long vectors in one pass (topk_stream.cuh) ----
+StArgs stream_args(const float* a, i64 pitch_a, const float* b, i64 pitch_b, float gamma, i64 d, int k, const TopkBuffers& B) {
+    StArgs p;
+    p.a = a; p.pitch_a = pitch_a; p.b = const_cast<float*>(b); p.pitch_b = pitch_b; p.d = d; p.k = k;
+    p.nreg = B.L.nreg; p.nreg_pitch = B.L.nreg_pitch; p.region_log = B.L.region_log; p.cap = B.L.cap; p.open_cap = (unsigned)B.L.open_cap; p.gamma = gamma;
+    p.ctl = reinterpret_cast<StCtl*>(B.base + B.L.ctl);
+    p.open_hist = reinterpret_cast<unsigned*>(B.base + B.L.open_hist);
+    p.open_list = reinterpret_cast<unsigned long long*>(B.base + B.L.open_list);
+    p.reg_cand = reinterpret_cast<unsigned*>(B.base + B.L.reg_cand);
+    p.reg_base = reinterpret_cast<unsigned*>(B.base + B.L.reg_base);
+    p.cand = reinterpret_cast<int4*>(B.base + B.L.cand);
+    p.slow_count = reinterpret_cast<unsigned*>(B.base + B.L.slow_count);
+    return p;
+}
+
+// The bracket (first of the five kernels): clusters of eight blocks, of four or two when there are many vectors (two of these
+// blocks fit on an SM).
+template <int MODE>
+ef21_status enqueue_stream_sample(cudaStream_t st, const StArgs& p, int batch, const TopkLayout& L, i64* launches) {
+    const double rank = (double)p.k * (double)L.samples / (double)p.d;
+    const int C = batch <= 37 ? 8 : (batch <= 74 ? 4 : 2);
+    const i64 per_thread = L.samples / (ST_SAMPLE_THREADS * C);
+    auto kern = C == 2 ? st_sample_kernel<MODE, 2, 32>
+                       : (C == 4 ? st_sample_kernel<MODE, 4, 16>
+                                 : (per_thread >= 32 ? st_sample_kernel<MODE, 8, 32>
+                                                     : (per_thread >= 16 ? st_sample_kernel<MODE, 8, 16> : st_sample_kernel<MODE, 8, 8>)));
+    CU(launch(kern, dim3((unsigned)(batch * C)), ST_SAMPLE_THREADS, 0, st, (unsigned)C, p, (float)rank, (float)st_margin(rank)));
+    if (launches) *launches += 1;
+    return EF21_OK;
+}
+
+template <int MODE>
+ef21_status enqueue_topk_stream(cudaStream_t st, const float* a, i64 pitch_a, const float* b, i64 pitch_b, float gamma, int batch, i64 d,
+                                int k, const StOut& out, const TopkBuffers& B, i64* launches, bool count_slow, bool sampled = false) {
+    StArgs p = stream_args(a, pitch_a, b, pitch_b, gamma, d, k, B);
+    if (!count_slow) p.slow_count = nullptr;
+    if (!sampled) EF(enqueue_stream_sample<MODE>(st, p, batch, B.L, launches));
+    const bool vec = aligned16(a) && (pitch_a % 4 == 0 || batch == 1) && (!b || (aligned16(b) && (pitch_b % 4 == 0 || batch == 1)));
+    // open entries of a vector: twice the margin's share of the message (and the sampled range's steps, hence the 30 %)
+    const double rank = (double)k * (double)B.L.samples / (double)d;
+    const double open = 2.6 * st_margin(rank) / rank * (double)k;
+    const i64 all_blocks = ceil_div(p.nreg, ST_WARPS);
+    int cut_blocks = batch > 37 ? 2 : 8;
+    bool classify = vec && p.region_log == ST_REGION_LOG_LARGE && p.cap > 0;
+    while (classify && cut_blocks < 8 && open > 0.8 * cut_blocks * ST_OPEN_STAGE) cut_blocks *= 2;
+    classify = classify && open <= 0.8 * cut_blocks * ST_OPEN_STAGE;
+    if (classify) {
+        CU(launch(st_collect_long_kernel<MODE>, dim3((unsigned)all_blocks, (unsigned)batch), ST_WARPS * 32, 0, st, 1, p));
+    } else {
+        auto collect = p.cap == 0 ? (vec ? st_collect_kernel<MODE, true, 4, false> : st_collect_kernel<MODE, false, 8, false>)
+                                  : (vec ? st_collect_kernel<MODE, true, 4, true> : st_collect_kernel<MODE, false, 8, true>);
+        // as many blocks as are resident, in turn; more where the open entries of one would not fit its buffer
+        const i64 resident = std::max<i64>(1, 148 * 4 / batch), for_open = (i64)(1.5 * open / ST_BLOCK_OPEN);
+        CU(launch(collect, dim3((unsigned)std::min(all_blocks, std::max(resident, for_open)), (unsigned)batch), ST_WARPS * 32, 0, st, 1, p));
+    }
+    typedef void (*CutKernel)(const StArgs);
+    static const CutKernel cut_kernels[2][3] = {{st_cut_kernel<2, false>, st_cut_kernel<4, false>, st_cut_kernel<8, false>},
+                                                {st_cut_kernel<2, true>, st_cut_kernel<4, true>, st_cut_kernel<8, true>}};
+    const CutKernel cut = cut_kernels[classify ? 1 : 0][cut_blocks == 2 ? 0 : (cut_blocks == 4 ? 1 : 2)];
+    EF(allow_smem(reinterpret_cast<const void*>(cut), st_cut_smem_bytes(classify)));
+    CU(launch(cut, dim3((unsigned)(batch * cut_blocks)), 1024, st_cut_smem_bytes(classify), st, (unsigned)cut_blocks, p));
+    if (p.cap > 0)
+        CU(launch(st_compact_kernel<MODE>, dim3((unsigned)ceil_div(p.nreg, 32), (unsigned)batch), 256, 0, st, 1, p, out));
+    else
+        CU(launch(st_reread_kernel<MODE>, dim3((unsigned)ceil_div(p.nreg, 8), (unsigned)batch), 256, 0, st, 1, p, out));
+    // vectors whose bracket missed: redone exactly (at once over where there is none)
+    TcArgs t = {};
+    t.a = a; t.pitch_a = pitch_a; t.b = const_cast<float*>(b); t.pitch_b = pitch_b; t.d = (int)d; t.k = k; t.batch = batch;
+    t.idx_out = out.idx_out; t.val_out = out.val_out; t.apply = out.apply; t.pitch_apply = out.pitch_apply; t.status = out.status;
+    t.flag = &p.ctl->slow; t.flag_pitch = sizeof(StCtl) / 4;
+    t.tile_off = out.tile_off; t.ntiles = out.ntiles; t.tile = AGG_TILE;
+    t.slice = (int)((ceil_div(d, 8) + 127) / 128 * 128);
+    CU(launch(tc_topk_kernel<MODE == TC_EF ? TC_SENT : MODE, 8, 1024, true>, dim3(8u * (unsigned)std::min(batch, 16)), 1024, tc_smem_bytes(8, 0), st, 8, t));
+    if (launches) *launches += 4;
+    return EF21_OK;
+}
+
+// The handle's count of vectors that took the slow way (long vectors only; null where the layout keeps none).
+unsigned* slow_counter(const TopkBuffers& B) { return B.L.fast ? reinterpret_cast<unsigned*>(B.base + B.L.slow_count) : nullptr; }
+
+// Exact Top-k of v = a - b for `batch` vectors (b may be null): one cluster per vector where it fits, else the
+// multi-pass radix select.
 ef21_status enqueue_topk_general(cudaStream_t st, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
                                  int batch, i64 d, int k, int* idx_out, float* val_out,
                                  const TopkBuffers& B, i64* launches, unsigned* status, float* apply_to = nullptr,
                                  i64 pitch_apply = 0, bool* applied = nullptr) {
     if (applied) *applied = false;
-    if (d <= TKS_MAX_D) {
-        // short vectors: the whole selection in one launch, one block per vector (no scratch); the same
-        // launch adds the messages to apply_to if the caller asks for it
-        tk_small_kernel<<<batch, TKS_BLOCK, (size_t)d * 4, st>>>(a, pitch_a, b, pitch_b, (int)d, k, idx_out, val_out,
-                                                                 apply_to, pitch_apply, status);
+    TcShape S;
+    if (tc_shape(batch, d, S)) {
+        // the whole selection in one launch (no scratch), which also adds the messages to apply_to if the caller asks for it
         if (applied) *applied = apply_to != nullptr;
-        if (launches) *launches += 1;
-        CU(cudaGetLastError());
-        return EF21_OK;
+        return enqueue_topk_cluster(st, b ? TC_DIFF : TC_PLAIN, S, a, pitch_a, b, pitch_b, 0.f, batch, d, k, idx_out, val_out, apply_to,
+                                    pitch_apply, launches, status, status ? slow_counter(B) : nullptr);
     }
     tk_reset_kernel<<<batch, 256, 0, st>>>(B.state, B.hist, batch, (unsigned)k);
     dim3 grid((unsigned)B.nchunks, (unsigned)batch);
@@ -389,14 +520,20 @@ ef21_status enqueue_minibatch_grads(ef21_ctx* c, const int* batch_dev, int tau) 
     return EF21_OK;
 }
 
+// Whether the handle's rounds take the one-pass Top-k of long vectors.
+bool long_topk(const ef21_ctx* c) {
+    TcShape S;
+    return c->L.tk.fast && !c->force_general_topk && !tc_shape(c->n, c->d, S);
+}
+
 // Selection half of a message round: c_i = C(a_i - g_i) and g_i += c_i.  sampled: the threshold
 // kernel of the one-pass Top-k has already run for these inputs.
 ef21_status enqueue_round_select(ef21_ctx* c, const float* a, i64 pitch_a, bool sampled) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
-    if (B.fast && !c->force_general_topk) {
+    if (long_topk(c)) {
         // the finish kernel also leaves the per-tile offsets of the messages for the aggregation
-        EF(enqueue_topk_fast(c->stream, a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->k, c->msg_idx(), c->msg_val(),
-                             c->gi(), c->L.ld, B, &c->launches, c->status(), sampled, c->at<int>(c->L.agg_off), c->L.agg_tiles));
+        const StOut out = {c->msg_idx(), c->msg_val(), c->gi(), c->L.ld, c->at<int>(c->L.agg_off), c->L.agg_tiles, c->status()};
+        EF(enqueue_topk_stream<TC_DIFF>(c->stream, a, pitch_a, c->gi(), c->L.ld, 0.f, c->n, c->d, c->k, out, B, &c->launches, true, sampled));
         c->agg_off_ready = true;
     } else {
         c->agg_off_ready = false;
@@ -452,10 +589,10 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
     int* idx_b = c->at<int>(c->L.msg2_idx);
     float* val_b = c->at<float>(c->L.msg2_val);
-    if (B.fast && !c->force_general_topk) {
-        EF(enqueue_topk_fast(c->stream, a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->k, c->msg_idx(), c->msg_val(),
-                             nullptr, 0, B, &c->launches, c->status()));
-        EF(enqueue_topk_fast(c->stream, a, pitch_a, nullptr, 0, c->n, c->d, c->k, idx_b, val_b, nullptr, 0, B, &c->launches, c->status()));
+    if (long_topk(c)) {
+        const StOut om = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status()}, ob = {idx_b, val_b, nullptr, 0, nullptr, 0, c->status()};
+        EF(enqueue_topk_stream<TC_DIFF>(c->stream, a, pitch_a, c->gi(), c->L.ld, 0.f, c->n, c->d, c->k, om, B, &c->launches, true));
+        EF(enqueue_topk_stream<TC_PLAIN>(c->stream, a, pitch_a, nullptr, 0, 0.f, c->n, c->d, c->k, ob, B, &c->launches, true));
     } else {
         EF(enqueue_topk_general(c->stream, a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->k, c->msg_idx(), c->msg_val(), B,
                                 &c->launches, c->status()));
@@ -479,9 +616,9 @@ ef21_status enqueue_ef_round(ef21_ctx* c, const float* a, i64 pitch_a) {
     const unsigned blocks = (unsigned)std::min<i64>(ceil_div((i64)c->n * c->d, 256), 148 * 16);
     ef_compose_kernel<<<blocks, 256, 0, c->stream>>>(a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->gamma);
     c->launches += 1;
-    if (B.fast && !c->force_general_topk) {
-        EF(enqueue_topk_fast(c->stream, c->gi(), c->L.ld, nullptr, 0, c->n, c->d, c->k, c->msg_idx(), c->msg_val(),
-                             nullptr, 0, B, &c->launches, c->status()));
+    if (long_topk(c)) {
+        const StOut out = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status()};
+        EF(enqueue_topk_stream<TC_PLAIN>(c->stream, c->gi(), c->L.ld, nullptr, 0, 0.f, c->n, c->d, c->k, out, B, &c->launches, true));
     } else {
         EF(enqueue_topk_general(c->stream, c->gi(), c->L.ld, nullptr, 0, c->n, c->d, c->k, c->msg_idx(), c->msg_val(), B,
                                 &c->launches, c->status()));
@@ -935,7 +1072,7 @@ static ef21_status enqueue_launch_iteration(ef21_ctx* c) {
 // plain launches, which give the same results.
 static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
     int done = 0;
-    const bool graphable = c->d <= TKS_MAX_D && steps >= 3 && !c->iter_graph_off;
+    const bool graphable = c->d <= GRAPH_MAX_D && steps >= 3 && !c->iter_graph_off;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (graphable && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         EF(enqueue_launch_iteration(c));
@@ -1017,7 +1154,7 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
         c->last_path = EF21_PATH_LAUNCHES;
         return EF21_OK;
     }
-    const bool fast = c->L.tk.fast && !c->force_general_topk;
+    const bool fast = long_topk(c);
     if (fast && steps > 1 && !c->aux_stream) {
         if (cudaStreamCreateWithFlags(&c->aux_stream, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1051,7 +1188,7 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
         EF(agg);
         CU(cudaEventRecord(c->ev_join, c->aux_stream));
         if (t + 1 < steps)
-            EF(enqueue_topk_fast_sample(main_stream, V_dev, c->d, c->gi(), c->L.ld, c->n, c->d, c->k, B, &c->launches));
+            EF(enqueue_stream_sample<TC_DIFF>(main_stream, stream_args(V_dev, c->d, c->gi(), c->L.ld, 0.f, c->d, c->k, B), c->n, B.L, &c->launches));
     }
     CU(cudaStreamWaitEvent(main_stream, c->ev_join, 0));
     c->last_path = EF21_PATH_LAUNCHES;
@@ -1134,8 +1271,10 @@ ef21_status ef21_topk(const float* v_dev, int32_t batch, int64_t d, int32_t k, i
         return EF21_ERR_WORKSPACE;
     TopkBuffers B = topk_buffers(static_cast<char*>(workspace_dev), L);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-    if (B.fast)
-        return enqueue_topk_fast(st, v_dev, d, nullptr, 0, batch, d, k, idx_out_dev, val_out_dev, nullptr, 0, B, nullptr, nullptr);
+    TcShape S;
+    if (L.fast && !tc_shape(batch, d, S))
+        return enqueue_topk_stream<TC_PLAIN>(st, v_dev, d, nullptr, 0, 0.f, batch, d, k, StOut{idx_out_dev, val_out_dev, nullptr, 0, nullptr, 0, nullptr}, B,
+                                             nullptr, false);
     return enqueue_topk_general(st, v_dev, d, nullptr, 0, batch, d, k, idx_out_dev, val_out_dev, B, nullptr, nullptr);
 }
 

@@ -1,0 +1,404 @@
+// Exact Top-k of vectors that fit into the shared memory of one thread-block cluster: the whole selection in ONE
+// launch, one cluster of C blocks per vector.
+//
+//   1. block r holds the coordinates [r * slice, (r + 1) * slice) of v in shared memory (v is formed once, on the way in;
+//      kept as its bits rotated left by one, so that an unsigned compare orders magnitudes) and counts the leading 11 bits
+//      of the magnitude keys in a shared-memory histogram;
+//   2. the non-empty bins are added up in the block that owns the bin (distributed shared memory, 2048 / C bins per block),
+//      every block reads the sums and finds the bin that holds the k-th largest key (redundantly: the barrier that handing
+//      the result around would need costs more than the reading);
+//   3. every block lists its own keys of that bin; every block then reads all C lists and finds the k-th largest key T by
+//      counting (up to TC_RANKED keys) or by two more histograms over the list.  More than TC_LIST keys in the bin (ties,
+//      narrow ranges): the two histograms run over the vector instead;
+//   4. ordered compaction: the lists also tell how many entries above T (and equal to T) the warps and blocks before this
+//      one hold; ties at T are taken in index order.
+// The same kernel, with the vector left in global memory, is the exact fallback of the streaming path (topk_stream.cuh).
+//
+// What bounds it: latencies and issue slots, not bandwidth.  A block executes each piece of code once, a cluster barrier
+// takes about 1,000 cycles (measured; __syncthreads 40), and what all 32 warps of a block execute redundantly costs eight
+// times what eight of them would pay.  Hence two cluster barriers on the path, few and short code paths, searches by eight
+// warps.
+#pragma once
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+
+namespace ef21 {
+
+constexpr int TC_BITS = 11, TC_BINS = 1 << TC_BITS;      // digits of 11 + 11 + 9 bits
+constexpr int TC_LIST = 2048;               // keys of the deciding bin that are handled as a list
+constexpr int TC_RANKED = 256;              // up to this many of them are ranked by counting (two more histograms: +1.2 us)
+constexpr int TC_MAX_CLUSTER = 16;          // 16 needs the non-portable cluster size; used only where 8 blocks cannot hold the vector
+constexpr int TC_MAX_SLICE = 47104;         // floats per block (184 KB)
+
+// How v is formed: TC_PLAIN v = a; TC_DIFF v = a - b; TC_EF v = b + gamma * a, and b takes v (Algorithm 4: the error vector
+// becomes the vector to be compressed); TC_SENT v = b, which a TC_EF pass has already formed.
+enum { TC_PLAIN = 0, TC_DIFF = 1, TC_EF = 2, TC_SENT = 3 };
+
+struct TcArgs {
+    const float* a; i64 pitch_a;
+    float* b; i64 pitch_b;                  // TC_EF: updated in place
+    int d, k, slice;
+    float gamma;
+    int* idx_out; float* val_out;
+    float* apply; i64 pitch_apply;          // TC_DIFF: receives b + v on the selected coordinates; TC_EF, TC_SENT: v - v there; may be null
+    unsigned* status;
+    unsigned* slow_count;                   // counts the vectors with more than TC_LIST entries equal to T; may be null
+    // STREAM only: vectors whose flag (one word every flag_pitch words) is zero are left alone; tile_off (may be null):
+    // [batch][ntiles + 1] first message position of every `tile` coordinates
+    const unsigned* flag; int flag_pitch, batch;
+    int* tile_off; int ntiles, tile;
+};
+
+__host__ __device__ constexpr size_t tc_smem_bytes(int C, int slice) {
+    return (size_t)slice * 4 + (size_t)TC_LIST * 5 + (size_t)TC_BINS * 4 + (C > 1 ? (size_t)(TC_LIST + TC_BINS) * 4 : 0);
+}
+
+// Bin of the histogram (bin 0 not counted in it) that holds the need-th largest of `population` entries: found[] = bin,
+// entries in higher bins, entries in the bin.  All threads call it; the first 256 search, eight bins each.
+__device__ __noinline__ void tc_find_bin(const unsigned* hist, unsigned need, unsigned population, unsigned* wsum, unsigned* found) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (warp < 8) {
+        // thread t owns the bins [2040 - 8 t, 2048 - 8 t), highest first
+        const uint4 hi = reinterpret_cast<const uint4*>(hist)[2 * (255 - tid) + 1], lo = reinterpret_cast<const uint4*>(hist)[2 * (255 - tid)];
+        const unsigned c[8] = {hi.w, hi.z, hi.y, hi.x, lo.w, lo.z, lo.y, lo.x};
+        unsigned sum = 0u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) sum += c[q];
+        const unsigned wtot = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0) wsum[warp] = wtot;
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        unsigned before = 0u, total = 0u;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) { const unsigned t = wsum[w]; if (w < warp) before += t; total += t; }
+        if (before < need && need <= before + wtot) {                // one warp
+            unsigned up = before + warp_incl_scan(sum) - sum;
+            if (up < need && need <= up + sum) {                     // one lane
+                bool open = true;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (open && need <= up + c[q]) { found[0] = (unsigned)(2047 - (8 * tid + q)); found[1] = up; found[2] = c[q]; open = false; }
+                    up += c[q];
+                }
+            }
+        } else if (need > total && tid == 0) {
+            found[0] = 0u; found[1] = total; found[2] = population - total;
+        }
+    }
+    __syncthreads();
+}
+
+// STREAM: the vector is longer than the cluster's shared memory; it stays in global memory and every sweep reads it again.
+template <int MODE, int C, int THREADS, bool STREAM>
+__device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
+    namespace cg = cooperative_groups;
+    constexpr int WARPS = THREADS / 32;
+    extern __shared__ __align__(16) unsigned char tc_smem[];
+    unsigned* ws = reinterpret_cast<unsigned*>(tc_smem);            // [slice] bits of v rotated left by one
+    unsigned* hist = ws + (STREAM ? 0 : p.slice);                   // [TC_BINS] this block's histogram
+    unsigned* list = hist + TC_BINS;                                // [TC_LIST] this block's keys of the deciding bin
+    unsigned* all = C > 1 ? list + TC_LIST : list;                  // [TC_LIST] the lists of all blocks
+    unsigned* hsum = C > 1 ? all + TC_LIST : hist;                  // [TC_BINS] the cluster's histogram (own bins first, then all)
+    unsigned char* lwarp = reinterpret_cast<unsigned char*>(C > 1 ? hsum + TC_BINS : all + TC_LIST);    // [TC_LIST] warp of a listed key
+    __shared__ unsigned list_n, above_n;                            // this block: keys in its list, entries in higher bins
+    __shared__ unsigned found[3], result[2], before_sh[2];
+    __shared__ unsigned wsum[8], wgt[WARPS], weq[WARPS];
+
+    __shared__ uint2 blk_counts;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = C > 1 ? (int)cluster.block_rank() : 0;
+    auto sync_all = [&]() { if (C > 1) cluster.sync(); else __syncthreads(); };
+
+    const int j0 = (int)min((i64)rank * p.slice, (i64)p.d), len = min(p.slice, p.d - j0);
+    const float* __restrict__ av = p.a + (i64)vec * p.pitch_a + j0;
+    float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + j0;
+#pragma unroll 1
+    for (int q = tid; q < TC_BINS; q += THREADS) { hist[q] = 0u; if (C > 1) hsum[q] = 0u; }
+    for (int j = len + tid; !STREAM && j < p.slice && j < len + 128; j += THREADS) ws[j] = 0u;       // the tail of the last tile
+    if (tid < WARPS) { wgt[tid] = 0u; weq[tid] = 0u; }
+    if (tid == 0) { list_n = 0u; above_n = 0u; before_sh[0] = 0u; before_sh[1] = 0u; result[0] = 0xffffffffu; }
+    __syncthreads();
+    if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // hsum is empty
+    if (!STREAM) { pdl_trigger(); pdl_wait(); }
+    // entries of bin 0 (zeros and the smallest magnitudes) are not counted: what the other bins leave over is theirs
+    auto take = [&](int j, float a, float b) {
+        float v = a;
+        if (MODE == TC_DIFF) v = __fsub_rn(a, b);
+        if (MODE == TC_EF) { v = __fadd_rn(b, __fmul_rn(p.gamma, a)); bv[j] = v; }
+        if (MODE == TC_SENT) v = b;
+        const unsigned w = __funnelshift_l(__float_as_uint(v), __float_as_uint(v), 1);
+        if (!STREAM) ws[j] = w;
+        if (w >> 21) atomicAdd(&hist[w >> 21], 1u);
+    };
+    {
+        constexpr int U = THREADS == 1024 ? 8 : 4;
+        int j = tid;
+#pragma unroll 1
+        for (; j + (U - 1) * THREADS < len; j += U * THREADS) {
+            float a[U], b[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) { a[u] = MODE == TC_SENT ? 0.f : av[j + u * THREADS]; b[u] = MODE == TC_PLAIN ? 0.f : bv[j + u * THREADS]; }
+#pragma unroll
+            for (int u = 0; u < U; ++u) take(j + u * THREADS, a[u], b[u]);
+        }
+#pragma unroll 1
+        for (; j < len; j += THREADS) take(j, MODE == TC_SENT ? 0.f : av[j], MODE == TC_PLAIN ? 0.f : bv[j]);
+    }
+    constexpr int OWN = TC_BINS / C;                                // bins summed by one block
+    auto sum_histograms = [&]() {                                   // hist of all blocks -> hsum
+        __syncthreads();
+        if (C > 1) {
+            // hsum of every block is empty here
+#pragma unroll 1
+            for (int q = tid; q < TC_BINS; q += THREADS) {
+                const unsigned c = hist[q];
+                if (c) atomicAdd(cluster.map_shared_rank(hsum, q / OWN) + q, c);
+            }
+            cluster.sync();
+#pragma unroll 1
+            for (int q = tid; q < TC_BINS; q += THREADS)            // hist becomes the cluster's histogram
+                hist[q] = cluster.map_shared_rank(hsum, q / OWN)[q];
+            __syncthreads();
+        }
+    };
+    if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    sum_histograms();
+    tc_find_bin(hist, (unsigned)p.k, (unsigned)p.d, wsum, found);
+    const unsigned bin0 = found[0], pop0 = found[2];
+    unsigned need = (unsigned)p.k - found[1];
+    const bool listed = pop0 <= (unsigned)TC_LIST;
+    // the word(s) of an entry (of four consecutive ones) again, zero behind the end
+    auto word = [&](int j) {
+        if (!STREAM) return ws[j];
+        if (j >= len) return 0u;
+        const float v = MODE == TC_SENT ? bv[j] : (MODE == TC_DIFF ? __fsub_rn(av[j], bv[j]) : av[j]);
+        return __funnelshift_l(__float_as_uint(v), __float_as_uint(v), 1);
+    };
+    auto word4 = [&](int j) {
+        if (!STREAM) return reinterpret_cast<const uint4*>(ws)[j >> 2];
+        return make_uint4(word(j), word(j + 1), word(j + 2), word(j + 3));
+    };
+    // warp w owns the entries [w * chunk, (w + 1) * chunk) of the slice, in tiles of 128, four consecutive ones per lane
+    const int chunk = ((len + WARPS - 1) / WARPS + 127) & ~127;
+    const int w0 = min(warp * chunk, len), w1 = min(w0 + chunk, len);
+    auto valid4 = [&](int j) { return j + 3 < w1 ? 15u : (j < w1 ? (1u << (w1 - j)) - 1u : 0u); };
+    unsigned T, need_ties;
+    unsigned gt_before = 0u, eq_before = 0u;                        // in the blocks before this one
+    if (listed) {
+        unsigned above = 0u;
+        const unsigned lo = bin0 << 21;
+#pragma unroll 1
+        for (int base = w0; base < w1; base += 128) {
+            const int j = base + 4 * lane;
+            const uint4 w = word4(j);
+            unsigned hit = 0u;
+            // (w - lo) < 2^21: in the bin; beyond that and not below lo: above it
+            const unsigned o[4] = {w.x - lo, w.y - lo, w.z - lo, w.w - lo};
+            hit = (o[0] < (1u << 21) ? 1u : 0u) | (o[1] < (1u << 21) ? 2u : 0u) | (o[2] < (1u << 21) ? 4u : 0u) | (o[3] < (1u << 21) ? 8u : 0u);
+            above += (w.x >= lo ? 1u : 0u) + (w.y >= lo ? 1u : 0u) + (w.z >= lo ? 1u : 0u) + (w.w >= lo ? 1u : 0u);
+            if (lo == 0u || hit) {
+                const unsigned ok = valid4(j);                      // zeros behind the end belong to no bin
+                if (lo == 0u) above -= 4u - (unsigned)__popc(ok);
+                hit &= ok;
+                above -= (unsigned)__popc(hit);
+                while (hit != 0u) {
+                    const int e = __ffs((int)hit) - 1;
+                    hit &= hit - 1u;
+                    const unsigned at = atomicAdd(&list_n, 1u);
+                    list[at] = word(j + e) >> 1;
+                    lwarp[at] = (unsigned char)warp;
+                }
+            }
+        }
+        above = __reduce_add_sync(0xffffffffu, above);
+        if (lane == 0) {
+            if (above) atomicAdd(&wgt[warp], above);
+            if (C > 1 && above) atomicAdd(&above_n, above);
+        }
+        sync_all();
+        unsigned first = 0u;                                        // where this block's keys start in `all`
+        if (C > 1) {
+            unsigned n_of[C], ab[C];
+#pragma unroll
+            for (int r = 0; r < C; ++r) { n_of[r] = *cluster.map_shared_rank(&list_n, r); ab[r] = *cluster.map_shared_rank(&above_n, r); }
+#pragma unroll
+            for (int r = 0; r < C; ++r) if (r < rank) { first += n_of[r]; gt_before += ab[r]; }
+#pragma unroll 1
+            for (unsigned e = tid; e < pop0; e += THREADS) {
+                unsigned off = e; int from = 0;
+#pragma unroll
+                for (int r = 0; r < C - 1; ++r) if (from == r && off >= n_of[r]) { off -= n_of[r]; from = r + 1; }
+                all[e] = cluster.map_shared_rank(list, from)[off];
+            }
+        }
+        if (tid < 4 && pop0 + tid < (unsigned)TC_LIST) all[pop0 + tid] = 0u;        // read in groups of four below
+        __syncthreads();
+        if (pop0 <= (unsigned)TC_RANKED) {
+            // one key per thread: T is the smallest key that fewer than `need` keys exceed
+            const bool have = tid < (int)pop0;
+            const unsigned mine = have ? all[tid] : 0u;
+            unsigned gt = 0u;
+            if (have) {
+#pragma unroll 2
+                for (unsigned o = 0; o < (pop0 + 3u) >> 2; ++o) {
+                    const uint4 x = reinterpret_cast<const uint4*>(all)[o];
+                    gt += x.x > mine ? 1u : 0u; gt += x.y > mine ? 1u : 0u; gt += x.z > mine ? 1u : 0u; gt += x.w > mine ? 1u : 0u;
+                }
+                if (gt < need) atomicMin(&result[0], mine);
+            }
+            __syncthreads();
+            T = result[0];
+            if (have && mine == T) result[1] = need - gt;
+            __syncthreads();
+            need_ties = result[1];
+        } else {
+            unsigned prefix = bin0, pop = pop0;
+#pragma unroll 1
+            for (int shift = 9; shift >= 0; shift -= 9) {           // bits 19..9, then 8..0
+#pragma unroll 1
+                for (int q = tid; q < TC_BINS; q += THREADS) hist[q] = 0u;
+                __syncthreads();
+                const int up = shift == 9 ? 20 : 9;
+                const unsigned mask = shift == 9 ? 2047u : 511u;
+#pragma unroll 1
+                for (unsigned e = tid; e < pop0; e += THREADS) {
+                    const unsigned key = all[e], bin = (key >> shift) & mask;
+                    if ((key >> up) == prefix && bin) atomicAdd(&hist[bin], 1u);
+                }
+                __syncthreads();
+                tc_find_bin(hist, need, pop, wsum, found);
+                prefix = (prefix << (shift == 9 ? 11 : 9)) | found[0]; need -= found[1]; pop = found[2];
+            }
+            T = prefix; need_ties = need;
+        }
+        // listed keys above and at T: this block's by warp, those of the blocks before it in total
+        const unsigned mine_n = C > 1 ? list_n : pop0;
+#pragma unroll 1
+        for (unsigned e = tid; e < mine_n; e += THREADS) {
+            const unsigned key = list[e];
+            if (key > T) atomicAdd(&wgt[lwarp[e]], 1u);
+            else if (key == T) atomicAdd(&weq[lwarp[e]], 1u);
+        }
+        if (C > 1) {
+#pragma unroll 1
+            for (unsigned e = tid; e < first; e += THREADS) {
+                const unsigned key = all[e];
+                if (key >= T) atomicAdd(&before_sh[key == T ? 1 : 0], 1u);
+            }
+        }
+        __syncthreads();
+        if (C > 1) { gt_before += before_sh[0]; eq_before += before_sh[1]; }
+    } else {
+        unsigned prefix = bin0, pop = pop0;
+#pragma unroll 1
+        for (int shift = 9; shift >= 0; shift -= 9) {
+            sync_all();                                             // everybody has read the histograms
+#pragma unroll 1
+            for (int q = tid; q < TC_BINS; q += THREADS) { hist[q] = 0u; if (C > 1) hsum[q] = 0u; }
+            sync_all();
+            const int up = shift == 9 ? 20 : 9;
+            const unsigned mask = shift == 9 ? 2047u : 511u;
+#pragma unroll 1
+            for (int j = tid; j < len; j += THREADS) {
+                const unsigned key = word(j) >> 1, bin = (key >> shift) & mask;
+                if ((key >> up) == prefix && bin) atomicAdd(&hist[bin], 1u);
+            }
+            sum_histograms();
+            tc_find_bin(hist, need, pop, wsum, found);
+            prefix = (prefix << (shift == 9 ? 11 : 9)) | found[0]; need -= found[1]; pop = found[2];
+        }
+        T = prefix; need_ties = need;
+        if (rank == 0 && tid == 0 && p.slow_count && pop > (unsigned)TC_LIST) atomicAdd(p.slow_count, 1u);
+        unsigned gt = 0u, eq = 0u;
+#pragma unroll 1
+        for (int j = w0 + lane; j < w1; j += 32) { const unsigned key = word(j) >> 1; gt += key > T ? 1u : 0u; eq += key == T ? 1u : 0u; }
+        gt = __reduce_add_sync(0xffffffffu, gt); eq = __reduce_add_sync(0xffffffffu, eq);
+        if (lane == 0) { wgt[warp] = gt; weq[warp] = eq; }
+        __syncthreads();
+        // the counts of the blocks before this one have to be handed around
+        if (C > 1) {
+            const unsigned bg = __reduce_add_sync(0xffffffffu, lane < WARPS ? wgt[lane] : 0u);
+            const unsigned be = __reduce_add_sync(0xffffffffu, lane < WARPS ? weq[lane] : 0u);
+            if (tid == 0) blk_counts = make_uint2(bg, be);
+            sync_all();
+            for (int r = 0; r < rank; ++r) { const uint2 o = *cluster.map_shared_rank(&blk_counts, r); gt_before += o.x; eq_before += o.y; }
+        }
+    }
+    if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");     // done with the other blocks' memory
+
+    // ordered compaction
+    if (wgt[warp] + weq[warp] != 0u) {
+        gt_before += __reduce_add_sync(0xffffffffu, lane < warp ? wgt[lane] : 0u);
+        eq_before += __reduce_add_sync(0xffffffffu, lane < warp ? weq[lane] : 0u);
+        int* __restrict__ io = p.idx_out + (i64)vec * p.k;
+        float* __restrict__ vo = p.val_out + (i64)vec * p.k;
+        float* app = (MODE != TC_PLAIN && p.apply) ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
+        const unsigned lo = T << 1;
+#pragma unroll 1
+        for (int base = w0; base < w1; base += 128) {
+            const int j = base + 4 * lane;
+            const uint4 w = word4(j);
+            if (!__any_sync(0xffffffffu, max(max(w.x, w.y), max(w.z, w.w)) >= lo)) continue;
+            unsigned m = (w.x >= lo ? 1u : 0u) | (w.y >= lo ? 2u : 0u) | (w.z >= lo ? 4u : 0u) | (w.w >= lo ? 8u : 0u);
+            m &= valid4(j);
+            unsigned ties = ((w.x >> 1) == T ? 1u : 0u) | ((w.y >> 1) == T ? 2u : 0u) | ((w.z >> 1) == T ? 4u : 0u) | ((w.w >> 1) == T ? 8u : 0u);
+            ties &= m;
+            // entries above T (low half) and at T (high half) in lower lanes
+            const unsigned mine = (unsigned)__popc(m & ~ties) | ((unsigned)__popc(ties) << 16);
+            const unsigned incl = warp_incl_scan(mine), excl = incl - mine;
+            const unsigned tile = __shfl_sync(0xffffffffu, incl, 31);
+            unsigned g0 = gt_before + (excl & 0xffffu), e0 = eq_before + (excl >> 16);
+            while (m != 0u) {
+                const int e = __ffs((int)m) - 1;
+                m &= m - 1u;
+                const bool tie = (ties >> e) & 1u;
+                if (!tie || e0 < need_ties) {
+                    const unsigned wv = word(j + e);
+                    const float v = __uint_as_float(__funnelshift_r(wv, wv, 1));
+                    const unsigned pos = g0 + min(e0, need_ties);
+                    io[pos] = j0 + j + e; vo[pos] = v;
+                    flag_nonfinite(p.status, v);
+                    if (app) app[j + e] = MODE == TC_DIFF ? __fadd_rn(app[j + e], v) : __fsub_rn(v, v);
+                }
+                g0 += tie ? 0u : 1u; e0 += tie ? 1u : 0u;
+            }
+            gt_before += tile & 0xffffu; eq_before += tile >> 16;
+        }
+    }
+    if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (STREAM && p.tile_off) {
+        cluster.sync();                                              // the message is complete and visible to the cluster
+        int* off = p.tile_off + (i64)vec * (p.ntiles + 1);
+        const int* io = p.idx_out + (i64)vec * p.k;
+        for (int b = rank * THREADS + tid; b <= p.ntiles; b += C * THREADS) {
+            const i64 bound = (i64)b * p.tile;
+            int lo = 0, hi = p.k;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if ((i64)__ldcg(&io[mid]) < bound) lo = mid + 1; else hi = mid;
+            }
+            off[b] = lo;
+        }
+    }
+}
+
+template <int MODE, int C, int THREADS, bool STREAM = false>
+__global__ void __launch_bounds__(THREADS)
+tc_topk_kernel(const __grid_constant__ TcArgs p) {
+    if (STREAM) {
+        // a few clusters look through the flags: as a rule there is nothing to do
+        pdl_trigger();
+        pdl_wait();
+        for (int vec = (int)(blockIdx.x / (unsigned)C); vec < p.batch; vec += (int)(gridDim.x / (unsigned)C))
+            if (p.flag[(i64)vec * p.flag_pitch] != 0u) {
+                tc_vector<MODE, C, THREADS, STREAM>(p, vec);
+                cooperative_groups::this_cluster().sync();
+            }
+    } else {
+        tc_vector<MODE, C, THREADS, STREAM>(p, (int)(blockIdx.x / (unsigned)C));
+    }
+}
+
+}  // namespace ef21
