@@ -327,7 +327,7 @@ int32_t ef21_get_persistent_body(const ef21_ctx* ctx);
 ef21_status ef21_set_path(ef21_ctx* ctx, int32_t path);
 /* The path the last ef21_step / ef21_step_grads actually used (EF21_PATH_*), 0 if none yet. */
 int32_t ef21_last_path(const ef21_ctx* ctx);
-/* Kernel launches enqueued by this handle since creation (copies are not counted). */
+/* Kernel launches enqueued by this handle since creation (host copies are not counted). */
 int64_t ef21_launch_count(const ef21_ctx* ctx);
 
 #ifdef __cplusplus

@@ -15,6 +15,8 @@ constexpr int AGG_BLOCK = 256;
 // g_i[idx] += val for all n*k message entries (indices within a worker are distinct).
 __global__ void apply_messages_kernel(const int* __restrict__ idx, const float* __restrict__ val,
                                       i64 total, int k, i64 ld, float* __restrict__ gi) {
+    pdl_trigger();
+    pdl_wait(idx, val, gi);
     const i64 e = blockIdx.x * (i64)blockDim.x + threadIdx.x;
     if (e >= total) return;
     const i64 i = e / k;
@@ -29,6 +31,8 @@ __global__ void apply_messages_kernel(const int* __restrict__ idx, const float* 
 __global__ void randk_select_kernel(const float* __restrict__ a, i64 pitch_a, float* __restrict__ gi, i64 ld,
                                     const int* __restrict__ sets, i64 total, int k, i64 d,
                                     int* __restrict__ idx_out, float* __restrict__ val_out, unsigned* status) {
+    pdl_trigger();
+    pdl_wait(a, gi, sets, idx_out, val_out, status);
     const i64 e = blockIdx.x * (i64)blockDim.x + threadIdx.x;
     if (e >= total) return;
     const i64 i = e / k;
@@ -47,6 +51,8 @@ __global__ void randk_select_kernel(const float* __restrict__ a, i64 pitch_a, fl
 // for b = 0 .. ntiles (so tile b owns entries [off[i][b], off[i][b+1])).
 __global__ void agg_offsets_kernel(const int* __restrict__ idx, int n, int k, int ntiles,
                                    int* __restrict__ off) {
+    pdl_trigger();
+    pdl_wait(idx, off);
     const i64 e = blockIdx.x * (i64)blockDim.x + threadIdx.x;
     const i64 total = (i64)n * (ntiles + 1);
     if (e >= total) return;
@@ -62,13 +68,18 @@ __global__ void agg_offsets_kernel(const int* __restrict__ idx, int n, int k, in
     off[e] = lo;
 }
 
-// One block per tile of AGG_TILE coordinates.  UPDATE_X: also perform x <- fma(-gamma, g_old, x)
-// on the tile before g changes (Algorithm 2 updates x from g^t, then g^{t+1} from the messages).
-template <bool UPDATE_X>
+// What an aggregation does to x besides: nothing; x <- fma(-gamma, g^t, x) before g changes (Algorithm 2 updates x from g^t, then
+// g^{t+1} from the messages); or the x update of the following iteration, from the new g.
+enum { AGG_X_KEEP = 0, AGG_X_BEFORE = 1, AGG_X_AFTER = 2 };
+
+// One block per tile of AGG_TILE coordinates.
+template <int XMODE>
 __global__ void __launch_bounds__(AGG_BLOCK)
 aggregate_kernel(const int* __restrict__ idx, const float* __restrict__ val, const int* __restrict__ off,
                  int n, int k, int ntiles, i64 d, float inv_n, float gamma,
                  float* __restrict__ g, float* __restrict__ x) {
+    pdl_trigger();
+    pdl_wait(idx, val, off, g, x);
     __shared__ float s[AGG_TILE];
     __shared__ unsigned char touched[AGG_TILE];
     const int b = blockIdx.x;
@@ -87,13 +98,10 @@ aggregate_kernel(const int* __restrict__ idx, const float* __restrict__ val, con
     for (int t = threadIdx.x; t < AGG_TILE; t += AGG_BLOCK) {
         const i64 j = j0 + t;
         if (j >= d) break;
-        if (UPDATE_X) {
-            const float gj = g[j];
-            x[j] = fmaf(-gamma, gj, x[j]);
-            if (touched[t]) g[j] = __fadd_rn(gj, __fmul_rn(s[t], inv_n));
-        } else if (touched[t]) {
-            g[j] = __fadd_rn(g[j], __fmul_rn(s[t], inv_n));
-        }
+        if (XMODE == AGG_X_KEEP && !touched[t]) continue;
+        const float old = g[j], now = touched[t] ? __fadd_rn(old, __fmul_rn(s[t], inv_n)) : old;
+        if (XMODE != AGG_X_KEEP) x[j] = fmaf(-gamma, XMODE == AGG_X_BEFORE ? old : now, x[j]);
+        if (touched[t]) g[j] = now;
     }
 }
 
@@ -104,11 +112,13 @@ constexpr int AGG_STAGE_MAX_N = 1024;
 constexpr int AGG_STAGE_CAP = 3072;
 constexpr int AGG_OWNER_SCAN_MAX = 512;   // tiles with at most this many entries skip the per-worker loop
 
-template <bool UPDATE_X>
+template <int XMODE>
 __global__ void __launch_bounds__(AGG_BLOCK)
 aggregate_staged_kernel(const int* __restrict__ idx, const float* __restrict__ val, const int* __restrict__ off,
                         int n, int k, int ntiles, i64 d, float inv_n, float gamma,
                         float* __restrict__ g, float* __restrict__ x) {
+    pdl_trigger();
+    pdl_wait(idx, val, off, g, x);
     __shared__ float s[AGG_TILE];
     __shared__ __align__(4) unsigned short touched[AGG_TILE];   // staged entries per coordinate
     __shared__ int w_start[AGG_STAGE_MAX_N + 1];
@@ -209,21 +219,75 @@ aggregate_staged_kernel(const int* __restrict__ idx, const float* __restrict__ v
         const int t = u * AGG_BLOCK + threadIdx.x;
         const i64 j = j0 + t;
         gv[u] = 0.f; xv[u] = 0.f;
-        if (j < d && (UPDATE_X || touched[t])) gv[u] = g[j];
-        if (UPDATE_X && j < d) xv[u] = x[j];
+        if (j < d && (XMODE != AGG_X_KEEP || touched[t])) gv[u] = g[j];
+        if (XMODE != AGG_X_KEEP && j < d) xv[u] = x[j];
     }
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
         const int t = u * AGG_BLOCK + threadIdx.x;
         const i64 j = j0 + t;
         if (j >= d) continue;
-        if (UPDATE_X) x[j] = fmaf(-gamma, gv[u], xv[u]);
-        if (touched[t]) g[j] = __fadd_rn(gv[u], __fmul_rn(s[t], inv_n));
+        const float now = touched[t] ? __fadd_rn(gv[u], __fmul_rn(s[t], inv_n)) : gv[u];
+        if (XMODE != AGG_X_KEEP) x[j] = fmaf(-gamma, XMODE == AGG_X_BEFORE ? gv[u] : now, xv[u]);
+        if (touched[t]) g[j] = now;
     }
+}
+
+// Short vectors: a block of AGG_TABLE_COLS coordinates scatters the messages that fall on them into a table [n][columns] in shared
+// memory and every thread adds up its column, workers ascending.  No tile offsets are needed, and the ordered sum is one
+// read per worker (20 workers, d = 5,001, Top-50: 3 us against 4 + 19 us for the offsets and the staged kernel).  Every block
+// goes through all n * k messages, hence only for few of them.
+constexpr int AGG_TABLE_COLS = 128;
+constexpr i64 AGG_TABLE_MAX_D = 16384, AGG_TABLE_MAX_MESSAGES = 65536;
+constexpr int AGG_TABLE_MAX_N = 400;                       // 200 KB of shared memory
+constexpr unsigned AGG_NO_ENTRY = 0xffffffffu;             // cell without a message (a NaN pattern no finite value has)
+
+template <int XMODE>
+__global__ void __launch_bounds__(AGG_BLOCK)
+aggregate_table_kernel(const int* __restrict__ idx, const float* __restrict__ val, int n, int k, int d, float inv_n, float gamma,
+                       float* __restrict__ g, float* __restrict__ x) {
+    extern __shared__ __align__(16) unsigned agg_table[];                 // [n][AGG_TABLE_COLS]
+    for (int e = threadIdx.x; e < n * (AGG_TABLE_COLS / 4); e += AGG_BLOCK)
+        reinterpret_cast<uint4*>(agg_table)[e] = make_uint4(AGG_NO_ENTRY, AGG_NO_ENTRY, AGG_NO_ENTRY, AGG_NO_ENTRY);
+    __syncthreads();
+    pdl_trigger();
+    pdl_wait(idx, val, g, x);
+    const int j0 = blockIdx.x * AGG_TABLE_COLS, total = n * k;
+    const unsigned magic = (unsigned)(((1ull << 32) + (unsigned)k - 1u) / (unsigned)k);      // e / k for e < 65,536: one high product
+    constexpr int U = 4;
+#pragma unroll 1
+    for (int e0 = threadIdx.x; e0 < total; e0 += U * AGG_BLOCK) {
+        int c[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) { const int e = e0 + u * AGG_BLOCK; c[u] = e < total ? idx[e] - j0 : -1; }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if ((unsigned)c[u] < (unsigned)AGG_TABLE_COLS) {
+                const int e = e0 + u * AGG_BLOCK;
+                const unsigned i = k == 1 ? (unsigned)e : __umulhi((unsigned)e, magic);
+                agg_table[i * AGG_TABLE_COLS + c[u]] = __float_as_uint(val[e]);
+            }
+    }
+    __syncthreads();
+    const int t = threadIdx.x, j = j0 + t;
+    if (t >= AGG_TABLE_COLS || j >= d) return;
+    const float old = g[j], xj = XMODE == AGG_X_KEEP ? 0.f : x[j];
+    float s = 0.f; bool hit = false;
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) {
+        const unsigned w = agg_table[i * AGG_TABLE_COLS + t];
+        const float sum = __fadd_rn(s, __uint_as_float(w));
+        if (w != AGG_NO_ENTRY) { s = sum; hit = true; }
+    }
+    const float now = hit ? __fadd_rn(old, __fmul_rn(s, inv_n)) : old;
+    if (XMODE != AGG_X_KEEP) x[j] = fmaf(-gamma, XMODE == AGG_X_BEFORE ? old : now, xj);
+    if (hit) g[j] = now;
 }
 
 // x <- fma(-gamma, g, x), elementwise.
 __global__ void x_update_kernel(const float* __restrict__ g, float* __restrict__ x, i64 d, float gamma) {
+    pdl_trigger();
+    pdl_wait(g, x);
     for (i64 j = blockIdx.x * (i64)blockDim.x + threadIdx.x; j < d; j += (i64)gridDim.x * blockDim.x)
         x[j] = fmaf(-gamma, g[j], x[j]);
 }
@@ -232,6 +296,8 @@ __global__ void x_update_kernel(const float* __restrict__ g, float* __restrict__
 // round applied to zero state.
 __global__ void dense_init_kernel(const float* __restrict__ V, i64 pitch_v, int n, i64 d, i64 ld,
                                   float inv_n, float* __restrict__ gi, float* __restrict__ g) {
+    pdl_trigger();
+    pdl_wait(V, gi, g);
     for (i64 j = blockIdx.x * (i64)blockDim.x + threadIdx.x; j < d; j += (i64)gridDim.x * blockDim.x) {
         float s = 0.f;
         for (int i = 0; i < n; ++i) {

@@ -12,7 +12,15 @@ typedef long long i64;
 // dependent it starts after 0.5 us.  Every kernel of the library calls pdl_wait() before it touches global memory (it
 // returns when the preceding kernels of the stream have completed and their writes are visible) and pdl_trigger() early,
 // so that the kernel behind it can be placed on the device meanwhile.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The kernel's pointers go through pdl_wait so that no load through them -- a read-only one (const __restrict__) is otherwise
+// free to move -- is placed in front of the wait.
+template <typename T>
+__device__ __forceinline__ void pdl_fresh(T& p) { asm volatile("" : "+l"(p)); }
+template <typename... P>
+__device__ __forceinline__ void pdl_wait(P&... pointers) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (pdl_fresh(pointers), ...);
+}
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Status word layout in the workspace (one 256-byte slot): word 0 = first error code seen.

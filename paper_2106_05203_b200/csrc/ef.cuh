@@ -13,6 +13,8 @@ namespace ef21 {
 // e_i <- e_i + gamma * grad_i, all n rows (grad has leading dimension pitch, e has ld).
 __global__ void ef_compose_kernel(const float* __restrict__ grad, i64 pitch, float* __restrict__ e, i64 ld,
                                   int n, i64 d, float gamma) {
+    pdl_trigger();
+    pdl_wait(grad, e);
     const i64 total = (i64)n * d;
     for (i64 t = blockIdx.x * (i64)blockDim.x + threadIdx.x; t < total; t += (i64)gridDim.x * blockDim.x) {
         const i64 i = t / d, j = t - i * d;
@@ -24,6 +26,8 @@ __global__ void ef_compose_kernel(const float* __restrict__ grad, i64 pitch, flo
 // e_i[idx] <- p_i[idx] - w_i[idx] on the n*k sent coordinates (the others keep p_i - 0 = p_i).
 __global__ void ef_subtract_sent_kernel(const int* __restrict__ idx, const float* __restrict__ val, i64 total, int k,
                                         i64 ld, float* __restrict__ e) {
+    pdl_trigger();
+    pdl_wait(idx, val, e);
     const i64 t = blockIdx.x * (i64)blockDim.x + threadIdx.x;
     if (t >= total) return;
     const i64 i = t / k;

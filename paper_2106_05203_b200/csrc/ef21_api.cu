@@ -12,6 +12,7 @@
 
 #include "apply.cuh"
 #include "common.cuh"
+#include "copy.cuh"
 #include "ef.cuh"
 #include "grad.cuh"
 #include "persistent.cuh"
@@ -172,7 +173,7 @@ struct Layout {
     int tile_rows;     // rows per gradient tile
     i64 max_tiles;     // capacity of the gradient tile table
     size_t status, x, g, gi, msg_idx, msg_val, topk, agg_off, eval_out, slots;
-    size_t msg2_idx, msg2_val, plus_old, plus_choice, plus_bitmap;    // EF21+ (Algorithm 3)
+    size_t msg2_idx, msg2_val, plus_cuts, plus_choice, plus_parts;    // EF21+ (Algorithm 3)
     size_t A, y, row_off, tile_begin, tiles, partial, loss_partial, grad, mb_tile_begin, mb_tiles;
     size_t total;
     TopkLayout tk;
@@ -197,9 +198,9 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.slots = take((size_t)2 * n * k * 8);
     L.msg2_idx = take((size_t)n * k * 4);
     L.msg2_val = take((size_t)n * k * 4);
-    L.plus_old = take((size_t)n * k * 4);
+    L.plus_cuts = take((size_t)2 * n * 8);
     L.plus_choice = take((size_t)n * 4);
-    L.plus_bitmap = take((size_t)n * ((d + 31) / 32) * 4);
+    L.plus_parts = take((size_t)n * PLUS_MAX_PARTS * sizeof(double2));
     L.tile_rows = 0; L.max_tiles = 0;
     L.A = L.y = L.row_off = L.tile_begin = L.tiles = L.partial = L.loss_partial = L.grad = L.mb_tile_begin = L.mb_tiles = 0;
     if (N > 0) {
@@ -245,7 +246,6 @@ struct ef21_ctx {
     int num_tiles;
     int path, last_path;
     bool agg_off_ready;                 // the last selection already wrote the aggregation's tile offsets
-    bool agg_off_static;                // one tile only: the offsets are (0, k) whatever the messages; written once
     int pk_cluster, pk_rb, pk_src, pk_threads;      // forced persistent-kernel shape (0 / -1 = automatic)
     int pk_used_cluster, pk_used_rb, pk_used_src, pk_used_threads;
     PersistPlan plan; bool plan_valid;  // cached plan of ef21_step's persistent launch
@@ -281,6 +281,28 @@ struct ef21_ctx {
 };
 
 namespace {
+
+// Several copies or clears as one launch; null destinations are left out, contiguous rows become one.
+struct Copies {
+    CopyArgs p;
+    i64 blocks = 0;
+    Copies() { p.count = 0; }
+    void add(void* dst, i64 dpitch, const void* src, i64 spitch, i64 width, i64 rows) {
+        if (!dst || width <= 0 || rows <= 0) return;
+        if (dpitch == width && (!src || spitch == width)) { width *= rows; dpitch = spitch = width; rows = 1; }
+        CopySeg& c = p.seg[p.count++];
+        c.dst = static_cast<unsigned*>(dst); c.src = static_cast<const unsigned*>(src);
+        c.dpitch = dpitch; c.spitch = spitch; c.width = width; c.rows = rows;
+        c.units = rows * ceil_div(width, COPY_UNIT);
+        blocks += c.units;
+    }
+    ef21_status run(cudaStream_t st, i64* launches) {
+        if (blocks == 0) return EF21_OK;
+        CU(launch(copy_segments_kernel, dim3((unsigned)blocks), COPY_THREADS, 0, st, 1, p));
+        *launches += 1;
+        return EF21_OK;
+    }
+};
 
 struct TopkBuffers {
     TkState* state; unsigned* hist; uint2* chunks; int nchunks;
@@ -334,14 +356,14 @@ TcKernel tc_lookup(const TcShape& S) {
 
 ef21_status enqueue_topk_cluster(cudaStream_t st, int mode, const TcShape& S, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
                                  float gamma, int batch, i64 d, int k, int* idx_out, float* val_out, float* apply, i64 pitch_apply,
-                                 i64* launches, unsigned* status, unsigned* slow_count = nullptr) {
+                                 i64* launches, unsigned* status, unsigned* slow_count = nullptr, unsigned long long* cut_out = nullptr) {
     const TcKernel kern = mode == TC_PLAIN ? tc_lookup<TC_PLAIN>(S) : (mode == TC_DIFF ? tc_lookup<TC_DIFF>(S) : tc_lookup<TC_EF>(S));
     const size_t smem = tc_smem_bytes(S.C, S.slice);
     EF(allow_smem(reinterpret_cast<const void*>(kern), tc_smem_bytes(S.C, S.C == 1 && S.threads < 1024 ? 8192 : TC_MAX_SLICE), S.C > 8));
     TcArgs p = {};
     p.a = a; p.pitch_a = pitch_a; p.b = const_cast<float*>(b); p.pitch_b = pitch_b;
     p.d = (int)d; p.k = k; p.slice = S.slice; p.gamma = gamma;
-    p.idx_out = idx_out; p.val_out = val_out; p.apply = apply; p.pitch_apply = pitch_apply; p.status = status; p.slow_count = slow_count;
+    p.idx_out = idx_out; p.val_out = val_out; p.apply = apply; p.pitch_apply = pitch_apply; p.status = status; p.slow_count = slow_count; p.cut_out = cut_out;
     CU(launch(kern, dim3((unsigned)batch * (unsigned)S.C), (unsigned)S.threads, smem, st, (unsigned)S.C, p));
     if (launches) *launches += 1;
     return EF21_OK;
@@ -417,7 +439,7 @@ ef21_status enqueue_topk_stream(cudaStream_t st, const float* a, i64 pitch_a, co
     t.a = a; t.pitch_a = pitch_a; t.b = const_cast<float*>(b); t.pitch_b = pitch_b; t.d = (int)d; t.k = k; t.batch = batch;
     t.idx_out = out.idx_out; t.val_out = out.val_out; t.apply = out.apply; t.pitch_apply = out.pitch_apply; t.status = out.status;
     t.flag = &p.ctl->slow; t.flag_pitch = sizeof(StCtl) / 4;
-    t.tile_off = out.tile_off; t.ntiles = out.ntiles; t.tile = AGG_TILE;
+    t.tile_off = out.tile_off; t.ntiles = out.ntiles; t.tile = AGG_TILE; t.cut_out = out.cut_out;
     t.slice = (int)((ceil_div(d, 8) + 127) / 128 * 128);
     CU(launch(tc_topk_kernel<MODE == TC_EF ? TC_SENT : MODE, 8, 1024, true>, dim3(8u * (unsigned)std::min(batch, 16)), 1024, tc_smem_bytes(8, 0), st, 8, t));
     if (launches) *launches += 4;
@@ -432,25 +454,25 @@ unsigned* slow_counter(const TopkBuffers& B) { return B.L.fast ? reinterpret_cas
 ef21_status enqueue_topk_general(cudaStream_t st, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
                                  int batch, i64 d, int k, int* idx_out, float* val_out,
                                  const TopkBuffers& B, i64* launches, unsigned* status, float* apply_to = nullptr,
-                                 i64 pitch_apply = 0, bool* applied = nullptr) {
+                                 i64 pitch_apply = 0, bool* applied = nullptr, unsigned long long* cut_out = nullptr) {
     if (applied) *applied = false;
     TcShape S;
     if (tc_shape(batch, d, S)) {
         // the whole selection in one launch (no scratch), which also adds the messages to apply_to if the caller asks for it
         if (applied) *applied = apply_to != nullptr;
         return enqueue_topk_cluster(st, b ? TC_DIFF : TC_PLAIN, S, a, pitch_a, b, pitch_b, 0.f, batch, d, k, idx_out, val_out, apply_to,
-                                    pitch_apply, launches, status, status ? slow_counter(B) : nullptr);
+                                    pitch_apply, launches, status, status ? slow_counter(B) : nullptr, cut_out);
     }
-    tk_reset_kernel<<<batch, 256, 0, st>>>(B.state, B.hist, batch, (unsigned)k);
+    CU(launch(tk_reset_kernel, dim3(batch), 256, 0, st, 1, B.state, B.hist, batch, (unsigned)k));
     dim3 grid((unsigned)B.nchunks, (unsigned)batch);
     for (int level = 0; level < 3; ++level) {
-        tk_hist_kernel<<<grid, TK_BLOCK, 0, st>>>(a, pitch_a, b, pitch_b, d, level, B.state, B.hist);
-        tk_find_kernel<<<batch, 1024, 0, st>>>(B.state, B.hist, level);
+        CU(launch(tk_hist_kernel, grid, TK_BLOCK, 0, st, 1, a, pitch_a, b, pitch_b, d, level, B.state, B.hist));
+        CU(launch(tk_find_kernel, dim3(batch), 1024, 0, st, 1, B.state, B.hist, level));
     }
-    tk_count_kernel<<<grid, TK_BLOCK, 0, st>>>(a, pitch_a, b, pitch_b, d, B.state, B.chunks, B.nchunks);
-    tk_scan_kernel<<<batch, 1024, 0, st>>>(B.chunks, B.nchunks);
-    tk_write_kernel<<<grid, TK_BLOCK, 0, st>>>(a, pitch_a, b, pitch_b, d, B.state, B.chunks, B.nchunks, k,
-                                               idx_out, val_out, status);
+    CU(launch(tk_count_kernel, grid, TK_BLOCK, 0, st, 1, a, pitch_a, b, pitch_b, d, B.state, B.chunks, B.nchunks));
+    CU(launch(tk_scan_kernel, dim3(batch), 1024, 0, st, 1, B.chunks, B.nchunks));
+    CU(launch(tk_write_kernel, grid, TK_BLOCK, 0, st, 1, a, pitch_a, b, pitch_b, d, B.state, B.chunks, B.nchunks, k,
+                                               idx_out, val_out, status, cut_out));
     if (launches) *launches += 10;
     CU(cudaGetLastError());
     return EF21_OK;
@@ -460,21 +482,21 @@ ef21_status enqueue_grads(ef21_ctx* c, bool with_loss) {
     if (c->num_tiles > 0) {
         GradTileKernel stream = grad_stream_lookup(c->L.ld);
         if (stream)
-            stream<<<c->num_tiles, GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * c->L.ld * 4, c->stream>>>(
+            CU(launch(stream, dim3(c->num_tiles), GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * c->L.ld * 4, c->stream, 1,
                 c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.tiles), (int)c->L.ld, c->objective,
                 c->at<float>(c->L.partial), with_loss ? c->at<double>(c->L.loss_partial) : nullptr, nullptr, 0,
-                c->at<i64>(c->L.row_off), c->status());
+                c->at<i64>(c->L.row_off), c->status()));
         else
-            grad_tiles_kernel<<<c->num_tiles, GRAD_BLOCK, 0, c->stream>>>(
+            CU(launch(grad_tiles_kernel, dim3(c->num_tiles), GRAD_BLOCK, 0, c->stream, 1,
                 c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.tiles), (int)c->L.ld, c->objective,
                 c->at<float>(c->L.partial), with_loss ? c->at<double>(c->L.loss_partial) : nullptr, nullptr, 0,
-                c->at<i64>(c->L.row_off), c->status());
+                c->at<i64>(c->L.row_off), c->status()));
         c->launches += 1;
     }
     dim3 grid((unsigned)ceil_div(c->L.ld, GRAD_FINISH_COLS), (unsigned)c->n);
-    grad_finish_kernel<<<grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream>>>(
+    CU(launch(grad_finish_kernel, grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream, 1,
         c->at<float>(c->L.partial), c->at<int>(c->L.tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d,
-        (int)c->L.ld, c->at<float>(c->L.grad), 0);
+        (int)c->L.ld, c->at<float>(c->L.grad), 0));
     c->launches += 1;
     CU(cudaGetLastError());
     return EF21_OK;
@@ -504,17 +526,17 @@ ef21_status enqueue_minibatch_grads(ef21_ctx* c, const int* batch_dev, int tau) 
     }
     GradTileKernel stream = grad_stream_lookup(c->L.ld);
     if (stream)
-        stream<<<(unsigned)c->mb_tiles.size(), GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * c->L.ld * 4, c->stream>>>(
+        CU(launch(stream, dim3((unsigned)c->mb_tiles.size()), GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * c->L.ld * 4, c->stream, 1,
             c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.mb_tiles), (int)c->L.ld, c->objective,
-            c->at<float>(c->L.partial), nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status());
+            c->at<float>(c->L.partial), nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status()));
     else
-        grad_tiles_kernel<<<(unsigned)c->mb_tiles.size(), GRAD_BLOCK, 0, c->stream>>>(
+        CU(launch(grad_tiles_kernel, dim3((unsigned)c->mb_tiles.size()), GRAD_BLOCK, 0, c->stream, 1,
             c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.mb_tiles), (int)c->L.ld, c->objective,
-            c->at<float>(c->L.partial), nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status());
+            c->at<float>(c->L.partial), nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status()));
     dim3 grid((unsigned)ceil_div(c->L.ld, GRAD_FINISH_COLS), (unsigned)c->n);
-    grad_finish_kernel<<<grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream>>>(
+    CU(launch(grad_finish_kernel, grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream, 1,
         c->at<float>(c->L.partial), c->at<int>(c->L.mb_tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d,
-        (int)c->L.ld, c->at<float>(c->L.grad), tau);
+        (int)c->L.ld, c->at<float>(c->L.grad), tau));
     c->launches += 2;
     CU(cudaGetLastError());
     return EF21_OK;
@@ -532,7 +554,7 @@ ef21_status enqueue_round_select(ef21_ctx* c, const float* a, i64 pitch_a, bool 
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
     if (long_topk(c)) {
         // the finish kernel also leaves the per-tile offsets of the messages for the aggregation
-        const StOut out = {c->msg_idx(), c->msg_val(), c->gi(), c->L.ld, c->at<int>(c->L.agg_off), c->L.agg_tiles, c->status()};
+        const StOut out = {c->msg_idx(), c->msg_val(), c->gi(), c->L.ld, c->at<int>(c->L.agg_off), c->L.agg_tiles, c->status(), nullptr};
         EF(enqueue_topk_stream<TC_DIFF>(c->stream, a, pitch_a, c->gi(), c->L.ld, 0.f, c->n, c->d, c->k, out, B, &c->launches, true, sampled));
         c->agg_off_ready = true;
     } else {
@@ -542,8 +564,8 @@ ef21_status enqueue_round_select(ef21_ctx* c, const float* a, i64 pitch_a, bool 
                                 c->msg_val(), B, &c->launches, c->status(), c->gi(), c->L.ld, &applied));
         if (!applied) {
             const i64 total = (i64)c->n * c->k;
-            apply_messages_kernel<<<(unsigned)ceil_div(total, 256), 256, 0, c->stream>>>(c->msg_idx(), c->msg_val(), total,
-                                                                                        c->k, c->L.ld, c->gi());
+            CU(launch(apply_messages_kernel, dim3((unsigned)ceil_div(total, 256)), 256, 0, c->stream, 1, c->msg_idx(), c->msg_val(), total,
+                                                                                        c->k, c->L.ld, c->gi()));
             c->launches += 1;
         }
     }
@@ -551,60 +573,79 @@ ef21_status enqueue_round_select(ef21_ctx* c, const float* a, i64 pitch_a, bool 
     return EF21_OK;
 }
 
-ef21_status enqueue_aggregate_into(ef21_ctx* c, float* target, float factor, bool update_x);
+ef21_status enqueue_aggregate_into(ef21_ctx* c, float* target, float factor, int xmode);
 
-// Aggregation half: g += (1/n) sum c_i (and, if update_x, x <- x - gamma g_old in the same kernel).
-ef21_status enqueue_round_aggregate(ef21_ctx* c, bool update_x) {
-    return enqueue_aggregate_into(c, c->g(), 1.0f / (float)c->n, update_x);
+// Aggregation half: g += (1/n) sum c_i (and, with xmode, an update of x in the same kernel).
+ef21_status enqueue_round_aggregate(ef21_ctx* c, int xmode) {
+    return enqueue_aggregate_into(c, c->g(), 1.0f / (float)c->n, xmode);
 }
 
 // target_j += factor * (sum over workers, ascending, of the values sent for coordinate j).
-ef21_status enqueue_aggregate_into(ef21_ctx* c, float* target, float factor, bool update_x) {
-    if (!c->agg_off_ready && !(c->L.agg_tiles == 1 && c->agg_off_static)) {
-        const i64 noff = (i64)c->n * (c->L.agg_tiles + 1);
-        agg_offsets_kernel<<<(unsigned)ceil_div(noff, 256), 256, 0, c->stream>>>(c->msg_idx(), c->n, c->k,
-                                                                                c->L.agg_tiles, c->at<int>(c->L.agg_off));
+ef21_status enqueue_aggregate_into(ef21_ctx* c, float* target, float factor, int xmode) {
+    if (c->d <= AGG_TABLE_MAX_D && c->n <= AGG_TABLE_MAX_N && (i64)c->n * c->k <= AGG_TABLE_MAX_MESSAGES) {
+        auto kern = xmode == AGG_X_KEEP ? aggregate_table_kernel<AGG_X_KEEP>
+                                        : (xmode == AGG_X_BEFORE ? aggregate_table_kernel<AGG_X_BEFORE> : aggregate_table_kernel<AGG_X_AFTER>);
+        const size_t smem = (size_t)c->n * AGG_TABLE_COLS * 4;
+        EF(allow_smem(reinterpret_cast<const void*>(kern), (size_t)AGG_TABLE_MAX_N * AGG_TABLE_COLS * 4));
+        CU(launch(kern, dim3((unsigned)ceil_div(c->d, AGG_TABLE_COLS)), AGG_BLOCK, smem, c->stream, 1, c->msg_idx(), c->msg_val(), c->n, c->k,
+                  (int)c->d, factor, c->gamma, target, c->x()));
         c->launches += 1;
-        c->agg_off_static = c->L.agg_tiles == 1;
+        return EF21_OK;
+    }
+    if (!c->agg_off_ready) {
+        const i64 noff = (i64)c->n * (c->L.agg_tiles + 1);
+        CU(launch(agg_offsets_kernel, dim3((unsigned)ceil_div(noff, 256)), 256, 0, c->stream, 1, c->msg_idx(), c->n, c->k,
+                  c->L.agg_tiles, c->at<int>(c->L.agg_off)));
+        c->launches += 1;
     }
     c->agg_off_ready = false;
     auto kern = c->n <= AGG_STAGE_MAX_N
-                    ? (update_x ? aggregate_staged_kernel<true> : aggregate_staged_kernel<false>)
-                    : (update_x ? aggregate_kernel<true> : aggregate_kernel<false>);
-    kern<<<c->L.agg_tiles, AGG_BLOCK, 0, c->stream>>>(c->msg_idx(), c->msg_val(), c->at<int>(c->L.agg_off), c->n, c->k,
-                                                      c->L.agg_tiles, c->d, factor, c->gamma, target, c->x());
+                    ? (xmode == AGG_X_KEEP ? aggregate_staged_kernel<AGG_X_KEEP>
+                                           : (xmode == AGG_X_BEFORE ? aggregate_staged_kernel<AGG_X_BEFORE> : aggregate_staged_kernel<AGG_X_AFTER>))
+                    : (xmode == AGG_X_KEEP ? aggregate_kernel<AGG_X_KEEP>
+                                           : (xmode == AGG_X_BEFORE ? aggregate_kernel<AGG_X_BEFORE> : aggregate_kernel<AGG_X_AFTER>));
+    CU(launch(kern, dim3(c->L.agg_tiles), AGG_BLOCK, 0, c->stream, 1, c->msg_idx(), c->msg_val(), c->at<int>(c->L.agg_off), c->n, c->k,
+              c->L.agg_tiles, c->d, factor, c->gamma, target, c->x()));
     c->launches += 1;
-    CU(cudaGetLastError());
     return EF21_OK;
 }
 
-ef21_status enqueue_round(ef21_ctx* c, const float* a, i64 pitch_a, bool update_x) {
+ef21_status enqueue_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmode) {
     EF(enqueue_round_select(c, a, pitch_a, false));
-    return enqueue_round_aggregate(c, update_x);
+    return enqueue_round_aggregate(c, xmode);
 }
 
 // One round of EF21+ (Algorithm 3) on local gradients a: both compressed vectors, the choice by
 // distortion, g_i <- chosen, g = (1/n) sum g_i.
-ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a) {
+ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmode) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
     int* idx_b = c->at<int>(c->L.msg2_idx);
     float* val_b = c->at<float>(c->L.msg2_val);
+    unsigned long long* cuts = c->at<unsigned long long>(c->L.plus_cuts);       // [2][n]: Markov, plain
     if (long_topk(c)) {
-        const StOut om = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status()}, ob = {idx_b, val_b, nullptr, 0, nullptr, 0, c->status()};
+        const StOut om = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status(), cuts};
+        const StOut ob = {idx_b, val_b, nullptr, 0, nullptr, 0, c->status(), cuts + c->n};
         EF(enqueue_topk_stream<TC_DIFF>(c->stream, a, pitch_a, c->gi(), c->L.ld, 0.f, c->n, c->d, c->k, om, B, &c->launches, true));
         EF(enqueue_topk_stream<TC_PLAIN>(c->stream, a, pitch_a, nullptr, 0, 0.f, c->n, c->d, c->k, ob, B, &c->launches, true));
     } else {
         EF(enqueue_topk_general(c->stream, a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->k, c->msg_idx(), c->msg_val(), B,
-                                &c->launches, c->status()));
-        EF(enqueue_topk_general(c->stream, a, pitch_a, nullptr, 0, c->n, c->d, c->k, idx_b, val_b, B, &c->launches, c->status()));
+                                &c->launches, c->status(), nullptr, 0, nullptr, cuts));
+        EF(enqueue_topk_general(c->stream, a, pitch_a, nullptr, 0, c->n, c->d, c->k, idx_b, val_b, B, &c->launches, c->status(), nullptr, 0,
+                                nullptr, cuts + c->n));
     }
-    plus_choose_kernel<<<c->n, PLUS_BLOCK, 0, c->stream>>>(a, pitch_a, c->gi(), c->L.ld, c->d, c->k, c->msg_idx(), c->msg_val(),
-                                                          idx_b, val_b, c->at<float>(c->L.plus_old), c->at<unsigned>(c->L.plus_bitmap),
-                                                          c->at<int>(c->L.plus_choice));
-    const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->d, 256), 148 * 8);
-    dense_mean_kernel<<<blocks, 256, 0, c->stream>>>(c->gi(), c->L.ld, c->n, c->d, 1.0f / (float)c->n, c->g());
-    c->launches += 2;
-    CU(cudaGetLastError());
+    // four blocks per SM over all workers, parts of at least 4,096 coordinates
+    const i64 parts = std::max<i64>(1, std::min<i64>(std::min<i64>(PLUS_MAX_PARTS, 148 * 4 / c->n), c->d / 4096));
+    double2* part = c->at<double2>(c->L.plus_parts);
+    CU(launch(plus_distortion_kernel, dim3((unsigned)parts, (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, a, pitch_a, c->gi(), c->L.ld, c->d,
+              ceil_div(c->d, parts), cuts, part));
+    CU(launch(plus_choose_kernel, dim3((unsigned)ceil_div(c->k, PLUS_BLOCK), (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, part, (int)parts, c->gi(),
+              c->L.ld, c->k, c->msg_idx(), c->msg_val(), idx_b, val_b, c->at<int>(c->L.plus_choice)));
+    const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->d, 1024), 148 * 8);
+    auto mean = xmode == AGG_X_KEEP ? plus_mean_kernel<AGG_X_KEEP>
+                                    : (xmode == AGG_X_BEFORE ? plus_mean_kernel<AGG_X_BEFORE> : plus_mean_kernel<AGG_X_AFTER>);
+    CU(launch(mean, dim3(blocks), 256, 0, c->stream, 1, a, pitch_a, cuts + c->n, c->at<int>(c->L.plus_choice), c->gi(), c->L.ld, c->n, c->d,
+              1.0f / (float)c->n, c->gamma, c->g(), c->x()));
+    c->launches += 3;
     return EF21_OK;
 }
 
@@ -613,47 +654,52 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a) {
 // x by -(1/n) sum w_i, and e_i <- p_i - w_i.
 ef21_status enqueue_ef_round(ef21_ctx* c, const float* a, i64 pitch_a) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
-    const unsigned blocks = (unsigned)std::min<i64>(ceil_div((i64)c->n * c->d, 256), 148 * 16);
-    ef_compose_kernel<<<blocks, 256, 0, c->stream>>>(a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->gamma);
-    c->launches += 1;
-    if (long_topk(c)) {
-        const StOut out = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status()};
-        EF(enqueue_topk_stream<TC_PLAIN>(c->stream, c->gi(), c->L.ld, nullptr, 0, 0.f, c->n, c->d, c->k, out, B, &c->launches, true));
+    TcShape S;
+    c->agg_off_ready = false;
+    if (tc_shape(c->n, c->d, S)) {
+        // the kernel that selects also forms p_i (kept as the new error) and clears the sent coordinates
+        EF(enqueue_topk_cluster(c->stream, TC_EF, S, a, pitch_a, c->gi(), c->L.ld, c->gamma, c->n, c->d, c->k, c->msg_idx(), c->msg_val(),
+                                c->gi(), c->L.ld, &c->launches, c->status(), slow_counter(B)));
+    } else if (long_topk(c)) {
+        const StOut out = {c->msg_idx(), c->msg_val(), c->gi(), c->L.ld, c->at<int>(c->L.agg_off), c->L.agg_tiles, c->status(), nullptr};
+        EF(enqueue_topk_stream<TC_EF>(c->stream, a, pitch_a, c->gi(), c->L.ld, c->gamma, c->n, c->d, c->k, out, B, &c->launches, true));
+        c->agg_off_ready = true;
     } else {
+        const unsigned blocks = (unsigned)std::min<i64>(ceil_div((i64)c->n * c->d, 256), 148 * 16);
+        CU(launch(ef_compose_kernel, dim3(blocks), 256, 0, c->stream, 1, a, pitch_a, c->gi(), c->L.ld, c->n, c->d, c->gamma));
         EF(enqueue_topk_general(c->stream, c->gi(), c->L.ld, nullptr, 0, c->n, c->d, c->k, c->msg_idx(), c->msg_val(), B,
                                 &c->launches, c->status()));
+        const i64 total = (i64)c->n * c->k;
+        CU(launch(ef_subtract_sent_kernel, dim3((unsigned)ceil_div(total, 256)), 256, 0, c->stream, 1, c->msg_idx(), c->msg_val(), total, c->k,
+                  c->L.ld, c->gi()));
+        c->launches += 2;
     }
-    const i64 total = (i64)c->n * c->k;
-    ef_subtract_sent_kernel<<<(unsigned)ceil_div(total, 256), 256, 0, c->stream>>>(c->msg_idx(), c->msg_val(), total, c->k,
-                                                                                  c->L.ld, c->gi());
-    c->launches += 1;
-    c->agg_off_ready = false;
-    CU(cudaGetLastError());
-    return enqueue_aggregate_into(c, c->x(), -(1.0f / (float)c->n), false);
+    return enqueue_aggregate_into(c, c->x(), -(1.0f / (float)c->n), AGG_X_KEEP);
 }
 
 ef21_status enqueue_x_update(ef21_ctx* c) {
     const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->d, 256), 148 * 8);
-    x_update_kernel<<<blocks, 256, 0, c->stream>>>(c->g(), c->x(), c->d, c->gamma);
+    CU(launch(x_update_kernel, dim3(blocks), 256, 0, c->stream, 1, c->g(), c->x(), c->d, c->gamma));
     c->launches += 1;
     CU(cudaGetLastError());
     return EF21_OK;
 }
 
 ef21_status zero_state(ef21_ctx* c) {
-    CU(cudaMemsetAsync(c->gi(), 0, (size_t)c->n * c->L.ld * 4, c->stream));
-    CU(cudaMemsetAsync(c->g(), 0, (size_t)c->L.ld * 4, c->stream));
-    return EF21_OK;
+    Copies m;
+    m.add(c->gi(), c->L.ld, nullptr, 0, c->L.ld, c->n);
+    m.add(c->g(), c->L.ld, nullptr, 0, c->L.ld, 1);
+    return m.run(c->stream, &c->launches);
 }
 
 ef21_status init_from(ef21_ctx* c, const float* V, i64 pitch, int mode) {
     EF(zero_state(c));
     if (mode == EF21_INIT_COMPRESSED) {
-        EF(enqueue_round(c, V, pitch, false));
+        EF(enqueue_round(c, V, pitch, AGG_X_KEEP));
     } else if (mode == EF21_INIT_GRADIENT) {
         const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->d, 256), 148 * 8);
-        dense_init_kernel<<<blocks, 256, 0, c->stream>>>(V, pitch, c->n, c->d, c->L.ld, 1.0f / (float)c->n,
-                                                        c->gi(), c->g());
+        CU(launch(dense_init_kernel, dim3(blocks), 256, 0, c->stream, 1, V, pitch, c->n, c->d, c->L.ld, 1.0f / (float)c->n,
+                                                        c->gi(), c->g()));
         c->launches += 1;
         CU(cudaGetLastError());
     }
@@ -911,10 +957,12 @@ ef21_status run_persistent(ef21_ctx* c, const PersistPlan& P, int steps, const i
     cfg.stream = c->stream;
     // A plain cluster launch: that all n clusters fit on the device at once was checked with the
     // occupancy query when the plan was made.
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)P.C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
     cudaError_t e = cudaLaunchKernelEx(&cfg, P.kernel, p);
     if (e != cudaSuccess) { cudaGetLastError(); return EF21_ERR_CUDA; }
     if (G) { G->any = true; G->detached = false; G->last_stream = c->stream; }
@@ -970,7 +1018,7 @@ ef21_status ef21_create(ef21_ctx** out, int32_t n, int64_t d, int32_t k, float g
     c->L = L;
     c->shards_loaded = false; c->inited = false; c->num_tiles = 0;
     c->path = EF21_PATH_AUTO; c->last_path = 0; c->launches = 0;
-    c->pk_cluster = 0; c->pk_rb = 0; c->pk_src = -1; c->pk_threads = 0; c->agg_off_ready = false; c->agg_off_static = false;
+    c->pk_cluster = 0; c->pk_rb = 0; c->pk_src = -1; c->pk_threads = 0; c->agg_off_ready = false;
     c->pk_used_cluster = c->pk_used_rb = 0; c->pk_used_src = -1; c->pk_used_threads = 0;
     c->pk_body = 0; c->pk_used_body = 0; c->pk_epoch = 0u; c->pk_par = 0u; c->plan_valid = false; c->mb_plan_valid = false; c->mb_plan_tau = 0;
     c->spin_limit = 1u << 22;
@@ -979,16 +1027,15 @@ ef21_status ef21_create(ef21_ctx** out, int32_t n, int64_t d, int32_t k, float g
     c->mb_tau = -1;
     c->objective = EF21_OBJECTIVE_LOGISTIC;
     c->aux_stream = nullptr; c->ev_fork = nullptr; c->ev_join = nullptr;
-    cudaError_t e = cudaMemsetAsync(c->ws + L.status, 0, 256, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->x(), 0, (size_t)L.ld * 4, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->g(), 0, (size_t)L.ld * 4, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->gi(), 0, (size_t)n * L.ld * 4, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->msg_idx(), 0, (size_t)n * k * 4, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->msg_val(), 0, (size_t)n * k * 4, c->stream);
-    if (e == cudaSuccess && L.tk.fast) e = cudaMemsetAsync(c->ws + L.topk + L.tk.slow_count, 0, 4, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.plus_choice, 0, (size_t)n * 4, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->ws + L.slots, 0, (size_t)2 * n * k * 8, c->stream);
-    if (e != cudaSuccess) { delete c; return EF21_ERR_CUDA; }
+    // x, g, g_i and the messages lie one behind the other, the words that have to start at zero elsewhere are few
+    Copies clear;
+    clear.add(c->ws + L.status, 64, nullptr, 0, 64, 1);
+    clear.add(c->ws + L.x, 1, nullptr, 0, 1, (i64)(L.topk - L.x) / 4);
+    if (L.tk.fast) clear.add(c->ws + L.topk + L.tk.slow_count, 1, nullptr, 0, 1, 1);
+    clear.add(c->ws + L.plus_choice, n, nullptr, 0, n, 1);
+    clear.add(c->ws + L.slots, 1, nullptr, 0, 1, (i64)4 * n * k);
+    const ef21_status e = clear.run(c->stream, &c->launches);
+    if (e != EF21_OK) { delete c; return e; }
     *out = c;
     return EF21_OK;
 }
@@ -1009,7 +1056,7 @@ ef21_status ef21_load_shards(ef21_ctx* c, const float* A_dev, const float* y_dev
     if (c->N == 0) return EF21_ERR_STATE;
     if (!A_dev || !y_dev) return EF21_ERR_INVALID_ARG;
     const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->N * c->L.ld, 256), 148 * 16);
-    pad_rows_kernel<<<blocks, 256, 0, c->stream>>>(A_dev, c->N, (int)c->d, (int)c->L.ld, c->at<float>(c->L.A));
+    CU(launch(pad_rows_kernel, dim3(blocks), 256, 0, c->stream, 1, A_dev, c->N, (int)c->d, (int)c->L.ld, c->at<float>(c->L.A)));
     c->launches += 1;
     CU(cudaGetLastError());
     CU(cudaMemcpyAsync(c->at<float>(c->L.y), y_dev, (size_t)c->N * 4, cudaMemcpyDeviceToDevice, c->stream));
@@ -1030,8 +1077,9 @@ ef21_status ef21_load_shards_host(ef21_ctx* c, const float* A_host, const float*
 
 ef21_status ef21_set_x(ef21_ctx* c, const float* x0_dev) {
     if (!c || !x0_dev) return EF21_ERR_INVALID_ARG;
-    CU(cudaMemcpyAsync(c->x(), x0_dev, (size_t)c->d * 4, cudaMemcpyDeviceToDevice, c->stream));
-    return EF21_OK;
+    Copies m;
+    m.add(c->x(), c->d, x0_dev, c->d, c->d, 1);
+    return m.run(c->stream, &c->launches);
 }
 
 ef21_status ef21_init(ef21_ctx* c, int32_t mode) {
@@ -1052,31 +1100,26 @@ ef21_status ef21_init_grads(ef21_ctx* c, const float* V_dev, int32_t mode) {
     return init_from(c, V_dev, c->d, mode);
 }
 
-// One iteration of ef21_step on the launch path, as plain kernel launches on the handle's stream.
-static ef21_status enqueue_launch_iteration(ef21_ctx* c) {
-    if (c->variant == EF21_VARIANT_EF) {
-        EF(enqueue_grads(c, false));
-        return enqueue_ef_round(c, c->at<float>(c->L.grad), c->L.ld);
-    }
-    EF(enqueue_x_update(c));
+// One iteration of ef21_step on the launch path, as plain kernel launches on the handle's stream.  The x update that opens the
+// iteration has already been enqueued (or does not exist: Algorithm 4); xmode AGG_X_AFTER: the one of the next iteration is
+// made by the kernel that updates g.
+static ef21_status enqueue_launch_iteration(ef21_ctx* c, int xmode) {
     EF(enqueue_grads(c, false));
-    if (c->variant == EF21_VARIANT_EF21_PLUS) return enqueue_plus_round(c, c->at<float>(c->L.grad), c->L.ld);
-    return enqueue_round(c, c->at<float>(c->L.grad), c->L.ld, false);
+    if (c->variant == EF21_VARIANT_EF) return enqueue_ef_round(c, c->at<float>(c->L.grad), c->L.ld);
+    if (c->variant == EF21_VARIANT_EF21_PLUS) return enqueue_plus_round(c, c->at<float>(c->L.grad), c->L.ld, xmode);
+    return enqueue_round(c, c->at<float>(c->L.grad), c->L.ld, xmode);
 }
 
-// `steps` launch-path iterations.  Short vectors (the one-launch Top-k) make an iteration a fixed list of
-// five to nine small kernels whose cost is their launches: from the second iteration of a call on, the
-// list is replayed as a CUDA graph captured once per handle and method.  The first iteration always
-// runs as plain launches (it may still write the one-time aggregation offsets).  Anything that stands
-// in the way (the caller's stream is itself being captured, capture or instantiation fails) leaves the
-// plain launches, which give the same results.
+// `steps` launch-path iterations.  Short vectors make an iteration a fixed list of a few small kernels whose cost is their
+// launches: the iterations before the last one are replayed as a CUDA graph captured once per handle and method.  Anything
+// that stands in the way (the caller's stream is itself being captured, capture or instantiation fails) leaves the plain
+// launches, which give the same results.
 static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
     int done = 0;
     const bool graphable = c->d <= GRAPH_MAX_D && steps >= 3 && !c->iter_graph_off;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (c->variant != EF21_VARIANT_EF) EF(enqueue_x_update(c));
     if (graphable && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-        EF(enqueue_launch_iteration(c));
-        done = 1;
         const int key = c->variant * 16 + c->objective;
         if (c->iter_graph && c->iter_graph_key != key) { cudaGraphExecDestroy(c->iter_graph); c->iter_graph = nullptr; }
         if (!c->iter_graph) {
@@ -1089,7 +1132,7 @@ static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
             if (ok) {
                 cudaStream_t user_stream = c->stream;
                 c->stream = c->cap_stream;
-                const ef21_status st = enqueue_launch_iteration(c);
+                const ef21_status st = enqueue_launch_iteration(c, AGG_X_AFTER);
                 c->stream = user_stream;
                 ok = cudaStreamEndCapture(c->cap_stream, &graph) == cudaSuccess && st == EF21_OK && graph != nullptr;
             }
@@ -1106,7 +1149,7 @@ static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
             }
         }
         if (c->iter_graph) {
-            for (; done < steps; ++done) {
+            for (; done + 1 < steps; ++done) {
                 CU(cudaGraphLaunch(c->iter_graph, c->stream));
                 c->launches += c->iter_graph_launches;
             }
@@ -1114,7 +1157,7 @@ static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
     } else {
         cudaGetLastError();
     }
-    for (; done < steps; ++done) EF(enqueue_launch_iteration(c));
+    for (; done < steps; ++done) EF(enqueue_launch_iteration(c, done + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;
 }
@@ -1147,10 +1190,7 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
         return EF21_OK;
     }
     if (c->variant == EF21_VARIANT_EF21_PLUS) {
-        for (int t = 0; t < steps; ++t) {
-            EF(enqueue_x_update(c));
-            EF(enqueue_plus_round(c, V_dev, c->d));
-        }
+        for (int t = 0; t < steps; ++t) EF(enqueue_plus_round(c, V_dev, c->d, AGG_X_BEFORE));
         c->last_path = EF21_PATH_LAUNCHES;
         return EF21_OK;
     }
@@ -1166,8 +1206,7 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
     if (!(fast && steps > 1)) {
         for (int t = 0; t < steps; ++t) {
-            EF(enqueue_round_select(c, V_dev, c->d, false));
-            EF(enqueue_round_aggregate(c, true));
+            EF(enqueue_round(c, V_dev, c->d, AGG_X_BEFORE));
         }
         c->last_path = EF21_PATH_LAUNCHES;
         return EF21_OK;
@@ -1183,7 +1222,7 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
         CU(cudaEventRecord(c->ev_fork, main_stream));
         CU(cudaStreamWaitEvent(c->aux_stream, c->ev_fork, 0));
         c->stream = c->aux_stream;
-        const ef21_status agg = enqueue_round_aggregate(c, true);
+        const ef21_status agg = enqueue_round_aggregate(c, AGG_X_BEFORE);
         c->stream = main_stream;
         EF(agg);
         CU(cudaEventRecord(c->ev_join, c->aux_stream));
@@ -1214,10 +1253,10 @@ ef21_status ef21_step_minibatches(ef21_ctx* c, const int32_t* batches_dev, int32
         }
     }
     if (c->path == EF21_PATH_PERSISTENT) return EF21_ERR_UNSUPPORTED;
+    EF(enqueue_x_update(c));
     for (int t = 0; t < steps; ++t) {
-        EF(enqueue_x_update(c));
         EF(enqueue_minibatch_grads(c, batches_dev + (size_t)t * c->n * tau, tau));
-        EF(enqueue_round(c, c->at<float>(c->L.grad), c->L.ld, false));
+        EF(enqueue_round(c, c->at<float>(c->L.grad), c->L.ld, t + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
     }
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;
@@ -1232,17 +1271,17 @@ ef21_status ef21_step_randk(ef21_ctx* c, const float* V_dev, const int32_t* sets
     if (!c->inited || (!V_dev && !c->shards_loaded)) return EF21_ERR_STATE;
     if (c->variant != EF21_VARIANT_EF21) return EF21_ERR_UNSUPPORTED;
     const i64 total = (i64)c->n * c->k;
+    if (!V_dev && steps > 0) EF(enqueue_x_update(c));
     for (int t = 0; t < steps; ++t) {
-        EF(enqueue_x_update(c));
         if (!V_dev) EF(enqueue_grads(c, false));
         const float* a = V_dev ? V_dev : c->at<float>(c->L.grad);
         const i64 pitch = V_dev ? c->d : c->L.ld;
-        randk_select_kernel<<<(unsigned)ceil_div(total, 256), 256, 0, c->stream>>>(
-            a, pitch, c->gi(), c->L.ld, sets_dev + (size_t)t * total, total, c->k, c->d, c->msg_idx(), c->msg_val(), c->status());
+        CU(launch(randk_select_kernel, dim3((unsigned)ceil_div(total, 256)), 256, 0, c->stream, 1,
+            a, pitch, c->gi(), c->L.ld, sets_dev + (size_t)t * total, total, c->k, c->d, c->msg_idx(), c->msg_val(), c->status()));
         c->launches += 1;
         CU(cudaGetLastError());
         c->agg_off_ready = false;
-        EF(enqueue_round_aggregate(c, false));
+        EF(enqueue_round_aggregate(c, V_dev ? AGG_X_BEFORE : (t + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP)));
     }
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;
@@ -1252,9 +1291,9 @@ ef21_status ef21_local_grads(ef21_ctx* c, float* grads_out_dev) {
     if (!c || !grads_out_dev) return EF21_ERR_INVALID_ARG;
     if (!c->shards_loaded) return EF21_ERR_STATE;
     EF(enqueue_grads(c, false));
-    CU(cudaMemcpy2DAsync(grads_out_dev, (size_t)c->d * 4, c->at<float>(c->L.grad), (size_t)c->L.ld * 4,
-                         (size_t)c->d * 4, (size_t)c->n, cudaMemcpyDeviceToDevice, c->stream));
-    return EF21_OK;
+    Copies m;
+    m.add(grads_out_dev, c->d, c->at<float>(c->L.grad), c->L.ld, c->d, c->n);
+    return m.run(c->stream, &c->launches);
 }
 
 size_t ef21_topk_workspace_bytes(int32_t batch, int64_t d, int32_t k) {
@@ -1273,7 +1312,7 @@ ef21_status ef21_topk(const float* v_dev, int32_t batch, int64_t d, int32_t k, i
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     TcShape S;
     if (L.fast && !tc_shape(batch, d, S))
-        return enqueue_topk_stream<TC_PLAIN>(st, v_dev, d, nullptr, 0, 0.f, batch, d, k, StOut{idx_out_dev, val_out_dev, nullptr, 0, nullptr, 0, nullptr}, B,
+        return enqueue_topk_stream<TC_PLAIN>(st, v_dev, d, nullptr, 0, 0.f, batch, d, k, StOut{idx_out_dev, val_out_dev, nullptr, 0, nullptr, 0, nullptr, nullptr}, B,
                                              nullptr, false);
     return enqueue_topk_general(st, v_dev, d, nullptr, 0, batch, d, k, idx_out_dev, val_out_dev, B, nullptr, nullptr);
 }
@@ -1325,33 +1364,37 @@ ef21_status ef21_topk_static(const float* v_dev, int32_t batch, int64_t d, int32
                                 idx_out_dev, val_out_dev, B, nullptr, nullptr);
 }
 
-static ef21_status copy_state_out(ef21_ctx* c, float* x, float* g, float* gi, int32_t* li, float* lv, cudaMemcpyKind kind) {
-    if (x) CU(cudaMemcpyAsync(x, c->x(), (size_t)c->d * 4, kind, c->stream));
-    if (g) CU(cudaMemcpyAsync(g, c->g(), (size_t)c->d * 4, kind, c->stream));
-    if (gi) CU(cudaMemcpy2DAsync(gi, (size_t)c->d * 4, c->gi(), (size_t)c->L.ld * 4, (size_t)c->d * 4, (size_t)c->n, kind, c->stream));
-    if (li) CU(cudaMemcpyAsync(li, c->msg_idx(), (size_t)c->n * c->k * 4, kind, c->stream));
-    if (lv) CU(cudaMemcpyAsync(lv, c->msg_val(), (size_t)c->n * c->k * 4, kind, c->stream));
-    return EF21_OK;
-}
-
 ef21_status ef21_get_state(ef21_ctx* c, float* x_dev, float* g_dev, float* gi_dev, int32_t* last_idx_dev, float* last_val_dev) {
     if (!c) return EF21_ERR_INVALID_ARG;
-    return copy_state_out(c, x_dev, g_dev, gi_dev, last_idx_dev, last_val_dev, cudaMemcpyDeviceToDevice);
+    const i64 nk = (i64)c->n * c->k;
+    Copies m;
+    m.add(x_dev, c->d, c->x(), c->d, c->d, 1);
+    m.add(g_dev, c->d, c->g(), c->d, c->d, 1);
+    m.add(gi_dev, c->d, c->gi(), c->L.ld, c->d, c->n);
+    m.add(last_idx_dev, nk, c->msg_idx(), nk, nk, 1);
+    m.add(last_val_dev, nk, c->msg_val(), nk, nk, 1);
+    return m.run(c->stream, &c->launches);
 }
 
 ef21_status ef21_get_state_host(ef21_ctx* c, float* x_host, float* g_host, float* gi_host, int32_t* last_idx_host, float* last_val_host) {
     if (!c) return EF21_ERR_INVALID_ARG;
-    EF(copy_state_out(c, x_host, g_host, gi_host, last_idx_host, last_val_host, cudaMemcpyDeviceToHost));
+    constexpr cudaMemcpyKind kind = cudaMemcpyDeviceToHost;
+    if (x_host) CU(cudaMemcpyAsync(x_host, c->x(), (size_t)c->d * 4, kind, c->stream));
+    if (g_host) CU(cudaMemcpyAsync(g_host, c->g(), (size_t)c->d * 4, kind, c->stream));
+    if (gi_host) CU(cudaMemcpy2DAsync(gi_host, (size_t)c->d * 4, c->gi(), (size_t)c->L.ld * 4, (size_t)c->d * 4, (size_t)c->n, kind, c->stream));
+    if (last_idx_host) CU(cudaMemcpyAsync(last_idx_host, c->msg_idx(), (size_t)c->n * c->k * 4, kind, c->stream));
+    if (last_val_host) CU(cudaMemcpyAsync(last_val_host, c->msg_val(), (size_t)c->n * c->k * 4, kind, c->stream));
     CU(cudaStreamSynchronize(c->stream));
     return EF21_OK;
 }
 
 ef21_status ef21_set_state(ef21_ctx* c, const float* x_dev, const float* g_dev, const float* gi_dev) {
     if (!c) return EF21_ERR_INVALID_ARG;
-    if (x_dev) CU(cudaMemcpyAsync(c->x(), x_dev, (size_t)c->d * 4, cudaMemcpyDeviceToDevice, c->stream));
-    if (g_dev) CU(cudaMemcpyAsync(c->g(), g_dev, (size_t)c->d * 4, cudaMemcpyDeviceToDevice, c->stream));
-    if (gi_dev) CU(cudaMemcpy2DAsync(c->gi(), (size_t)c->L.ld * 4, gi_dev, (size_t)c->d * 4, (size_t)c->d * 4, (size_t)c->n,
-                                     cudaMemcpyDeviceToDevice, c->stream));
+    Copies m;
+    if (x_dev) m.add(c->x(), c->d, x_dev, c->d, c->d, 1);
+    if (g_dev) m.add(c->g(), c->d, g_dev, c->d, c->d, 1);
+    if (gi_dev) m.add(c->gi(), c->L.ld, gi_dev, c->d, c->d, c->n);
+    EF(m.run(c->stream, &c->launches));
     c->inited = true;
     return EF21_OK;
 }
@@ -1360,9 +1403,9 @@ ef21_status ef21_eval(ef21_ctx* c, double* f, double* grad_norm2, double* G) {
     if (!c) return EF21_ERR_INVALID_ARG;
     if (!c->shards_loaded) return EF21_ERR_STATE;
     EF(enqueue_grads(c, true));
-    eval_reduce_kernel<<<1, 1024, 0, c->stream>>>(c->at<double>(c->L.loss_partial), c->at<int>(c->L.tile_begin),
+    CU(launch(eval_reduce_kernel, dim3(1), 1024, 0, c->stream, 1, c->at<double>(c->L.loss_partial), c->at<int>(c->L.tile_begin),
                                                   c->at<i64>(c->L.row_off), c->at<float>(c->L.grad), c->gi(), c->x(),
-                                                  c->lambda, c->n, (int)c->d, (int)c->L.ld, c->at<double>(c->L.eval_out));
+                                                  c->lambda, c->n, (int)c->d, (int)c->L.ld, c->at<double>(c->L.eval_out)));
     c->launches += 1;
     CU(cudaGetLastError());
     double out[3];
@@ -1471,7 +1514,7 @@ ef21_status ef21_clear_status(ef21_ctx* c) {
 ef21_status ef21_selftest_bounded_wait(ef21_ctx* c, uint32_t spin_limit) {
     if (!c || spin_limit == 0 || spin_limit > (1u << 24)) return EF21_ERR_INVALID_ARG;
     CU(cudaMemsetAsync(c->at<unsigned long long>(c->L.slots), 0, 8, c->stream));
-    bounded_wait_selftest_kernel<<<1, 1, 0, c->stream>>>(c->at<unsigned long long>(c->L.slots), c->status(), spin_limit);
+    CU(launch(bounded_wait_selftest_kernel, dim3(1), 1, 0, c->stream, 1, c->at<unsigned long long>(c->L.slots), c->status(), spin_limit));
     c->launches += 1;
     CU(cudaGetLastError());
     return EF21_OK;

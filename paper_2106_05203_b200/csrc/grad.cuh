@@ -37,6 +37,8 @@ grad_tiles_kernel(const float* __restrict__ A, const float* __restrict__ y, cons
                   const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                   double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
                   const i64* __restrict__ row_off, unsigned* __restrict__ status) {
+    pdl_trigger();
+    pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
     __shared__ float rho[GRAD_TILE_MAX_ROWS];
     __shared__ i64 rowid[GRAD_TILE_MAX_ROWS];
     __shared__ double loss_w[GRAD_BLOCK / 32];
@@ -61,7 +63,7 @@ grad_tiles_kernel(const float* __restrict__ A, const float* __restrict__ y, cons
         float z = 0.f;
         for (int c = lane; c < chunks; c += 32) {
             float4 a = row[c];
-            float4 xv = __ldg(x4 + c);
+            float4 xv = x4[c];
             z = fmaf(a.x, xv.x, z); z = fmaf(a.y, xv.y, z); z = fmaf(a.z, xv.z, z); z = fmaf(a.w, xv.w, z);
         }
         z = warp_sum(z);
@@ -115,6 +117,8 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
                    const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                    double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
                    const i64* __restrict__ row_off, unsigned* __restrict__ status) {
+    pdl_trigger();
+    pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
     constexpr int SH = (RB == 32) ? 0 : (RB == 16 ? 1 : (RB == 8 ? 2 : (RB == 4 ? 3 : 4)));    // log2(32/RB)
     constexpr int WARPS = GRAD_STREAM_BLOCK / 32;
     static_assert(RB == 2 || RB == 4 || RB == 8 || RB == 16, "RB");
@@ -141,7 +145,7 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
 #pragma unroll
     for (int cs = 0; cs < CHUNKS; ++cs) {
         const int c = lane + 32 * cs;
-        xr[cs] = c < chunks ? __ldg(reinterpret_cast<const float4*>(x) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xr[cs] = c < chunks ? reinterpret_cast<const float4*>(x)[c] : make_float4(0.f, 0.f, 0.f, 0.f);
         acc[cs] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     double loss_acc = 0.0;
@@ -227,6 +231,8 @@ __global__ void __launch_bounds__(GRAD_FINISH_COLS * GRAD_FINISH_LANES)
 grad_finish_kernel(const float* __restrict__ partial, const int* __restrict__ tile_begin,
                    const i64* __restrict__ row_off, const float* __restrict__ x,
                    float lambda, int d, int ld, float* __restrict__ grad, int batch_rows) {
+    pdl_trigger();
+    pdl_wait(partial, tile_begin, row_off, x, grad);
     __shared__ float part[GRAD_FINISH_LANES][GRAD_FINISH_COLS];
     const int i = blockIdx.y;
     const int col = threadIdx.x % GRAD_FINISH_COLS, q = threadIdx.x / GRAD_FINISH_COLS;
@@ -254,6 +260,8 @@ grad_finish_kernel(const float* __restrict__ partial, const int* __restrict__ ti
 
 // Copies A[N][d] into the padded layout Ap[N][ld], zero-filling the padding columns.
 __global__ void pad_rows_kernel(const float* __restrict__ A, i64 N, int d, int ld, float* __restrict__ Ap) {
+    pdl_trigger();
+    pdl_wait(A, Ap);
     const i64 total = N * (i64)ld;
     for (i64 e = blockIdx.x * (i64)blockDim.x + threadIdx.x; e < total; e += (i64)gridDim.x * blockDim.x) {
         const i64 r = e / ld;
@@ -269,6 +277,8 @@ eval_reduce_kernel(const double* __restrict__ loss_partial, const int* __restric
                    const i64* __restrict__ row_off, const float* __restrict__ grad,
                    const float* __restrict__ gi, const float* __restrict__ x, float lambda,
                    int n, int d, int ld, double* __restrict__ out) {
+    pdl_trigger();
+    pdl_wait(loss_partial, tile_begin, row_off, grad, gi, x, out);
     __shared__ double red[3][32];
     double f = 0.0, nrm = 0.0, G = 0.0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {

@@ -2,12 +2,19 @@
 // Markov compressor m_i = g_i + C(grad_i - g_i), judged by the distortions
 //     B_i = ||b_i - grad_i||^2,   M_i = ||m_i - grad_i||^2      (fp64 sums of fp32 terms),
 // g_i <- m_i if M_i <= B_i else b_i; the master recomputes g = (1/n) sum_i g_i.
+//
+// Both messages come from the Top-k kernels, which also leave the cut of each selection -- entry j is in the message if and only
+// if (key << 32 | ~j) >= cut -- so that membership is one compare.  Then three kernels: the distortions, several blocks per
+// worker; the choice and the sparse update of the Markov workers; the dense mean, which also rewrites the rows of workers that
+// took the plain branch.  Bound by HBM / L2: g_i and grad_i are read once for the distortions, g_i once for the mean (one block per
+// worker did all of it before: 1,170 us for 16 workers of 1,000,003 entries against about 35 us).
 #pragma once
 #include "common.cuh"
 
 namespace ef21 {
 
 constexpr int PLUS_BLOCK = 256;
+constexpr int PLUS_MAX_PARTS = 64;          // blocks per worker in the distortion pass
 
 // Deterministic block sum of doubles (fixed tree): result valid in thread 0.
 __device__ __forceinline__ double block_sum_f64(double v, double* scratch /* [PLUS_BLOCK/32] */) {
@@ -21,74 +28,107 @@ __device__ __forceinline__ double block_sum_f64(double v, double* scratch /* [PL
     return s;
 }
 
-// One block per worker.  a: local gradients (pitch_a), gi: worker states (pitch ld).
-// (idx_m, val_m): C(grad_i - g_i); (idx_b, val_b): C(grad_i).  On exit g_i holds the chosen vector,
-// (idx_m, val_m) holds the compressed vector that was used and choice[i] is 0 (Markov) or 1 (plain).
+// grid = (parts, n); part p of worker i covers the coordinates [p * len, (p + 1) * len).  part_out[i][p] = (M, B) of the part.  M and B
+// are summed over the same coordinates in the same order, so that they are bit-identical whenever the two candidates coincide
+// (e.g. g_i = 0).
 __global__ void __launch_bounds__(PLUS_BLOCK)
-plus_choose_kernel(const float* __restrict__ a, i64 pitch_a, float* gi, i64 ld, i64 d, int k,
-                   int* __restrict__ idx_m, float* __restrict__ val_m,
-                   const int* __restrict__ idx_b, const float* __restrict__ val_b,
-                   float* __restrict__ old_vals, unsigned* __restrict__ bitmap, int* __restrict__ choice) {
+plus_distortion_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict__ gi, i64 ld, i64 d, i64 len,
+                       const unsigned long long* __restrict__ cuts /* [2][n]: Markov, plain */, double2* __restrict__ part_out) {
+    pdl_trigger();
+    pdl_wait(a, gi, cuts, part_out);
     __shared__ double scratch[PLUS_BLOCK / 32];
-    __shared__ int take_plain;
-    const int i = blockIdx.x;
+    const int i = blockIdx.y, n = gridDim.y;
+    const unsigned long long cut_m = cuts[i], cut_b = cuts[n + i];
+    const unsigned km = (unsigned)(cut_m >> 32), jm = 0xffffffffu - (unsigned)cut_m, kb = (unsigned)(cut_b >> 32), jb = 0xffffffffu - (unsigned)cut_b;
     const float* __restrict__ grad = a + (i64)i * pitch_a;
-    float* g = gi + (i64)i * ld;
-    int* im = idx_m + (i64)i * k;
-    float* vm = val_m + (i64)i * k;
-    const int* ib = idx_b + (i64)i * k;
-    const float* vb = val_b + (i64)i * k;
-    float* old = old_vals + (i64)i * k;
-
-    // mark the entries kept by the plain compressor (bitmap row of this worker)
-    const i64 words = (d + 31) >> 5;
-    unsigned* bm = bitmap + (i64)i * words;
-    for (i64 w = threadIdx.x; w < words; w += PLUS_BLOCK) bm[w] = 0u;
-    __syncthreads();
-    for (int t = threadIdx.x; t < k; t += PLUS_BLOCK) atomicOr(&bm[ib[t] >> 5], 1u << (ib[t] & 31));
-    // tentatively g_i <- m_i, remembering the k overwritten entries
-    for (int t = threadIdx.x; t < k; t += PLUS_BLOCK) {
-        const int j = im[t];
-        const float o = g[j];
-        old[t] = o;
-        g[j] = __fadd_rn(o, vm[t]);
-    }
-    __syncthreads();
-    // M = sum_j (m_j - grad_j)^2 and B = sum_j (b_j - grad_j)^2 over the same coordinates in the same order,
-    // so that the two sums are bit-identical whenever the two candidates coincide (e.g. g_i = 0)
+    const float* __restrict__ g = gi + (i64)i * ld;
+    const i64 j_end = min((i64)(blockIdx.x + 1) * len, d);
     double m_part = 0.0, b_part = 0.0;
-    for (i64 j = threadIdx.x; j < d; j += PLUS_BLOCK) {
-        const double gr = (double)grad[j];
-        const double e = (double)g[j] - gr;
-        m_part += e * e;
-        const bool kept = (bm[j >> 5] >> (j & 31)) & 1u;
-        b_part += kept ? 0.0 : gr * gr;
-    }
-    const double M = block_sum_f64(m_part, scratch);
-    const double B = block_sum_f64(b_part, scratch);
-    if (threadIdx.x == 0) {
-        take_plain = (M <= B) ? 0 : 1;
-        choice[i] = take_plain;
-    }
-    __syncthreads();
-    if (take_plain) {
-        for (i64 j = threadIdx.x; j < d; j += PLUS_BLOCK) g[j] = 0.f;
-        __syncthreads();
-        for (int t = threadIdx.x; t < k; t += PLUS_BLOCK) {
-            g[ib[t]] = vb[t];
-            im[t] = ib[t];
-            vm[t] = vb[t];
+    constexpr int U = 8;
+    for (i64 j0 = (i64)blockIdx.x * len + threadIdx.x; j0 < j_end; j0 += U * PLUS_BLOCK) {
+        float x[U], o[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const i64 j = j0 + u * PLUS_BLOCK;
+            x[u] = j < j_end ? grad[j] : 0.f; o[u] = j < j_end ? g[j] : 0.f;
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned j = (unsigned)(j0 + u * PLUS_BLOCK);
+            const float v = __fsub_rn(x[u], o[u]);
+            const unsigned kv = mag_key(v), kx = mag_key(x[u]);
+            const bool in_m = kv > km || (kv == km && j <= jm), in_b = kx > kb || (kx == kb && j <= jb);
+            const double e = (double)(in_m ? __fadd_rn(o[u], v) : o[u]) - (double)x[u];       // entries behind the end are 0 - 0
+            m_part += e * e;
+            b_part += in_b ? 0.0 : (double)x[u] * (double)x[u];
+        }
+    }
+    const double M = block_sum_f64(m_part, scratch), B = block_sum_f64(b_part, scratch);
+    if (threadIdx.x == 0) part_out[(i64)i * PLUS_MAX_PARTS + blockIdx.x] = make_double2(M, B);
+}
+
+// grid = (ceil(k / 256), n).  Every block adds up the parts of its worker in the same fixed order; a Markov worker's entries are
+// added to g_i, a plain worker's message takes the place of the Markov one (the rows are rewritten by plus_mean_kernel).
+__global__ void __launch_bounds__(PLUS_BLOCK)
+plus_choose_kernel(const double2* __restrict__ parts_in, int parts, float* __restrict__ gi, i64 ld, int k,
+                   int* __restrict__ idx_m, float* __restrict__ val_m, const int* __restrict__ idx_b, const float* __restrict__ val_b,
+                   int* __restrict__ choice) {
+    pdl_trigger();
+    pdl_wait(parts_in, gi, idx_m, val_m, idx_b, val_b, choice);
+    const int i = blockIdx.y, lane = threadIdx.x & 31;
+    double M = 0.0, B = 0.0;
+    for (int q = lane; q < parts; q += 32) { const double2 s = parts_in[(i64)i * PLUS_MAX_PARTS + q]; M += s.x; B += s.y; }
+    M = warp_sum(M); B = warp_sum(B);
+    const int plain = M <= B ? 0 : 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) choice[i] = plain;
+    const int t = blockIdx.x * PLUS_BLOCK + threadIdx.x;
+    if (t >= k) return;
+    const i64 e = (i64)i * k + t;
+    if (plain) {
+        idx_m[e] = idx_b[e]; val_m[e] = val_b[e];
+    } else {
+        float* p = gi + (i64)i * ld + idx_m[e];
+        *p = __fadd_rn(*p, val_m[e]);
     }
 }
 
-// g_j = (sum over workers, ascending, of g_ij) * (1/n).
-__global__ void dense_mean_kernel(const float* __restrict__ gi, i64 ld, int n, i64 d, float inv_n,
-                                  float* __restrict__ g) {
-    for (i64 j = blockIdx.x * (i64)blockDim.x + threadIdx.x; j < d; j += (i64)gridDim.x * blockDim.x) {
-        float s = 0.f;
-        for (int i = 0; i < n; ++i) s = __fadd_rn(s, gi[(i64)i * ld + j]);
-        g[j] = __fmul_rn(s, inv_n);
+// g_j = (sum over workers, ascending, of g_ij) * (1/n), four coordinates per thread (ld is a multiple of four); g_ij of a worker that took
+// the plain branch becomes C(grad_i)_j first.  XMODE as in the aggregation kernels.
+template <int XMODE>
+__global__ void __launch_bounds__(256)
+plus_mean_kernel(const float* __restrict__ a, i64 pitch_a, const unsigned long long* __restrict__ cut_b, const int* __restrict__ choice,
+                 float* __restrict__ gi, i64 ld, int n, i64 d, float inv_n, float gamma, float* __restrict__ g, float* __restrict__ x) {
+    pdl_trigger();
+    pdl_wait(a, cut_b, choice, gi, g, x);
+    for (i64 j = 4 * (blockIdx.x * (i64)blockDim.x + threadIdx.x); j < d; j += 4 * (i64)gridDim.x * blockDim.x) {
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+            float4* row = reinterpret_cast<float4*>(gi + (i64)i * ld + j);
+            float4 w;
+            if (choice[i]) {
+                const unsigned long long cut = cut_b[i];
+                float b[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float v = j + e < d ? a[(i64)i * pitch_a + j + e] : 0.f;
+                    const unsigned long long c = ((unsigned long long)mag_key(v) << 32) | (0xffffffffu - (unsigned)(j + e));
+                    b[e] = j + e < d && c >= cut ? v : 0.f;
+                }
+                w = make_float4(b[0], b[1], b[2], b[3]);
+                *row = w;
+            } else {
+                w = *row;
+            }
+            s[0] = __fadd_rn(s[0], w.x); s[1] = __fadd_rn(s[1], w.y); s[2] = __fadd_rn(s[2], w.z); s[3] = __fadd_rn(s[3], w.w);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (j + e >= d) break;
+            const float now = __fmul_rn(s[e], inv_n);
+            if (XMODE != 0) x[j + e] = fmaf(-gamma, XMODE == 1 ? g[j + e] : now, x[j + e]);
+            g[j + e] = now;
+        }
     }
 }
 

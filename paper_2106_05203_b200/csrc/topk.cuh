@@ -34,6 +34,8 @@ __host__ __device__ inline int tk_level_shift(int level) { return level == 0 ? 2
 __host__ __device__ inline int tk_level_bits(int level) { return level == 0 ? 11 : 10; }
 
 __global__ void tk_reset_kernel(TkState* __restrict__ st, unsigned* __restrict__ hist, int batch, unsigned k) {
+    pdl_trigger();
+    pdl_wait(st, hist);
     const int v = blockIdx.x;
     if (v >= batch) return;
     for (int b = threadIdx.x; b < TK_BINS; b += blockDim.x) hist[(i64)v * TK_BINS + b] = 0u;
@@ -48,6 +50,8 @@ __global__ void tk_reset_kernel(TkState* __restrict__ st, unsigned* __restrict__
 __global__ void __launch_bounds__(TK_BLOCK)
 tk_hist_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict__ b, i64 pitch_b, i64 d,
                int level, const TkState* __restrict__ st, unsigned* __restrict__ hist) {
+    pdl_trigger();
+    pdl_wait(a, b, st, hist);
     __shared__ unsigned sh[TK_BINS];
     const int v = blockIdx.y;
     const TkState s = st[v];
@@ -79,6 +83,8 @@ tk_hist_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict
 // and clear the histogram for the next level.
 __global__ void __launch_bounds__(1024)
 tk_find_kernel(TkState* __restrict__ st, unsigned* __restrict__ hist, int level) {
+    pdl_trigger();
+    pdl_wait(st, hist);
     __shared__ unsigned scratch[33];
     const int v = blockIdx.x;
     TkState s = st[v];
@@ -110,6 +116,8 @@ tk_find_kernel(TkState* __restrict__ st, unsigned* __restrict__ hist, int level)
 __global__ void __launch_bounds__(TK_BLOCK)
 tk_count_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict__ b, i64 pitch_b, i64 d,
                 const TkState* __restrict__ st, uint2* __restrict__ chunk_counts, int nchunks) {
+    pdl_trigger();
+    pdl_wait(a, b, st, chunk_counts);
     __shared__ unsigned wsum[2][TK_BLOCK / 32];
     const int v = blockIdx.y;
     const TkState s = st[v];
@@ -141,6 +149,8 @@ tk_count_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restric
 // Exclusive scan of the chunk counts of one vector (one block per vector), in place.
 __global__ void __launch_bounds__(1024)
 tk_scan_kernel(uint2* __restrict__ chunk_counts, int nchunks) {
+    pdl_trigger();
+    pdl_wait(chunk_counts);
     __shared__ unsigned scratch[33];
     uint2* __restrict__ cc = chunk_counts + (i64)blockIdx.x * nchunks;
     unsigned base_ge = 0u, base_tie = 0u;
@@ -159,13 +169,16 @@ tk_scan_kernel(uint2* __restrict__ chunk_counts, int nchunks) {
 __global__ void __launch_bounds__(TK_BLOCK)
 tk_write_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict__ b, i64 pitch_b, i64 d,
                 const TkState* __restrict__ st, const uint2* __restrict__ chunk_prefix, int nchunks,
-                int k, int* __restrict__ idx_out, float* __restrict__ val_out, unsigned* status) {
+                int k, int* __restrict__ idx_out, float* __restrict__ val_out, unsigned* status, unsigned long long* cut_out) {
+    pdl_trigger();
+    pdl_wait(a, b, st, chunk_prefix, idx_out, val_out, status, cut_out);
     __shared__ unsigned scratch[33];
     const int v = blockIdx.y;
     const TkState s = st[v];
     const float* __restrict__ av = a + (i64)v * pitch_a;
     const float* __restrict__ bv = b ? b + (i64)v * pitch_b : nullptr;
     const uint2 pre = chunk_prefix[(i64)v * nchunks + blockIdx.x];
+    if (cut_out && s.need_ties == 0u && blockIdx.x == 0 && threadIdx.x == 0) cut_out[v] = (unsigned long long)s.lo_ge << 32;
     unsigned ge_before = pre.x, tie_before = pre.y;
     int* __restrict__ io = idx_out + (i64)v * k;
     float* __restrict__ vo = val_out + (i64)v * k;
@@ -190,6 +203,7 @@ tk_write_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restric
         } else if (is_tie && my_tie < s.need_ties) {
             const unsigned pos = my_ge + my_tie;
             if (pos < (unsigned)k) { io[pos] = (int)j; vo[pos] = val; flag_nonfinite(status, val); }
+            if (cut_out && my_tie + 1u == s.need_ties) cut_out[v] = ((unsigned long long)s.T << 32) | (0xffffffffu - (unsigned)j);
         }
         ge_before += tot & 0xffffu;
         tie_before += tot >> 16;

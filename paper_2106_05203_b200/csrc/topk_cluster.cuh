@@ -43,6 +43,7 @@ struct TcArgs {
     int* idx_out; float* val_out;
     float* apply; i64 pitch_apply;          // TC_DIFF: receives b + v on the selected coordinates; TC_EF, TC_SENT: v - v there; may be null
     unsigned* status;
+    unsigned long long* cut_out;            // [batch]: an entry is selected if and only if (key << 32 | ~index) >= cut; may be null
     unsigned* slow_count;                   // counts the vectors with more than TC_LIST entries equal to T; may be null
     // STREAM only: vectors whose flag (one word every flag_pitch words) is zero are left alone; tile_off (may be null):
     // [batch][ntiles + 1] first message position of every `tile` coordinates
@@ -360,6 +361,8 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
                     const unsigned pos = g0 + min(e0, need_ties);
                     io[pos] = j0 + j + e; vo[pos] = v;
                     flag_nonfinite(p.status, v);
+                    if (tie && e0 + 1u == need_ties && p.cut_out)
+                        p.cut_out[vec] = ((unsigned long long)T << 32) | (0xffffffffu - (unsigned)(j0 + j + e));
                     if (app) app[j + e] = MODE == TC_DIFF ? __fadd_rn(app[j + e], v) : __fsub_rn(v, v);
                 }
                 g0 += tie ? 0u : 1u; e0 += tie ? 1u : 0u;

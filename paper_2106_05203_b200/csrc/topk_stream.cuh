@@ -547,6 +547,7 @@ struct StOut {
     float* apply; i64 pitch_apply;      // receives b + v on the selected coordinates (TC_EF: zero); may be null
     int* tile_off; int ntiles;          // [batch][ntiles + 1] first message position of every 2,048 coordinates; may be null
     unsigned* status;
+    unsigned long long* cut_out;        // [batch] the cut of every vector; may be null
 };
 
 // grid = (ceil(nreg / 32), batch), 256 threads: eight lanes per region.
@@ -560,6 +561,7 @@ st_compact_kernel(const __grid_constant__ StArgs p, const StOut o) {
     const StCtl& ct = p.ctl[vec];
     if (ct.slow) return;
     const unsigned long long cut = ct.cut;
+    if (o.cut_out && blockIdx.x == 0 && threadIdx.x == 0) o.cut_out[vec] = cut;
     const bool have = region < p.nreg;
     const unsigned n = have ? p.reg_cand[(i64)vec * p.nreg_pitch + region] : 0u;
     unsigned pos = have ? p.reg_base[(i64)vec * p.nreg_pitch + region] : 0u;
@@ -636,6 +638,7 @@ st_reread_kernel(const __grid_constant__ StArgs p, const StOut o) {
     const StCtl& ct = p.ctl[vec];
     if (ct.slow || region >= p.nreg) return;
     const unsigned long long cut = ct.cut;
+    if (o.cut_out && blockIdx.x == 0 && threadIdx.x == 0) o.cut_out[vec] = cut;
     const unsigned cut_key = (unsigned)(cut >> 32), cut_idx = 0xffffffffu - (unsigned)cut;
     const unsigned first = p.reg_base[(i64)vec * p.nreg_pitch + region];
     unsigned pos = first;

@@ -8,6 +8,8 @@ namespace ef21 {
 // with EF21_ERR_TIMEOUT in the status word instead of hanging.
 __global__ void bounded_wait_selftest_kernel(const unsigned long long* never_written, unsigned* status,
                                              unsigned spin_limit) {
+    pdl_trigger();
+    pdl_wait(never_written, status);
     unsigned spins = 0;
     while (true) {
         const unsigned long long w = ld_relaxed_u64(never_written);
