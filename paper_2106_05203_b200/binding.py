@@ -8,6 +8,7 @@ paper_2106_05203_b200.build``) importing this module raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional, Tuple
 
@@ -99,7 +100,7 @@ def _check(status: int, where: str) -> None:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _np_ptr(a: Optional[np.ndarray]):
@@ -108,7 +109,7 @@ def _np_ptr(a: Optional[np.ndarray]):
 
 def _stream_handle(stream: Optional[torch.cuda.Stream]):
     s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return s.cuda_stream
 
 
 def _dev_f32(t: torch.Tensor, shape=None) -> torch.Tensor:
@@ -331,23 +332,59 @@ class EF21:
         return int(_lib.ef21_launch_count(self._h))
 
 
+_NO_SCRATCH = 256            # workspace size of shapes whose selection uses no scratch (the pointer still has to be valid)
+_no_scratch_memory = {}      # device index -> one 512-byte tensor, never written
+
+
+def _no_scratch(index: int) -> int:
+    t = _no_scratch_memory.get(index)
+    if t is None:
+        t = _no_scratch_memory.setdefault(index, torch.empty(512, dtype=torch.uint8, device=torch.device("cuda", index)))
+    return (t.data_ptr() + 255) // 256 * 256
+
+
+def _current_raw_stream(index: int) -> int:
+    return torch.cuda.current_stream(index).cuda_stream
+
+
+if hasattr(torch._C, "_cuda_getCurrentRawStream"):          # the same handle without a Stream object around it
+    _current_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
+@functools.lru_cache(maxsize=1024)
+def _topk_workspace_bytes(batch: int, d: int, k: int) -> int:
+    nbytes = int(_lib.ef21_topk_workspace_bytes(batch, d, k))
+    if nbytes == 0:
+        raise Ef21Error(1, "ef21_topk_workspace_bytes")
+    return nbytes
+
+
 def topk(v: torch.Tensor, k: int, stream: Optional[torch.cuda.Stream] = None):
     """Top-k compressor on a batch of vectors v[batch, d] -> (idx[batch, k] int32, val[batch, k])."""
     if v.dim() == 1:
         v = v.unsqueeze(0)
     _dev_f32(v)
     batch, d = v.shape
-    nbytes = int(_lib.ef21_topk_workspace_bytes(batch, d, k))
-    if nbytes == 0:
-        raise Ef21Error(1, "ef21_topk_workspace_bytes")
-    with torch.cuda.device(v.device):
-        ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=v.device)
+    nbytes = _topk_workspace_bytes(batch, d, k)
+    device = v.device
+    if device.index != torch.cuda.current_device():
+        with torch.cuda.device(device):
+            return topk(v, k, stream)
+    # On short vectors the call is bound by this function (the kernel takes 3-5 us): no scratch is allocated where the
+    # library needs none, and nothing is recorded on the stream that everything was allocated on.
+    idx = torch.empty_strided((batch, k), (k, 1), dtype=torch.int32, device=device)
+    val = torch.empty_strided((batch, k), (k, 1), dtype=torch.float32, device=device)
+    if nbytes <= _NO_SCRATCH:
+        ws_ptr = _no_scratch(device.index)
+    else:
+        ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
         ws_ptr = (ws.data_ptr() + 255) // 256 * 256
-        idx = torch.empty((batch, k), dtype=torch.int32, device=v.device)
-        val = torch.empty((batch, k), dtype=torch.float32, device=v.device)
-        _check(_lib.ef21_topk(_ptr(v), batch, d, k, _ptr(idx), _ptr(val), ctypes.c_void_p(ws_ptr), nbytes,
-                              _stream_handle(stream)), "ef21_topk")
-        ws.record_stream(stream if stream is not None else torch.cuda.current_stream())
+        if stream is not None:
+            ws.record_stream(stream)
+    handle = stream.cuda_stream if stream is not None else _current_raw_stream(device.index)
+    status = _lib.ef21_topk(v.data_ptr(), batch, d, k, idx.data_ptr(), val.data_ptr(), ws_ptr, nbytes, handle)
+    if status != EF21_OK:
+        raise Ef21Error(status, "ef21_topk")
     return idx, val
 
 

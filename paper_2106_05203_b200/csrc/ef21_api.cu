@@ -1298,6 +1298,8 @@ ef21_status ef21_local_grads(ef21_ctx* c, float* grads_out_dev) {
 
 size_t ef21_topk_workspace_bytes(int32_t batch, int64_t d, int32_t k) {
     if (batch < 1 || batch > 65535 || !valid_shape(1, d, k, 0)) return 0;
+    TcShape S;
+    if (tc_shape(batch, d, S)) return ALIGN;         // one launch, no scratch
     return topk_layout(batch, d, k).total;
 }
 
@@ -1305,15 +1307,19 @@ ef21_status ef21_topk(const float* v_dev, int32_t batch, int64_t d, int32_t k, i
                       float* val_out_dev, void* workspace_dev, size_t workspace_bytes, void* cuda_stream) {
     if (!v_dev || !idx_out_dev || !val_out_dev || batch < 1 || batch > 65535 || !valid_shape(1, d, k, 0))
         return EF21_ERR_INVALID_ARG;
-    TopkLayout L = topk_layout(batch, d, k);
-    if (!workspace_dev || workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(workspace_dev) % ALIGN) != 0)
-        return EF21_ERR_WORKSPACE;
-    TopkBuffers B = topk_buffers(static_cast<char*>(workspace_dev), L);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     TcShape S;
-    if (L.fast && !tc_shape(batch, d, S))
-        return enqueue_topk_stream<TC_PLAIN>(st, v_dev, d, nullptr, 0, 0.f, batch, d, k, StOut{idx_out_dev, val_out_dev, nullptr, 0, nullptr, 0, nullptr, nullptr}, B,
-                                             nullptr, false);
+    const bool one_launch = tc_shape(batch, d, S);
+    TopkLayout L{};
+    if (one_launch) L.total = ALIGN; else L = topk_layout(batch, d, k);
+    if (!workspace_dev || workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(workspace_dev) % ALIGN) != 0)
+        return EF21_ERR_WORKSPACE;
+    if (one_launch)
+        return enqueue_topk_cluster(st, TC_PLAIN, S, v_dev, d, nullptr, 0, 0.f, batch, d, k, idx_out_dev, val_out_dev, nullptr, 0, nullptr, nullptr);
+    TopkBuffers B = topk_buffers(static_cast<char*>(workspace_dev), L);
+    if (L.fast)
+        return enqueue_topk_stream<TC_PLAIN>(st, v_dev, d, nullptr, 0, 0.f, batch, d, k,
+                                             StOut{idx_out_dev, val_out_dev, nullptr, 0, nullptr, 0, nullptr, nullptr}, B, nullptr, false);
     return enqueue_topk_general(st, v_dev, d, nullptr, 0, batch, d, k, idx_out_dev, val_out_dev, B, nullptr, nullptr);
 }
 
