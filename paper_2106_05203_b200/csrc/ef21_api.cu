@@ -144,22 +144,30 @@ TopkLayout topk_layout(i64 batch, i64 d, i64 k) {
 typedef void (*GradTileKernel)(const float*, const float*, const float*, const RowTile*, int, int, float*, double*,
                                const int*, int, const i64*, unsigned*);
 
-// The one-read gradient kernel for rows of up to 1,024 columns (chunk slots = float4 per lane and row); wider
-// rows use the two-sweep kernel.
-GradTileKernel grad_stream_lookup(i64 ld) {
-    const i64 slots = (ld / 4 + 31) / 32;
-    if (slots <= 1) return grad_stream_kernel<1, 16>;
-    if (slots == 2) return grad_stream_kernel<2, 8>;
-    if (slots == 3) return grad_stream_kernel<3, 4>;
-    if (slots == 4) return grad_stream_kernel<4, 4>;
-    if (slots <= 6) return grad_stream_kernel<6, 2>;
-    if (slots <= 8) return grad_stream_kernel<8, 2>;
-    return nullptr;
+// The gradient kernel for a row width: kernel, threads and shared memory per block; wide: a block works on whole rows and goes
+// through a long tile, `resident` blocks per SM and `rows` rows at a time (0: short tiles, several per SM).
+struct GradPlan { GradTileKernel kernel; unsigned threads; size_t smem; int resident, rows; };
+
+GradPlan grad_plan(i64 ld) {
+    const i64 slots = (ld / 4 + 31) / 32, wide = ceil_div(ld / 4, GRAD_WIDE_BLOCK);
+    if (slots <= 4) {
+        // rows of up to 512 columns, a warp per batch of rows
+        const GradTileKernel k = slots <= 1 ? grad_stream_kernel<1, 16>
+                                            : (slots == 2 ? grad_stream_kernel<2, 8> : (slots == 3 ? grad_stream_kernel<3, 4> : grad_stream_kernel<4, 4>));
+        return {k, GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * ld * 4, 0, 0};
+    }
+    static const GradTileKernel kernels[8] = {grad_wide_kernel<1>, grad_wide_kernel<2>, grad_wide_kernel<3>, grad_wide_kernel<4>,
+                                              grad_wide_kernel<5>, grad_wide_kernel<6>, grad_wide_kernel<7>, grad_wide_kernel<8>};
+    if (wide <= 8) return {kernels[wide - 1], GRAD_WIDE_BLOCK, 0, wide <= 2 ? 2 : 1, grad_wide_rows((int)wide)};
+    return {grad_tiles_kernel, GRAD_BLOCK, 0, 0, 0};
 }
 
 int grad_tile_rows(i64 N, i64 ld) {
+    const GradPlan P = grad_plan(ld);
+    // a wide tile: the rows of one resident block (the tiles of a load are cut when the shards are known, never shorter)
+    if (P.resident) return (int)std::max<i64>(P.rows, ceil_div(N, 148 * P.resident));
     // two-sweep kernel: a tile's rows should stay in L1 for the second sweep; one-read kernel: any size
-    i64 cap = grad_stream_lookup(ld) ? GRAD_TILE_MAX_ROWS : 65536 / (ld * 4);
+    i64 cap = P.kernel != grad_tiles_kernel ? GRAD_TILE_MAX_ROWS : 65536 / (ld * 4);
     if (cap < 1) cap = 1;
     if (cap > GRAD_TILE_MAX_ROWS) cap = GRAD_TILE_MAX_ROWS;
     i64 want = ceil_div(N, 4 * 148);
@@ -205,7 +213,8 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.A = L.y = L.row_off = L.tile_begin = L.tiles = L.partial = L.loss_partial = L.grad = L.mb_tile_begin = L.mb_tiles = 0;
     if (N > 0) {
         L.tile_rows = grad_tile_rows(N, L.ld);
-        L.max_tiles = N / L.tile_rows + n;
+        // (the tiles of minibatch lists are shorter than those of the shards, but no more of them are made than fit the device)
+        L.max_tiles = std::max<i64>(N / L.tile_rows, grad_plan(L.ld).resident * 148) + n;
         L.A = take((size_t)N * L.ld * 4);
         L.y = take((size_t)N * 4);
         L.row_off = take((size_t)(n + 1) * 8);
@@ -478,34 +487,47 @@ ef21_status enqueue_topk_general(cudaStream_t st, const float* a, i64 pitch_a, c
     return EF21_OK;
 }
 
-ef21_status enqueue_grads(ef21_ctx* c, bool with_loss) {
-    if (c->num_tiles > 0) {
-        GradTileKernel stream = grad_stream_lookup(c->L.ld);
-        if (stream)
-            CU(launch(stream, dim3(c->num_tiles), GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * c->L.ld * 4, c->stream, 1,
-                c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.tiles), (int)c->L.ld, c->objective,
-                c->at<float>(c->L.partial), with_loss ? c->at<double>(c->L.loss_partial) : nullptr, nullptr, 0,
-                c->at<i64>(c->L.row_off), c->status()));
-        else
-            CU(launch(grad_tiles_kernel, dim3(c->num_tiles), GRAD_BLOCK, 0, c->stream, 1,
-                c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.tiles), (int)c->L.ld, c->objective,
-                c->at<float>(c->L.partial), with_loss ? c->at<double>(c->L.loss_partial) : nullptr, nullptr, 0,
-                c->at<i64>(c->L.row_off), c->status()));
+// Rows per tile for workers of m(i) rows: short tiles as the layout has them; wide ones as long as it takes for all tiles to be
+// resident at once (a tile more than that would make a second wave of a few blocks).
+template <typename Rows>
+int cut_tile_rows(const ef21_ctx* c, Rows m) {
+    const GradPlan P = grad_plan(c->L.ld);
+    if (!P.resident) return c->L.tile_rows;
+    i64 total = 0, longest = 1;
+    for (int i = 0; i < c->n; ++i) { total += m(i); longest = std::max<i64>(longest, m(i)); }
+    i64 R = std::max<i64>(P.rows, ceil_div(total, 148 * P.resident));
+    for (; R < longest; R += std::max<i64>(1, R / 32)) {
+        i64 tiles = 0;
+        for (int i = 0; i < c->n; ++i) tiles += ceil_div(m(i), R);
+        if (tiles <= 148 * P.resident) break;
+    }
+    return (int)R;
+}
+
+// Tile partials and their sums.  batch_dev: the tau sampled rows of every worker instead of its shard.
+ef21_status launch_grads(ef21_ctx* c, int num_tiles, size_t tiles, size_t tile_begin, bool with_loss, const int* batch_dev, int tau) {
+    const GradPlan P = grad_plan(c->L.ld);
+    if (num_tiles > 0) {
+        CU(launch(P.kernel, dim3((unsigned)num_tiles), P.threads, P.smem, c->stream, 1, c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(),
+                  c->at<RowTile>(tiles), (int)c->L.ld, c->objective, c->at<float>(c->L.partial),
+                  with_loss ? c->at<double>(c->L.loss_partial) : nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status()));
         c->launches += 1;
     }
     dim3 grid((unsigned)ceil_div(c->L.ld, GRAD_FINISH_COLS), (unsigned)c->n);
-    CU(launch(grad_finish_kernel, grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream, 1,
-        c->at<float>(c->L.partial), c->at<int>(c->L.tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d,
-        (int)c->L.ld, c->at<float>(c->L.grad), 0));
+    CU(launch(grad_finish_kernel, grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream, 1, c->at<float>(c->L.partial),
+              c->at<int>(tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d, (int)c->L.ld, c->at<float>(c->L.grad), tau));
     c->launches += 1;
-    CU(cudaGetLastError());
     return EF21_OK;
+}
+
+ef21_status enqueue_grads(ef21_ctx* c, bool with_loss) {
+    return launch_grads(c, c->num_tiles, c->L.tiles, c->L.tile_begin, with_loss, nullptr, 0);
 }
 
 // Minibatch gradients (Algorithm 5): worker i averages over the tau rows batch[i][0..tau) of its shard.
 ef21_status enqueue_minibatch_grads(ef21_ctx* c, const int* batch_dev, int tau) {
     if (c->mb_tau != tau) {            // (re)build the tile table of the batch lists
-        const int R = c->L.tile_rows;
+        const int R = cut_tile_rows(c, [&](int) { return (i64)tau; });
         c->mb_tiles.clear();
         c->mb_tile_begin.assign(c->n + 1, 0);
         for (int i = 0; i < c->n; ++i) {
@@ -524,22 +546,7 @@ ef21_status enqueue_minibatch_grads(ef21_ctx* c, const int* batch_dev, int tau) 
         CU(cudaStreamSynchronize(c->stream));      // the host vectors may be rebuilt by the next call
         c->mb_tau = tau;
     }
-    GradTileKernel stream = grad_stream_lookup(c->L.ld);
-    if (stream)
-        CU(launch(stream, dim3((unsigned)c->mb_tiles.size()), GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * c->L.ld * 4, c->stream, 1,
-            c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.mb_tiles), (int)c->L.ld, c->objective,
-            c->at<float>(c->L.partial), nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status()));
-    else
-        CU(launch(grad_tiles_kernel, dim3((unsigned)c->mb_tiles.size()), GRAD_BLOCK, 0, c->stream, 1,
-            c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(), c->at<RowTile>(c->L.mb_tiles), (int)c->L.ld, c->objective,
-            c->at<float>(c->L.partial), nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status()));
-    dim3 grid((unsigned)ceil_div(c->L.ld, GRAD_FINISH_COLS), (unsigned)c->n);
-    CU(launch(grad_finish_kernel, grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream, 1,
-        c->at<float>(c->L.partial), c->at<int>(c->L.mb_tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d,
-        (int)c->L.ld, c->at<float>(c->L.grad), tau));
-    c->launches += 2;
-    CU(cudaGetLastError());
-    return EF21_OK;
+    return launch_grads(c, (int)c->mb_tiles.size(), c->L.mb_tiles, c->L.mb_tile_begin, false, batch_dev, tau);
 }
 
 // Whether the handle's rounds take the one-pass Top-k of long vectors.
@@ -715,7 +722,7 @@ ef21_status finish_load(ef21_ctx* c, const i64* row_offsets_host) {
     c->row_off.assign(row_offsets_host, row_offsets_host + c->n + 1);
     c->tiles.clear();
     c->tile_begin.assign(c->n + 1, 0);
-    const int R = c->L.tile_rows;
+    const int R = cut_tile_rows(c, [&](int i) { return c->row_off[i + 1] - c->row_off[i]; });
     for (int i = 0; i < c->n; ++i) {
         c->tile_begin[i] = (int)c->tiles.size();
         for (i64 r = c->row_off[i]; r < c->row_off[i + 1]; r += R) {

@@ -5,8 +5,9 @@
 //   rho_r = -y_r / (1 + exp(y_r a_r.x)).
 //
 // Rows are cut into tiles that never straddle two workers; one block handles one tile and leaves the
-// tile's partial sum of rho_r a_r.  Rows of up to 1,024 columns go through grad_stream_kernel (one
-// read of every row, rows held in registers between the margin and the accumulation); wider rows
+// tile's partial sum of rho_r a_r.  Rows of up to 512 columns go through grad_stream_kernel (one
+// read of every row, rows held in registers between the margin and the accumulation), rows of up to
+// 8,192 through grad_wide_kernel (the same with the block sharing a row); wider rows
 // through grad_tiles_kernel: a warp per row forms the margin a_r.x and the residual rho_r, then
 // every thread owns column chunks and accumulates rho_r a_r over the tile's rows in ascending row
 // order (the second sweep hits L1/L2).  A second kernel adds the tile partials of a worker in a
@@ -104,7 +105,7 @@ grad_tiles_kernel(const float* __restrict__ A, const float* __restrict__ y, cons
     }
 }
 
-// The same tile partials for rows of up to 1,024 columns, from ONE read of every row: a warp takes RB rows
+// The same tile partials for rows of up to 512 columns, from ONE read of every row: a warp takes RB rows
 // at a time into registers (CHUNKS float4 per lane and row), forms the RB margins by a transposed warp
 // reduction, the residuals, and adds rho_r a_r from the registers into its own accumulator; the warps'
 // accumulators are added in ascending warp order.  RB * CHUNKS * 16 bytes per lane are in flight per warp,
@@ -121,7 +122,7 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
     pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
     constexpr int SH = (RB == 32) ? 0 : (RB == 16 ? 1 : (RB == 8 ? 2 : (RB == 4 ? 3 : 4)));    // log2(32/RB)
     constexpr int WARPS = GRAD_STREAM_BLOCK / 32;
-    static_assert(RB == 2 || RB == 4 || RB == 8 || RB == 16, "RB");
+    static_assert(RB == 4 || RB == 8 || RB == 16, "RB");
     static_assert(RB * CHUNKS <= 16, "register budget");
     extern __shared__ __align__(16) unsigned char grad_smem[];
     float* red = reinterpret_cast<float*>(grad_smem);                       // [WARPS][ld]
@@ -217,6 +218,113 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
             sum.z = __fadd_rn(sum.z, o.z); sum.w = __fadd_rn(sum.w, o.w);
         }
         out[c] = sum;
+    }
+}
+
+// Rows of 513 to 8,192 columns, one read of every row: the whole block works on RB rows at a time, thread t holds the float4 columns
+// t, t + 256, ... of each in registers; the margins are summed over the block (transposed warp reduction, then over the warps
+// through shared memory, one barrier), every warp forms the residuals, and rho_r a_r is added from the registers.  The next RB
+// rows are on their way meanwhile (a second register buffer: 40-80 KB per SM in flight), and a block goes through a long
+// tile, so that few partials are written (6,000 x 5,001: 65 us with a tile of three rows per block, two sweeps and 40 MB of
+// partials; bound by reading the rows).
+constexpr int GRAD_WIDE_BLOCK = 256;
+__host__ __device__ constexpr int grad_wide_rows(int nc) { return nc == 1 ? 8 : (nc <= 5 ? 4 : 2); }
+
+template <int NC>
+__global__ void __launch_bounds__(GRAD_WIDE_BLOCK, NC <= 2 ? 2 : 1)
+grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
+                 const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
+                 double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
+                 const i64* __restrict__ row_off, unsigned* __restrict__ status) {
+    pdl_trigger();
+    pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
+    constexpr int RB = grad_wide_rows(NC), WARPS = GRAD_WIDE_BLOCK / 32;
+    constexpr int LOG_GROUP = RB == 8 ? 2 : (RB == 4 ? 3 : 4);                  // log2(32 / RB): lanes that end up with one row
+    __shared__ float red[2][WARPS][RB];
+    const RowTile t = tiles[blockIdx.x];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int chunks = ld >> 2;
+    const i64 lo = gather ? row_off[t.worker] : 0, m = gather ? row_off[t.worker + 1] - lo : 0;
+    auto row_id = [&](int r) -> i64 {
+        if (!gather) return t.row0 + r;
+        i64 pick = gather[(i64)t.worker * gather_pitch + t.row0 + r];
+        if (pick < 0 || pick >= m) { record_error(status, 1u /* EF21_ERR_INVALID_ARG */); pick = 0; }
+        return lo + pick;
+    };
+    float4 xr[NC], acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const int at = tid + c * GRAD_WIDE_BLOCK;
+        xr[c] = at < chunks ? reinterpret_cast<const float4*>(x)[at] : make_float4(0.f, 0.f, 0.f, 0.f);
+        acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    double loss_acc = 0.0;
+    float4 a[2][RB][NC];
+    float yb[2];                                               // label of the row whose margin this lane ends up with
+    auto load = [&](int r0, float4 (&buf)[RB][NC], float& label) {
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const bool in = r0 + r < t.rows;
+            const float4* __restrict__ src = reinterpret_cast<const float4*>(A + (in ? row_id(r0 + r) : 0) * (i64)ld);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const int at = tid + c * GRAD_WIDE_BLOCK;
+                buf[r][c] = in && at < chunks ? __ldg(src + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        const int mine = r0 + (lane >> LOG_GROUP);
+        label = mine < t.rows ? __ldg(y + row_id(mine)) : 0.f;
+    };
+    auto use = [&](int r0, int half, const float4 (&buf)[RB][NC], float label) {
+        float pd[RB];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            float z = 0.f;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) z = dot4(buf[r][c], xr[c], z);
+            pd[r] = z;
+        }
+        const float zw = reduce_rows<RB>(pd, lane);             // this warp's part of the margin of row lane >> LOG_GROUP
+        if ((lane & ((1 << LOG_GROUP) - 1)) == 0) red[half][warp][lane >> LOG_GROUP] = zw;
+        __syncthreads();
+        float z = red[half][0][lane >> LOG_GROUP];
+#pragma unroll
+        for (int w = 1; w < WARPS; ++w) z += red[half][w][lane >> LOG_GROUP];
+        const float rho = loss_residual(objective, label, z);   // 0 for a row past the end (y = 0, a = 0)
+        if (loss_partial && warp == 0 && (lane & ((1 << LOG_GROUP) - 1)) == 0 && r0 + (lane >> LOG_GROUP) < t.rows) {
+            if (objective == 0) {
+                const double u = -(double)label * (double)z;
+                loss_acc += (u > 0.0 ? u : 0.0) + log1p(exp(-fabs(u)));
+            } else {
+                const double e = (double)z - (double)label;
+                loss_acc += e * e;
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+            const float pr = __shfl_sync(0xffffffffu, rho, r << LOG_GROUP);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c] = fma4(pr, buf[r][c], acc[c]);
+        }
+    };
+    load(0, a[0], yb[0]);
+#pragma unroll 1
+    for (int r0 = 0; r0 < t.rows; r0 += 2 * RB) {
+        load(r0 + RB, a[1], yb[1]);
+        use(r0, 0, a[0], yb[0]);
+        if (r0 + RB >= t.rows) break;
+        load(r0 + 2 * RB, a[0], yb[0]);
+        use(r0 + RB, 1, a[1], yb[1]);
+    }
+    float4* __restrict__ out = reinterpret_cast<float4*>(partial + (i64)blockIdx.x * ld);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const int at = tid + c * GRAD_WIDE_BLOCK;
+        if (at < chunks) out[at] = acc[c];
+    }
+    if (loss_partial && warp == 0) {
+        loss_acc = warp_sum(loss_acc);
+        if (lane == 0) loss_partial[blockIdx.x] = loss_acc;
     }
 }
 
