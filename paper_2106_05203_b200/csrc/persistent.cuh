@@ -48,9 +48,11 @@ constexpr int PK_MAX_MSGS = 2048;       // n*k words staged in shared memory
 constexpr int PK_SCAN_MAX_MSGS = 128;   // up to this many messages every coordinate thread scans them all
 constexpr int PK_TABLE_MAX_BYTES = 64 * 1024;   // largest [n][ld] message table kept in shared memory
 constexpr unsigned PK_NO_ENTRY = 0xffffffffu;   // table cell without a message (a NaN pattern no finite value has)
-// where a block's rows come from: registers / shared memory (loaded once), global memory (every iteration), or global
-// memory through a per-iteration list of sampled row numbers (stochastic variant, Algorithm 5)
-enum { PK_SRC_REG = 0, PK_SRC_SMEM = 1, PK_SRC_GMEM = 2, PK_SRC_SAMPLED = 3 };
+// where a block's rows come from: registers / shared memory (loaded once), global memory (every iteration), global
+// memory through a per-iteration list of sampled row numbers (stochastic variant, Algorithm 5), or global memory through
+// a ring in shared memory (RowRing)
+enum { PK_SRC_REG = 0, PK_SRC_SMEM = 1, PK_SRC_GMEM = 2, PK_SRC_SAMPLED = 3, PK_SRC_RING = 4 };
+constexpr int PK_RING_MAX_STAGES = 8;
 
 struct PersistParams {
     const float* A;            // [N][ld], padded, read-only
@@ -74,6 +76,7 @@ struct PersistParams {
     int* plus_choice;          // [n] EF21+: branch taken at the final iteration (0 Markov compressor, 1 plain)
     const int* batch;          // stochastic variant (Algorithm 5): [steps][n][tau] row numbers inside each shard; null: all rows
     int tau;                   // rows per worker and iteration of the stochastic variant
+    int ring_stages;           // RING source: batches in flight per warp
 };
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
@@ -120,6 +123,67 @@ __device__ __forceinline__ void st_async_f4(unsigned remote_dst, float4 v, unsig
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                  ::"r"(remote_dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(remote_bar) : "memory");
 }
+
+// Rows from global memory through shared memory: every warp owns a ring of `stages` batches, filled by bulk copies (a batch is
+// contiguous) that one lane issues as soon as the batch before it in the stage has been taken into registers.  The rows are
+// the same in every iteration, so the ring runs on from one sweep into the next: while a block exchanges messages, the
+// first batches of its next sweep arrive (a third of a block's rows on the w8a-shaped workload), and neither registers nor
+// issue slots are spent on loads in flight.  Every wait is bounded; a wait that gives up records EF21_ERR_TIMEOUT.
+struct RowRing {
+    float* stage0;                 // this warp's first stage
+    unsigned long long* bars;      // its barriers, one per stage
+    const float* rows;             // the block's slice
+    int batch_words, rows_total, batch_rows, ld, first, step, count;    // batches first, first + step, ... (`count` of them)
+    int stages, at;                // the stage the next batch is taken from
+    unsigned parity;
+    int next;                      // which batch of the sweep (0 .. count - 1) is issued next
+    long long to_issue, to_take;
+
+    __device__ __forceinline__ void issue(int stage) {
+        const int b = first + next * step;
+        next = next + 1 == count ? 0 : next + 1;
+        --to_issue;
+        const unsigned bytes = (unsigned)min(batch_rows, rows_total - b * batch_rows) * (unsigned)ld * 4u;
+        const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage), dst = (unsigned)__cvta_generic_to_shared(stage0 + stage * batch_words);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(dst), "l"(rows + (i64)b * batch_words), "r"(bytes), "r"(bar) : "memory");
+    }
+    // all lanes keep the same counters; lane 0 issues
+    __device__ __forceinline__ void start(int lane) {
+        at = 0; parity = 0u; next = 0;
+        const int n = (int)min((long long)stages, to_issue);
+        for (int q = 0; q < n; ++q) {
+            if (lane == 0) issue(q); else { next = next + 1 == count ? 0 : next + 1; --to_issue; }
+        }
+    }
+    __device__ __forceinline__ bool wait(unsigned limit, unsigned* status) {
+        const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + at);
+        unsigned spins = 0u, ok = 0u;
+        while (true) {
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+            if (ok) return true;
+            if (++spins > limit) { record_error(status, 5u /* EF21_ERR_TIMEOUT */); return false; }
+        }
+    }
+    __device__ __forceinline__ const float* stage() const { return stage0 + at * batch_words; }
+    // the batch of the current stage is in registers: the stage takes the next one
+    __device__ __forceinline__ void taken(int lane) {
+        __syncwarp();
+        if (to_issue > 0) { if (lane == 0) issue(at); else { next = next + 1 == count ? 0 : next + 1; --to_issue; } }
+        --to_take;
+        if (++at == stages) { at = 0; parity ^= 1u; }
+    }
+    // nothing may be in flight when the block ends (an aborted run leaves batches behind)
+    __device__ __forceinline__ void drain(unsigned limit, unsigned* status) {
+        long long left = to_take - to_issue;
+        for (; left > 0; --left) {
+            if (!wait(limit, status)) return;
+            if (++at == stages) { at = 0; parity ^= 1u; }
+        }
+    }
+};
 
 // Named barriers of a block (id 1..15; 0 belongs to __syncthreads): `count` threads take part, some only announce
 // their arrival (producers), the others wait for everybody (consumers).  Shared-memory writes made before the
