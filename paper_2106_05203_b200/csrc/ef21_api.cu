@@ -756,6 +756,7 @@ ef21_status finish_load(ef21_ctx* c, const i64* row_offsets_host) {
 
 // From two entries per worker on, the received messages are scattered into a [n][ld] table in shared
 // memory (if that table is small): aggregation then costs n reads per coordinate instead of n*k.
+constexpr int PK_STATIC_SMEM = 2048;                  // room for the kernels' static shared memory
 constexpr i64 PK_RING_MAX_BYTES = (i64)110 << 20;      // shards that an L2 of 126 MB holds
 
 bool pk_use_table(int n, int ld, int k) { return k >= 2 && (size_t)n * ld * 4 <= (size_t)PK_TABLE_MAX_BYTES; }
@@ -837,7 +838,7 @@ PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau) {
             rb = max_rb512; threads = 512;
             const size_t with_slice = roles ? pk_roles_smem_bytes(ld, C, PK_SRC_SMEM, rows_cta, threads)
                                             : pk_smem_bytes(plus, c->n, c->k, ld, C, nmsg, PK_SRC_SMEM, rows_cta, threads);
-            src = with_slice <= (size_t)max_smem - 1024 ? PK_SRC_SMEM : PK_SRC_GMEM;
+            src = with_slice <= (size_t)max_smem - PK_STATIC_SMEM ? PK_SRC_SMEM : PK_SRC_GMEM;
         }
         if (c->pk_threads > 0) {
             threads = c->pk_threads;
@@ -861,7 +862,7 @@ PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau) {
                                       : pk_smem_bytes(plus, c->n, c->k, ld, C, nmsg, src, rows_cta, threads);
             for (int cand = max_rb512; cand >= 8 && stages < 2; cand /= 2) {
                 stages = 0;
-                while (stages < PK_RING_MAX_STAGES && rest + pk_ring_bytes(ld, threads, cand, stages + 1) <= (size_t)max_smem - 1024) ++stages;
+                while (stages < PK_RING_MAX_STAGES && rest + pk_ring_bytes(ld, threads, cand, stages + 1) <= (size_t)max_smem - PK_STATIC_SMEM) ++stages;
                 if (stages >= 2) { src = PK_SRC_RING; rb = cand; }
             }
             if (src != PK_SRC_RING) stages = 0;
@@ -896,7 +897,7 @@ PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau) {
         const size_t smem = (roles ? pk_roles_smem_bytes(ld, C, src, rows_cta, threads)
                                    : pk_smem_bytes(plus, c->n, c->k, ld, C, nmsg, src, rows_cta, threads)) +
                             (src == PK_SRC_RING ? pk_ring_bytes(ld, threads, rb, stages) : 0);
-        if (smem > (size_t)max_smem - 1024) continue;
+        if (smem > (size_t)max_smem - PK_STATIC_SMEM) continue;
         PersistKernel kern;
         if (roles)
             kern = c->variant == EF21_VARIANT_EF ? pk_lookup_ef(chunk_slots, rb, src, threads, extra)
@@ -909,7 +910,7 @@ PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau) {
         const int block_threads = threads;
         // the device's opt-in limit (less the kernel's static part), so that no other handle's plan for the same
         // kernel can lower it under this one's need
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - 1024) != cudaSuccess) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - PK_STATIC_SMEM) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -1571,7 +1572,7 @@ ef21_status ef21_selftest_exchange_floor(ef21_ctx* c, int32_t steps) {
     int dev = 0, max_smem = 0;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    CU(cudaFuncSetAttribute(P.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - 1024));
+    CU(cudaFuncSetAttribute(P.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - PK_STATIC_SMEM));
     return run_persistent(c, P, steps);
 }
 
