@@ -70,7 +70,8 @@ __global__ void agg_offsets_kernel(const int* __restrict__ idx, int n, int k, in
 
 // What an aggregation does to x besides: nothing; x <- fma(-gamma, g^t, x) before g changes (Algorithm 2 updates x from g^t, then
 // g^{t+1} from the messages); or the x update of the following iteration, from the new g.
-enum { AGG_X_KEEP = 0, AGG_X_BEFORE = 1, AGG_X_AFTER = 2 };
+// AGG_INIT (table kernel only): x stays, and g starts from zero.
+enum { AGG_X_KEEP = 0, AGG_X_BEFORE = 1, AGG_X_AFTER = 2, AGG_INIT = 3 };
 
 // One block per tile of AGG_TILE coordinates.
 template <int XMODE>
@@ -271,7 +272,8 @@ aggregate_table_kernel(const int* __restrict__ idx, const float* __restrict__ va
     __syncthreads();
     const int t = threadIdx.x, j = j0 + t;
     if (t >= AGG_TABLE_COLS || j >= d) return;
-    const float old = g[j], xj = XMODE == AGG_X_KEEP ? 0.f : x[j];
+    constexpr bool MOVE_X = XMODE == AGG_X_BEFORE || XMODE == AGG_X_AFTER;
+    const float old = XMODE == AGG_INIT ? 0.f : g[j], xj = MOVE_X ? x[j] : 0.f;
     float s = 0.f; bool hit = false;
 #pragma unroll 8
     for (int i = 0; i < n; ++i) {
@@ -280,8 +282,8 @@ aggregate_table_kernel(const int* __restrict__ idx, const float* __restrict__ va
         if (w != AGG_NO_ENTRY) { s = sum; hit = true; }
     }
     const float now = hit ? __fadd_rn(old, __fmul_rn(s, inv_n)) : old;
-    if (XMODE != AGG_X_KEEP) x[j] = fmaf(-gamma, XMODE == AGG_X_BEFORE ? old : now, xj);
-    if (hit) g[j] = now;
+    if (MOVE_X) x[j] = fmaf(-gamma, XMODE == AGG_X_BEFORE ? old : now, xj);
+    if (hit || XMODE == AGG_INIT) g[j] = now;
 }
 
 // x <- fma(-gamma, g, x), elementwise.

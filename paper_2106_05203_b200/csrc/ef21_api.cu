@@ -252,7 +252,7 @@ struct ef21_ctx {
     char* ws;
     Layout L;
     bool shards_loaded, inited;
-    int num_tiles;
+    int num_tiles, worker_tiles;        // gradient tiles: all, and the most that one worker has
     int path, last_path;
     bool agg_off_ready;                 // the last selection already wrote the aggregation's tile offsets
     int pk_cluster, pk_rb, pk_src, pk_threads;      // forced persistent-kernel shape (0 / -1 = automatic)
@@ -504,28 +504,61 @@ int cut_tile_rows(const ef21_ctx* c, Rows m) {
     return (int)R;
 }
 
-// Tile partials and their sums.  batch_dev: the tau sampled rows of every worker instead of its shard.
-ef21_status launch_grads(ef21_ctx* c, int num_tiles, size_t tiles, size_t tile_begin, bool with_loss, const int* batch_dev, int tau) {
+// What the gradients of a step are taken over: the shards' tiles, or those of the minibatch lists.
+struct GradSource { int num_tiles, worker_tiles; size_t tiles, tile_begin; const int* batch_dev; int tau; };
+
+GradSource full_source(const ef21_ctx* c) { return {c->num_tiles, c->worker_tiles, c->L.tiles, c->L.tile_begin, nullptr, 0}; }
+
+ef21_status launch_grad_tiles(ef21_ctx* c, const GradSource& G, bool with_loss) {
+    if (G.num_tiles == 0) return EF21_OK;
     const GradPlan P = grad_plan(c->L.ld);
-    if (num_tiles > 0) {
-        CU(launch(P.kernel, dim3((unsigned)num_tiles), P.threads, P.smem, c->stream, 1, c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(),
-                  c->at<RowTile>(tiles), (int)c->L.ld, c->objective, c->at<float>(c->L.partial),
-                  with_loss ? c->at<double>(c->L.loss_partial) : nullptr, batch_dev, tau, c->at<i64>(c->L.row_off), c->status()));
-        c->launches += 1;
-    }
+    CU(launch(P.kernel, dim3((unsigned)G.num_tiles), P.threads, P.smem, c->stream, 1, c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(),
+              c->at<RowTile>(G.tiles), (int)c->L.ld, c->objective, c->at<float>(c->L.partial),
+              with_loss ? c->at<double>(c->L.loss_partial) : nullptr, G.batch_dev, G.tau, c->at<i64>(c->L.row_off), c->status()));
+    c->launches += 1;
+    return EF21_OK;
+}
+
+ef21_status launch_grad_finish(ef21_ctx* c, const GradSource& G) {
     dim3 grid((unsigned)ceil_div(c->L.ld, GRAD_FINISH_COLS), (unsigned)c->n);
     CU(launch(grad_finish_kernel, grid, GRAD_FINISH_COLS * GRAD_FINISH_LANES, 0, c->stream, 1, c->at<float>(c->L.partial),
-              c->at<int>(tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d, (int)c->L.ld, c->at<float>(c->L.grad), tau));
+              c->at<int>(G.tile_begin), c->at<i64>(c->L.row_off), c->x(), c->lambda, (int)c->d, (int)c->L.ld, c->at<float>(c->L.grad), G.tau));
+    c->launches += 1;
+    return EF21_OK;
+}
+
+// Whether the Top-k kernel can form the gradients from the tile partials itself (one block per worker, two columns per thread):
+// vectors of up to 512 columns with up to 32 tiles per worker, where a thread needs no more dependent rounds of reading than
+// in a kernel of its own and a launch is saved.  (Rows of 600 to 1,000 columns took 2 us longer that way, 5,001 columns 8 us: a
+// kernel of its own spreads the sums over the device.)
+bool select_can_form_grads(const ef21_ctx* c, const GradSource& G, TcShape& S) {
+    return tc_shape(c->n, c->d, S) && S.threads == 256 && c->d <= 512 && G.worker_tiles <= 4 * GRAD_FINISH_LANES;
+}
+
+// Tile partials -> messages and worker states in one kernel (see select_can_form_grads).  mode: TC_DIFF, TC_EF, or TC_PLAIN for
+// g_i = C(grad_i) from nothing.
+ef21_status enqueue_grad_select(ef21_ctx* c, const GradSource& G, const TcShape& S, int mode) {
+    typedef void (*Kernel)(const TcArgs);
+    static const Kernel kernels[3] = {tc_topk_kernel<TC_PLAIN, 1, 256, false, true>, tc_topk_kernel<TC_DIFF, 1, 256, false, true>,
+                                      tc_topk_kernel<TC_EF, 1, 256, false, true>};
+    const Kernel kern = kernels[mode];
+    TcArgs p = {};
+    p.b = c->gi(); p.pitch_b = c->L.ld; p.d = (int)c->d; p.k = c->k; p.slice = S.slice; p.gamma = c->gamma;
+    p.idx_out = c->msg_idx(); p.val_out = c->msg_val(); p.apply = c->gi(); p.pitch_apply = c->L.ld; p.status = c->status();
+    p.partial = c->at<float>(c->L.partial); p.tile_begin = c->at<int>(G.tile_begin); p.row_off = c->at<i64>(c->L.row_off); p.x = c->x();
+    p.lambda = c->lambda; p.ld = (int)c->L.ld; p.batch_rows = G.tau;
+    CU(launch(kern, dim3((unsigned)c->n), (unsigned)S.threads, tc_smem_bytes(1, S.slice), c->stream, 1, p));
     c->launches += 1;
     return EF21_OK;
 }
 
 ef21_status enqueue_grads(ef21_ctx* c, bool with_loss) {
-    return launch_grads(c, c->num_tiles, c->L.tiles, c->L.tile_begin, with_loss, nullptr, 0);
+    EF(launch_grad_tiles(c, full_source(c), with_loss));
+    return launch_grad_finish(c, full_source(c));
 }
 
 // Minibatch gradients (Algorithm 5): worker i averages over the tau rows batch[i][0..tau) of its shard.
-ef21_status enqueue_minibatch_grads(ef21_ctx* c, const int* batch_dev, int tau) {
+ef21_status minibatch_source(ef21_ctx* c, const int* batch_dev, int tau, GradSource& G) {
     if (c->mb_tau != tau) {            // (re)build the tile table of the batch lists
         const int R = cut_tile_rows(c, [&](int) { return (i64)tau; });
         c->mb_tiles.clear();
@@ -546,7 +579,10 @@ ef21_status enqueue_minibatch_grads(ef21_ctx* c, const int* batch_dev, int tau) 
         CU(cudaStreamSynchronize(c->stream));      // the host vectors may be rebuilt by the next call
         c->mb_tau = tau;
     }
-    return launch_grads(c, (int)c->mb_tiles.size(), c->L.mb_tiles, c->L.mb_tile_begin, false, batch_dev, tau);
+    int worker_tiles = 0;
+    for (int i = 0; i < c->n; ++i) worker_tiles = std::max(worker_tiles, c->mb_tile_begin[i + 1] - c->mb_tile_begin[i]);
+    G = {(int)c->mb_tiles.size(), worker_tiles, c->L.mb_tiles, c->L.mb_tile_begin, batch_dev, tau};
+    return EF21_OK;
 }
 
 // Whether the handle's rounds take the one-pass Top-k of long vectors.
@@ -587,10 +623,15 @@ ef21_status enqueue_round_aggregate(ef21_ctx* c, int xmode) {
     return enqueue_aggregate_into(c, c->g(), 1.0f / (float)c->n, xmode);
 }
 
+bool agg_by_table(const ef21_ctx* c) {
+    return c->d <= AGG_TABLE_MAX_D && c->n <= AGG_TABLE_MAX_N && (i64)c->n * c->k <= AGG_TABLE_MAX_MESSAGES;
+}
+
 // target_j += factor * (sum over workers, ascending, of the values sent for coordinate j).
 ef21_status enqueue_aggregate_into(ef21_ctx* c, float* target, float factor, int xmode) {
-    if (c->d <= AGG_TABLE_MAX_D && c->n <= AGG_TABLE_MAX_N && (i64)c->n * c->k <= AGG_TABLE_MAX_MESSAGES) {
+    if (agg_by_table(c)) {
         auto kern = xmode == AGG_X_KEEP ? aggregate_table_kernel<AGG_X_KEEP>
+                    : xmode == AGG_INIT ? aggregate_table_kernel<AGG_INIT>
                                         : (xmode == AGG_X_BEFORE ? aggregate_table_kernel<AGG_X_BEFORE> : aggregate_table_kernel<AGG_X_AFTER>);
         const size_t smem = (size_t)c->n * AGG_TABLE_COLS * 4;
         EF(allow_smem(reinterpret_cast<const void*>(kern), (size_t)AGG_TABLE_MAX_N * AGG_TABLE_COLS * 4));
@@ -735,6 +776,8 @@ ef21_status finish_load(ef21_ctx* c, const i64* row_offsets_host) {
     }
     c->tile_begin[c->n] = (int)c->tiles.size();
     c->num_tiles = (int)c->tiles.size();
+    c->worker_tiles = 0;
+    for (int i = 0; i < c->n; ++i) c->worker_tiles = std::max(c->worker_tiles, c->tile_begin[i + 1] - c->tile_begin[i]);
     if ((i64)c->num_tiles > c->L.max_tiles) return EF21_ERR_WORKSPACE;
     // a captured launch-path iteration has the old tile count baked into its grid
     if (c->iter_graph) { cudaGraphExecDestroy(c->iter_graph); c->iter_graph = nullptr; }
@@ -1049,7 +1092,7 @@ ef21_status ef21_create(ef21_ctx** out, int32_t n, int64_t d, int32_t k, float g
     if (cudaGetDevice(&c->device) != cudaSuccess) { cudaGetLastError(); c->device = -1; }
     c->ws = static_cast<char*>(workspace_dev);
     c->L = L;
-    c->shards_loaded = false; c->inited = false; c->num_tiles = 0;
+    c->shards_loaded = false; c->inited = false; c->num_tiles = 0; c->worker_tiles = 0;
     c->path = EF21_PATH_AUTO; c->last_path = 0; c->launches = 0;
     c->pk_cluster = 0; c->pk_rb = 0; c->pk_src = -1; c->pk_threads = 0; c->agg_off_ready = false;
     c->pk_used_cluster = c->pk_used_rb = 0; c->pk_used_src = -1; c->pk_used_threads = 0;
@@ -1123,6 +1166,15 @@ ef21_status ef21_init(ef21_ctx* c, int32_t mode) {
         return EF21_OK;
     }
     if (!c->shards_loaded) return EF21_ERR_STATE;
+    TcShape S;
+    if (mode == EF21_INIT_COMPRESSED && agg_by_table(c) && select_can_form_grads(c, full_source(c), S)) {
+        // three launches: the selection writes g_i whole, the aggregation g
+        EF(launch_grad_tiles(c, full_source(c), false));
+        EF(enqueue_grad_select(c, full_source(c), S, TC_PLAIN));
+        EF(enqueue_round_aggregate(c, AGG_INIT));
+        c->inited = true;
+        return EF21_OK;
+    }
     EF(enqueue_grads(c, false));
     return init_from(c, c->at<float>(c->L.grad), c->L.ld, mode);
 }
@@ -1136,8 +1188,16 @@ ef21_status ef21_init_grads(ef21_ctx* c, const float* V_dev, int32_t mode) {
 // One iteration of ef21_step on the launch path, as plain kernel launches on the handle's stream.  The x update that opens the
 // iteration has already been enqueued (or does not exist: Algorithm 4); xmode AGG_X_AFTER: the one of the next iteration is
 // made by the kernel that updates g.
-static ef21_status enqueue_launch_iteration(ef21_ctx* c, int xmode) {
-    EF(enqueue_grads(c, false));
+static ef21_status enqueue_launch_iteration(ef21_ctx* c, const GradSource& G, int xmode) {
+    EF(launch_grad_tiles(c, G, false));
+    TcShape S;
+    if (c->variant != EF21_VARIANT_EF21_PLUS && select_can_form_grads(c, G, S)) {
+        c->agg_off_ready = false;
+        const bool ef = c->variant == EF21_VARIANT_EF;
+        EF(enqueue_grad_select(c, G, S, ef ? TC_EF : TC_DIFF));
+        return ef ? enqueue_aggregate_into(c, c->x(), -(1.0f / (float)c->n), AGG_X_KEEP) : enqueue_round_aggregate(c, xmode);
+    }
+    EF(launch_grad_finish(c, G));
     if (c->variant == EF21_VARIANT_EF) return enqueue_ef_round(c, c->at<float>(c->L.grad), c->L.ld);
     if (c->variant == EF21_VARIANT_EF21_PLUS) return enqueue_plus_round(c, c->at<float>(c->L.grad), c->L.ld, xmode);
     return enqueue_round(c, c->at<float>(c->L.grad), c->L.ld, xmode);
@@ -1165,7 +1225,7 @@ static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
             if (ok) {
                 cudaStream_t user_stream = c->stream;
                 c->stream = c->cap_stream;
-                const ef21_status st = enqueue_launch_iteration(c, AGG_X_AFTER);
+                const ef21_status st = enqueue_launch_iteration(c, full_source(c), AGG_X_AFTER);
                 c->stream = user_stream;
                 ok = cudaStreamEndCapture(c->cap_stream, &graph) == cudaSuccess && st == EF21_OK && graph != nullptr;
             }
@@ -1190,7 +1250,7 @@ static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
     } else {
         cudaGetLastError();
     }
-    for (; done < steps; ++done) EF(enqueue_launch_iteration(c, done + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
+    for (; done < steps; ++done) EF(enqueue_launch_iteration(c, full_source(c), done + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;
 }
@@ -1288,8 +1348,9 @@ ef21_status ef21_step_minibatches(ef21_ctx* c, const int32_t* batches_dev, int32
     if (c->path == EF21_PATH_PERSISTENT) return EF21_ERR_UNSUPPORTED;
     EF(enqueue_x_update(c));
     for (int t = 0; t < steps; ++t) {
-        EF(enqueue_minibatch_grads(c, batches_dev + (size_t)t * c->n * tau, tau));
-        EF(enqueue_round(c, c->at<float>(c->L.grad), c->L.ld, t + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
+        GradSource G;
+        EF(minibatch_source(c, batches_dev + (size_t)t * c->n * tau, tau, G));
+        EF(enqueue_launch_iteration(c, G, t + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
     }
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;

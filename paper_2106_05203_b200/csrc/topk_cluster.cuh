@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "grad.cuh"
 
 namespace ef21 {
 
@@ -41,10 +42,13 @@ struct TcArgs {
     int d, k, slice;
     float gamma;
     int* idx_out; float* val_out;
-    float* apply; i64 pitch_apply;          // TC_DIFF: receives b + v on the selected coordinates; TC_EF, TC_SENT: v - v there; may be null
+    float* apply; i64 pitch_apply;          // TC_DIFF: receives b + v on the selected coordinates; TC_EF, TC_SENT: v - v there; TC_PLAIN: v there and 0 elsewhere; may be null
     unsigned* status;
     unsigned long long* cut_out;            // [batch]: an entry is selected if and only if (key << 32 | ~index) >= cut; may be null
     unsigned* slow_count;                   // counts the vectors with more than TC_LIST entries equal to T; may be null
+    // GRAD only: a is the mean of worker i's tile partials plus the regulariser term at x (the sums of grad_finish_kernel)
+    const float* partial; const int* tile_begin; const i64* row_off; const float* x;
+    float lambda; int ld, batch_rows;
     // STREAM only: vectors whose flag (one word every flag_pitch words) is zero are left alone; tile_off (may be null):
     // [batch][ntiles + 1] first message position of every `tile` coordinates
     const unsigned* flag; int flag_pitch, batch;
@@ -90,7 +94,8 @@ __device__ __noinline__ void tc_find_bin(const unsigned* hist, unsigned need, un
 }
 
 // STREAM: the vector is longer than the cluster's shared memory; it stays in global memory and every sweep reads it again.
-template <int MODE, int C, int THREADS, bool STREAM>
+// GRAD: the local gradients are formed from the tile partials on the way in (no kernel and no array for them).
+template <int MODE, int C, int THREADS, bool STREAM, bool GRAD>
 __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     namespace cg = cooperative_groups;
     constexpr int WARPS = THREADS / 32;
@@ -113,7 +118,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     auto sync_all = [&]() { if (C > 1) cluster.sync(); else __syncthreads(); };
 
     const int j0 = (int)min((i64)rank * p.slice, (i64)p.d), len = min(p.slice, p.d - j0);
-    const float* __restrict__ av = p.a + (i64)vec * p.pitch_a + j0;
+    const float* __restrict__ av = GRAD ? nullptr : p.a + (i64)vec * p.pitch_a + j0;
     float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + j0;
 #pragma unroll 1
     for (int q = tid; q < TC_BINS; q += THREADS) { hist[q] = 0u; if (C > 1) hsum[q] = 0u; }
@@ -123,6 +128,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     __syncthreads();
     if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // hsum is empty
     if (!STREAM) { pdl_trigger(); pdl_wait(); }
+    float* dense = MODE == TC_PLAIN && !STREAM && p.apply ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
     // entries of bin 0 (zeros and the smallest magnitudes) are not counted: what the other bins leave over is theirs
     auto take = [&](int j, float a, float b) {
         float v = a;
@@ -131,9 +137,43 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         if (MODE == TC_SENT) v = b;
         const unsigned w = __funnelshift_l(__float_as_uint(v), __float_as_uint(v), 1);
         if (!STREAM) ws[j] = w;
+        if (MODE == TC_PLAIN && dense) dense[j] = 0.f;
         if (w >> 21) atomicAdd(&hist[w >> 21], 1u);
     };
-    {
+    if (GRAD) {
+        const int t0 = p.tile_begin[vec], t1 = p.tile_begin[vec + 1];
+        const i64 m = p.batch_rows > 0 ? (i64)p.batch_rows : p.row_off[vec + 1] - p.row_off[vec];
+        // two columns at a time: sixteen partials in flight per thread
+#pragma unroll 1
+        for (int jj = tid; jj < len; jj += 2 * THREADS) {
+            const int js[2] = {jj, min(jj + THREADS, len - 1)};
+            float acc[2][GRAD_FINISH_LANES], b[2], xj[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                b[u] = MODE == TC_PLAIN ? 0.f : bv[js[u]]; xj[u] = p.x[js[u]];
+#pragma unroll
+                for (int q = 0; q < GRAD_FINISH_LANES; ++q) acc[u][q] = 0.f;
+            }
+            const float* row = p.partial + (i64)t0 * p.ld;
+#pragma unroll 1
+            for (int t = t0; t < t1; t += GRAD_FINISH_LANES) {
+#pragma unroll
+                for (int q = 0; q < GRAD_FINISH_LANES; ++q)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (t + q < t1) acc[u][q] = __fadd_rn(acc[u][q], row[(i64)q * p.ld + js[u]]);
+                row += (i64)GRAD_FINISH_LANES * p.ld;
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (u == 1 && jj + THREADS >= len) break;
+#pragma unroll
+                for (int q = 1; q < GRAD_FINISH_LANES; ++q) acc[u][0] = __fadd_rn(acc[u][0], acc[u][q]);
+                const float data = m > 0 ? __fdiv_rn(acc[u][0], (float)m) : 0.f;
+                take(js[u], __fadd_rn(data, regulariser_grad(p.lambda, xj[u])), b[u]);
+            }
+        }
+    } else {
         constexpr int U = THREADS == 1024 ? 8 : 4;
         int j = tid;
 #pragma unroll 1
@@ -335,7 +375,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         eq_before += __reduce_add_sync(0xffffffffu, lane < warp ? weq[lane] : 0u);
         int* __restrict__ io = p.idx_out + (i64)vec * p.k;
         float* __restrict__ vo = p.val_out + (i64)vec * p.k;
-        float* app = (MODE != TC_PLAIN && p.apply) ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
+        float* app = p.apply ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
         const unsigned lo = T << 1;
 #pragma unroll 1
         for (int base = w0; base < w1; base += 128) {
@@ -363,7 +403,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
                     flag_nonfinite(p.status, v);
                     if (tie && e0 + 1u == need_ties && p.cut_out)
                         p.cut_out[vec] = ((unsigned long long)T << 32) | (0xffffffffu - (unsigned)(j0 + j + e));
-                    if (app) app[j + e] = MODE == TC_DIFF ? __fadd_rn(app[j + e], v) : __fsub_rn(v, v);
+                    if (app) app[j + e] = MODE == TC_DIFF ? __fadd_rn(app[j + e], v) : (MODE == TC_PLAIN ? __fadd_rn(0.f, v) : __fsub_rn(v, v));
                 }
                 g0 += tie ? 0u : 1u; e0 += tie ? 1u : 0u;
             }
@@ -387,7 +427,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     }
 }
 
-template <int MODE, int C, int THREADS, bool STREAM = false>
+template <int MODE, int C, int THREADS, bool STREAM = false, bool GRAD = false>
 __global__ void __launch_bounds__(THREADS)
 tc_topk_kernel(const __grid_constant__ TcArgs p) {
     if (STREAM) {
@@ -396,11 +436,11 @@ tc_topk_kernel(const __grid_constant__ TcArgs p) {
         pdl_wait();
         for (int vec = (int)(blockIdx.x / (unsigned)C); vec < p.batch; vec += (int)(gridDim.x / (unsigned)C))
             if (p.flag[(i64)vec * p.flag_pitch] != 0u) {
-                tc_vector<MODE, C, THREADS, STREAM>(p, vec);
+                tc_vector<MODE, C, THREADS, STREAM, GRAD>(p, vec);
                 cooperative_groups::this_cluster().sync();
             }
     } else {
-        tc_vector<MODE, C, THREADS, STREAM>(p, (int)(blockIdx.x / (unsigned)C));
+        tc_vector<MODE, C, THREADS, STREAM, GRAD>(p, (int)(blockIdx.x / (unsigned)C));
     }
 }
 
