@@ -240,6 +240,7 @@ bool valid_shape(i64 n, i64 d, i64 k, i64 N) {
 struct PersistPlan {
     bool ok;
     bool roles;         // persistent_roles.inc (the last warp serves the block) instead of whole-block steps
+    bool local;         // all workers in one cluster
     int C, rb, src, chunks, threads, extra, stages;
     size_t smem;
     PersistKernel kernel;
@@ -827,6 +828,15 @@ size_t pk_roles_smem_bytes(int ld, int C, int src, i64 rows_cta, int threads) {
 
 PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau = 0);
 
+PersistKernel persistent_kernel_of(const ef21_ctx* c, bool roles, bool local, int chunks, int rb, int src, int threads, int extra) {
+    const bool ef = c->variant == EF21_VARIANT_EF, plus = c->variant == EF21_VARIANT_EF21_PLUS;
+    auto lookup = roles ? (ef ? (local ? pk_lookup_local_ef : pk_lookup_ef) : (local ? pk_lookup_local_ef21 : pk_lookup_ef21))
+                  : ef  ? (local ? pk_lookup_local_wide_ef : pk_lookup_wide_ef)
+                  : plus ? (local ? pk_lookup_local_plus : pk_lookup_plus)
+                         : (local ? pk_lookup_local_wide_ef21 : pk_lookup_wide_ef21);
+    return lookup(chunks, rb, src, threads, extra);
+}
+
 // Chooses the kernel body, cluster size, block size, rows per batch and the source of the shard rows; checks
 // that all n clusters can be resident at once (the blocks wait on one another through global memory).
 PersistPlan plan_persistent(ef21_ctx* c) {
@@ -839,13 +849,13 @@ PersistPlan plan_persistent(ef21_ctx* c) {
         PersistPlan P = plan_persistent_body(c, true);
         if (P.ok || c->pk_body == 1) return P;
     }
-    if (c->pk_body == 1) { PersistPlan P; P.ok = false; return P; }
+    if (c->pk_body == 1) { PersistPlan P{}; return P; }
     return plan_persistent_body(c, false);
 }
 
 // tau > 0: plan for the stochastic variant (tau sampled rows per worker and iteration, read from global memory).
 PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau) {
-    PersistPlan P; P.ok = false; P.roles = roles;
+    PersistPlan P{}; P.roles = roles;
     const int ld = (int)c->L.ld;
     if (!c->shards_loaded || ld > 512 || c->k > PK_MAX_K || (i64)c->n * c->k > PK_MAX_MSGS) return P;
     const bool plus = c->variant == EF21_VARIANT_EF21_PLUS;
@@ -941,33 +951,35 @@ PersistPlan plan_persistent_body(ef21_ctx* c, bool roles, int tau) {
                                    : pk_smem_bytes(plus, c->n, c->k, ld, C, nmsg, src, rows_cta, threads)) +
                             (src == PK_SRC_RING ? pk_ring_bytes(ld, threads, rb, stages) : 0);
         if (smem > (size_t)max_smem - PK_STATIC_SMEM) continue;
-        PersistKernel kern;
-        if (roles)
-            kern = c->variant == EF21_VARIANT_EF ? pk_lookup_ef(chunk_slots, rb, src, threads, extra)
-                                                   : pk_lookup_ef21(chunk_slots, rb, src, threads, extra);
-        else
-            kern = c->variant == EF21_VARIANT_EF ? pk_lookup_wide_ef(chunk_slots, rb, src, threads, extra)
-                   : (plus ? pk_lookup_plus(chunk_slots, rb, src, threads, extra)
-                           : pk_lookup_wide_ef21(chunk_slots, rb, src, threads, extra));
-        if (!kern) continue;
-        const int block_threads = threads;
-        // the device's opt-in limit (less the kernel's static part), so that no other handle's plan for the same
-        // kernel can lower it under this one's need
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - PK_STATIC_SMEM) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
+        // All workers in one cluster where it holds them and the kernel exists (rows in registers, or sampled), else a cluster per
+        // worker.  A message then takes a store to shared memory instead of a trip through L2: 4 workers, d = 64, Top-4 2.55 ->
+        // 2.17 us per iteration, 8 x 64 Top-2 2.45 -> 1.99, 10 x 112 Top-1 2.23 -> 2.00, 32 sampled rows 2.32 -> 2.00.  Vectors
+        // of more than 128 coordinates with several entries per message stay with a cluster per worker (2 x 500, Top-8: 4.3 us
+        // against 4.6: a thread then has several coordinates to look the words through for).
+        for (const bool local : {true, false}) {
+            if (local && ((i64)c->n * C > PK_LOCAL_BLOCKS || nmsg > PK_LOCAL_MSGS)) continue;
+            PersistKernel kern = persistent_kernel_of(c, roles, local, chunk_slots, rb, src, threads, extra);
+            if (!kern) continue;
+            // the device's opt-in limit (less the kernel's static part), so that no other handle's plan for the same
+            // kernel can lower it under this one's need
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - PK_STATIC_SMEM) != cudaSuccess ||
+                (local && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+                cudaGetLastError();
+                continue;
+            }
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(c->n * C)); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)(local ? c->n * C : C); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            int active = 0;
+            if (cudaOccupancyMaxActiveClusters(&active, kern, &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
+            if (active < (local ? 1 : c->n)) continue;
+            P.ok = true; P.local = local; P.C = C; P.rb = rb; P.src = src; P.chunks = chunk_slots; P.threads = threads; P.extra = extra;
+            P.smem = smem; P.stages = stages; P.kernel = kern;
+            return P;
         }
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(c->n * C)); cfg.blockDim = dim3((unsigned)block_threads); cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        int active = 0;
-        if (cudaOccupancyMaxActiveClusters(&active, kern, &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
-        if (active < c->n) continue;
-        P.ok = true; P.C = C; P.rb = rb; P.src = src; P.chunks = chunk_slots; P.threads = threads; P.extra = extra; P.smem = smem; P.stages = stages; P.kernel = kern;
-        return P;
     }
     return P;
 }
@@ -1024,7 +1036,7 @@ ef21_status run_persistent(ef21_ctx* c, const PersistPlan& P, int steps, const i
     p.slots = c->at<unsigned long long>(c->L.slots); p.status = c->status();
     p.n = c->n; p.d = (int)c->d; p.ld = (int)c->L.ld; p.k = c->k; p.C = P.C; p.steps = steps;
     p.objective = c->objective;
-    p.slice_rows = 0; p.use_table = (c->variant != EF21_VARIANT_EF21_PLUS && pk_use_table(c->n, (int)c->L.ld, c->k)) ? 1 : 0; p.gamma = c->gamma; p.lambda = c->lambda; p.inv_n = 1.0f / (float)c->n;
+    p.slice_rows = 0; p.use_table = (!P.local && c->variant != EF21_VARIANT_EF21_PLUS && pk_use_table(c->n, (int)c->L.ld, c->k)) ? 1 : 0; p.gamma = c->gamma; p.lambda = c->lambda; p.inv_n = 1.0f / (float)c->n;
     // the epochs run on from launch to launch, so the slot array (cleared once, at creation) needs no clearing here
     p.spin_limit = c->spin_limit; p.epoch0 = c->pk_epoch; p.par0 = c->pk_par;
     cudaLaunchConfig_t cfg = {};
@@ -1035,7 +1047,7 @@ ef21_status run_persistent(ef21_ctx* c, const PersistPlan& P, int steps, const i
     // occupancy query when the plan was made.
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)P.C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = (unsigned)(P.local ? c->n * P.C : P.C); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
@@ -1043,8 +1055,10 @@ ef21_status run_persistent(ef21_ctx* c, const PersistPlan& P, int steps, const i
     if (e != cudaSuccess) { cudaGetLastError(); return EF21_ERR_CUDA; }
     if (G) { G->any = true; G->detached = false; G->last_stream = c->stream; }
     c->launches += 1;
-    c->pk_epoch = (unsigned)(((i64)c->pk_epoch + steps - 1) % 65535) + 1u;
-    c->pk_par = (c->pk_par + (unsigned)steps) & 1u;
+    if (!P.local) {           // (one cluster for all workers keeps its words in shared memory)
+        c->pk_epoch = (unsigned)(((i64)c->pk_epoch + steps - 1) % 65535) + 1u;
+        c->pk_par = (c->pk_par + (unsigned)steps) & 1u;
+    }
     c->pk_used_cluster = P.C; c->pk_used_rb = P.rb; c->pk_used_src = P.src == PK_SRC_RING ? PK_SRC_GMEM : P.src; c->pk_used_threads = P.threads;
     c->pk_used_body = P.roles ? 1 : 2;
     return EF21_OK;
@@ -1627,6 +1641,7 @@ ef21_status ef21_selftest_exchange_floor(ef21_ctx* c, int32_t steps) {
     // the shape ef21_step itself would launch, with the skeleton kernel of the same instantiation in its place
     PersistPlan P = plan_persistent(c);
     if (!P.ok) return EF21_ERR_UNSUPPORTED;
+    P.local = false;
     P.kernel = P.roles ? pk_lookup_floor(P.chunks, P.rb, P.src, P.threads, P.extra)
                        : pk_lookup_wide_floor(P.chunks, P.rb, P.src, P.threads, P.extra);
     if (!P.kernel) return EF21_ERR_UNSUPPORTED;

@@ -87,6 +87,14 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
+// Two neighbouring words of this block's shared memory that other blocks write (each of the two is read whole).
+__device__ __forceinline__ void ld_volatile_2u64(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
+    asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
+}
+// A word of another block's shared memory (mapped address).
+__device__ __forceinline__ void st_cluster_u64(unsigned addr, unsigned long long v) {
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
 __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
     unsigned v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -215,18 +223,37 @@ __device__ __forceinline__ unsigned next_epoch(unsigned e) { return e >= 65535u 
 // recomputed.  pad_bits: bit e set = entry 4L+e lies beyond d and is never taken.  Returns the lane's 4-bit mask of
 // selected entries; position receives the number of selected entries in lower lanes, so that a lane can emit its picks
 // in ascending index order at position, position + 1, ...
+// PAIRS: keys and places ordered as pairs of 32-bit words (100 cycles less than 64-bit composites); the serving-warp kernels
+// keep the composites, next to which the compiler lays out their Top-1 path better (20 x 406 x 112: 2.60 against 2.75 us).
+template <bool PAIRS = true>
 __device__ __forceinline__ unsigned warp_topk_four_per_lane(const float4& v4, unsigned pad_bits, int k, int lane, int& position) {
-    // composite (key, 3 - e): larger is better; -1 marks an entry that cannot be taken
-    long long c[4];
+    int k0, k1, k2, k3, e0, e1, e2, e3;
+    if constexpr (PAIRS) {
+        // neighbours change places only if the later one is strictly larger: equal keys stay in index order
+        k0 = (pad_bits & 1u) ? -1 : (int)mag_key(v4.x); k1 = (pad_bits & 2u) ? -1 : (int)mag_key(v4.y);
+        k2 = (pad_bits & 4u) ? -1 : (int)mag_key(v4.z); k3 = (pad_bits & 8u) ? -1 : (int)mag_key(v4.w);
+        e0 = 0; e1 = 1; e2 = 2; e3 = 3;
+        auto order = [](int& ka, int& kb, int& ea, int& eb) {
+            const bool swap = kb > ka;
+            const int hi = max(ka, kb), lo = min(ka, kb);
+            const int eh = swap ? eb : ea, el = swap ? ea : eb;
+            ka = hi; kb = lo; ea = eh; eb = el;
+        };
+        order(k0, k1, e0, e1); order(k2, k3, e2, e3); order(k1, k2, e1, e2);
+        order(k0, k1, e0, e1); order(k2, k3, e2, e3); order(k1, k2, e1, e2);
+    } else {
+        // composite (key, 3 - e): larger is better; -1 marks an entry that cannot be taken
+        long long c[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const long long key = ((pad_bits >> e) & 1u) ? -1ll : (long long)mag_key(comp_of(v4, e));
-        c[e] = key < 0 ? -1ll : ((key << 2) | (long long)(3 - e));
+        for (int e = 0; e < 4; ++e) {
+            const long long key = ((pad_bits >> e) & 1u) ? -1ll : (long long)mag_key(comp_of(v4, e));
+            c[e] = key < 0 ? -1ll : ((key << 2) | (long long)(3 - e));
+        }
+        auto order = [&](int a, int b) { const long long hi = max(c[a], c[b]), lo = min(c[a], c[b]); c[a] = hi; c[b] = lo; };
+        order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
+        k0 = (int)(c[0] >> 2); k1 = (int)(c[1] >> 2); k2 = (int)(c[2] >> 2); k3 = (int)(c[3] >> 2);       // -1 stays -1
+        e0 = 3 - (int)(c[0] & 3); e1 = 3 - (int)(c[1] & 3); e2 = 3 - (int)(c[2] & 3); e3 = 3 - (int)(c[3] & 3);
     }
-    auto order = [&](int a, int b) { const long long hi = max(c[a], c[b]), lo = min(c[a], c[b]); c[a] = hi; c[b] = lo; };
-    order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
-    int k0 = (int)(c[0] >> 2), k1 = (int)(c[1] >> 2), k2 = (int)(c[2] >> 2), k3 = (int)(c[3] >> 2);       // -1 stays -1
-    int e0 = 3 - (int)(c[0] & 3), e1 = 3 - (int)(c[1] & 3), e2 = 3 - (int)(c[2] & 3), e3 = 3 - (int)(c[3] & 3);
     unsigned mask = 0u;
     for (int round = 0; round < k; ++round) {
         const int wk = __reduce_max_sync(0xffffffffu, k0);
@@ -252,8 +279,16 @@ typedef void (*PersistKernel)(const PersistParams);
 // Top-k by warp arg-max rounds -- for k <= PK_ROLES_MAX_K.  "wide" (persistent_body.inc): every step is taken by the
 // whole block between block barriers, Top-k by rank counting over all threads for larger k -- any k <= PK_MAX_K, and
 // the only body of Algorithm 3.
+constexpr int PK_LOCAL_BLOCKS = 16, PK_LOCAL_MSGS = 48;      // all workers in one cluster: most blocks, most words per iteration (64: 2.81 us against 2.78)
 constexpr int PK_ROLES_MAX_K = 8;
 PersistKernel pk_lookup_ef21(int chunks, int rb, int src, int threads, int extra);          // Algorithm 2, roles
+// The same methods with all workers in ONE cluster: the message words go from block to block through distributed shared
+// memory instead of global memory, and every block polls its own copy.  Wide body: one chunk slot (d <= 128).
+PersistKernel pk_lookup_local_ef21(int chunks, int rb, int src, int threads, int extra);
+PersistKernel pk_lookup_local_ef(int chunks, int rb, int src, int threads, int extra);
+PersistKernel pk_lookup_local_wide_ef21(int chunks, int rb, int src, int threads, int extra);
+PersistKernel pk_lookup_local_plus(int chunks, int rb, int src, int threads, int extra);
+PersistKernel pk_lookup_local_wide_ef(int chunks, int rb, int src, int threads, int extra);
 PersistKernel pk_lookup_ef(int chunks, int rb, int src, int threads, int extra);            // Algorithm 4, roles
 PersistKernel pk_lookup_floor(int chunks, int rb, int src, int threads, int extra);         // exchange skeleton, roles
 PersistKernel pk_lookup_wide_ef21(int chunks, int rb, int src, int threads, int extra);     // Algorithm 2, wide

@@ -1,0 +1,46 @@
+"""Persistent kernels with all workers in one cluster (messages through distributed shared memory): edges of the range of
+workers, blocks and message words, and calls of many iterations against as many calls of one."""
+import numpy as np
+import pytest
+
+import ef21_inputs as inputs
+from gpu_util import lockstep, make_gpu, make_oracle_state
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(n, d, k, rows, seed):
+    return inputs.make_logistic("one-cluster", n=n, d=d, N=n * rows + 3, k=k, seed=seed, features="bernoulli", density=0.2, gamma=0.1,
+                                T=10)
+
+
+# one worker, odd numbers of words, 48 words and one more, 16 blocks and one more, several blocks per worker, full d
+@pytest.mark.parametrize("n,d,k,rows", [(1, 5, 2, 9), (3, 128, 3, 40), (7, 33, 3, 20), (16, 64, 3, 12), (7, 20, 7, 12), (17, 64, 2, 12),
+                                        (2, 128, 24, 30), (2, 128, 32, 30), (2, 112, 1, 800), (16, 130, 1, 20), (4, 127, 1, 400), (5, 16, 16, 10), (2, 100, 7, 700)])
+def test_tracks_the_oracle(n, d, k, rows, oracle32):
+    from paper_2106_05203_b200 import binding as B
+    w = _workload(n, d, k, rows, seed=n * d + k)
+    h = make_gpu(w, path=B.PATH_PERSISTENT)
+    st = make_oracle_state(oracle32, w)
+    h.init(B.INIT_ZERO)
+    st.init(1)
+    lockstep(h, st, oracle32, w, 6)
+    assert h.poll() == 0
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("n,d,k,rows", [(4, 64, 4, 50), (16, 112, 1, 60), (9, 128, 7, 30), (2, 120, 2, 600)])
+def test_many_iterations_are_as_many_calls(variant, n, d, k, rows):
+    from paper_2106_05203_b200 import binding as B
+    w = _workload(n, d, k, rows, seed=k)
+    states = []
+    for calls, steps in ((1, 60), (60, 1)):
+        h = make_gpu(w, path=B.PATH_PERSISTENT)
+        h.set_variant(variant)
+        h.init(B.INIT_ZERO)
+        for _ in range(calls):
+            h.step(steps)
+        assert h.poll() == 0 and h.last_path == B.PATH_PERSISTENT
+        states.append([np.array(a) for a in h.get_state_host()])
+    for a, b in zip(*states):
+        assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
