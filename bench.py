@@ -293,7 +293,7 @@ def run_ours(args):
                               "data": "synthetic", "config": {"workload": r["workload"]},
                               "roofline": {"bound": "hbm", "achieved": r["algorithmic_GBps"], "peak": peak, "unit": "GB/s",
                                            "frac": r["frac_of_hbm_peak"], "traffic": NCU_TRAFFIC["stress_collect"]["bytes"], "peak_kind": f"of {peak_kind}",
-                                           "kernel": "st_collect_kernel (dominant) + sample/finish/aggregate"},
+                                           "kernel": "st_collect_long_kernel (dominant) + sample/cut/compact/aggregate"},
                               "gpu_launches": r["launches"], "fallbacks": r["fallbacks"]}), flush=True)
         if world > 1:
             dist.destroy_process_group()
