@@ -405,16 +405,22 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
     unsigned sure, open, my_open;                                    // of the vector; open entries this block goes through
     bool slow;
     if (CLASSIFY) {
-        // one thread per region
+        // 2^group lanes per region, as many as there are threads for; neighbouring regions go to different blocks, so that every
+        // block has its share of the open entries (a lane per region and block 0 taking the first 1,024 of them: 64 x 1,024
+        // regions 20 us, 16 x 1,024 35 us, and more open entries than one block holds from k = d / 400 on)
+        int group = 0;
+        while (group < 5 && (p.nreg << (group + 1)) <= C * 1024) ++group;
+        const unsigned lanes = 1u << group, sub = (unsigned)tid & (lanes - 1u);
         unsigned sure_mine = 0u;
         bool over = false;
-        for (int r = rk * 1024 + tid; r < p.nreg; r += C * 1024) {
-            const unsigned n = p.reg_cand[(i64)vec * p.nreg_pitch + r];
+        for (int r0 = 0; r0 < p.nreg; r0 += (C * 1024) >> group) {
+            const int r = r0 + (tid >> group) * C + rk;
+            const unsigned n = r < p.nreg ? p.reg_cand[(i64)vec * p.nreg_pitch + r] : 0u;
             const int2* rec = reinterpret_cast<const int2*>(p.cand + ((i64)vec * p.nreg + r) * p.cap);
             unsigned s = 0u;
             over |= n > (unsigned)p.cap;
-#pragma unroll 8
-            for (unsigned e = 0; e < min(n, (unsigned)p.cap); ++e) {
+#pragma unroll 4
+            for (unsigned e = sub; e < min(n, (unsigned)p.cap); e += lanes) {
                 const int2 w = rec[2 * e];
                 const unsigned key = (unsigned)w.y & 0x7fffffffu;
                 if (key >= hi) ++s;
@@ -424,8 +430,10 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
                     if (at < (unsigned)ST_OPEN_STAGE) mine_open[at] = st_composite(key, (unsigned)w.x);
                 }
             }
-            base[r] = s;
             sure_mine += s;
+            __syncwarp();
+            for (unsigned off = 1u; off < lanes; off <<= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            if (r < p.nreg && sub == 0u) base[r] = s;
         }
         sure_mine = __reduce_add_sync(0xffffffffu, sure_mine);
         if ((tid & 31) == 0 && sure_mine) atomicAdd(&sure_sh, sure_mine);

@@ -65,3 +65,21 @@ def test_rounds_on_the_long_paths(variant, n, d, k, oracle32):
     if variant != B.VARIANT_EF:
         np.testing.assert_array_equal(g.view(np.uint32), st.g.view(np.uint32))
     assert h.poll() == 0
+
+
+@pytest.mark.parametrize("n,d,k", [(16, 4194304, 40000), (24, 3000000, 12000), (64, 1200000, 12000)])
+def test_larger_messages_stay_on_the_streaming_path(n, d, k):
+    """Large batches of aligned vectors with up to 1 % of the entries per message: exact, and no vector needs a second look."""
+    import torch
+    from paper_2106_05203_b200 import binding as B
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(k)
+    V = torch.randn(n, d, device="cuda", generator=gen)
+    h = B.EF21(n, d, k, 0.05)
+    h.init_grads(None, B.INIT_ZERO)
+    h.step_grads(V, 1)
+    assert h.fallback_count() == 0 and h.poll() == 0
+    idx, val = h.get_state(messages=True)[3:5]
+    for i in (0, n // 2, n - 1):
+        order = torch.sort(V[i].abs(), descending=True, stable=True).indices[:k].sort().values
+        assert torch.equal(idx[i].long(), order) and torch.equal(val[i], V[i][order])
