@@ -421,10 +421,13 @@ ef21_status enqueue_topk_stream(cudaStream_t st, const float* a, i64 pitch_a, co
     const double rank = (double)k * (double)B.L.samples / (double)d;
     const double open = 2.6 * st_margin(rank) / rank * (double)k;
     const i64 all_blocks = ceil_div(p.nreg, ST_WARPS);
-    int cut_blocks = batch > 37 ? 2 : 8;
     bool classify = vec && p.region_log == ST_REGION_LOG_LARGE && p.cap > 0;
+    // blocks of the cut kernel's cluster: as few as hold the open entries where it classifies (16 x 4,194,304: 24 us with eight, 15 with
+    // two), eight for the long lists of a few vectors
+    int cut_blocks = classify || batch > 37 ? 2 : 8;
     while (classify && cut_blocks < 8 && open > 0.8 * cut_blocks * ST_OPEN_STAGE) cut_blocks *= 2;
     classify = classify && open <= 0.8 * cut_blocks * ST_OPEN_STAGE;
+    if (!classify) cut_blocks = batch > 37 ? 2 : 8;
     if (classify) {
         CU(launch(st_collect_long_kernel<MODE>, dim3((unsigned)all_blocks, (unsigned)batch), ST_WARPS * 32, 0, st, 1, p));
     } else {
@@ -1318,25 +1321,35 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
         c->last_path = EF21_PATH_LAUNCHES;
         return EF21_OK;
     }
-    // Same V at every step: the threshold estimate of round t+1 needs V and g_i^{t+1} only, so it
-    // follows the finish kernel of round t directly on this stream, and the aggregation of round t (g
-    // and x) runs beside it on the second stream; the streaming pass of round t+1 waits for both.
+    // Same V at every step: the threshold estimate of round t+1 needs V and g_i^{t+1} only, so it runs beside the aggregation of
+    // round t (g and x); the streaming pass of round t+1 waits for both.  The longer of the two follows the selection on
+    // this stream, without an event in between: the aggregation where there are many message entries (64 x 4,194: 395 us a round
+    // against 398, 24 x 40,000: 293 against 300), else the estimate (16 x 4,194: 132 against 142).
     cudaStream_t main_stream = c->stream;
+    const bool agg_first = (i64)c->n * c->k > 131072;
     for (int t = 0; t < steps; ++t) {
         // (letting the streaming pass start while the aggregation still runs made the pass 15-20 % slower)
         if (t > 0) CU(cudaStreamWaitEvent(main_stream, c->ev_join, 0));
         EF(enqueue_round_select(c, V_dev, c->d, t > 0));
+        if (t + 1 == steps) {
+            EF(enqueue_round_aggregate(c, AGG_X_BEFORE));
+            break;
+        }
         CU(cudaEventRecord(c->ev_fork, main_stream));
         CU(cudaStreamWaitEvent(c->aux_stream, c->ev_fork, 0));
-        c->stream = c->aux_stream;
-        const ef21_status agg = enqueue_round_aggregate(c, AGG_X_BEFORE);
-        c->stream = main_stream;
-        EF(agg);
+        const StArgs next = stream_args(V_dev, c->d, c->gi(), c->L.ld, 0.f, c->d, c->k, B);
+        if (agg_first) {
+            EF(enqueue_stream_sample<TC_DIFF>(c->aux_stream, next, c->n, B.L, &c->launches));
+            EF(enqueue_round_aggregate(c, AGG_X_BEFORE));
+        } else {
+            c->stream = c->aux_stream;
+            const ef21_status agg = enqueue_round_aggregate(c, AGG_X_BEFORE);
+            c->stream = main_stream;
+            EF(agg);
+            EF(enqueue_stream_sample<TC_DIFF>(main_stream, next, c->n, B.L, &c->launches));
+        }
         CU(cudaEventRecord(c->ev_join, c->aux_stream));
-        if (t + 1 < steps)
-            EF(enqueue_stream_sample<TC_DIFF>(main_stream, stream_args(V_dev, c->d, c->gi(), c->L.ld, 0.f, c->d, c->k, B), c->n, B.L, &c->launches));
     }
-    CU(cudaStreamWaitEvent(main_stream, c->ev_join, 0));
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;
 }

@@ -392,7 +392,7 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
     if (tid == 0) { stage_n = 0u; sure_sh = 0u; open_sh = 0u; over_sh = 0u; }
     if (CLASSIFY) { hist[tid] = 0u; hist[tid + 1024] = 0u; }
     __syncthreads();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");                // block 0's counter is ready
+    if (!CLASSIFY) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); // block 0's counter is ready
     pdl_trigger();
     pdl_wait();
     StCtl& ct = p.ctl[vec];
@@ -441,7 +441,6 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
         __syncthreads();
         if (tid == 0 && open_sh > (unsigned)ST_OPEN_STAGE) over_sh = 1u;
         __threadfence();
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         cluster.sync();
         sure = open = 0u; slow = false;
         c = make_uint2(0u, 0u);
@@ -453,7 +452,6 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
             c.x += o.x; c.y += o.y;
         }
         my_open = open_sh;
-        cluster.sync();                                              // (a slow vector's blocks leave below)
         slow |= sure > k || sure + open < k;
     } else {
         x0 = e0 < p.open_cap ? list[e0] : 0ull;                      // on its way while the counters and the histogram arrive
@@ -477,6 +475,7 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
         slow = pop > (unsigned)ST_OPEN_STAGE;
     }
     if (slow) {
+        if (CLASSIFY) cluster.sync();                                // (the others may still read this block's counters)
         if (rk == 0 && tid == 0) { ct.slow = 1u; if (p.slow_count) atomicAdd(p.slow_count, 1u); }
         return;
     }
@@ -529,7 +528,10 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
         }
         __threadfence();
         __syncthreads();
-    } else if (rk != 0) return;
+    } else {
+        if (CLASSIFY) cluster.sync();
+        if (rk != 0) return;
+    }
     if (tid == 0) ct.cut = cut;
     // counts -> first positions (the counts were changed by atomics: read them from L2)
     unsigned before = 0u;
@@ -558,7 +560,7 @@ struct StOut {
     unsigned long long* cut_out;        // [batch] the cut of every vector; may be null
 };
 
-// grid = (ceil(nreg / 32), batch), 256 threads: eight lanes per region.
+// grid = (ceil(nreg / 32), batch), 256 threads: eight lanes per region (four in one wave instead of two: no faster).
 template <int MODE>
 __global__ void __launch_bounds__(256)
 st_compact_kernel(const __grid_constant__ StArgs p, const StOut o) {
