@@ -102,25 +102,39 @@ plus_mean_kernel(const float* __restrict__ a, i64 pitch_a, const unsigned long l
     pdl_wait(a, cut_b, choice, gi, g, x);
     for (i64 j = 4 * (blockIdx.x * (i64)blockDim.x + threadIdx.x); j < d; j += 4 * (i64)gridDim.x * blockDim.x) {
         float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int i = 0; i < n; ++i) {
-            float4* row = reinterpret_cast<float4*>(gi + (i64)i * ld + j);
-            float4 w;
-            if (choice[i]) {
-                const unsigned long long cut = cut_b[i];
-                float b[4];
+        // eight rows on their way at a time (a load behind the branch of every row: 100 workers, d = 356, 49 us a round)
+        for (int i0 = 0; i0 < n; i0 += 8) {
+            float4 w[8];
+            bool plain[8], any = false;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float v = j + e < d ? a[(i64)i * pitch_a + j + e] : 0.f;
-                    const unsigned long long c = ((unsigned long long)mag_key(v) << 32) | (0xffffffffu - (unsigned)(j + e));
-                    b[e] = j + e < d && c >= cut ? v : 0.f;
-                }
-                w = make_float4(b[0], b[1], b[2], b[3]);
-                *row = w;
-            } else {
-                w = *row;
+            for (int q = 0; q < 8; ++q) {
+                plain[q] = i0 + q < n && choice[i0 + q] != 0;
+                w[q] = i0 + q < n ? *reinterpret_cast<const float4*>(gi + (i64)(i0 + q) * ld + j) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            s[0] = __fadd_rn(s[0], w.x); s[1] = __fadd_rn(s[1], w.y); s[2] = __fadd_rn(s[2], w.z); s[3] = __fadd_rn(s[3], w.w);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) any = any || plain[q];
+            if (any) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (!plain[q]) continue;
+                    const int i = i0 + q;
+                    const unsigned long long cut = cut_b[i];
+                    float b[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float v = j + e < d ? a[(i64)i * pitch_a + j + e] : 0.f;
+                        const unsigned long long c = ((unsigned long long)mag_key(v) << 32) | (0xffffffffu - (unsigned)(j + e));
+                        b[e] = j + e < d && c >= cut ? v : 0.f;
+                    }
+                    w[q] = make_float4(b[0], b[1], b[2], b[3]);
+                    *reinterpret_cast<float4*>(gi + (i64)i * ld + j) = w[q];
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (i0 + q < n) {
+                    s[0] = __fadd_rn(s[0], w[q].x); s[1] = __fadd_rn(s[1], w[q].y); s[2] = __fadd_rn(s[2], w[q].z); s[3] = __fadd_rn(s[3], w[q].w);
+                }
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
