@@ -12,8 +12,10 @@ typedef long long i64;
 // dependent it starts after 0.5 us.  Every kernel of the library calls pdl_wait() before it touches global memory (it
 // returns when the preceding kernels of the stream have completed and their writes are visible) and pdl_trigger() early,
 // so that the kernel behind it can be placed on the device meanwhile.
-// The kernel's pointers go through pdl_wait so that no load through them -- a read-only one (const __restrict__) is otherwise
-// free to move -- is placed in front of the wait.
+// The kernel's pointers go through pdl_wait so that no load through them -- a read-only one (const __restrict__, __ldg, __ldcs) is
+// otherwise free to move -- is placed in front of the wait.  Where they come in a struct, the local pointer that such loads
+// start from is made by pdl_ptr, behind the wait; or the loads are plain ones, which the wait's memory clobber keeps behind it
+// (the persistent kernels: the rows' address in a register cost the w8a-shaped run 5 %, 547 -> 574 us).
 template <typename T>
 __device__ __forceinline__ void pdl_fresh(T& p) { asm volatile("" : "+l"(p)); }
 template <typename... P>
@@ -21,6 +23,8 @@ __device__ __forceinline__ void pdl_wait(P&... pointers) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     (pdl_fresh(pointers), ...);
 }
+template <typename T>
+__device__ __forceinline__ T* pdl_ptr(T* p) { pdl_fresh(p); return p; }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Status word layout in the workspace (one 256-byte slot): word 0 = first error code seen.

@@ -27,7 +27,7 @@ copy_segments_kernel(const __grid_constant__ CopyArgs p) {
     const i64 row = u / per_row, w0 = (u - row * per_row) * COPY_UNIT;
     const int len = (int)min((i64)COPY_UNIT, c.width - w0);
     unsigned* dst = c.dst + row * c.dpitch + w0;
-    const unsigned* src = c.src ? c.src + row * c.spitch + w0 : nullptr;
+    const unsigned* src = pdl_ptr(c.src ? c.src + row * c.spitch + w0 : nullptr);
     int done = 0;
     if (((reinterpret_cast<size_t>(dst) | reinterpret_cast<size_t>(src)) & 15u) == 0u) {
         const int quads = len >> 2;

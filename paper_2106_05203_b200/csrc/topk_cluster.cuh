@@ -118,8 +118,6 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     auto sync_all = [&]() { if (C > 1) cluster.sync(); else __syncthreads(); };
 
     const int j0 = (int)min((i64)rank * p.slice, (i64)p.d), len = min(p.slice, p.d - j0);
-    const float* __restrict__ av = GRAD ? nullptr : p.a + (i64)vec * p.pitch_a + j0;
-    float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + j0;
 #pragma unroll 1
     for (int q = tid; q < TC_BINS; q += THREADS) { hist[q] = 0u; if (C > 1) hsum[q] = 0u; }
     for (int j = len + tid; !STREAM && j < p.slice && j < len + 128; j += THREADS) ws[j] = 0u;       // the tail of the last tile
@@ -128,6 +126,8 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     __syncthreads();
     if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // hsum is empty
     if (!STREAM) { pdl_trigger(); pdl_wait(); }
+    const float* __restrict__ av = GRAD ? nullptr : pdl_ptr(p.a + (i64)vec * p.pitch_a + j0);
+    float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + j0;
     float* dense = MODE == TC_PLAIN && !STREAM && p.apply ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
     // entries of bin 0 (zeros and the smallest magnitudes) are not counted: what the other bins leave over is theirs
     auto take = [&](int j, float a, float b) {
@@ -414,7 +414,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     if (STREAM && p.tile_off) {
         cluster.sync();                                              // the message is complete and visible to the cluster
         int* off = p.tile_off + (i64)vec * (p.ntiles + 1);
-        const int* io = p.idx_out + (i64)vec * p.k;
+        const int* io = pdl_ptr(p.idx_out + (i64)vec * p.k);
         for (int b = rank * THREADS + tid; b <= p.ntiles; b += C * THREADS) {
             const i64 bound = (i64)b * p.tile;
             int lo = 0, hi = p.k;

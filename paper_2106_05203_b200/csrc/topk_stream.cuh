@@ -93,8 +93,8 @@ st_sample_kernel(const __grid_constant__ StArgs p, float rank, float margin) {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // block 0's words are ready
     pdl_trigger();
     pdl_wait();
-    const float* __restrict__ av = p.a + (i64)vec * p.pitch_a;
-    const float* __restrict__ bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b;
+    const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a);
+    const float* __restrict__ bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b);
     const int warps = C * (ST_SAMPLE_THREADS / 32), w = rk * (ST_SAMPLE_THREADS / 32) + (tid >> 5);
     const i64 stride = p.d / ((i64)warps * PT);                     // >= 32: a quarter of the vector at most is sampled
     unsigned key[PT];
@@ -168,8 +168,8 @@ st_collect_long_kernel(const __grid_constant__ StArgs p) {
     if (region >= p.nreg) return;
     const unsigned lo = p.ctl[vec].lo;
     const i64 base = (i64)region << ST_REGION_LOG_LARGE;
-    const float* __restrict__ av = p.a + (i64)vec * p.pitch_a;
-    float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b;
+    const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a);
+    float* bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b);
     int4* out = p.cand + ((i64)vec * p.nreg + region) * p.cap;
     const unsigned lt = (1u << lane) - 1u;
     int cnt = 0;
@@ -251,8 +251,8 @@ st_collect_kernel(const __grid_constant__ StArgs p) {
         const unsigned lo = p.ctl[vec].lo;
         const i64 base = (i64)region << p.region_log;
         const int end = (int)min((i64)1 << p.region_log, p.d - base);           // positions below are relative to the region
-        const float* __restrict__ av = p.a + (i64)vec * p.pitch_a + base;
-        float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + base;
+        const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a + base);
+        float* bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b + base);
         int4* out = p.cand + ((i64)vec * p.nreg + region) * p.cap;
         unsigned cnt = 0u, sure = 0u;
         // listed candidates are classified behind the loop, by lanes side by side
@@ -533,7 +533,8 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
         if (rk != 0) return;
     }
     if (tid == 0) ct.cut = cut;
-    // counts -> first positions (the counts were changed by atomics: read them from L2)
+    // counts -> first positions (the counts were changed by atomics: read them from L2, behind the barrier)
+    base = pdl_ptr(base);
     unsigned before = 0u;
     for (int r0 = 0; r0 < p.nreg; r0 += 8192) {
         const int r = r0 + 8 * tid;                                  // the padding behind the last region is added up and ignored
@@ -605,7 +606,7 @@ st_compact_kernel(const __grid_constant__ StArgs p, const StOut o) {
     }
     // regions whose list overflowed (or that keep none): all four groups of the warp stay together, each reads its own
     if (__any_sync(0xffffffffu, !listed)) {
-        const float* __restrict__ av = p.a + (i64)vec * p.pitch_a;
+        const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a);
         const float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b;
         for (int s = 0; s < 1 << (p.region_log - 3); s += 4) {
             float v[4], nw[4];
@@ -654,7 +655,7 @@ st_reread_kernel(const __grid_constant__ StArgs p, const StOut o) {
     unsigned pos = first;
     const i64 base = (i64)region << p.region_log;
     const int end = (int)min((i64)1 << p.region_log, p.d - base);
-    const float* __restrict__ av = p.a + (i64)vec * p.pitch_a + base;
+    const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a + base);
     const float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + base;
     int* io = o.idx_out + (i64)vec * p.k;
     float* vo = o.val_out + (i64)vec * p.k;
