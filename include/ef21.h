@@ -309,6 +309,11 @@ ef21_status ef21_set_persistent_shape(ef21_ctx* ctx, int32_t cluster_blocks, int
 ef21_status ef21_get_persistent_shape(const ef21_ctx* ctx, int32_t* cluster_blocks,
                                       int32_t* rows_per_batch, int32_t* row_source);
 
+/* Diagnostics of the last persistent launch beyond its shape: one_cluster 1 if all workers ran in one thread-block cluster
+ * (messages through distributed shared memory), else 0; ring_stages: batches in flight per warp where rows from global
+ * memory (row source 2) came through a ring in shared memory, 0 where they did not.  Both 0 before the first launch. */
+ef21_status ef21_get_persistent_form(const ef21_ctx* ctx, int32_t* one_cluster, int32_t* ring_stages);
+
 /* Threads per block of the persistent path: 256, 512 or 0 = automatic (512 exists only for batches
  * of at most 16 float4 registers per lane).  get_ reports what the last persistent launch used. */
 ef21_status ef21_set_persistent_threads(ef21_ctx* ctx, int32_t threads_per_block);

@@ -65,6 +65,7 @@ SIGNATURES = {
     "ef21_get_persistent_body": (ctypes.c_int32, [_vp]),
     "ef21_set_persistent_shape": (ctypes.c_int, [_vp, _i32, _i32, _i32]),
     "ef21_get_persistent_shape": (ctypes.c_int, [_vp, ctypes.POINTER(_i32), ctypes.POINTER(_i32), ctypes.POINTER(_i32)]),
+    "ef21_get_persistent_form": (ctypes.c_int, [_vp, ctypes.POINTER(_i32), ctypes.POINTER(_i32)]),
     "ef21_set_persistent_threads": (ctypes.c_int, [_vp, _i32]),
     "ef21_get_persistent_threads": (_i32, [_vp]),
     "ef21_set_path": (ctypes.c_int, [_vp, _i32]),
@@ -313,6 +314,12 @@ class EF21:
         _check(_lib.ef21_get_persistent_shape(self._h, ctypes.byref(c), ctypes.byref(r), ctypes.byref(s)),
                "ef21_get_persistent_shape")
         return c.value, r.value, s.value
+
+    def get_persistent_form(self):
+        """(all workers in one cluster, ring stages per warp) of the last persistent launch."""
+        one, stages = _i32(), _i32()
+        _check(_lib.ef21_get_persistent_form(self._h, ctypes.byref(one), ctypes.byref(stages)), "ef21_get_persistent_form")
+        return bool(one.value), stages.value
 
     def set_persistent_threads(self, threads_per_block: int) -> None:
         _check(_lib.ef21_set_persistent_threads(self._h, threads_per_block), "ef21_set_persistent_threads")

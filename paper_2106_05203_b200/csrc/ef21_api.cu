@@ -261,6 +261,7 @@ struct ef21_ctx {
     bool agg_off_ready;                 // the last selection already wrote the aggregation's tile offsets
     int pk_cluster, pk_rb, pk_src, pk_threads;      // forced persistent-kernel shape (0 / -1 = automatic)
     int pk_used_cluster, pk_used_rb, pk_used_src, pk_used_threads;
+    int pk_used_local, pk_used_stages;
     PersistPlan plan; bool plan_valid;  // cached plan of ef21_step's persistent launch
     PersistPlan mb_plan; bool mb_plan_valid; int mb_plan_tau;      // the same for the stochastic variant with mb_plan_tau rows
     unsigned pk_epoch, pk_par;          // epoch and slot half of the last persistent iteration (see PersistParams)
@@ -1067,6 +1068,7 @@ ef21_status run_persistent(ef21_ctx* c, const PersistPlan& P, int steps, const i
     }
     c->pk_used_cluster = P.C; c->pk_used_rb = P.rb; c->pk_used_src = P.src == PK_SRC_RING ? PK_SRC_GMEM : P.src; c->pk_used_threads = P.threads;
     c->pk_used_body = P.roles ? 1 : 2;
+    c->pk_used_local = P.local ? 1 : 0; c->pk_used_stages = P.src == PK_SRC_RING ? P.stages : 0;
     return EF21_OK;
 }
 
@@ -1116,6 +1118,7 @@ ef21_status ef21_create(ef21_ctx** out, int32_t n, int64_t d, int32_t k, float g
     c->path = EF21_PATH_AUTO; c->last_path = 0; c->launches = 0;
     c->pk_cluster = 0; c->pk_rb = 0; c->pk_src = -1; c->pk_threads = 0; c->agg_off_ready = false;
     c->pk_used_cluster = c->pk_used_rb = 0; c->pk_used_src = -1; c->pk_used_threads = 0;
+    c->pk_used_local = c->pk_used_stages = 0;
     c->pk_body = 0; c->pk_used_body = 0; c->pk_epoch = 0u; c->pk_par = 0u; c->plan_valid = false; c->mb_plan_valid = false; c->mb_plan_tau = 0;
     c->spin_limit = 1u << 22;
     c->force_general_topk = false;
@@ -1595,6 +1598,13 @@ ef21_status ef21_get_persistent_shape(const ef21_ctx* c, int32_t* cluster_blocks
     if (cluster_blocks) *cluster_blocks = c->pk_used_cluster;
     if (rows_per_batch) *rows_per_batch = c->pk_used_rb;
     if (row_source) *row_source = c->pk_used_src;
+    return EF21_OK;
+}
+
+ef21_status ef21_get_persistent_form(const ef21_ctx* c, int32_t* one_cluster, int32_t* ring_stages) {
+    if (!c) return EF21_ERR_INVALID_ARG;
+    if (one_cluster) *one_cluster = c->pk_used_local;
+    if (ring_stages) *ring_stages = c->pk_used_stages;
     return EF21_OK;
 }
 

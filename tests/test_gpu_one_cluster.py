@@ -15,9 +15,11 @@ def _workload(n, d, k, rows, seed):
 
 
 # one worker, odd numbers of words, 48 words and one more, 16 blocks and one more, several blocks per worker, full d
-@pytest.mark.parametrize("n,d,k,rows", [(1, 5, 2, 9), (3, 128, 3, 40), (7, 33, 3, 20), (16, 64, 3, 12), (7, 20, 7, 12), (17, 64, 2, 12),
-                                        (2, 128, 24, 30), (2, 128, 32, 30), (2, 112, 1, 800), (16, 130, 1, 20), (4, 127, 1, 400), (5, 16, 16, 10), (2, 100, 7, 700)])
-def test_tracks_the_oracle(n, d, k, rows, oracle32):
+@pytest.mark.parametrize("n,d,k,rows,one_cluster",
+                         [(1, 5, 2, 9, True), (3, 128, 3, 40, True), (7, 33, 3, 20, True), (16, 64, 3, 12, True), (7, 20, 7, 12, False),
+                          (17, 64, 2, 12, False), (2, 128, 24, 30, True), (2, 128, 32, 30, False), (2, 112, 1, 800, True),
+                          (16, 130, 1, 20, True), (4, 127, 1, 400, True), (5, 16, 16, 10, False), (2, 100, 7, 700, True)])
+def test_tracks_the_oracle(n, d, k, rows, one_cluster, oracle32):
     from paper_2106_05203_b200 import binding as B
     w = _workload(n, d, k, rows, seed=n * d + k)
     h = make_gpu(w, path=B.PATH_PERSISTENT)
@@ -26,6 +28,7 @@ def test_tracks_the_oracle(n, d, k, rows, oracle32):
     st.init(1)
     lockstep(h, st, oracle32, w, 6)
     assert h.poll() == 0
+    assert h.get_persistent_form()[0] == one_cluster
 
 
 @pytest.mark.parametrize("variant", [0, 1, 2])
@@ -40,7 +43,7 @@ def test_many_iterations_are_as_many_calls(variant, n, d, k, rows):
         h.init(B.INIT_ZERO)
         for _ in range(calls):
             h.step(steps)
-        assert h.poll() == 0 and h.last_path == B.PATH_PERSISTENT
+        assert h.poll() == 0 and h.last_path == B.PATH_PERSISTENT and h.get_persistent_form()[0] == (n * k <= 48)
         states.append([np.array(a) for a in h.get_state_host()])
     for a, b in zip(*states):
         assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
