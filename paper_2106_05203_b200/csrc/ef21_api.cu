@@ -1667,14 +1667,14 @@ ef21_status ef21_selftest_exchange_floor(ef21_ctx* c, int32_t steps) {
     // the shape ef21_step itself would launch, with the skeleton kernel of the same instantiation in its place
     PersistPlan P = plan_persistent(c);
     if (!P.ok) return EF21_ERR_UNSUPPORTED;
-    P.local = false;
-    P.kernel = P.roles ? pk_lookup_floor(P.chunks, P.rb, P.src, P.threads, P.extra)
-                       : pk_lookup_wide_floor(P.chunks, P.rb, P.src, P.threads, P.extra);
+    const auto lookup = P.roles ? (P.local ? pk_lookup_local_floor : pk_lookup_floor) : (P.local ? pk_lookup_local_wide_floor : pk_lookup_wide_floor);
+    P.kernel = lookup(P.chunks, P.rb, P.src, P.threads, P.extra);
     if (!P.kernel) return EF21_ERR_UNSUPPORTED;
     int dev = 0, max_smem = 0;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     CU(cudaFuncSetAttribute(P.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem - PK_STATIC_SMEM));
+    if (P.local) CU(cudaFuncSetAttribute(P.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return run_persistent(c, P, steps);
 }
 

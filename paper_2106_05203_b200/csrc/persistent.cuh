@@ -289,6 +289,8 @@ PersistKernel pk_lookup_local_ef(int chunks, int rb, int src, int threads, int e
 PersistKernel pk_lookup_local_wide_ef21(int chunks, int rb, int src, int threads, int extra);
 PersistKernel pk_lookup_local_plus(int chunks, int rb, int src, int threads, int extra);
 PersistKernel pk_lookup_local_wide_ef(int chunks, int rb, int src, int threads, int extra);
+PersistKernel pk_lookup_local_floor(int chunks, int rb, int src, int threads, int extra);
+PersistKernel pk_lookup_local_wide_floor(int chunks, int rb, int src, int threads, int extra);
 PersistKernel pk_lookup_ef(int chunks, int rb, int src, int threads, int extra);            // Algorithm 4, roles
 PersistKernel pk_lookup_floor(int chunks, int rb, int src, int threads, int extra);         // exchange skeleton, roles
 PersistKernel pk_lookup_wide_ef21(int chunks, int rb, int src, int threads, int extra);     // Algorithm 2, wide

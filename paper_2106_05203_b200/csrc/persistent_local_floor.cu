@@ -1,0 +1,9 @@
+// Exchange skeleton of the persistent cluster kernel with all workers in one cluster (no arithmetic of the method).
+#define PK_BODY_FILE "persistent_roles.inc"
+#define PK_KERNEL_NAME persistent_local_floor_kernel
+#define PK_LOOKUP_NAME pk_lookup_local_floor
+#define PK_PLUS 0
+#define PK_EF 0
+#define PK_FLOOR 1
+#define PK_LOCAL 1
+#include "persistent_method.inc"

@@ -47,3 +47,26 @@ def test_many_iterations_are_as_many_calls(variant, n, d, k, rows):
         states.append([np.array(a) for a in h.get_state_host()])
     for a, b in zip(*states):
         assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
+
+
+# both bodies (Top-1: serving warp), one and several blocks per worker, and a shape with a cluster per worker
+@pytest.mark.parametrize("n,d,k,rows,one_cluster", [(4, 64, 4, 50, True), (2, 112, 1, 800, True), (16, 130, 1, 20, True), (2, 100, 7, 700, True),
+                                                    (20, 112, 1, 40, False)])
+def test_exchange_skeleton_has_the_form_of_the_run(n, d, k, rows, one_cluster):
+    from paper_2106_05203_b200 import binding as B
+    w = _workload(n, d, k, rows, seed=3)
+    forms, states = [], []
+    for floor in (True, False):
+        h = make_gpu(w, path=B.PATH_PERSISTENT)
+        h.init(B.INIT_ZERO)
+        h.step(3)
+        forms.append((h.get_persistent_form(), h.get_persistent_shape(), h.get_persistent_body()))
+        if floor:
+            h.selftest_exchange_floor(70)
+            forms.append((h.get_persistent_form(), h.get_persistent_shape(), h.get_persistent_body()))
+        h.step(4)                           # the skeleton leaves the state and the order of epochs alone
+        assert h.poll() == 0
+        states.append([np.array(a) for a in h.get_state_host()])
+    assert forms[0] == forms[1] == forms[2] and forms[0][0][0] == one_cluster
+    for a, b in zip(*states):
+        assert np.array_equal(a.view(np.uint32), b.view(np.uint32))
