@@ -109,6 +109,11 @@ aggregate_kernel(const int* __restrict__ idx, const float* __restrict__ val, con
 // The same aggregation with the tile's message entries first staged in shared memory (one
 // parallel gather), so that the ordered pass over the workers touches shared memory only.
 // Needs n <= AGG_STAGE_MAX_N; a tile with more than AGG_STAGE_CAP entries takes the direct loop.
+// alone: nothing may be placed beside the blocks (no pdl_trigger), for handles whose rounds have a streaming pass.  A block takes 39 KB
+// of shared memory, and an SM that never runs empty keeps that split: the streaming pass of the next round, two kernels further on, ran
+// with an L1 too small for its loads in flight.  Calls of one round each, us a round, alone / not: 64 x 4,194,304 393 / 459,
+// 64 x 1,000,000 121 / 158, 20 x 1,000,000 59 / 75, 1 x 25,000,000 141 / 161; with Algorithm 4 64 x 4,194,304 597 / 680.  Shorter vectors,
+// whose selection is one kernel, lose the overlap: 20 x 200,000 62.2 / 61.3, 5 x 50,000 34.1 / 33.6.
 constexpr int AGG_STAGE_MAX_N = 1024;
 constexpr int AGG_STAGE_CAP = 3072;
 constexpr int AGG_OWNER_SCAN_MAX = 512;   // tiles with at most this many entries skip the per-worker loop
@@ -117,8 +122,8 @@ template <int XMODE>
 __global__ void __launch_bounds__(AGG_BLOCK)
 aggregate_staged_kernel(const int* __restrict__ idx, const float* __restrict__ val, const int* __restrict__ off,
                         int n, int k, int ntiles, i64 d, float inv_n, float gamma,
-                        float* __restrict__ g, float* __restrict__ x) {
-    pdl_trigger();
+                        float* __restrict__ g, float* __restrict__ x, int alone) {
+    if (!alone) pdl_trigger();
     pdl_wait(idx, val, off, g, x);
     __shared__ float s[AGG_TILE];
     __shared__ __align__(4) unsigned short touched[AGG_TILE];   // staged entries per coordinate

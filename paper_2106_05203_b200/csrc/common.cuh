@@ -10,8 +10,8 @@ typedef long long i64;
 // Programmatic dependent launch.  Launched the plain way, a kernel that follows another one in a stream starts 2-4 us after
 // its predecessor's end (in steps of about 1 us; measured with spinning kernels of 0.3-10 us); launched as a programmatic
 // dependent it starts after 0.5 us.  Every kernel of the library calls pdl_wait() before it touches global memory (it
-// returns when the preceding kernels of the stream have completed and their writes are visible) and pdl_trigger() early,
-// so that the kernel behind it can be placed on the device meanwhile.
+// returns when the preceding kernels of the stream have completed and their writes are visible) and pdl_trigger() early (the
+// staged aggregation only where that pays, see apply.cuh), so that the kernel behind it can be placed on the device meanwhile.
 // The kernel's pointers go through pdl_wait so that no load through them -- a read-only one (const __restrict__, __ldg, __ldcs) is
 // otherwise free to move -- is placed in front of the wait.  Where they come in a struct, the local pointer that such loads
 // start from is made by pdl_ptr, behind the wait; or the loads are plain ones, which the wait's memory clobber keeps behind it

@@ -655,13 +655,19 @@ ef21_status enqueue_aggregate_into(ef21_ctx* c, float* target, float factor, int
         c->launches += 1;
     }
     c->agg_off_ready = false;
-    auto kern = c->n <= AGG_STAGE_MAX_N
-                    ? (xmode == AGG_X_KEEP ? aggregate_staged_kernel<AGG_X_KEEP>
-                                           : (xmode == AGG_X_BEFORE ? aggregate_staged_kernel<AGG_X_BEFORE> : aggregate_staged_kernel<AGG_X_AFTER>))
-                    : (xmode == AGG_X_KEEP ? aggregate_kernel<AGG_X_KEEP>
-                                           : (xmode == AGG_X_BEFORE ? aggregate_kernel<AGG_X_BEFORE> : aggregate_kernel<AGG_X_AFTER>));
-    CU(launch(kern, dim3(c->L.agg_tiles), AGG_BLOCK, 0, c->stream, 1, c->msg_idx(), c->msg_val(), c->at<int>(c->L.agg_off), c->n, c->k,
-              c->L.agg_tiles, c->d, factor, c->gamma, target, c->x()));
+    const dim3 tiles(c->L.agg_tiles);
+    const int* off = c->at<int>(c->L.agg_off);
+    if (c->n <= AGG_STAGE_MAX_N) {
+        auto kern = xmode == AGG_X_KEEP ? aggregate_staged_kernel<AGG_X_KEEP>
+                                        : (xmode == AGG_X_BEFORE ? aggregate_staged_kernel<AGG_X_BEFORE> : aggregate_staged_kernel<AGG_X_AFTER>);
+        CU(launch(kern, tiles, AGG_BLOCK, 0, c->stream, 1, c->msg_idx(), c->msg_val(), off, c->n, c->k, c->L.agg_tiles, c->d, factor, c->gamma,
+                  target, c->x(), long_topk(c) ? 1 : 0));
+    } else {
+        auto kern = xmode == AGG_X_KEEP ? aggregate_kernel<AGG_X_KEEP>
+                                        : (xmode == AGG_X_BEFORE ? aggregate_kernel<AGG_X_BEFORE> : aggregate_kernel<AGG_X_AFTER>);
+        CU(launch(kern, tiles, AGG_BLOCK, 0, c->stream, 1, c->msg_idx(), c->msg_val(), off, c->n, c->k, c->L.agg_tiles, c->d, factor, c->gamma,
+                  target, c->x()));
+    }
     c->launches += 1;
     return EF21_OK;
 }
