@@ -5,9 +5,10 @@
 //   2. st_collect_kernel: the streaming pass.  A warp owns a region of 1,024 or 4,096 consecutive entries and lists those with
 //      key >= lo in index order (ballot ranks); a record is (index, v, b + v), so the updated state value travels with the
 //      candidate.  Entries with key >= hi are in the message for sure and only counted; those in between ("open" ones) also go
-//      to a list of the vector and into a histogram of 2,048 steps of [lo, hi).  st_cut_kernel, a
-//      cluster per vector, finds the exact cut from that histogram and list -- a composite of key and index, so ties at the
-//      k-th key go to the lower index -- and the position in the message at which every region's entries begin.
+//      to a list of the vector and into a histogram of 2,048 steps of [lo, hi).  (Large batches: st_collect_long_kernel only
+//      lists, and st_cut_kernel tells the sure entries from the open ones.)  st_cut_kernel, a cluster per vector, finds the
+//      exact cut from that histogram and list -- a composite of key and index, so ties at the k-th key go to the lower
+//      index -- and the position in the message at which every region's entries begin.
 //   3. st_compact_kernel: eight lanes per region write the selected entries to their places, store b + v (Algorithm 4: zero)
 //      on the selected coordinates and, on request, where each tile of coordinates begins in the message.  A region with more
 //      candidates than its list holds is read again; where more than a tenth of the entries are wanted no lists are kept
@@ -16,7 +17,7 @@
 //      the k-th key or whose open list overflowed (masses of ties, fewer than k non-zeros); for the others it returns at once.
 // The bracket only decides speed, never the result.
 //
-// What bounds it: HBM in step 2 (64 vectors of 4 million entries: 321 us, 1.02 of the copy peak); steps 1 and 3 are a few
+// What bounds it: HBM in step 2 (64 vectors of 4 million entries: 306 us, 7.0 TB/s of reading); steps 1 and 3 are a few
 // microseconds each and take no part of a vector's length.
 #pragma once
 #include <cooperative_groups.h>
@@ -155,63 +156,90 @@ st_sample_kernel(const __grid_constant__ StArgs p, float rank, float margin) {
 
 // ---- 2. streaming pass --------------------------------------------------------------------------
 // The streaming pass for large batches of aligned rows, regions of 4,096 entries, one warp each; grid = (ceil(nreg / 8), batch).
-// The loop only lists candidates and so stays within 32 registers: eight blocks per SM with one 16-byte load per array in
-// flight per lane saturate HBM.  (With the open entries counted on the way, which spills, or behind the loop, where a warp
-// stops streaming, the pass over 64 x 4,194,304 entries took 350-390 us instead of 320; st_cut_kernel<C, true> counts them.)
+// HBM bounds it.  The loop only lists candidates; four 16-byte loads per array are in flight per lane (64-68 registers, no spills,
+// three or four blocks per SM).  64 x 4,194,304 entries, V and g_i: 306 us, 7.0 TB/s; one load per array and eight blocks of 32
+// registers, which spilt, 331 us (a round 393 -> 379, of Algorithm 4 597 -> 564); two loads and five blocks 313.  (With the open
+// entries counted on the way, or behind the loop, where a warp stops streaming, the pass takes longer; st_cut_kernel<C, true>
+// counts them.)
+constexpr int ST_LONG_LOADS = 4, ST_LONG_BLOCKS = 3;
+
 template <int MODE>
-__global__ void __launch_bounds__(ST_WARPS * 32, 8)
+__global__ void __launch_bounds__(ST_WARPS * 32, ST_LONG_BLOCKS)
 st_collect_long_kernel(const __grid_constant__ StArgs p) {
+    constexpr int U = ST_LONG_LOADS, REGION = 1 << ST_REGION_LOG_LARGE;
     pdl_trigger();
     pdl_wait();
     const int lane = threadIdx.x & 31;
     const int vec = blockIdx.y, region = blockIdx.x * ST_WARPS + (threadIdx.x >> 5);
     if (region >= p.nreg) return;
     const unsigned lo = p.ctl[vec].lo;
-    const i64 base = (i64)region << ST_REGION_LOG_LARGE;
-    const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a);
-    float* bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b);
+    const int first = region << ST_REGION_LOG_LARGE, end = (int)min((i64)REGION, p.d - first);    // positions below are relative to `first`
+    const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a + first);
+    float* bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b + first);
     int4* out = p.cand + ((i64)vec * p.nreg + region) * p.cap;
-    const unsigned lt = (1u << lane) - 1u;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     int cnt = 0;
-    for (int it = 0; it < 32; ++it) {
-        const i64 j0 = base + it * 128 + 4 * lane;
-        float v[4], old[4];
-        if (j0 + 3 < p.d) {
-            const float4 x = __ldcs(reinterpret_cast<const float4*>(av + j0));
-            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-            if (MODE != TC_PLAIN) {
-                const float4 g = __ldcs(reinterpret_cast<const float4*>(bv + j0));
-                old[0] = g.x; old[1] = g.y; old[2] = g.z; old[3] = g.w;
-            } else {
-                old[0] = old[1] = old[2] = old[3] = 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = st_value<MODE>(v[e], old[e], p.gamma);
-            if (MODE == TC_EF) __stcs(reinterpret_cast<float4*>(bv + j0), make_float4(v[0], v[1], v[2], v[3]));
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                old[e] = (MODE != TC_PLAIN && j0 + e < p.d) ? bv[j0 + e] : 0.f;
-                v[e] = j0 + e < p.d ? st_value<MODE>(av[j0 + e], old[e], p.gamma) : 0.f;
-                if (MODE == TC_EF && j0 + e < p.d) bv[j0 + e] = v[e];
-            }
-        }
+    auto form = [&](float4 x, const float4& g) {
+        x.x = st_value<MODE>(x.x, g.x, p.gamma); x.y = st_value<MODE>(x.y, g.y, p.gamma);
+        x.z = st_value<MODE>(x.z, g.z, p.gamma); x.w = st_value<MODE>(x.w, g.w, p.gamma);
+        return x;
+    };
+    // the candidates among 128 entries, four consecutive ones (from j0 on) per lane
+    auto list = [&](int j0, const float4& x, const float4& g) {
+        const float v[4] = {x.x, x.y, x.z, x.w}, old[4] = {g.x, g.y, g.z, g.w};
         bool pr[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) pr[e] = mag_key(v[e]) >= lo;       // lo >= 1: the zeros behind the end never are
-        const unsigned any = __ballot_sync(0xffffffffu, pr[0] | pr[1] | pr[2] | pr[3]);
-        if (any) {
-            unsigned bm[4];
+        if (__any_sync(0xffffffffu, pr[0] | pr[1] | pr[2] | pr[3])) {
+            const unsigned lt = (1u << lane) - 1u;
+            int pos = cnt;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) bm[e] = __ballot_sync(0xffffffffu, pr[e]);
-            int pos = cnt + __popc(bm[0] & lt) + __popc(bm[1] & lt) + __popc(bm[2] & lt) + __popc(bm[3] & lt);
+            for (int e = 0; e < 4; ++e) {
+                const unsigned bm = __ballot_sync(0xffffffffu, pr[e]);
+                pos += __popc(bm & lt); cnt += __popc(bm);
+            }
 #pragma unroll
             for (int e = 0; e < 4; ++e)
                 if (pr[e]) {
-                    if (pos < p.cap) out[pos] = make_int4((int)(j0 + e), __float_as_int(v[e]), __float_as_int(__fadd_rn(old[e], v[e])), 0);
+                    if (pos < p.cap) out[pos] = make_int4(first + j0 + e, __float_as_int(v[e]), __float_as_int(__fadd_rn(old[e], v[e])), 0);
                     ++pos;
                 }
-            cnt += __popc(bm[0]) + __popc(bm[1]) + __popc(bm[2]) + __popc(bm[3]);
+        }
+    };
+    if (end == REGION) {
+#pragma unroll 1
+        for (int j0 = 4 * lane; j0 < REGION; j0 += 128 * U) {
+            float4 x[U], g[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                x[u] = __ldcs(reinterpret_cast<const float4*>(av + j0 + 128 * u));
+                g[u] = MODE == TC_PLAIN ? zero : __ldcs(reinterpret_cast<const float4*>(bv + j0 + 128 * u));
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                x[u] = form(x[u], g[u]);
+                if (MODE == TC_EF) __stcs(reinterpret_cast<float4*>(bv + j0 + 128 * u), x[u]);
+                list(j0 + 128 * u, x[u], g[u]);
+            }
+        }
+    } else {
+        // the last region of a vector whose length is no multiple of 4,096
+#pragma unroll 1
+        for (int j0 = 4 * lane; j0 - 4 * lane < end; j0 += 128) {
+            const int left = end - j0;
+            float4 x = zero, g = zero;
+            if (left > 0) { x.x = av[j0]; if (MODE != TC_PLAIN) g.x = bv[j0]; }
+            if (left > 1) { x.y = av[j0 + 1]; if (MODE != TC_PLAIN) g.y = bv[j0 + 1]; }
+            if (left > 2) { x.z = av[j0 + 2]; if (MODE != TC_PLAIN) g.z = bv[j0 + 2]; }
+            if (left > 3) { x.w = av[j0 + 3]; if (MODE != TC_PLAIN) g.w = bv[j0 + 3]; }
+            x = form(x, g);
+            if (MODE == TC_EF) {
+                if (left > 0) bv[j0] = x.x;
+                if (left > 1) bv[j0 + 1] = x.y;
+                if (left > 2) bv[j0 + 2] = x.z;
+                if (left > 3) bv[j0 + 3] = x.w;
+            }
+            list(j0, x, g);
         }
     }
     if (lane == 0) p.reg_cand[(i64)vec * p.nreg_pitch + region] = (unsigned)cnt;
