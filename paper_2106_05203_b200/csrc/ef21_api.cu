@@ -47,10 +47,7 @@ inline i64 ceil_div(i64 a, i64 b) { return (a + b - 1) / b; }
 // Workspace layouts
 // ---------------------------------------------------------------------------------------------
 
-// Kernel launch as a programmatic dependent of whatever precedes it in the stream (see pdl_wait), with clusters of C blocks.  C = 0: not
-// a programmatic dependent.  For long passes over memory: their first blocks would move in beside the last ones of a kernel that
-// uses much shared memory, find the SM split in its favour and keep that, and an L1 too small for the loads in flight (64 x
-// 4,194,304: 125 us more for the copy of the state behind an aggregation).
+// Kernel launch as a programmatic dependent of whatever precedes it in the stream (see pdl_wait), with clusters of C blocks.
 template <typename... Params, typename... Args>
 cudaError_t launch(void (*kern)(Params...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, unsigned C, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -60,7 +57,7 @@ cudaError_t launch(void (*kern)(Params...), dim3 grid, unsigned block, size_t sm
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = C > 1 ? 2 : C;
+    cfg.attrs = attr; cfg.numAttrs = C > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
 }
 
@@ -312,7 +309,7 @@ struct Copies {
     }
     ef21_status run(cudaStream_t st, i64* launches) {
         if (blocks == 0) return EF21_OK;
-        CU(launch(copy_segments_kernel, dim3((unsigned)blocks), COPY_THREADS, 0, st, blocks > 148 * 16 ? 0 : 1, p));
+        CU(launch(copy_segments_kernel, dim3((unsigned)blocks), COPY_THREADS, 0, st, 1, p));
         *launches += 1;
         return EF21_OK;
     }
