@@ -42,9 +42,9 @@ NCU_TRAFFIC = {
     "headline": {"per": "launch", "bytes": 3746048},
     # persistent_kernel<3,4,GMEM,512,0>, launches of 50 iterations: 30,100,547,840 B read + 4,156,416 B written
     "hbm_persistent": {"per": "iteration", "bytes": 602094085},
-    # st_collect_kernel<true> captured at n = 16 workers (537.12 MB read + 4.64 MB written per launch), scaled by
+    # st_collect_long_kernel captured at n = 16 workers (537.04 MB read + 3.90 MB written per launch), scaled by
     # 64 / 16: the pass reads every vector once, so its traffic grows with the number of workers
-    "stress_collect": {"per": "iteration", "bytes": 2167040000},
+    "stress_collect": {"per": "iteration", "bytes": 2163761152},
 }
 
 

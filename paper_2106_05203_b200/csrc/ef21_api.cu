@@ -601,7 +601,7 @@ bool long_topk(const ef21_ctx* c) {
 ef21_status enqueue_round_select(ef21_ctx* c, const float* a, i64 pitch_a, bool sampled) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
     if (long_topk(c)) {
-        // the finish kernel also leaves the per-tile offsets of the messages for the aggregation
+        // the compaction also leaves the per-tile offsets of the messages for the aggregation
         const StOut out = {c->msg_idx(), c->msg_val(), c->gi(), c->L.ld, c->at<int>(c->L.agg_off), c->L.agg_tiles, c->status(), nullptr};
         EF(enqueue_topk_stream<TC_DIFF>(c->stream, a, pitch_a, c->gi(), c->L.ld, 0.f, c->n, c->d, c->k, out, B, &c->launches, true, sampled));
         c->agg_off_ready = true;
@@ -852,7 +852,8 @@ PersistKernel persistent_kernel_of(const ef21_ctx* c, bool roles, bool local, in
 PersistPlan plan_persistent(ef21_ctx* c) {
     // Automatic choice: the serving-warp body for Top-1 (2.6 against 3.2 us per iteration on the mushrooms-shaped
     // workload, 3.4 against 4.0 on the a9a-shaped one, the same 10.4 on the w8a-shaped one, measured); with more
-    // entries per message its k arg-max rounds in one warp cost more than the whole block counting ranks.
+    // entries per message the three polling rounds of a single warp cost more than the whole block's table (a9a-shaped, Top-4:
+    // 5.6 against 4.5 us).
     const bool roles_can = c->variant != EF21_VARIANT_EF21_PLUS && c->k <= PK_ROLES_MAX_K;
     const bool roles_first = c->pk_body == 1 || (c->pk_body == 0 && c->k == 1);
     if (roles_can && roles_first) {
@@ -1332,8 +1333,8 @@ ef21_status ef21_step_grads(ef21_ctx* c, const float* V_dev, int32_t steps) {
     }
     // Same V at every step: the threshold estimate of round t+1 needs V and g_i^{t+1} only, so it runs beside the aggregation of
     // round t (g and x); the streaming pass of round t+1 waits for both.  The longer of the two follows the selection on
-    // this stream, without an event in between: the aggregation where there are many message entries (64 x 4,194: 395 us a round
-    // against 398, 24 x 40,000: 293 against 300), else the estimate (16 x 4,194: 132 against 142).
+    // this stream, without an event in between: the aggregation where there are many message entries (64 x 4,194: 376.8 us a round
+    // against 377.6, 24 x 40,000: 283 against 289), else the estimate (16 x 4,194: 125 against 135, 64 x 1,000: 121 against 125).
     cudaStream_t main_stream = c->stream;
     const bool agg_first = (i64)c->n * c->k > 131072;
     for (int t = 0; t < steps; ++t) {

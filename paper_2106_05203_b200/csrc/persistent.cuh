@@ -14,8 +14,8 @@
 //      memory that credit an mbarrier there; the senders do not wait, the leader waits (bounded) for
 //      the byte count of all partials
 //   4. leader block: grad_i = sum/m_i + regulariser' and v = grad_i - g_i, one coordinate per
-//      thread; Top-k either by k rounds of a warp arg-max on (|v| bits, lower index wins) or, for
-//      larger k, by rank counting (every coordinate counts the entries ahead of it); g_i += c_i;
+//      thread; Top-k by rounds of a warp arg-max on (|v| bits, lower index wins), for five and more
+//      entries of wide vectors in two steps (per 128 coordinates, then among the picks); g_i += c_i;
 //      k packed 64-bit words (epoch:16 | index:16 | value bits:32) go into a double-buffered global
 //      slot array
 //   5. every block polls the n*k words of this iteration's epoch (bounded spin); then each
@@ -135,8 +135,8 @@ __device__ __forceinline__ void st_async_f4(unsigned remote_dst, float4 v, unsig
 // Rows from global memory through shared memory: every warp owns a ring of `stages` batches, filled by bulk copies (a batch is
 // contiguous) that one lane issues as soon as the batch before it in the stage has been taken into registers.  The rows are
 // the same in every iteration, so the ring runs on from one sweep into the next: while a block exchanges messages, the
-// first batches of its next sweep arrive (a third of a block's rows on the w8a-shaped workload), and neither registers nor
-// issue slots are spent on loads in flight.  Every wait is bounded; a wait that gives up records EF21_ERR_TIMEOUT.
+// first batches of its next sweep arrive, and neither registers nor issue slots are spent on loads in flight.  Chosen for rows of
+// up to 190 columns (plan_persistent_body).  Every wait is bounded; a wait that gives up records EF21_ERR_TIMEOUT.
 struct RowRing {
     float* stage0;                 // this warp's first stage
     unsigned long long* bars;      // its barriers, one per stage
@@ -277,8 +277,8 @@ typedef void (*PersistKernel)(const PersistParams);
 // extra rows per batch), or nullptr if that shape is not instantiated.
 // Two bodies exist.  "roles" (persistent_roles.inc): the last warp of a block serves it, the others only sweep rows;
 // Top-k by warp arg-max rounds -- for k <= PK_ROLES_MAX_K.  "wide" (persistent_body.inc): every step is taken by the
-// whole block between block barriers, Top-k by rank counting over all threads for larger k -- any k <= PK_MAX_K, and
-// the only body of Algorithm 3.
+// whole block between block barriers, Top-k by one warp, or in two steps by several -- any k <= PK_MAX_K, and the only
+// body of Algorithm 3.
 constexpr int PK_LOCAL_BLOCKS = 16, PK_LOCAL_MSGS = 48;      // all workers in one cluster: most blocks, most words per iteration (64: 2.81 us against 2.78)
 constexpr int PK_ROLES_MAX_K = 8;
 PersistKernel pk_lookup_ef21(int chunks, int rb, int src, int threads, int extra);          // Algorithm 2, roles
