@@ -413,11 +413,11 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
     unsigned long long* stage = reinterpret_cast<unsigned long long*>(st_cut_smem);      // block 0: open entries of the deciding step
     unsigned long long* mine_open = stage + ST_OPEN_STAGE;                               // CLASSIFY: this block's open entries
     unsigned* hist = reinterpret_cast<unsigned*>(mine_open + ST_OPEN_STAGE);             // CLASSIFY: their histogram
-    __shared__ unsigned scratch[33], found[3], stage_n, sure_sh, open_sh, over_sh;
-    __shared__ unsigned long long cut_sh;
+    __shared__ unsigned scratch[33], scratch_b[32], found[3], stage_n, sure_sh, open_sh, over_sh;
+    __shared__ unsigned long long cut_sh, differ_sh;
     cg::cluster_group cluster = cg::this_cluster();
     const int tid = threadIdx.x, rk = (int)cluster.block_rank(), vec = (int)(blockIdx.x / (unsigned)C);
-    if (tid == 0) { stage_n = 0u; sure_sh = 0u; open_sh = 0u; over_sh = 0u; }
+    if (tid == 0) { stage_n = 0u; sure_sh = 0u; open_sh = 0u; over_sh = 0u; differ_sh = 0ull; }
     if (CLASSIFY) { hist[tid] = 0u; hist[tid + 1024] = 0u; }
     __syncthreads();
     if (!CLASSIFY) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); // block 0's counter is ready
@@ -534,20 +534,37 @@ st_cut_kernel(const __grid_constant__ StArgs p) {
             __syncthreads();
             cut = cut_sh;
         } else {
-            // largest cut with at least `need` entries at or above it, bit by bit from the step's lower end
-            const unsigned long long low = (unsigned long long)(lo + (step << shift)) << 32;
-            cut = low;
+            // Largest cut with at least `need` entries at or above it.  Bits that all of them share are the cut's; the others are
+            // found two at a time.  (All bits of the step, one at a time: rounds on 64 x 4,194,304 values of bf16, whose groups of
+            // equal keys share all but the index, 395 us instead of 388.)
+            const unsigned long long any = stage[0];
+            unsigned long long differ = 0ull;
+            for (unsigned e = tid; e < pop; e += 1024u) differ |= stage[e] ^ any;
+            const unsigned dh = __reduce_or_sync(0xffffffffu, (unsigned)(differ >> 32)), dl = __reduce_or_sync(0xffffffffu, (unsigned)differ);
+            if ((tid & 31) == 0) atomicOr(&differ_sh, ((unsigned long long)dh << 32) | dl);
+            __syncthreads();
+            differ = differ_sh;
+            cut = any & ~differ;
 #pragma unroll 1
-            for (int bit = 31 + (int)shift; bit >= 0; --bit) {
-                const unsigned long long c0 = cut + (1ull << bit);
-                unsigned cnt = 0u;
-                for (unsigned e = tid; e < pop; e += 1024u) cnt += stage[e] >= c0 ? 1u : 0u;
-                cnt = __reduce_add_sync(0xffffffffu, cnt);
-                if ((tid & 31) == 0) scratch[tid >> 5] = cnt;
+            while (differ != 0ull) {
+                const unsigned long long b1 = 1ull << (63 - __clzll((long long)differ));
+                differ ^= b1;
+                const unsigned long long b0 = differ != 0ull ? 1ull << (63 - __clzll((long long)differ)) : 0ull;
+                differ ^= b0;
+                unsigned two = 0u, one = 0u;                         // at or above cut + b1 + b0 (low half) and cut + b1; cut + b0
+                for (unsigned e = tid; e < pop; e += 1024u) {
+                    const unsigned long long x = stage[e];
+                    two += (x >= (cut | b1 | b0) ? 1u : 0u) + (x >= (cut | b1) ? 0x10000u : 0u);
+                    one += x >= (cut | b0) ? 1u : 0u;
+                }
+                two = __reduce_add_sync(0xffffffffu, two); one = __reduce_add_sync(0xffffffffu, one);
+                if ((tid & 31) == 0) { scratch[tid >> 5] = two; scratch_b[tid >> 5] = one; }
                 __syncthreads();
-                cnt = __reduce_add_sync(0xffffffffu, scratch[tid & 31]);
+                two = __reduce_add_sync(0xffffffffu, scratch[tid & 31]); one = __reduce_add_sync(0xffffffffu, scratch_b[tid & 31]);
                 __syncthreads();
-                if (cnt >= need) cut = c0;
+                if ((two & 0xffffu) >= need) cut |= b1 | b0;
+                else if ((two >> 16) >= need) cut |= b1;
+                else if (one >= need) cut |= b0;
             }
         }
         for (unsigned e = tid; e < pop; e += 1024u) {
