@@ -37,6 +37,7 @@ constexpr int ST_SAMPLE_STEPS = 1024;   // steps of the sampled range
 constexpr int ST_OPEN_BINS = 2048;
 constexpr int ST_OPEN_STAGE = 8192;     // open entries of the deciding step that are ranked in shared memory
 constexpr int ST_BLOCK_OPEN = 2048;     // open entries a block of the streaming pass gathers before they go to the list
+constexpr int ST_GATHER = 160;          // a warp's buffer for candidates: emptied from 32 on, after at most 128 more
 constexpr i64 ST_MIN_D = 262144;        // shorter vectors always fit into a cluster
 
 // Per vector: the bracket, the counters of the streaming pass, the exact cut.
@@ -248,47 +249,68 @@ st_collect_long_kernel(const __grid_constant__ StArgs p) {
 // The streaming pass for everything else: grid = (blocks per vector, batch), 256 threads, one warp per region, in turn.  VEC: both
 // rows 16-byte aligned.  U loads per array are in flight per lane: short regions and 4-byte loads (rows of odd length) need
 // more of them and leave room for four blocks per SM.
-// LISTS: candidates are listed (else every region is read again).
+// LISTS: candidates are listed (else every region is read again, the sure entries are only counted and the open ones gathered).
+// Short of HBM it is the number of instructions that bounds it, above all of those that few lanes take part in: candidates go to a
+// buffer in shared memory, and whenever it holds 32 of them the lanes write and classify them side by side; whole batches of loads go
+// without a bounds check.  Before, a lane wrote and classified its candidate alone: 20 x 2,642,533 with a tenth wanted 119 us, now 61;
+// 16 x 1,000,003 (odd rows, one in a hundred) V and g_i 25.3 -> 22.7 us, V alone 23.3 -> 21.0; 4 x 1,461,252 14.7 -> 13.6.
 template <int MODE, bool VEC, int U, bool LISTS>
 __global__ void __launch_bounds__(ST_WARPS * 32, 4)
 st_collect_kernel(const __grid_constant__ StArgs p) {
     __shared__ unsigned long long stage[ST_BLOCK_OPEN];
+    __shared__ __align__(16) int4 gather_sh[ST_WARPS][ST_GATHER];
     __shared__ unsigned sure_sh, open_sh, open_at;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int vec = blockIdx.y;
+    int4* gather = gather_sh[warp];
     if (tid == 0) { sure_sh = 0u; open_sh = 0u; }
     __syncthreads();
     pdl_trigger();
     pdl_wait();
-    // an entry above lo: sure, or open (gathered per block: one counter in global memory for every one would serialise them)
-    auto classify = [&](unsigned key, unsigned j) {
-        const StCtl& ct = p.ctl[vec];
-        if (key >= ct.hi) return 1u;
-        atomicAdd(&p.open_hist[(i64)vec * ST_OPEN_BINS + ((key - ct.lo) >> ct.shift)], 1u);
-        const unsigned long long x = st_composite(key, j);
-        const unsigned at = atomicAdd(&open_sh, 1u);
-        if (at < (unsigned)ST_BLOCK_OPEN) stage[at] = x;
-        else {
-            const unsigned to = atomicAdd(&p.ctl[vec].open, 1u);
-            if (to < p.open_cap) p.open_list[(i64)vec * p.open_cap + to] = x;
-        }
-        return 0u;
-    };
 #pragma unroll 1
     for (int region = blockIdx.x * ST_WARPS + warp; region < p.nreg; region += gridDim.x * ST_WARPS) {
-        const unsigned lo = p.ctl[vec].lo;
+        const unsigned lo = p.ctl[vec].lo, hi = LISTS ? 0u : p.ctl[vec].hi;
         const i64 base = (i64)region << p.region_log;
         const int end = (int)min((i64)1 << p.region_log, p.d - base);           // positions below are relative to the region
         const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a + base);
         float* bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b + base);
-        int4* out = p.cand + ((i64)vec * p.nreg + region) * p.cap;
-        unsigned cnt = 0u, sure = 0u;
-        // listed candidates are classified behind the loop, by lanes side by side
-        auto candidate = [&](unsigned pos, int j, float v, float old) {
-            if (LISTS && pos < (unsigned)p.cap)
-                out[pos] = make_int4((int)base + j, __float_as_int(v), __float_as_int(__fadd_rn(old, v)), 0);
-            if (!LISTS) sure += classify(mag_key(v), (unsigned)base + (unsigned)j);
+        unsigned held = 0u, done = 0u, sure = 0u;                               // in the buffer, written before, sure entries (per lane)
+        // the buffer's candidates: records to the region's list; an entry is sure, or open (gathered per block: one counter in
+        // global memory for every one would serialise them)
+        auto empty = [&]() {
+            __syncwarp();
+            const StCtl& ct = p.ctl[vec];
+            int4* out = p.cand + ((i64)vec * p.nreg + region) * p.cap;
+            for (unsigned e = lane; e < held; e += 32u) {
+                const int4 w = gather[e];
+                const unsigned key = (unsigned)w.y & 0x7fffffffu;
+                if (LISTS) {
+                    if (done + e < (unsigned)p.cap) out[done + e] = w;
+                    if (key >= ct.hi) { ++sure; continue; }
+                }
+                atomicAdd(&p.open_hist[(i64)vec * ST_OPEN_BINS + ((key - ct.lo) >> ct.shift)], 1u);
+                const unsigned long long x = st_composite(key, (unsigned)w.x);
+                const unsigned at = atomicAdd(&open_sh, 1u);
+                if (at < (unsigned)ST_BLOCK_OPEN) stage[at] = x;
+                else {
+                    const unsigned to = atomicAdd(&p.ctl[vec].open, 1u);
+                    if (to < p.open_cap) p.open_list[(i64)vec * p.open_cap + to] = x;
+                }
+            }
+            done += held; held = 0u;
+            __syncwarp();
         };
+        auto put = [&](unsigned at, int j, float v, float old) {
+            gather[at] = make_int4((int)base + j, __float_as_int(v), __float_as_int(__fadd_rn(old, v)), 0);
+        };
+        // wanted: a candidate (no lists: an open entry)
+        auto wanted = [&](float v) {
+            const unsigned key = mag_key(v);
+            if (LISTS) return key >= lo;
+            if (key >= hi) ++sure;
+            return key >= lo && key < hi;
+        };
+        // 128 entries, four consecutive ones per lane
         auto four = [&](int j0, const float4& x, const float4& g) {
             const float old[4] = {g.x, g.y, g.z, g.w};
             const float v[4] = {st_value<MODE>(x.x, old[0], p.gamma), st_value<MODE>(x.y, old[1], p.gamma),
@@ -299,34 +321,62 @@ st_collect_kernel(const __grid_constant__ StArgs p) {
             }
             bool pr[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) pr[e] = mag_key(v[e]) >= lo;               // lo >= 1: the zeros behind the end never are
+            for (int e = 0; e < 4; ++e) pr[e] = wanted(v[e]);                      // lo >= 1: the zeros behind the end never are
             if (__any_sync(0xffffffffu, pr[0] | pr[1] | pr[2] | pr[3])) {
                 const unsigned lt = (1u << lane) - 1u;
-                unsigned pos = cnt;
+                unsigned pos = held;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const unsigned bm = __ballot_sync(0xffffffffu, pr[e]);
-                    pos += (unsigned)__popc(bm & lt); cnt += (unsigned)__popc(bm);
+                    pos += (unsigned)__popc(bm & lt); held += (unsigned)__popc(bm);
                 }
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (pr[e]) { candidate(pos, j0 + e, v[e], old[e]); ++pos; }
+                    if (pr[e]) { put(pos, j0 + e, v[e], old[e]); ++pos; }
+                if (held >= 32u) empty();
+            }
+        };
+        // 32 * U entries, a lane's 32 apart
+        auto apart = [&](int j0, float (&v)[U], const float (&old)[U], int left) {
+            bool any = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                v[u] = st_value<MODE>(v[u], old[u], p.gamma);
+                if (MODE == TC_EF && 32 * u < left) __stcs(bv + j0 + 32 * u, v[u]);
+                any |= LISTS ? mag_key(v[u]) >= lo : wanted(v[u]);
+            }
+            if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const unsigned key = mag_key(v[u]);
+                    const bool pr = key >= lo && (LISTS || key < hi);
+                    const unsigned bm = __ballot_sync(0xffffffffu, pr);
+                    if (pr) put(held + (unsigned)__popc(bm & ((1u << lane) - 1u)), j0 + 32 * u, v[u], old[u]);
+                    held += (unsigned)__popc(bm);
+                    if (u % 4 == 3 && held >= 32u) empty();
+                }
             }
         };
         if (VEC) {
 #pragma unroll 1
             for (int i0 = 0; i0 < end; i0 += 128 * U) {
                 float4 x[U], g[U];
+                if (i0 + 128 * U <= end) {
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int j0 = i0 + 128 * u + 4 * lane;
-                    x[u] = g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (j0 + 3 < end) {
+                    for (int u = 0; u < U; ++u) {
+                        const int j0 = i0 + 128 * u + 4 * lane;
                         x[u] = __ldcs(reinterpret_cast<const float4*>(av + j0));
-                        if (MODE != TC_PLAIN) g[u] = __ldcs(reinterpret_cast<const float4*>(bv + j0));
-                    } else if (j0 < end) {
-                        x[u].x = av[j0]; if (j0 + 1 < end) x[u].y = av[j0 + 1]; if (j0 + 2 < end) x[u].z = av[j0 + 2];
-                        if (MODE != TC_PLAIN) { g[u].x = bv[j0]; if (j0 + 1 < end) g[u].y = bv[j0 + 1]; if (j0 + 2 < end) g[u].z = bv[j0 + 2]; }
+                        g[u] = MODE == TC_PLAIN ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldcs(reinterpret_cast<const float4*>(bv + j0));
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int j0 = i0 + 128 * u + 4 * lane, left = end - j0;
+                        x[u] = g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (left > 0) { x[u].x = av[j0]; if (MODE != TC_PLAIN) g[u].x = bv[j0]; }
+                        if (left > 1) { x[u].y = av[j0 + 1]; if (MODE != TC_PLAIN) g[u].y = bv[j0 + 1]; }
+                        if (left > 2) { x[u].z = av[j0 + 2]; if (MODE != TC_PLAIN) g[u].z = bv[j0 + 2]; }
+                        if (left > 3) { x[u].w = av[j0 + 3]; if (MODE != TC_PLAIN) g[u].w = bv[j0 + 3]; }
                     }
                 }
 #pragma unroll
@@ -334,54 +384,27 @@ st_collect_kernel(const __grid_constant__ StArgs p) {
             }
         } else {
 #pragma unroll 1
-            for (int j0 = lane; j0 - lane < end; j0 += 32 * U) {
+            for (int i0 = 0; i0 < end; i0 += 32 * U) {
+                const int j0 = i0 + lane, left = end - j0;
                 float v[U], old[U];
+                if (i0 + 32 * U <= end) {
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int j = j0 + 32 * u;
-                    v[u] = j < end ? __ldcs(av + j) : 0.f;
-                    old[u] = (MODE != TC_PLAIN && j < end) ? __ldcs(bv + j) : 0.f;
-                }
-                bool any = false;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    v[u] = st_value<MODE>(v[u], old[u], p.gamma);
-                    if (MODE == TC_EF && j0 + 32 * u < end) __stcs(bv + j0 + 32 * u, v[u]);
-                    any |= mag_key(v[u]) >= lo;
-                }
-                if (__any_sync(0xffffffffu, any)) {
+                    for (int u = 0; u < U; ++u) { v[u] = __ldcs(av + j0 + 32 * u); old[u] = MODE == TC_PLAIN ? 0.f : __ldcs(bv + j0 + 32 * u); }
+                    apart(j0, v, old, 32 * U);
+                } else {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const bool pr = mag_key(v[u]) >= lo;
-                        const unsigned bm = __ballot_sync(0xffffffffu, pr);
-                        if (bm) {
-                            if (pr) candidate(cnt + (unsigned)__popc(bm & ((1u << lane) - 1u)), j0 + 32 * u, v[u], old[u]);
-                            cnt += (unsigned)__popc(bm);
-                        }
+                        v[u] = 32 * u < left ? __ldcs(av + j0 + 32 * u) : 0.f;
+                        old[u] = MODE != TC_PLAIN && 32 * u < left ? __ldcs(bv + j0 + 32 * u) : 0.f;
                     }
+                    apart(j0, v, old, left);
                 }
             }
         }
-        if (LISTS) {
-            __syncwarp();
-            if (cnt <= (unsigned)p.cap) {
-#pragma unroll 1
-                for (unsigned e = lane; e < cnt; e += 32u) {
-                    const int2 r = *reinterpret_cast<const int2*>(&out[e]);
-                    sure += classify((unsigned)r.y & 0x7fffffffu, (unsigned)r.x);
-                }
-            } else {
-                // the region's list overflowed: its entries once more (TC_EF: v is in b by now)
-#pragma unroll 1
-                for (int j = lane; j < end; j += 32) {
-                    const float v = MODE == TC_EF ? bv[j] : st_value<MODE>(av[j], MODE == TC_PLAIN ? 0.f : bv[j], p.gamma);
-                    if (mag_key(v) >= lo) sure += classify(mag_key(v), (unsigned)base + (unsigned)j);
-                }
-            }
-        }
+        empty();
         sure = __reduce_add_sync(0xffffffffu, sure);
         if (lane == 0) {
-            p.reg_cand[(i64)vec * p.nreg_pitch + region] = cnt;
+            if (LISTS) p.reg_cand[(i64)vec * p.nreg_pitch + region] = done;
             p.reg_base[(i64)vec * p.nreg_pitch + region] = sure;
             if (sure) atomicAdd(&sure_sh, sure);
         }
@@ -682,11 +705,16 @@ st_compact_kernel(const __grid_constant__ StArgs p, const StOut o) {
     }
 }
 
-// The same where no lists are kept (more than a tenth of the entries are wanted): one warp per region reads it again.
+// The same where no lists are kept (more than a tenth of the entries are wanted): one warp per region reads it again, and gathers
+// the selected ones of 256 entries in shared memory before they are written side by side.  Bound by instructions (20 x 2,642,533, a
+// tenth wanted: 83 us with a store per lane and entry, now 73).
 // grid = (ceil(nreg / 8), batch), 256 threads.
+constexpr int ST_REREAD_LOADS = 8;
+
 template <int MODE>
 __global__ void __launch_bounds__(256)
 st_reread_kernel(const __grid_constant__ StArgs p, const StOut o) {
+    __shared__ int2 gather_sh[8][32 * ST_REREAD_LOADS];
     pdl_trigger();
     pdl_wait();
     const int vec = blockIdx.y, lane = threadIdx.x & 31;
@@ -705,31 +733,40 @@ st_reread_kernel(const __grid_constant__ StArgs p, const StOut o) {
     int* io = o.idx_out + (i64)vec * p.k;
     float* vo = o.val_out + (i64)vec * p.k;
     float* app = o.apply ? o.apply + (i64)vec * o.pitch_apply + base : nullptr;
-    constexpr int U = 8;
-    for (int j0 = lane; j0 - lane < end; j0 += 32 * U) {
-        if (o.tile_off && lane == 0 && j0 == 2048) o.tile_off[(i64)vec * (o.ntiles + 1) + 2 * region + 1] = (int)pos;
+    constexpr int U = ST_REREAD_LOADS;
+    int2* gather = gather_sh[threadIdx.x >> 5];
+    const i64 tie = (i64)cut_idx - base;                            // an entry at the cut's key is in the message up to here
+#pragma unroll 1
+    for (int i0 = 0; i0 < end; i0 += 32 * U) {
+        const int j0 = i0 + lane;
+        const int left = i0 + 32 * U <= end ? 32 * U : end - j0;
+        if (o.tile_off && j0 == 2048) o.tile_off[(i64)vec * (o.ntiles + 1) + 2 * region + 1] = (int)pos;
         float v[U], b[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int j = j0 + 32 * u;
-            b[u] = (MODE != TC_PLAIN && j < end) ? bv[j] : 0.f;                      // TC_EF: v itself by now
-            v[u] = j < end ? (MODE == TC_EF ? b[u] : st_value<MODE>(av[j], b[u], p.gamma)) : 0.f;
+            b[u] = MODE != TC_PLAIN && 32 * u < left ? bv[j0 + 32 * u] : 0.f;        // TC_EF: v itself by now
+            v[u] = MODE != TC_EF && 32 * u < left ? av[j0 + 32 * u] : 0.f;
         }
+        unsigned n = 0u;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int j = j0 + 32 * u;
-            const unsigned key = mag_key(v[u]);
-            const bool sel = j < end && (key > cut_key || (key == cut_key && (unsigned)(base + j) <= cut_idx));
+            v[u] = MODE == TC_EF ? b[u] : st_value<MODE>(v[u], b[u], p.gamma);
+            const bool sel = 32 * u < left && mag_key(v[u]) >= cut_key + (j0 + 32 * u > tie ? 1u : 0u);
             const unsigned bal = __ballot_sync(0xffffffffu, sel);
-            if (bal == 0u) continue;
             if (sel) {
-                const unsigned at = pos + (unsigned)__popc(bal & ((1u << lane) - 1u));
-                io[at] = (int)(base + j); vo[at] = v[u];
-                flag_nonfinite(o.status, v[u]);
-                if (app) app[j] = MODE == TC_EF ? __fsub_rn(v[u], v[u]) : __fadd_rn(b[u], v[u]);
+                gather[n + (unsigned)__popc(bal & ((1u << lane) - 1u))] = make_int2((int)base + j0 + 32 * u, __float_as_int(v[u]));
+                if (app) app[j0 + 32 * u] = MODE == TC_EF ? __fsub_rn(v[u], v[u]) : __fadd_rn(b[u], v[u]);
             }
-            pos += (unsigned)__popc(bal);
+            n += (unsigned)__popc(bal);
         }
+        __syncwarp();
+        for (unsigned e = lane; e < n; e += 32u) {
+            const int2 w = gather[e];
+            io[pos + e] = w.x; vo[pos + e] = __int_as_float(w.y);
+            flag_nonfinite(o.status, __int_as_float(w.y));
+        }
+        pos += n;
+        __syncwarp();
     }
     if (o.tile_off && lane == 0) {
         int* off = o.tile_off + (i64)vec * (o.ntiles + 1);
