@@ -39,7 +39,10 @@ using namespace ef21;
 namespace {
 
 constexpr size_t ALIGN = 256;
-constexpr i64 GRAPH_MAX_D = 8192;      // launch-path iterations up to this dimension are replayed as a CUDA graph
+// Launch-path iterations up to this dimension are replayed as a CUDA graph.  Wider ones are launched one by one: a graph per iteration is
+// a full stop between iterations, across which the gradient kernel could not fetch its first rows (20 x 300 x 5,001: 41.2 us an
+// iteration without the graph, 43.1 with it; three launches take the host about 7 us).
+constexpr i64 GRAPH_MAX_D = 512;
 inline size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 inline i64 ceil_div(i64 a, i64 b) { return (a + b - 1) / b; }
 
@@ -142,23 +145,27 @@ TopkLayout topk_layout(i64 batch, i64 d, i64 k) {
 }
 
 typedef void (*GradTileKernel)(const float*, const float*, const float*, const RowTile*, int, int, float*, double*,
-                               const int*, int, const i64*, unsigned*);
+                               const int*, int, const i64*, unsigned*, int);
 
 // The gradient kernel for a row width: kernel, threads and shared memory per block; wide: a block works on whole rows and goes
 // through a long tile, `resident` blocks per SM and `rows` rows at a time (0: short tiles, several per SM).
 struct GradPlan { GradTileKernel kernel; unsigned threads; size_t smem; int resident, rows; };
 
 GradPlan grad_plan(i64 ld) {
-    const i64 slots = (ld / 4 + 31) / 32, wide = ceil_div(ld / 4, GRAD_WIDE_BLOCK);
+    const i64 slots = (ld / 4 + 31) / 32;
     if (slots <= 4) {
         // rows of up to 512 columns, a warp per batch of rows
         const GradTileKernel k = slots <= 1 ? grad_stream_kernel<1, 16>
                                             : (slots == 2 ? grad_stream_kernel<2, 8> : (slots == 3 ? grad_stream_kernel<3, 4> : grad_stream_kernel<4, 4>));
         return {k, GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * ld * 4, 0, 0};
     }
-    static const GradTileKernel kernels[8] = {grad_wide_kernel<1>, grad_wide_kernel<2>, grad_wide_kernel<3>, grad_wide_kernel<4>,
-                                              grad_wide_kernel<5>, grad_wide_kernel<6>, grad_wide_kernel<7>, grad_wide_kernel<8>};
-    if (wide <= 8) return {kernels[wide - 1], GRAD_WIDE_BLOCK, 0, wide <= 2 ? 2 : 1, grad_wide_rows((int)wide)};
+    // rows of up to 8,192 columns: 256 threads hold 1,024 columns, 512 threads 2,048 a chunk
+    static const GradTileKernel kernels[5] = {grad_wide_kernel<1, 256>, grad_wide_kernel<1, 512>, grad_wide_kernel<2, 512>, grad_wide_kernel<3, 512>,
+                                              grad_wide_kernel<4, 512>};
+    if (ld <= 8192) {
+        const int nc = (int)ceil_div(ld, 2048), rows = grad_wide_rows(nc);
+        return {kernels[ld <= 1024 ? 0 : nc], ld <= 1024 ? 256u : 512u, (size_t)grad_wide_stages(rows, (int)ld) * rows * ld * 4, 1, rows};
+    }
     return {grad_tiles_kernel, GRAD_BLOCK, 0, 0, 0};
 }
 
@@ -365,6 +372,18 @@ TcKernel tc_lookup(const TcShape& S) {
     }
 }
 
+// The same with the gradients formed on the way in.
+template <int MODE>
+TcKernel tc_grad_lookup(const TcShape& S) {
+    if (S.threads == 256) return tc_topk_kernel<MODE, 1, 256, false, 1>;
+    switch (S.C) {
+        case 1: return tc_topk_kernel<MODE, 1, 512, false, 1>;
+        case 2: return tc_topk_kernel<MODE, 1, 512, false, 2>;
+        case 4: return tc_topk_kernel<MODE, 1, 512, false, 4>;
+        default: return tc_topk_kernel<MODE, 1, 512, false, 8>;
+    }
+}
+
 ef21_status enqueue_topk_cluster(cudaStream_t st, int mode, const TcShape& S, const float* a, i64 pitch_a, const float* b, i64 pitch_b,
                                  float gamma, int batch, i64 d, int k, int* idx_out, float* val_out, float* apply, i64 pitch_apply,
                                  i64* launches, unsigned* status, unsigned* slow_count = nullptr, unsigned long long* cut_out = nullptr) {
@@ -514,12 +533,13 @@ struct GradSource { int num_tiles, worker_tiles; size_t tiles, tile_begin; const
 
 GradSource full_source(const ef21_ctx* c) { return {c->num_tiles, c->worker_tiles, c->L.tiles, c->L.tile_begin, nullptr, 0}; }
 
-ef21_status launch_grad_tiles(ef21_ctx* c, const GradSource& G, bool with_loss) {
+ef21_status launch_grad_tiles(ef21_ctx* c, const GradSource& G, bool with_loss, bool early = false) {
     if (G.num_tiles == 0) return EF21_OK;
     const GradPlan P = grad_plan(c->L.ld);
+    if (P.resident) EF(allow_smem(reinterpret_cast<const void*>(P.kernel), GRAD_WIDE_SMEM));
     CU(launch(P.kernel, dim3((unsigned)G.num_tiles), P.threads, P.smem, c->stream, 1, c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(),
               c->at<RowTile>(G.tiles), (int)c->L.ld, c->objective, c->at<float>(c->L.partial),
-              with_loss ? c->at<double>(c->L.loss_partial) : nullptr, G.batch_dev, G.tau, c->at<i64>(c->L.row_off), c->status()));
+              with_loss ? c->at<double>(c->L.loss_partial) : nullptr, G.batch_dev, G.tau, c->at<i64>(c->L.row_off), c->status(), early ? 1 : 0));
     c->launches += 1;
     return EF21_OK;
 }
@@ -532,27 +552,32 @@ ef21_status launch_grad_finish(ef21_ctx* c, const GradSource& G) {
     return EF21_OK;
 }
 
-// Whether the Top-k kernel can form the gradients from the tile partials itself (one block per worker, two columns per thread):
-// vectors of up to 512 columns with up to 32 tiles per worker, where a thread needs no more dependent rounds of reading than
-// in a kernel of its own and a launch is saved.  (Rows of 600 to 1,000 columns took 2 us longer that way, 5,001 columns 8 us: a
-// kernel of its own spreads the sums over the device.)
+// Whether the Top-k kernel can form the gradients from the tile partials itself, and in which shape: a thread then needs few dependent
+// rounds of reading (eight tiles each), and a launch is saved.  Up to 512 columns and 32 tiles per worker one block per worker, two columns
+// per thread.  Up to 8,192 columns and 40 tiles a cluster of up to eight blocks forms them, the first of which selects; no more blocks
+// than SMs, since they are placed as the blocks of the gradient kernel end (20 x 5,001: 32.7 us an iteration with clusters of four, 35.0 of
+// eight, 39.0 of two; 10 x 4,180: 16.1 with eight, 17.1 with four; two kernels 36.5 and 21.3).
 bool select_can_form_grads(const ef21_ctx* c, const GradSource& G, TcShape& S) {
-    return tc_shape(c->n, c->d, S) && S.threads == 256 && c->d <= 512 && G.worker_tiles <= 4 * GRAD_FINISH_LANES;
+    if (c->d <= 512) return tc_shape(c->n, c->d, S) && S.threads == 256 && G.worker_tiles <= 4 * GRAD_FINISH_LANES;
+    if (c->d > 8192 || G.worker_tiles > 5 * GRAD_FINISH_LANES) return false;
+    i64 C = 1;
+    while (C < 8 && c->n * C * 2 <= 148 && c->d / (2 * C) >= 128) C *= 2;
+    S.C = (int)C; S.threads = 512;
+    S.slice = (int)((c->d + 127) / 128 * 128);
+    return ceil_div(c->d, C) <= 2048;
 }
 
 // Tile partials -> messages and worker states in one kernel (see select_can_form_grads).  mode: TC_DIFF, TC_EF, or TC_PLAIN for
 // g_i = C(grad_i) from nothing.
 ef21_status enqueue_grad_select(ef21_ctx* c, const GradSource& G, const TcShape& S, int mode) {
-    typedef void (*Kernel)(const TcArgs);
-    static const Kernel kernels[3] = {tc_topk_kernel<TC_PLAIN, 1, 256, false, true>, tc_topk_kernel<TC_DIFF, 1, 256, false, true>,
-                                      tc_topk_kernel<TC_EF, 1, 256, false, true>};
-    const Kernel kern = kernels[mode];
+    const TcKernel kern = mode == TC_PLAIN ? tc_grad_lookup<TC_PLAIN>(S) : (mode == TC_DIFF ? tc_grad_lookup<TC_DIFF>(S) : tc_grad_lookup<TC_EF>(S));
+    EF(allow_smem(reinterpret_cast<const void*>(kern), tc_smem_bytes(1, 8192)));
     TcArgs p = {};
     p.b = c->gi(); p.pitch_b = c->L.ld; p.d = (int)c->d; p.k = c->k; p.slice = S.slice; p.gamma = c->gamma;
     p.idx_out = c->msg_idx(); p.val_out = c->msg_val(); p.apply = c->gi(); p.pitch_apply = c->L.ld; p.status = c->status();
     p.partial = c->at<float>(c->L.partial); p.tile_begin = c->at<int>(G.tile_begin); p.row_off = c->at<i64>(c->L.row_off); p.x = c->x();
     p.lambda = c->lambda; p.ld = (int)c->L.ld; p.batch_rows = G.tau;
-    CU(launch(kern, dim3((unsigned)c->n), (unsigned)S.threads, tc_smem_bytes(1, S.slice), c->stream, 1, p));
+    CU(launch(kern, dim3((unsigned)c->n * (unsigned)S.C), (unsigned)S.threads, tc_smem_bytes(1, S.slice), c->stream, (unsigned)S.C, p));
     c->launches += 1;
     return EF21_OK;
 }
@@ -1214,9 +1239,9 @@ ef21_status ef21_init_grads(ef21_ctx* c, const float* V_dev, int32_t mode) {
 
 // One iteration of ef21_step on the launch path, as plain kernel launches on the handle's stream.  The x update that opens the
 // iteration has already been enqueued (or does not exist: Algorithm 4); xmode AGG_X_AFTER: the one of the next iteration is
-// made by the kernel that updates g.
-static ef21_status enqueue_launch_iteration(ef21_ctx* c, const GradSource& G, int xmode) {
-    EF(launch_grad_tiles(c, G, false));
+// made by the kernel that updates g.  early: an iteration of the same call has been enqueued before (see grad_wide_kernel).
+static ef21_status enqueue_launch_iteration(ef21_ctx* c, const GradSource& G, int xmode, bool early = false) {
+    EF(launch_grad_tiles(c, G, false, early));
     TcShape S;
     if (c->variant != EF21_VARIANT_EF21_PLUS && select_can_form_grads(c, G, S)) {
         c->agg_off_ready = false;
@@ -1277,7 +1302,7 @@ static ef21_status run_launch_iterations(ef21_ctx* c, int steps) {
     } else {
         cudaGetLastError();
     }
-    for (; done < steps; ++done) EF(enqueue_launch_iteration(c, full_source(c), done + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
+    for (; done < steps; ++done) EF(enqueue_launch_iteration(c, full_source(c), done + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP, done > 0));
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;
 }
@@ -1387,7 +1412,7 @@ ef21_status ef21_step_minibatches(ef21_ctx* c, const int32_t* batches_dev, int32
     for (int t = 0; t < steps; ++t) {
         GradSource G;
         EF(minibatch_source(c, batches_dev + (size_t)t * c->n * tau, tau, G));
-        EF(enqueue_launch_iteration(c, G, t + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP));
+        EF(enqueue_launch_iteration(c, G, t + 1 < steps ? AGG_X_AFTER : AGG_X_KEEP, t > 0));
     }
     c->last_path = EF21_PATH_LAUNCHES;
     return EF21_OK;

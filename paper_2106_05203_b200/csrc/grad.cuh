@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(GRAD_BLOCK)
 grad_tiles_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
                   const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                   double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
-                  const i64* __restrict__ row_off, unsigned* __restrict__ status) {
+                  const i64* __restrict__ row_off, unsigned* __restrict__ status, int early) {
     pdl_trigger();
     pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
     __shared__ float rho[GRAD_TILE_MAX_ROWS];
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(GRAD_STREAM_BLOCK)
 grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
                    const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                    double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
-                   const i64* __restrict__ row_off, unsigned* __restrict__ status) {
+                   const i64* __restrict__ row_off, unsigned* __restrict__ status, int early) {
     pdl_trigger();
     pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
     constexpr int SH = (RB == 32) ? 0 : (RB == 16 ? 1 : (RB == 8 ? 2 : (RB == 4 ? 3 : 4)));    // log2(32/RB)
@@ -222,28 +222,49 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
 }
 
 // Rows of 513 to 8,192 columns, one read of every row: the whole block works on RB rows at a time, thread t holds the float4 columns
-// t, t + 256, ... of each in registers; the margins are summed over the block (transposed warp reduction, then over the warps
-// through shared memory, one barrier), every warp forms the residuals, and rho_r a_r is added from the registers.  The next RB
-// rows are on their way meanwhile (a second register buffer: 40-80 KB per SM in flight), and a block goes through a long
-// tile, so that few partials are written (6,000 x 5,001: 65 us with a tile of three rows per block, two sweeps and 40 MB of
-// partials; bound by reading the rows).
-constexpr int GRAD_WIDE_BLOCK = 256;
-__host__ __device__ constexpr int grad_wide_rows(int nc) { return nc == 1 ? 8 : (nc <= 5 ? 4 : 2); }
+// t, t + THREADS, ... of each in registers; the margins are summed over the block (transposed warp reduction, then over the warps
+// through shared memory, one barrier), every warp forms the residuals, and rho_r a_r is added from the registers.  A block goes
+// through a long tile, so that few partials are written, and its rows arrive through a ring in shared memory: bulk copies, a row
+// each, that refill a stage as soon as the barrier shows that it has been taken into registers.
+// early: the rows (and labels, tile table and sampled row numbers) were complete before an earlier gradient kernel of the same call
+// passed its wait, so the ring is filled before this kernel waits for the one in front of it, while that selects and aggregates: up
+// to 160 KB per SM, 24 MB in all, arrive in time in which HBM and L2 would idle.  The first kernel of a call (early == 0) waits first,
+// and lets nothing behind it start before.
+// 20 x 300 x 5,001 (120 MB, more than stays in L2): 26.2 us with the next rows in a second register buffer, 24.2 through the ring,
+// 19.6 with the early start, of which HBM takes 15; 20 x 285 x 2,625: 13.2, 11.1; 20 x 208 x 1,463: 8.4, 6.0 (latencies: x, two to four
+// batches of 0.5 us, launch).
+constexpr int GRAD_WIDE_SMEM = 160 * 1024, GRAD_WIDE_MAX_STAGES = 8, GRAD_WIDE_SPINS = 1 << 22;
+__host__ __device__ constexpr int grad_wide_rows(int nc) { return nc == 1 ? 8 : (nc <= 3 ? 4 : 2); }
+__host__ __device__ inline int grad_wide_stages(int rows, int ld) {
+    const int fit = GRAD_WIDE_SMEM / (rows * ld * 4);
+    return fit < GRAD_WIDE_MAX_STAGES ? fit : GRAD_WIDE_MAX_STAGES;
+}
 
-template <int NC>
-__global__ void __launch_bounds__(GRAD_WIDE_BLOCK, NC <= 2 ? 2 : 1)
+template <int NC, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1)
 grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
                  const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                  double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
-                 const i64* __restrict__ row_off, unsigned* __restrict__ status) {
-    pdl_trigger();
-    pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
-    constexpr int RB = grad_wide_rows(NC), WARPS = GRAD_WIDE_BLOCK / 32;
+                 const i64* __restrict__ row_off, unsigned* __restrict__ status, int early) {
+    constexpr int RB = grad_wide_rows(NC), WARPS = THREADS / 32;
     constexpr int LOG_GROUP = RB == 8 ? 2 : (RB == 4 ? 3 : 4);                  // log2(32 / RB): lanes that end up with one row
+    extern __shared__ __align__(128) unsigned char grad_smem[];
     __shared__ float red[2][WARPS][RB];
-    const RowTile t = tiles[blockIdx.x];
+    __shared__ unsigned long long bars[GRAD_WIDE_MAX_STAGES];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int chunks = ld >> 2;
+    if (tid < GRAD_WIDE_MAX_STAGES)
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(bars + tid)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (early) {
+        pdl_trigger();
+    } else {
+        pdl_wait(A, y, x, tiles, partial, loss_partial, gather, row_off, status);
+        pdl_trigger();
+    }
+    const RowTile t = tiles[blockIdx.x];
+    const int chunks = ld >> 2, batches = (t.rows + RB - 1) / RB, stages = grad_wide_stages(RB, ld);
     const i64 lo = gather ? row_off[t.worker] : 0, m = gather ? row_off[t.worker + 1] - lo : 0;
     auto row_id = [&](int r) -> i64 {
         if (!gather) return t.row0 + r;
@@ -251,47 +272,71 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         if (pick < 0 || pick >= m) { record_error(status, 1u /* EF21_ERR_INVALID_ARG */); pick = 0; }
         return lo + pick;
     };
+    // the first warp fetches batch b into `stage`, a lane per row
+    auto fetch = [&](int b, int stage) {
+        const int r = b * RB + lane, bytes = ld * 4;
+        const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage);
+        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(min(RB, t.rows - b * RB) * bytes) : "memory");
+        __syncwarp();
+        if (lane < RB && r < t.rows)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"((unsigned)__cvta_generic_to_shared(grad_smem) + (unsigned)((stage * RB + lane) * bytes)), "l"(A + row_id(r) * (i64)ld),
+                           "r"(bytes), "r"(bar) : "memory");
+    };
+    if (warp == 0) for (int b = 0; b < min(stages, batches); ++b) fetch(b, b);
+    if (early) pdl_wait(x, partial, loss_partial);
     float4 xr[NC], acc[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        const int at = tid + c * GRAD_WIDE_BLOCK;
+        const int at = tid + c * THREADS;
         xr[c] = at < chunks ? reinterpret_cast<const float4*>(x)[at] : make_float4(0.f, 0.f, 0.f, 0.f);
         acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     double loss_acc = 0.0;
-    float4 a[2][RB][NC];
-    float yb[2];                                               // label of the row whose margin this lane ends up with
-    auto load = [&](int r0, float4 (&buf)[RB][NC], float& label) {
+    // label of the row whose margin this lane ends up with, a batch ahead
+    auto label_of = [&](int b) { const int r = b * RB + (lane >> LOG_GROUP); return r < t.rows ? __ldg(y + row_id(r)) : 0.f; };
+    float next_label = label_of(0);
+    int stage = 0;
+    unsigned parity = 0u;
+#pragma unroll 1
+    for (int b = 0; b < batches; ++b) {
+        const float label = next_label;
+        next_label = label_of(b + 1);
+        const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage);
+        unsigned ok = 0u;
+        for (int spins = 0; spins < GRAD_WIDE_SPINS && !ok; ++spins)
+            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (!ok) record_error(status, 5u /* EF21_ERR_TIMEOUT */);
+        const float4* rows = reinterpret_cast<const float4*>(grad_smem) + stage * RB * chunks;
+        const int left = t.rows - b * RB;
+        float4 a[RB][NC];
+        float pd[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
-            const bool in = r0 + r < t.rows;
-            const float4* __restrict__ src = reinterpret_cast<const float4*>(A + (in ? row_id(r0 + r) : 0) * (i64)ld);
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                const int at = tid + c * GRAD_WIDE_BLOCK;
-                buf[r][c] = in && at < chunks ? __ldg(src + at) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const int at = tid + c * THREADS;
+                a[r][c] = r < left && at < chunks ? rows[r * chunks + at] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
-        const int mine = r0 + (lane >> LOG_GROUP);
-        label = mine < t.rows ? __ldg(y + row_id(mine)) : 0.f;
-    };
-    auto use = [&](int r0, int half, const float4 (&buf)[RB][NC], float label) {
-        float pd[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) {
             float z = 0.f;
 #pragma unroll
-            for (int c = 0; c < NC; ++c) z = dot4(buf[r][c], xr[c], z);
+            for (int c = 0; c < NC; ++c) z = dot4(a[r][c], xr[c], z);
             pd[r] = z;
         }
         const float zw = reduce_rows<RB>(pd, lane);             // this warp's part of the margin of row lane >> LOG_GROUP
+        const int half = b & 1;
         if ((lane & ((1 << LOG_GROUP) - 1)) == 0) red[half][warp][lane >> LOG_GROUP] = zw;
         __syncthreads();
+        if (warp == 0 && b + stages < batches) fetch(b + stages, stage);        // the rows are in registers
         float z = red[half][0][lane >> LOG_GROUP];
 #pragma unroll
         for (int w = 1; w < WARPS; ++w) z += red[half][w][lane >> LOG_GROUP];
         const float rho = loss_residual(objective, label, z);   // 0 for a row past the end (y = 0, a = 0)
-        if (loss_partial && warp == 0 && (lane & ((1 << LOG_GROUP) - 1)) == 0 && r0 + (lane >> LOG_GROUP) < t.rows) {
+        if (loss_partial && warp == 0 && (lane & ((1 << LOG_GROUP) - 1)) == 0 && (lane >> LOG_GROUP) < left) {
             if (objective == 0) {
                 const double u = -(double)label * (double)z;
                 loss_acc += (u > 0.0 ? u : 0.0) + log1p(exp(-fabs(u)));
@@ -304,22 +349,14 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         for (int r = 0; r < RB; ++r) {
             const float pr = __shfl_sync(0xffffffffu, rho, r << LOG_GROUP);
 #pragma unroll
-            for (int c = 0; c < NC; ++c) acc[c] = fma4(pr, buf[r][c], acc[c]);
+            for (int c = 0; c < NC; ++c) acc[c] = fma4(pr, a[r][c], acc[c]);
         }
-    };
-    load(0, a[0], yb[0]);
-#pragma unroll 1
-    for (int r0 = 0; r0 < t.rows; r0 += 2 * RB) {
-        load(r0 + RB, a[1], yb[1]);
-        use(r0, 0, a[0], yb[0]);
-        if (r0 + RB >= t.rows) break;
-        load(r0 + 2 * RB, a[0], yb[0]);
-        use(r0 + RB, 1, a[1], yb[1]);
+        if (++stage == stages) { stage = 0; parity ^= 1u; }
     }
     float4* __restrict__ out = reinterpret_cast<float4*>(partial + (i64)blockIdx.x * ld);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        const int at = tid + c * GRAD_WIDE_BLOCK;
+        const int at = tid + c * THREADS;
         if (at < chunks) out[at] = acc[c];
     }
     if (loss_partial && warp == 0) {

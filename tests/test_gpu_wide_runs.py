@@ -1,0 +1,74 @@
+"""Runs on rows of 513 to 8,192 columns (gradient tiles through a ring that later iterations of a call fill ahead of time, gradients
+formed by the selecting cluster), and the selection of few entries in one block: at the edges of their shapes."""
+import numpy as np
+import pytest
+import torch
+
+import ef21_inputs as inputs
+from gpu_util import dev, lockstep, make_gpu, make_oracle_state
+
+pytestmark = pytest.mark.gpu
+
+# d, n, rows, k: clusters of 8, 4, 2 and 1 forming blocks; k up to and beyond a quarter of 512 threads; tiles from one row on; up to 40
+# tiles per worker and more
+SHAPES = [(513, 3, 40, 5), (700, 2, 900, 7), (1025, 37, 500, 20), (2047, 75, 300, 128), (2048, 75, 160, 129), (2049, 9, 70, 1), (4100, 4, 700, 41),
+          (5001, 20, 900, 50), (6145, 40, 300, 60), (8192, 5, 333, 128)]
+
+
+def _workload(d, n, rows, k):
+    return inputs.make_logistic("wide", n=n, d=d, N=rows, k=k, seed=d + n, features="bernoulli", density=0.1, gamma=0.05, T=10)
+
+
+@pytest.mark.parametrize("d,n,rows,k", SHAPES)
+def test_wide_runs_track_the_oracle(d, n, rows, k, oracle32):
+    from paper_2106_05203_b200 import binding as B
+    w = _workload(d, n, rows, k)
+    h = make_gpu(w)
+    st = make_oracle_state(oracle32, w)
+    h.init(B.INIT_COMPRESSED)
+    st.init(0)
+    lockstep(h, st, oracle32, w, 4)
+    assert h.last_path == B.PATH_LAUNCHES and h.poll() == 0
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("d,n,rows,k", SHAPES[:4] + SHAPES[7:])
+def test_one_call_gives_the_bits_of_many(d, n, rows, k, variant):
+    from paper_2106_05203_b200 import binding as B
+    w = _workload(d, n, rows, k)
+    states = []
+    for calls, steps in ((1, 7), (7, 1)):
+        h = make_gpu(w)
+        h.set_variant(variant)
+        h.init(B.INIT_ZERO)
+        for _ in range(calls):
+            h.step(steps)
+        assert h.poll() == 0
+        states.append(h.get_state())
+    for a, b in zip(*states):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
+
+
+# blocks of 256, 512 and 1,024 threads: k at a quarter of them and one more, lengths at the values a thread holds
+@pytest.mark.parametrize("kind", ["gauss", "ties", "signs", "few nonzero", "zeros", "spread"])
+@pytest.mark.parametrize("batch,d,k", [(3, 7, 7), (3, 257, 64), (5, 2048, 64), (5, 2048, 65), (3, 2049, 128), (3, 8192, 128), (3, 8192, 129), (150, 8193, 256),
+                                       (150, 16384, 256), (150, 16384, 257), (150, 16385, 20), (2, 5000, 1)])
+def test_few_entries_of_short_vectors(batch, d, k, kind, oracle32):
+    from paper_2106_05203_b200 import binding as B
+    rng = np.random.default_rng(d + k)
+    v = rng.standard_normal((batch, d), dtype=np.float32)
+    if kind == "ties":
+        v = np.round(v * 2).astype(np.float32) * np.float32(0.5)
+    elif kind == "signs":
+        v = np.sign(v).astype(np.float32)
+    elif kind == "few nonzero":
+        v *= rng.random((batch, d)) < 0.5 * k / d
+    elif kind == "zeros":
+        v *= np.float32(0)                                     # of both signs
+    elif kind == "spread":
+        v = (v * np.exp2(rng.integers(-140, 100, (batch, d)).astype(np.float64))).astype(np.float32)      # subnormals among them
+    idx, val = B.topk(dev(v), k)
+    for i in sorted({0, batch // 2, batch - 1}):
+        oi, ov = oracle32.topk(v[i], k)
+        np.testing.assert_array_equal(idx[i].cpu().numpy(), oi)
+        np.testing.assert_array_equal(val[i].cpu().numpy().view(np.uint32), ov.view(np.uint32))
