@@ -102,6 +102,7 @@ TopkLayout topk_layout_general(i64 batch, i64 d) {
     TopkLayout L{};
     L.nchunks = (int)ceil_div(d, TK_CHUNK);
     size_t o = 0;
+    L.slow_count = o; o += align_up(4);                    // (in the same place for every batch: a handle's count runs on)
     L.state = o; o += align_up((size_t)batch * sizeof(TkState));
     L.hist = o; o += align_up((size_t)batch * TK_BINS * sizeof(unsigned));
     L.chunks = o; o += align_up((size_t)batch * (size_t)L.nchunks * sizeof(uint2));
@@ -137,7 +138,6 @@ TopkLayout topk_layout(i64 batch, i64 d, i64 k) {
         L.open_list = o; o += align_up((size_t)batch * L.open_cap * 8);
         L.reg_cand = o; o += align_up((size_t)batch * L.nreg_pitch * 4);
         L.reg_base = o; o += align_up((size_t)batch * L.nreg_pitch * 4);
-        L.slow_count = o; o += align_up(4);
         L.cand = o; o += align_up((size_t)batch * L.nreg * L.cap * sizeof(int4));
     }
     L.total = o;
@@ -188,10 +188,11 @@ struct Layout {
     int tile_rows;     // rows per gradient tile
     i64 max_tiles;     // capacity of the gradient tile table
     size_t status, x, g, gi, msg_idx, msg_val, topk, agg_off, eval_out, slots;
-    size_t msg2_idx, msg2_val, plus_cuts, plus_choice, plus_parts;    // EF21+ (Algorithm 3)
+    size_t msg2_idx, msg2_val, plus_cuts, plus_choice, plus_parts, plus_low, plus_nonzero, plus_cand;    // EF21+ (Algorithm 3)
+    int plus_pitch;
     size_t A, y, row_off, tile_begin, tiles, partial, loss_partial, grad, mb_tile_begin, mb_tiles;
     size_t total;
-    TopkLayout tk;
+    TopkLayout tk, tk2;                   // of n vectors; of the 2 n vectors of EF21+ (the same memory)
 };
 
 Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
@@ -199,6 +200,7 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.ld = (d + 3) / 4 * 4;
     L.agg_tiles = (int)ceil_div(d, AGG_TILE);
     L.tk = topk_layout(n, d, k);
+    L.tk2 = topk_layout(2 * n, d, k);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o += align_up(bytes); return at; };
     L.status = take(256);
@@ -207,7 +209,7 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.gi = take((size_t)n * L.ld * 4);
     L.msg_idx = take((size_t)n * k * 4);
     L.msg_val = take((size_t)n * k * 4);
-    L.topk = take(L.tk.total);
+    L.topk = take(std::max(L.tk.total, L.tk2.total));
     L.agg_off = take((size_t)n * (L.agg_tiles + 1) * 4);
     L.eval_out = take(256);
     L.slots = take((size_t)2 * n * k * 8);
@@ -216,6 +218,10 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.plus_cuts = take((size_t)2 * n * 8);
     L.plus_choice = take((size_t)n * 4);
     L.plus_parts = take((size_t)n * PLUS_MAX_PARTS * sizeof(double2));
+    L.plus_pitch = (int)std::max<i64>(1, 148 * 4 / n);         // blocks per worker: four per SM in one wave
+    L.plus_low = take(L.tk2.fast ? (size_t)n * L.plus_pitch * sizeof(double2) : 0);
+    L.plus_nonzero = take(L.tk2.fast ? (size_t)n * L.plus_pitch * 4 : 0);
+    L.plus_cand = take(L.tk2.fast ? (size_t)2 * n * ceil_div(L.tk2.nreg, 32) * 8 : 0);
     L.tile_rows = 0; L.max_tiles = 0;
     L.A = L.y = L.row_off = L.tile_begin = L.tiles = L.partial = L.loss_partial = L.grad = L.mb_tile_begin = L.mb_tiles = 0;
     if (N > 0) {
@@ -402,7 +408,7 @@ ef21_status enqueue_topk_cluster(cudaStream_t st, int mode, const TcShape& S, co
 // ---- Top-k of long vectors in one pass (topk_stream.cuh) ----
 StArgs stream_args(const float* a, i64 pitch_a, const float* b, i64 pitch_b, float gamma, i64 d, int k, const TopkBuffers& B) {
     StArgs p;
-    p.a = a; p.pitch_a = pitch_a; p.b = const_cast<float*>(b); p.pitch_b = pitch_b; p.d = d; p.k = k;
+    p.a = a; p.pitch_a = pitch_a; p.b = const_cast<float*>(b); p.pitch_b = pitch_b; p.d = d; p.k = k; p.pair = 0;
     p.nreg = B.L.nreg; p.nreg_pitch = B.L.nreg_pitch; p.region_log = B.L.region_log; p.cap = B.L.cap; p.open_cap = (unsigned)B.L.open_cap; p.gamma = gamma;
     p.ctl = reinterpret_cast<StCtl*>(B.base + B.L.ctl);
     p.open_hist = reinterpret_cast<unsigned*>(B.base + B.L.open_hist);
@@ -699,6 +705,40 @@ ef21_status enqueue_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmode) {
     return enqueue_round_aggregate(c, xmode);
 }
 
+// Both selections of EF21+ on long vectors, as a batch of 2 n, and the distortions' sums (topk_stream.cuh): five launches.
+ef21_status enqueue_plus_select(ef21_ctx* c, const float* a, i64 pitch_a, unsigned long long* cuts, PlusSums& sums) {
+    const TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk2);
+    const int n = c->n;
+    StArgs p = stream_args(a, pitch_a, c->gi(), c->L.ld, 0.f, c->d, c->k, B);
+    p.pair = n;
+    const unsigned groups = (unsigned)ceil_div(p.nreg, 32);
+    sums.low = c->at<double2>(c->L.plus_low); sums.nonzero = c->at<int>(c->L.plus_nonzero); sums.low_pitch = c->L.plus_pitch;
+    // as many blocks as are resident at most, every warp with the same number of regions
+    const i64 rounds = ceil_div(ceil_div(p.nreg, ST_WARPS), c->L.plus_pitch);
+    sums.low_parts = (int)ceil_div(ceil_div(p.nreg, ST_WARPS), rounds);
+    sums.cand = c->at<double>(c->L.plus_cand); sums.groups = (int)groups; sums.ctl = p.ctl;
+    EF(enqueue_stream_sample<TC_PAIR>(c->stream, p, 2 * n, B.L, &c->launches));
+    EF(allow_smem(reinterpret_cast<const void*>(st_collect_pair_kernel), sizeof(StPairShared)));
+    CU(launch(st_collect_pair_kernel, dim3((unsigned)sums.low_parts, (unsigned)n), ST_WARPS * 32, sizeof(StPairShared), c->stream, 1, p, sums));
+    const int cut_blocks = 2 * n > 37 ? 2 : 8;
+    auto cut = cut_blocks == 2 ? st_cut_kernel<2, false> : st_cut_kernel<8, false>;
+    EF(allow_smem(reinterpret_cast<const void*>(cut), st_cut_smem_bytes(false)));
+    CU(launch(cut, dim3((unsigned)(2 * n * cut_blocks)), 1024, st_cut_smem_bytes(false), c->stream, (unsigned)cut_blocks, p));
+    int* idx_b = c->at<int>(c->L.msg2_idx);
+    float* val_b = c->at<float>(c->L.msg2_val);
+    CU(launch(st_compact_pair_kernel, dim3(groups, (unsigned)(2 * n)), 256, 0, c->stream, 1, p, sums, c->msg_idx(), c->msg_val(), idx_b, val_b, cuts,
+              c->status()));
+    TcArgs m = {};
+    m.a = a; m.pitch_a = pitch_a; m.b = c->gi(); m.pitch_b = c->L.ld; m.d = (int)c->d; m.k = c->k; m.batch = n;
+    m.idx_out = c->msg_idx(); m.val_out = c->msg_val(); m.status = c->status(); m.cut_out = cuts;
+    m.flag = &p.ctl->slow; m.flag_pitch = sizeof(StCtl) / 4; m.slice = (int)((ceil_div(c->d, 8) + 127) / 128 * 128);
+    TcArgs b = m;
+    b.b = nullptr; b.pitch_b = 0; b.idx_out = idx_b; b.val_out = val_b; b.cut_out = cuts + n; b.flag = &p.ctl[n].slow;
+    CU(launch(tc_pair_kernel<8, 1024>, dim3(8u * (unsigned)std::min(2 * n, 16)), 1024, tc_smem_bytes(8, 0), c->stream, 8, m, b));
+    c->launches += 4;
+    return EF21_OK;
+}
+
 // One round of EF21+ (Algorithm 3) on local gradients a: both compressed vectors, the choice by
 // distortion, g_i <- chosen, g = (1/n) sum g_i.
 ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmode) {
@@ -706,7 +746,10 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmo
     int* idx_b = c->at<int>(c->L.msg2_idx);
     float* val_b = c->at<float>(c->L.msg2_val);
     unsigned long long* cuts = c->at<unsigned long long>(c->L.plus_cuts);       // [2][n]: Markov, plain
-    if (long_topk(c)) {
+    PlusSums sums = {};
+    if (long_topk(c) && c->L.tk2.cap > 0) {
+        EF(enqueue_plus_select(c, a, pitch_a, cuts, sums));
+    } else if (long_topk(c)) {
         const StOut om = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status(), cuts};
         const StOut ob = {idx_b, val_b, nullptr, 0, nullptr, 0, c->status(), cuts + c->n};
         EF(enqueue_topk_stream<TC_DIFF>(c->stream, a, pitch_a, c->gi(), c->L.ld, 0.f, c->n, c->d, c->k, om, B, &c->launches, true));
@@ -721,9 +764,9 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmo
     const i64 parts = std::max<i64>(1, std::min<i64>(std::min<i64>(PLUS_MAX_PARTS, 148 * 4 / c->n), c->d / 4096));
     double2* part = c->at<double2>(c->L.plus_parts);
     CU(launch(plus_distortion_kernel, dim3((unsigned)parts, (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, a, pitch_a, c->gi(), c->L.ld, c->d,
-              ceil_div(c->d, parts), cuts, part));
+              ceil_div(c->d, parts), cuts, part, sums));
     CU(launch(plus_choose_kernel, dim3((unsigned)ceil_div(c->k, PLUS_BLOCK), (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, part, (int)parts, c->gi(),
-              c->L.ld, c->k, c->msg_idx(), c->msg_val(), idx_b, val_b, c->at<int>(c->L.plus_choice)));
+              c->L.ld, c->k, c->msg_idx(), c->msg_val(), idx_b, val_b, c->at<int>(c->L.plus_choice), sums));
     const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->d, 1024), 148 * 8);
     auto mean = xmode == AGG_X_KEEP ? plus_mean_kernel<AGG_X_KEEP>
                                     : (xmode == AGG_X_BEFORE ? plus_mean_kernel<AGG_X_BEFORE> : plus_mean_kernel<AGG_X_AFTER>);

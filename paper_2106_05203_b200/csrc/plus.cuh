@@ -10,6 +10,7 @@
 // worker did all of it before: 1,170 us for 16 workers of 1,000,003 entries against about 35 us).
 #pragma once
 #include "common.cuh"
+#include "topk_stream.cuh"
 
 namespace ef21 {
 
@@ -28,16 +29,42 @@ __device__ __forceinline__ double block_sum_f64(double v, double* scratch /* [PL
     return s;
 }
 
-// grid = (parts, n); part p of worker i covers the coordinates [p * len, (p + 1) * len).  part_out[i][p] = (M, B) of the part.  M and B
+// 0: Markov, 1: plain, 2: to be decided by the ordered sums (the whole warp calls it).  The sums that the selecting kernels leave decide
+// where they differ by more than one part in 10,000.  They are off by less than a tenth of that: a term is a rounded difference squared and
+// added to at most 128 others per lane in 32 bits, each rounding 2^-24 of a sum of non-negative terms, 131 x 2^-24 = 8e-6 in all, the
+// rest is 64 bits; squares below the normal range lose at most 2^-150 each, 1e-30 for every vector that fits the device; an
+// overflow makes the sum infinite.  Closer distortions, and vectors that the exact fallback has selected from, go through the ordered 64-bit
+// sums below, where M and B are bit-identical whenever the candidates coincide.  (g_i = 0, the state of the first round: they coincide
+// term by term, and a tie goes to the Markov compressor.)
+__device__ __forceinline__ int plus_decision(const PlusSums& s, int i, int n) {
+    if (s.low == nullptr) return 2;
+    const int lane = threadIdx.x & 31;
+    double M = 0.0, B = 0.0;
+    bool nonzero = false;
+    for (int q = lane; q < s.low_parts; q += 32) {
+        const double2 w = s.low[(i64)i * s.low_pitch + q];
+        M += w.x; B += w.y;
+        nonzero |= s.nonzero[(i64)i * s.low_pitch + q] != 0;
+    }
+    for (int q = lane; q < s.groups; q += 32) { M += s.cand[(i64)i * s.groups + q]; B += s.cand[(i64)(n + i) * s.groups + q]; }
+    M = warp_sum(M); B = warp_sum(B);
+    if (s.ctl[i].slow || s.ctl[n + i].slow || !(M + B <= 1.7e308)) return 2;
+    if (!__any_sync(0xffffffffu, nonzero)) return 0;
+    if (!(fabs(M - B) > 1e-4 * (M + B) + 1e-30)) return 2;
+    return M <= B ? 0 : 1;
+}
+
+// The ordered sums.  grid = (parts, n); part p of worker i covers the coordinates [p * len, (p + 1) * len).  part_out[i][p] = (M, B) of the part.  M and B
 // are summed over the same coordinates in the same order, so that they are bit-identical whenever the two candidates coincide
 // (e.g. g_i = 0).
 __global__ void __launch_bounds__(PLUS_BLOCK)
 plus_distortion_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict__ gi, i64 ld, i64 d, i64 len,
-                       const unsigned long long* __restrict__ cuts /* [2][n]: Markov, plain */, double2* __restrict__ part_out) {
+                       const unsigned long long* __restrict__ cuts /* [2][n]: Markov, plain */, double2* __restrict__ part_out, const __grid_constant__ PlusSums sums) {
     pdl_trigger();
     pdl_wait(a, gi, cuts, part_out);
     __shared__ double scratch[PLUS_BLOCK / 32];
     const int i = blockIdx.y, n = gridDim.y;
+    if (plus_decision(sums, i, n) != 2) return;                      // as a rule
     const unsigned long long cut_m = cuts[i], cut_b = cuts[n + i];
     const unsigned km = (unsigned)(cut_m >> 32), jm = 0xffffffffu - (unsigned)cut_m, kb = (unsigned)(cut_b >> 32), jb = 0xffffffffu - (unsigned)cut_b;
     const float* __restrict__ grad = a + (i64)i * pitch_a;
@@ -72,14 +99,17 @@ plus_distortion_kernel(const float* __restrict__ a, i64 pitch_a, const float* __
 __global__ void __launch_bounds__(PLUS_BLOCK)
 plus_choose_kernel(const double2* __restrict__ parts_in, int parts, float* __restrict__ gi, i64 ld, int k,
                    int* __restrict__ idx_m, float* __restrict__ val_m, const int* __restrict__ idx_b, const float* __restrict__ val_b,
-                   int* __restrict__ choice) {
+                   int* __restrict__ choice, const __grid_constant__ PlusSums sums) {
     pdl_trigger();
     pdl_wait(parts_in, gi, idx_m, val_m, idx_b, val_b, choice);
     const int i = blockIdx.y, lane = threadIdx.x & 31;
-    double M = 0.0, B = 0.0;
-    for (int q = lane; q < parts; q += 32) { const double2 s = parts_in[(i64)i * PLUS_MAX_PARTS + q]; M += s.x; B += s.y; }
-    M = warp_sum(M); B = warp_sum(B);
-    const int plain = M <= B ? 0 : 1;
+    int plain = plus_decision(sums, i, gridDim.y);
+    if (plain == 2) {
+        double M = 0.0, B = 0.0;
+        for (int q = lane; q < parts; q += 32) { const double2 s = parts_in[(i64)i * PLUS_MAX_PARTS + q]; M += s.x; B += s.y; }
+        M = warp_sum(M); B = warp_sum(B);
+        plain = M <= B ? 0 : 1;
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) choice[i] = plain;
     const int t = blockIdx.x * PLUS_BLOCK + threadIdx.x;
     if (t >= k) return;
@@ -93,9 +123,10 @@ plus_choose_kernel(const double2* __restrict__ parts_in, int parts, float* __res
 }
 
 // g_j = (sum over workers, ascending, of g_ij) * (1/n), four coordinates per thread (ld is a multiple of four); g_ij of a worker that took
-// the plain branch becomes C(grad_i)_j first.  XMODE as in the aggregation kernels.
+// the plain branch becomes C(grad_i)_j first.  XMODE as in the aggregation kernels.  Four blocks per SM (107 registers and two blocks:
+// 16.9 us for 16 x 1,000,003, now 14.2).
 template <int XMODE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 plus_mean_kernel(const float* __restrict__ a, i64 pitch_a, const unsigned long long* __restrict__ cut_b, const int* __restrict__ choice,
                  float* __restrict__ gi, i64 ld, int n, i64 d, float inv_n, float gamma, float* __restrict__ g, float* __restrict__ x) {
     pdl_trigger();

@@ -33,8 +33,9 @@ constexpr int TC_MAX_CLUSTER = 16;          // 16 needs the non-portable cluster
 constexpr int TC_MAX_SLICE = 47104;         // floats per block (184 KB)
 
 // How v is formed: TC_PLAIN v = a; TC_DIFF v = a - b; TC_EF v = b + gamma * a, and b takes v (Algorithm 4: the error vector
-// becomes the vector to be compressed); TC_SENT v = b, which a TC_EF pass has already formed.
-enum { TC_PLAIN = 0, TC_DIFF = 1, TC_EF = 2, TC_SENT = 3 };
+// becomes the vector to be compressed); TC_SENT v = b, which a TC_EF pass has already formed; TC_PAIR (long vectors of EF21+): the
+// first half of the batch is a - b, the second half the same a once more.
+enum { TC_PLAIN = 0, TC_DIFF = 1, TC_EF = 2, TC_SENT = 3, TC_PAIR = 4 };
 
 struct TcArgs {
     const float* a; i64 pitch_a;
@@ -574,6 +575,23 @@ tc_topk_kernel(const __grid_constant__ TcArgs p) {
             }
     } else {
         tc_vector<MODE, C, THREADS, STREAM, GRAD>(p, (int)(blockIdx.x / (unsigned)(GRAD > 1 ? GRAD : C)));
+    }
+}
+
+// The exact fallback of both selections of EF21+ in one launch: flags of the vectors a - b (pm), then of the vectors a (pb).
+template <int C, int THREADS>
+__global__ void __launch_bounds__(THREADS)
+tc_pair_kernel(const __grid_constant__ TcArgs pm, const __grid_constant__ TcArgs pb) {
+    pdl_trigger();
+    pdl_wait();
+    for (int v = (int)(blockIdx.x / (unsigned)C); v < 2 * pm.batch; v += (int)(gridDim.x / (unsigned)C)) {
+        const bool plain = v >= pm.batch;
+        const int vec = plain ? v - pm.batch : v;
+        const TcArgs& p = plain ? pb : pm;
+        if (p.flag[(i64)vec * p.flag_pitch] == 0u) continue;
+        if (plain) tc_vector<TC_PLAIN, C, THREADS, true, 0>(pb, vec);
+        else tc_vector<TC_DIFF, C, THREADS, true, 0>(pm, vec);
+        cooperative_groups::this_cluster().sync();
     }
 }
 

@@ -56,6 +56,7 @@ struct StArgs {
     i64 d; int k, nreg, nreg_pitch, region_log, cap;    // nreg_pitch: nreg rounded up to 8; cap: records per region (0: regions are always read again)
     unsigned open_cap;
     float gamma;
+    int pair;                           // TC_PAIR: vectors in each half of the batch
     StCtl* ctl;                         // [batch]
     unsigned* open_hist;                // [batch][ST_OPEN_BINS]
     unsigned long long* open_list;      // [batch][open_cap]
@@ -71,7 +72,7 @@ __device__ __forceinline__ unsigned long long st_composite(unsigned key, unsigne
 
 template <int MODE>
 __device__ __forceinline__ float st_value(float a, float b, float gamma) {
-    return MODE == TC_DIFF ? __fsub_rn(a, b) : (MODE == TC_EF ? __fadd_rn(b, __fmul_rn(gamma, a)) : a);
+    return MODE == TC_DIFF || MODE == TC_PAIR ? __fsub_rn(a, b) : (MODE == TC_EF ? __fadd_rn(b, __fmul_rn(gamma, a)) : a);
 }
 
 // ---- 1. bracket ---------------------------------------------------------------------------------
@@ -95,15 +96,16 @@ st_sample_kernel(const __grid_constant__ StArgs p, float rank, float margin) {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // block 0's words are ready
     pdl_trigger();
     pdl_wait();
-    const float* __restrict__ av = pdl_ptr(p.a + (i64)vec * p.pitch_a);
-    const float* __restrict__ bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)vec * p.pitch_b);
+    const bool second = MODE == TC_PAIR && vec >= p.pair;
+    const float* __restrict__ av = pdl_ptr(p.a + (i64)(second ? vec - p.pair : vec) * p.pitch_a);
+    const float* __restrict__ bv = MODE == TC_PLAIN ? nullptr : pdl_ptr(p.b + (i64)(second ? 0 : vec) * p.pitch_b);
     const int warps = C * (ST_SAMPLE_THREADS / 32), w = rk * (ST_SAMPLE_THREADS / 32) + (tid >> 5);
     const i64 stride = p.d / ((i64)warps * PT);                     // >= 32: a quarter of the vector at most is sampled
     unsigned key[PT];
 #pragma unroll
     for (int s = 0; s < PT; ++s) {
         const i64 j = ((i64)s * warps + w) * stride + lane;
-        key[s] = mag_key(st_value<MODE>(av[j], MODE == TC_PLAIN ? 0.f : bv[j], p.gamma));
+        key[s] = mag_key(st_value<MODE>(av[j], MODE == TC_PLAIN || second ? 0.f : bv[j], p.gamma));
     }
     // open histogram of this vector, for the streaming pass
     for (int q = rk * ST_SAMPLE_THREADS + tid; q < ST_OPEN_BINS; q += C * ST_SAMPLE_THREADS) p.open_hist[(i64)vec * ST_OPEN_BINS + q] = 0u;
@@ -420,6 +422,162 @@ st_collect_kernel(const __grid_constant__ StArgs p) {
         if (open_at + e < p.open_cap) p.open_list[(i64)vec * p.open_cap + open_at + e] = stage[e];
 }
 
+// ---- EF21+: both selections and the distortions from one pass -------------------------------------
+// Worker i compresses a_i - g_i (vector i of the batch) and a_i (vector n + i).  One pass over a_i and g_i lists the candidates of both
+// and adds up the distortions' terms of the entries below each bracket, which are not in that message for sure; those of the candidates
+// are added by st_compact_pair_kernel, which knows the cuts.  The terms of a region are squared and added in 32 bits, the regions in 64:
+// these sums only tell apart distortions that differ by more than their rounding can be, the others are decided by the ordered 64-bit
+// sums as ever (plus_decision).  (All in 64 bits the pass took 65 us for 16 x 1,000,003, conversions and all.)
+struct PlusSums {
+    double2* low; int* nonzero;         // [n][low_pitch]: (M, B) of the entries below the brackets, per block of the pass; whether g_i has a non-zero there
+    int low_pitch, low_parts;
+    double* cand; int groups;           // [2 n][groups]: M, then B, of the candidates
+    const StCtl* ctl;                   // [2 n]
+};
+
+constexpr int ST_PAIR_LOADS = 8, ST_PAIR_OPEN = 1024, ST_PAIR_GATHER = 32 + 32 * ST_PAIR_LOADS;      // (emptied from 32 on)
+
+// A warp's buffer of candidates, and the block's open entries.
+struct StPairShared {
+    float a[2][ST_WARPS][ST_PAIR_GATHER], g[ST_WARPS][ST_PAIR_GATHER];
+    unsigned short at[2][ST_WARPS][ST_PAIR_GATHER];
+    unsigned long long open[2][ST_PAIR_OPEN];
+};
+
+// grid = (blocks per worker, n), 256 threads, one warp per region, in turn, all blocks resident and every warp with the same number of
+// regions (a few blocks more than fit made a second wave: 61 us).  Bound by instructions, about fifty per 32 entries: 16 x 1,000,003,
+// one in a hundred, 44 us against 24 + 21 + 32 for two passes and the distortions' own (65 with a call of the emptying code in every
+// quarter of a batch, which is more code than the instruction cache takes well; the next batch fetched ahead costs the fourth
+// block per SM: 45).
+__global__ void __launch_bounds__(ST_WARPS * 32, 4)
+st_collect_pair_kernel(const __grid_constant__ StArgs p, const __grid_constant__ PlusSums sums) {
+    constexpr int U = ST_PAIR_LOADS;
+    extern __shared__ __align__(16) unsigned char st_pair_smem[];
+    StPairShared& sh = *reinterpret_cast<StPairShared*>(st_pair_smem);
+    __shared__ unsigned sure_sh[2], open_sh[2], open_at[2];
+    __shared__ double low_sh[2][ST_WARPS];
+    __shared__ int nonzero_sh;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, worker = blockIdx.y;
+    if (tid < 2) { sure_sh[tid] = 0u; open_sh[tid] = 0u; }
+    if (tid == 0) nonzero_sh = 0;
+    __syncthreads();
+    pdl_trigger();
+    pdl_wait();
+    double low[2] = {0.0, 0.0};
+    unsigned bits = 0u;                                              // of g_i, without the signs
+    const int vecs[2] = {worker, p.pair + worker};
+    const int first = blockIdx.x * ST_WARPS + warp, step = gridDim.x * ST_WARPS;
+    const float* __restrict__ av = pdl_ptr(p.a + (i64)worker * p.pitch_a);
+    const float* __restrict__ bv = pdl_ptr(p.b + (i64)worker * p.pitch_b);
+    // the entries i0 + lane, 32 apart, of a region; zeros behind the end of the vector
+    float a_next[U], g_next[U];
+    auto fetch = [&](int region, int i0) {
+        const i64 j = ((i64)region << p.region_log) + i0 + lane, left = p.d - j;
+        if (left + lane >= 32 * U) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) { a_next[u] = av[j + 32 * u]; g_next[u] = bv[j + 32 * u]; }
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) { a_next[u] = 32 * u < left ? av[j + 32 * u] : 0.f; g_next[u] = 32 * u < left ? bv[j + 32 * u] : 0.f; }
+        }
+    };
+#pragma unroll 1
+    for (int region = first; region < p.nreg; region += step) {
+        const unsigned lo[2] = {p.ctl[vecs[0]].lo, p.ctl[vecs[1]].lo};
+        const i64 base = (i64)region << p.region_log;
+        const int end = (int)min((i64)1 << p.region_log, p.d - base);           // positions below are relative to the region
+        unsigned held[2] = {0u, 0u}, done[2] = {0u, 0u}, sure[2] = {0u, 0u};
+        float below[2] = {0.f, 0.f};                                            // this region's terms, 32 or 128 per lane
+        // a buffer's candidates: records to the region's list; an entry is sure, or open
+        auto empty = [&](int s) {
+            __syncwarp();
+            const StCtl& ct = p.ctl[vecs[s]];
+            int4* out = p.cand + ((i64)vecs[s] * p.nreg + region) * p.cap;
+#pragma unroll 1
+            for (unsigned e = lane; e < held[s]; e += 32u) {
+                const float a = sh.a[s][warp][e], g = s == 0 ? sh.g[warp][e] : 0.f, v = __fsub_rn(a, g);
+                const int j = (int)base + sh.at[s][warp][e];
+                const unsigned key = mag_key(v);
+                if (done[s] + e < (unsigned)p.cap) out[done[s] + e] = make_int4(j, __float_as_int(v), __float_as_int(g), __float_as_int(a));
+                if (key >= ct.hi) { ++sure[s]; continue; }
+                atomicAdd(&p.open_hist[(i64)vecs[s] * ST_OPEN_BINS + ((key - ct.lo) >> ct.shift)], 1u);
+                const unsigned long long x = st_composite(key, (unsigned)j);
+                const unsigned at = atomicAdd(&open_sh[s], 1u);
+                if (at < (unsigned)ST_PAIR_OPEN) sh.open[s][at] = x;
+                else {
+                    const unsigned to = atomicAdd(&p.ctl[vecs[s]].open, 1u);
+                    if (to < p.open_cap) p.open_list[(i64)vecs[s] * p.open_cap + to] = x;
+                }
+            }
+            done[s] += held[s]; held[s] = 0u;
+            __syncwarp();
+        };
+#pragma unroll 1
+        for (int i0 = 0; i0 < end; i0 += 32 * U) {
+            const int j0 = i0 + lane;
+            const bool last = i0 + 32 * U >= end;
+            fetch(region, i0);
+            float (&a)[U] = a_next, (&g)[U] = g_next;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {                                       // entries behind the end are zeros
+                const float v = __fsub_rn(a[u], g[u]);
+                const bool pr[2] = {mag_key(v) >= lo[0], mag_key(a[u]) >= lo[1]};
+                if (!pr[0]) below[0] = fmaf(v, v, below[0]);
+                if (!pr[1]) below[1] = fmaf(a[u], a[u], below[1]);
+                bits |= __float_as_uint(g[u]);
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    const unsigned bm = __ballot_sync(0xffffffffu, pr[s]);
+                    if (bm == 0u) continue;
+                    if (pr[s]) {
+                        const unsigned to = held[s] + (unsigned)__popc(bm & ((1u << lane) - 1u));
+                        sh.a[s][warp][to] = a[u];
+                        if (s == 0) sh.g[warp][to] = g[u];
+                        sh.at[s][warp][to] = (unsigned short)(j0 + 32 * u);
+                    }
+                    held[s] += (unsigned)__popc(bm);
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                if (held[s] >= 32u || last) empty(s);
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            low[s] += (double)below[s];
+            const unsigned all = __reduce_add_sync(0xffffffffu, sure[s]);
+            if (lane == 0) {
+                p.reg_cand[(i64)vecs[s] * p.nreg_pitch + region] = done[s];
+                p.reg_base[(i64)vecs[s] * p.nreg_pitch + region] = all;
+                if (all) atomicAdd(&sure_sh[s], all);
+            }
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        low[s] = warp_sum(low[s]);
+        if (lane == 0) low_sh[s][warp] = low[s];
+    }
+    if (__any_sync(0xffffffffu, (bits << 1) != 0u) && lane == 0) nonzero_sh = 1;
+    __syncthreads();
+    if (tid == 0) {
+        double2 sum = make_double2(0.0, 0.0);
+        for (int w = 0; w < ST_WARPS; ++w) { sum.x += low_sh[0][w]; sum.y += low_sh[1][w]; }
+        sums.low[(i64)worker * sums.low_pitch + blockIdx.x] = sum;
+        sums.nonzero[(i64)worker * sums.low_pitch + blockIdx.x] = nonzero_sh;
+    }
+    if (tid < 2) {
+        const unsigned n = min(open_sh[tid], (unsigned)ST_PAIR_OPEN);
+        open_at[tid] = n ? atomicAdd(&p.ctl[vecs[tid]].open, n) : 0u;
+        if (sure_sh[tid]) atomicAdd(&p.ctl[vecs[tid]].sure, sure_sh[tid]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+        for (unsigned e = tid; e < min(open_sh[s], (unsigned)ST_PAIR_OPEN); e += ST_WARPS * 32)
+            if (open_at[s] + e < p.open_cap) p.open_list[(i64)vecs[s] * p.open_cap + open_at[s] + e] = sh.open[s][e];
+}
+
 // ---- exact cut and the regions' first positions ---------------------------------------------------
 // One cluster of C blocks of 1,024 threads per vector; dynamic shared memory for ST_OPEN_STAGE composites.  CLASSIFY: the streaming
 // pass has only listed the candidates; they are divided into sure and open ones here, the open ones of a block stay in its
@@ -705,7 +863,75 @@ st_compact_kernel(const __grid_constant__ StArgs p, const StOut o) {
     }
 }
 
-// The same where no lists are kept (more than a tenth of the entries are wanted): one warp per region reads it again, and gathers
+// The messages of EF21+ and the candidates' terms of the distortions; grid = (ceil(nreg / 32), 2 n), 256 threads, eight lanes per region.
+// A Markov record is (index, v, g, a), a plain one (index, a, g, a).
+__global__ void __launch_bounds__(256)
+st_compact_pair_kernel(const __grid_constant__ StArgs p, const __grid_constant__ PlusSums sums, int* idx_m, float* val_m, int* idx_b, float* val_b,
+                       unsigned long long* cut_out, unsigned* status) {
+    pdl_trigger();
+    pdl_wait(idx_m, val_m, idx_b, val_b, cut_out, status);
+    __shared__ double sum_sh[8];
+    const int vec = blockIdx.y, lane = threadIdx.x & 31, sub = lane & 7, group = lane & ~7;
+    const bool plain = vec >= p.pair;
+    const int worker = plain ? vec - p.pair : vec;
+    const int region = blockIdx.x * 32 + (threadIdx.x >> 3);
+    const StCtl& ct = p.ctl[vec];
+    if (ct.slow) return;
+    const unsigned long long cut = ct.cut;
+    const unsigned lo = ct.lo;
+    if (blockIdx.x == 0 && threadIdx.x == 0) cut_out[vec] = cut;
+    const bool have = region < p.nreg;
+    const unsigned n = have ? p.reg_cand[(i64)vec * p.nreg_pitch + region] : 0u;
+    unsigned pos = have ? p.reg_base[(i64)vec * p.nreg_pitch + region] : 0u;
+    int* io = (plain ? idx_b : idx_m) + (i64)worker * p.k;
+    float* vo = (plain ? val_b : val_m) + (i64)worker * p.k;
+    const i64 base = (i64)region << p.region_log;
+    double sum = 0.0;
+    auto emit = [&](bool mine, int j, float v, float g, float a) {
+        const bool sel = mine && st_composite(mag_key(v), (unsigned)j) >= cut;
+        const unsigned bal = (__ballot_sync(0xffffffffu, sel) >> group) & 0xffu;
+        if (sel) {
+            const unsigned at = pos + (unsigned)__popc(bal & ((1u << sub) - 1u));
+            io[at] = j; vo[at] = v;
+            flag_nonfinite(status, v);
+        }
+        if (mine) {
+            const double e = plain ? (sel ? 0.0 : (double)a) : (double)(sel ? __fadd_rn(g, v) : g) - (double)a;
+            sum = fma(e, e, sum);
+        }
+        pos += (unsigned)__popc(bal);
+    };
+    const bool listed = n <= (unsigned)p.cap;
+    const unsigned steps = __reduce_max_sync(0xffffffffu, listed ? (n + 7u) / 8u : 0u);
+    const int4* in = p.cand + ((i64)vec * p.nreg + (have ? region : 0)) * p.cap;
+    for (unsigned s = 0; s < steps; ++s) {
+        const unsigned e = 8u * s + (unsigned)sub;
+        const bool mine = listed && e < n;
+        const int4 w = mine ? in[e] : make_int4(0, 0, 0, 0);
+        emit(mine, w.x, __int_as_float(w.y), __int_as_float(w.z), __int_as_float(w.w));
+    }
+    // regions whose list overflowed: all four groups of the warp stay together, each reads its own
+    if (__any_sync(0xffffffffu, !listed)) {
+        const float* __restrict__ av = pdl_ptr(p.a + (i64)worker * p.pitch_a);
+        const float* __restrict__ bv = pdl_ptr(p.b + (i64)worker * p.pitch_b);
+        for (int s = 0; s < 1 << (p.region_log - 3); ++s) {
+            const i64 j = base + 8 * s + sub;
+            const bool in_range = !listed && j < p.d;
+            const float a = in_range ? av[j] : 0.f, g = in_range ? bv[j] : 0.f, v = plain ? a : __fsub_rn(a, g);
+            emit(in_range && mag_key(v) >= lo, (int)j, v, g, a);
+        }
+    }
+    sum = warp_sum(sum);
+    if (lane == 0) sum_sh[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double all = 0.0;
+        for (int w = 0; w < 8; ++w) all += sum_sh[w];
+        sums.cand[(i64)vec * sums.groups + blockIdx.x] = all;
+    }
+}
+
+// The compaction where no lists are kept (more than a tenth of the entries are wanted): one warp per region reads it again, and gathers
 // the selected ones of 256 entries in shared memory before they are written side by side.  Bound by instructions (20 x 2,642,533, a
 // tenth wanted: 83 us with a store per lane and entry, now 73).
 // grid = (ceil(nreg / 8), batch), 256 threads.
