@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.util
 import os
 from typing import Optional, Tuple
 
@@ -92,7 +93,20 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     return lib
 
 
+def _load_call():
+    """The native form of topk() for the usual arguments (csrc/topk_call.cpp)."""
+    path = os.path.join(_HERE, "_topk_call.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with `python -m paper_2106_05203_b200.build`")
+    spec = importlib.util.spec_from_file_location("_topk_call", path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    module.set_entry(*(ctypes.cast(f, _vp).value for f in (_lib.ef21_topk_workspace_bytes, _lib.ef21_topk)))
+    return module.topk
+
+
 _lib = load_library()
+_topk_call = _load_call()
 
 
 def _check(status: int, where: str) -> None:
@@ -368,6 +382,12 @@ def _topk_workspace_bytes(batch: int, d: int, k: int) -> int:
 
 def topk(v: torch.Tensor, k: int, stream: Optional[torch.cuda.Stream] = None):
     """Top-k compressor on a batch of vectors v[batch, d] -> (idx[batch, k] int32, val[batch, k])."""
+    if stream is None:
+        out = _topk_call(v, k)                              # None: not one of the usual calls
+        if out is not None:
+            if type(out) is tuple:
+                return out
+            raise Ef21Error(out, "ef21_topk")
     if v.dim() == 1:
         v = v.unsqueeze(0)
     _dev_f32(v)
@@ -377,8 +397,7 @@ def topk(v: torch.Tensor, k: int, stream: Optional[torch.cuda.Stream] = None):
     if device.index != torch.cuda.current_device():
         with torch.cuda.device(device):
             return topk(v, k, stream)
-    # On short vectors the call is bound by this function (the kernel takes 3-5 us): no scratch is allocated where the
-    # library needs none, and nothing is recorded on the stream that everything was allocated on.
+    # No scratch is allocated where the library needs none, and nothing is recorded on the stream that everything was allocated on.
     idx = torch.empty_strided((batch, k), (k, 1), dtype=torch.int32, device=device)
     val = torch.empty_strided((batch, k), (k, 1), dtype=torch.float32, device=device)
     if nbytes <= _NO_SCRATCH:

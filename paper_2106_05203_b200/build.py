@@ -1,4 +1,5 @@
-"""Builds libef21.so (sm_100a) next to this file with nvcc.  No GPU is needed to build."""
+"""Builds libef21.so (sm_100a, nvcc) and the Python call of its standalone Top-k (_topk_call.so, the C++ compiler, against
+torch's headers) next to this file.  No GPU is needed to build."""
 from __future__ import annotations
 
 import glob
@@ -10,6 +11,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libef21.so")
+CALL = os.path.join(HERE, "_topk_call.so")
+CALL_SOURCE = os.path.join(CSRC, "topk_call.cpp")
 
 
 def nvcc_path() -> str:
@@ -24,11 +27,34 @@ def sources():
 
 
 def _newest_source_mtime() -> float:
-    files = glob.glob(os.path.join(CSRC, "*")) + [os.path.join(HERE, "..", "include", "ef21.h")]
+    files = [f for f in glob.glob(os.path.join(CSRC, "*")) if f != CALL_SOURCE] + [os.path.join(HERE, "..", "include", "ef21.h")]
     return max(os.path.getmtime(f) for f in files)
 
 
+def build_call(force: bool = False) -> str:
+    if not force and os.path.exists(CALL) and os.path.getmtime(CALL) >= os.path.getmtime(CALL_SOURCE):
+        return CALL
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
+    include = [sysconfig.get_paths()["include"], *cpp_extension.include_paths(), cuda]
+    tmp = CALL + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                    f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{i}" for i in include), CALL_SOURCE,
+                    *(f"-L{p}" for p in cpp_extension.library_paths()), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+                    "-o", tmp], check=True)         # (found by name at run time: the import of torch has loaded them)
+    os.replace(tmp, CALL)
+    return CALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    """Builds both; returns the path of the library."""
+    build_call(force)
+    return build_library(force, verbose)
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compiles every csrc/*.cu to an object file (side by side: the persistent kernels of the three
     methods are translation units of their own) and links libef21.so."""
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
