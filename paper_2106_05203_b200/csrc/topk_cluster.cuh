@@ -37,6 +37,8 @@ constexpr int TC_MAX_SLICE = 47104;         // floats per block (184 KB)
 // first half of the batch is a - b, the second half the same a once more.
 enum { TC_PLAIN = 0, TC_DIFF = 1, TC_EF = 2, TC_SENT = 3, TC_PAIR = 4 };
 
+template <bool V> struct TcFlag { static constexpr bool value = V; };
+
 struct TcArgs {
     const float* a; i64 pitch_a;
     float* b; i64 pitch_b;                  // TC_EF: updated in place
@@ -176,6 +178,142 @@ __device__ __forceinline__ bool tc_few(const TcArgs& p, int vec, const unsigned*
     return true;
 }
 
+// The same for a cluster: every block finds a floor that at least k / C of its entries reach, the lowest of the C floors is the cluster's (k
+// entries or more reach it), and the entries from there on are handed around.  Every block finds the k-th of them by a histogram of 2,047
+// even steps between the floor and the maximum and by ranking the few in the deciding step, and places its own through a bitmap of its
+// share.  Two cluster barriers as without, but no atomic per entry, no histogram over distributed shared memory, no sweep for the list and
+// none for the compaction.  (Every own candidate ranked against all: a quarter of a million comparisons per block.)
+// 20 x 70,001, Top-700: 14.0 -> 11.5 us; 1 x 81,822, Top-818: 16.2 -> 14.0 with the call.
+// False (for the whole cluster): too many candidates, as where the large entries sit together in one block's share.
+constexpr int TC_FEW_OWN = 1024, TC_FEW_ALL = 2048;
+
+template <int MODE, int C, int THREADS>
+__device__ __forceinline__ bool tc_few_cluster(const TcArgs& p, int vec, int rank, int j0, int len, const unsigned* ws, unsigned* hist, unsigned* list,
+                                               unsigned long long* all, unsigned largest, unsigned* wmin, unsigned* wmax, unsigned* wsum, unsigned* found,
+                                               unsigned& list_n) {
+    namespace cg = cooperative_groups;
+    constexpr int WARPS = THREADS / 32, BITMAP = TC_MAX_SLICE / 32, GROUPS = BITMAP / 4;
+    static_assert(BITMAP + GROUPS <= TC_BINS, "bitmap and its prefix sums take the histogram's place");
+    __shared__ unsigned floor_sh, top_sh, before_sh, step_n, scratch[33];
+    __shared__ unsigned long long kth_sh, step_sh[TC_RANKED];
+    cg::cluster_group cluster = cg::this_cluster();
+    unsigned long long* cand = reinterpret_cast<unsigned long long*>(list);     // this block's (key << 32 | ~index), [TC_FEW_OWN]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = p.k, share = (k + C - 1) / C;
+    {
+        const unsigned hi = __reduce_max_sync(0xffffffffu, largest), lo = __reduce_min_sync(0xffffffffu, largest);
+        if (lane == 0) { wmax[warp] = hi; wmin[warp] = lo; }
+        if (tid == 0) { before_sh = 0u; step_n = 0u; }
+        hist[tid] = 0u; hist[tid + THREADS] = 0u;
+        static_assert(TC_BINS == 2 * THREADS, "two bins per thread");
+    }
+    __syncthreads();
+    unsigned floor = __reduce_min_sync(0xffffffffu, wmin[lane]), top = __reduce_max_sync(0xffffffffu, wmax[lane]);
+    static_assert(WARPS == 32, "a lane per warp");
+    if (tid == 0) top_sh = top;
+#pragma unroll 1
+    while (floor < top) {
+        const unsigned mid = floor + (top - floor + 1u) / 2u;
+        const int n = __syncthreads_count(largest >= mid);
+        if (n >= share) { floor = mid; if (n <= share + share / 4 + 4) break; }
+        else top = mid - 1u;
+    }
+    if (tid == 0) floor_sh = floor & ~1u;                                       // both signs of a magnitude
+    cluster.sync();
+    floor = 0xffffffffu; top = 0u;
+#pragma unroll
+    for (int r = 0; r < C; ++r) { floor = min(floor, *cluster.map_shared_rank(&floor_sh, r)); top = max(top, *cluster.map_shared_rank(&top_sh, r)); }
+    if (largest >= floor) {
+#pragma unroll 4
+        for (int j = tid; j < len; j += THREADS) {
+            const unsigned w = ws[j];
+            if (w >= floor) {
+                const unsigned at = atomicAdd(&list_n, 1u);
+                if (at < (unsigned)TC_FEW_OWN) cand[at] = ((unsigned long long)(w >> 1) << 32) | (0xffffffffu - (unsigned)(j0 + j));
+            }
+        }
+    }
+    cluster.sync();
+    unsigned n_of[C], total = 0u, first = 0u;
+    bool fits = true;
+#pragma unroll
+    for (int r = 0; r < C; ++r) {
+        n_of[r] = *cluster.map_shared_rank(&list_n, r);
+        fits = fits && n_of[r] <= (unsigned)TC_FEW_OWN;
+        if (r < rank) first += n_of[r];
+        total += n_of[r];
+    }
+    if (!fits || total > (unsigned)TC_FEW_ALL) return false;
+    const unsigned c = list_n, low = floor >> 1;
+    int shift = 0;
+    while ((((top >> 1) - low) >> shift) >= (unsigned)TC_BINS - 1u) ++shift;
+    auto step_of = [&](unsigned long long x) { return 1u + (((unsigned)(x >> 32) - low) >> shift); };
+#pragma unroll 1
+    for (unsigned e = tid; e < total; e += THREADS) {
+        unsigned off = e; int from = 0;
+#pragma unroll
+        for (int r = 0; r < C - 1; ++r) if (from == r && off >= n_of[r]) { off -= n_of[r]; from = r + 1; }
+        const unsigned long long x = cluster.map_shared_rank(cand, from)[off];
+        all[e] = x;
+        atomicAdd(&hist[step_of(x)], 1u);
+    }
+    // this block's own, one per thread
+    const bool have = tid < (int)c;
+    const unsigned long long mine = have ? cand[tid] : 0ull;
+    const int j = (int)(0xffffffffu - (unsigned)mine);
+    float* app = p.apply ? p.apply + (i64)vec * p.pitch_apply : nullptr;
+    const float old = MODE == TC_DIFF && have && app ? app[j] : 0.f;
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");       // done with the other blocks' memory
+    tc_find_bin(hist, (unsigned)k, total, wsum, found);
+    const unsigned step = found[0], need = (unsigned)k - found[1], pop = found[2];
+    if (pop > (unsigned)TC_RANKED) {                                            // (the same in all blocks)
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        return false;
+    }
+#pragma unroll 1
+    for (unsigned e = tid; e < total; e += THREADS) {
+        const unsigned long long x = all[e];
+        if (step_of(x) == step) step_sh[atomicAdd(&step_n, 1u)] = x;
+    }
+    hist[tid] = 0u; hist[tid + THREADS] = 0u;                                   // from here on the bitmap
+    __syncthreads();
+    if (tid < (int)pop) {
+        const unsigned long long x = step_sh[tid];
+        unsigned above = 0u;
+        for (unsigned o = 0; o < pop; ++o) above += step_sh[o] > x ? 1u : 0u;
+        if (above + 1u == need) kth_sh = x;
+    }
+    __syncthreads();
+    const unsigned long long kth = kth_sh;
+    const bool sel = have && mine >= kth;
+    if (sel) atomicOr(&hist[(j - j0) >> 5], 1u << ((j - j0) & 31));
+    unsigned before = 0u;                                                       // selected entries of the blocks before this one
+    for (unsigned o = tid; o < first; o += THREADS) before += all[o] >= kth ? 1u : 0u;
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 0 && before) atomicAdd(&before_sh, before);
+    __syncthreads();
+    {
+        const uint4 w = tid < GROUPS ? reinterpret_cast<const uint4*>(hist)[tid] : make_uint4(0u, 0u, 0u, 0u);
+        unsigned sum;
+        const unsigned up = block_excl_scan((unsigned)(__popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w)), scratch, sum);
+        if (tid < GROUPS) hist[BITMAP + tid] = up;
+    }
+    __syncthreads();
+    if (sel) {
+        const int word = (j - j0) >> 5;
+        unsigned pos = before_sh + hist[BITMAP + (word >> 2)] + (unsigned)__popc(hist[word] & ((1u << ((j - j0) & 31)) - 1u));
+        for (int q = word & ~3; q < word; ++q) pos += (unsigned)__popc(hist[q]);
+        const unsigned wv = ws[j - j0];
+        const float v = __uint_as_float(__funnelshift_r(wv, wv, 1));
+        p.idx_out[(i64)vec * k + pos] = j; p.val_out[(i64)vec * k + pos] = v;
+        flag_nonfinite(p.status, v);
+        if (mine == kth && p.cut_out) p.cut_out[vec] = mine;
+        if (app) app[j] = MODE == TC_DIFF ? __fadd_rn(old, v) : (MODE == TC_PLAIN ? __fadd_rn(0.f, v) : __fsub_rn(v, v));
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");         // nobody reads this block's list any more
+    return true;
+}
+
 // STREAM: the vector is longer than the cluster's shared memory; it stays in global memory and every sweep reads it again.
 // GRAD > 0: the local gradients are formed from the tile partials on the way in (no kernel and no array for them), by a cluster of GRAD
 // blocks that each take a share of the columns and leave v in the first one's shared memory; that one selects alone (C = 1).
@@ -203,11 +341,16 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
 
     const int j0 = (int)min((i64)rank * p.slice, (i64)p.d), len = min(p.slice, p.d - j0);
     const bool few = C == 1 && !STREAM && p.k <= THREADS / 4 && p.d <= THREADS * tc_few_values(THREADS);
+    // (sixteen blocks: a share of a few dozen entries makes an uneven floor, and every exchange goes to sixteen: 4 x 452,034, Top-452, 29.2
+    // against 30.0 us a round)
+    constexpr bool MAY_FEW = C > 1 && C <= 8 && !STREAM;
+    const bool few_cluster = MAY_FEW && p.k <= TC_FEW_OWN && (p.k + C - 1) / C <= THREADS / 5;
+    unsigned largest = 0u;
     auto clear = [&]() {
 #pragma unroll 1
         for (int q = tid; q < TC_BINS; q += THREADS) { hist[q] = 0u; if (C > 1) hsum[q] = 0u; }
     };
-    if (!few) clear();
+    if (!few && !few_cluster) clear();
     for (int j = len + tid; !STREAM && j < p.slice && j < len + 128; j += THREADS) ws[j] = 0u;       // the tail of the last tile
     if (tid < WARPS) { wgt[tid] = 0u; weq[tid] = 0u; }
     if (tid == 0) { list_n = 0u; above_n = 0u; before_sh[0] = 0u; before_sh[1] = 0u; result[0] = 0xffffffffu; }
@@ -226,7 +369,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     float* dense = MODE == TC_PLAIN && !STREAM && p.apply ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
     // entries of bin 0 (zeros and the smallest magnitudes) are not counted: what the other bins leave over is theirs
     auto count = [&](unsigned w) { if (!few && (w >> 21)) atomicAdd(&hist[w >> 21], 1u); };
-    auto take = [&](int j, float a, float b) {
+    auto take = [&](int j, float a, float b, auto only_largest) {
         float v = a;
         if (MODE == TC_DIFF) v = __fsub_rn(a, b);
         if (MODE == TC_EF) { v = __fadd_rn(b, __fmul_rn(p.gamma, a)); bv[j] = v; }
@@ -235,8 +378,10 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         if (MODE == TC_PLAIN && dense) dense[j] = 0.f;
         if (GRAD > 1) { cluster.map_shared_rank(ws, 0)[j] = w; return; }
         if (!STREAM) ws[j] = w;
-        count(w);
+        if (decltype(only_largest)::value) largest = max(largest, w);
+        else count(w);
     };
+    const TcFlag<false> all_counted;
     if (GRAD > 0) {
         const i64 m = p.batch_rows > 0 ? (i64)p.batch_rows : m_all;
         const int share = GRAD > 1 ? (len + GRAD - 1) / GRAD : len;
@@ -285,8 +430,8 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
                 for (int q = 1; q < Q; ++q) acc[u][0] = __fadd_rn(acc[u][0], acc[u][q]);
                 g[u] = __fadd_rn(m > 0 ? __fdiv_rn(acc[u][0], (float)m) : 0.f, regulariser_grad(p.lambda, xj[u]));
             }
-            take(js[0], g[0], b[0]);
-            if (jj + THREADS < c1) take(js[1], g[1], b[1]);
+            take(js[0], g[0], b[0], all_counted);
+            if (jj + THREADS < c1) take(js[1], g[1], b[1], all_counted);
         }
         // Behind the aggregation waits grad_wide_kernel, which fetches rows as soon as it is placed: not before this kernel's own
         // loads are through (20 x 5,001: 38.4 us an iteration instead of 39.4).
@@ -298,17 +443,20 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         }
     } else {
         constexpr int U = THREADS == 1024 ? 8 : 4;
-        int j = tid;
+        auto sweep = [&](auto only_largest) {
+            int j = tid;
 #pragma unroll 1
-        for (; j + (U - 1) * THREADS < len; j += U * THREADS) {
-            float a[U], b[U];
+            for (; j + (U - 1) * THREADS < len; j += U * THREADS) {
+                float a[U], b[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) { a[u] = MODE == TC_SENT ? 0.f : av[j + u * THREADS]; b[u] = MODE == TC_PLAIN ? 0.f : bv[j + u * THREADS]; }
+                for (int u = 0; u < U; ++u) { a[u] = MODE == TC_SENT ? 0.f : av[j + u * THREADS]; b[u] = MODE == TC_PLAIN ? 0.f : bv[j + u * THREADS]; }
 #pragma unroll
-            for (int u = 0; u < U; ++u) take(j + u * THREADS, a[u], b[u]);
-        }
+                for (int u = 0; u < U; ++u) take(j + u * THREADS, a[u], b[u], only_largest);
+            }
 #pragma unroll 1
-        for (; j < len; j += THREADS) take(j, MODE == TC_SENT ? 0.f : av[j], MODE == TC_PLAIN ? 0.f : bv[j]);
+            for (; j < len; j += THREADS) take(j, MODE == TC_SENT ? 0.f : av[j], MODE == TC_PLAIN ? 0.f : bv[j], only_largest);
+        };
+        if (MAY_FEW && few_cluster) sweep(TcFlag<MAY_FEW>()); else sweep(all_counted);
     }
     constexpr int OWN = TC_BINS / C;                                // bins summed by one block
     auto sum_histograms = [&]() {                                   // hist of all blocks -> hsum
@@ -339,6 +487,17 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         for (int j = tid; j < len; j += THREADS) { const unsigned w = ws[j]; if (w >> 21) atomicAdd(&hist[w >> 21], 1u); }
     }
     if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if constexpr (MAY_FEW) if (few_cluster) {
+        if (tc_few_cluster<MODE, C, THREADS>(p, vec, rank, j0, len, ws, hist, list, reinterpret_cast<unsigned long long*>(all), largest, wgt, weq, wsum, found, list_n))
+            return;
+        cluster.sync();                                             // (nobody reads this block's words any more)
+        clear();
+        if (tid == 0) list_n = 0u;
+        if (tid < WARPS) { wgt[tid] = 0u; weq[tid] = 0u; }
+        cluster.sync();
+#pragma unroll 1
+        for (int j = tid; j < len; j += THREADS) { const unsigned w = ws[j]; if (w >> 21) atomicAdd(&hist[w >> 21], 1u); }
+    }
     sum_histograms();
     tc_find_bin(hist, (unsigned)p.k, (unsigned)p.d, wsum, found);
     const unsigned bin0 = found[0], pop0 = found[2];

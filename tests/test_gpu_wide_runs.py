@@ -72,3 +72,51 @@ def test_few_entries_of_short_vectors(batch, d, k, kind, oracle32):
         oi, ov = oracle32.topk(v[i], k)
         np.testing.assert_array_equal(idx[i].cpu().numpy(), oi)
         np.testing.assert_array_equal(val[i].cpu().numpy().view(np.uint32), ov.view(np.uint32))
+
+
+# clusters of 2, 4, 8 and 16 blocks; k up to what the cluster's floors are used for and one more; the large entries in one block's
+# share (more candidates than it lists), ties at the cut in several blocks
+@pytest.mark.parametrize("kind", ["gauss", "ties", "signs", "layers", "bf16", "few nonzero"])
+@pytest.mark.parametrize("batch,d,k", [(1, 16384, 1), (40, 16385, 408), (3, 65537, 700), (20, 70001, 816), (20, 70001, 817), (2, 94209, 1024), (2, 376833, 1024),
+                                       (1, 376833, 1025), (1, 753664, 753)])
+def test_few_entries_in_a_cluster(batch, d, k, kind, oracle32):
+    from paper_2106_05203_b200 import binding as B
+    rng = np.random.default_rng(d + k)
+    v = rng.standard_normal((batch, d), dtype=np.float32)
+    if kind == "ties":
+        v = np.round(v * 4).astype(np.float32) * np.float32(0.25)
+    elif kind == "signs":
+        v = np.sign(v).astype(np.float32)
+    elif kind == "layers":
+        v[:, d // 3:d // 3 + max(2 * k, 1500)] *= np.float32(100)
+    elif kind == "bf16":
+        v = (v.view(np.uint32) & np.uint32(0xffff0000)).view(np.float32)
+    elif kind == "few nonzero":
+        v *= rng.random((batch, d)) < 0.5 * k / d
+    idx, val = B.topk(dev(v), k)
+    for i in sorted({0, batch // 2, batch - 1}):
+        oi, ov = oracle32.topk(v[i], k)
+        np.testing.assert_array_equal(idx[i].cpu().numpy(), oi)
+        np.testing.assert_array_equal(val[i].cpu().numpy().view(np.uint32), ov.view(np.uint32))
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("n,d,k", [(20, 70001, 700), (8, 95620, 95), (3, 376833, 1000)])
+def test_rounds_with_few_entries_in_a_cluster(n, d, k, variant):
+    from paper_2106_05203_b200 import binding as B
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    states = []
+    V = [torch.randn(n, d, device="cuda", generator=gen) * (1 + 3 * t) for t in range(3)]
+    V[1][0, d // 2:d // 2 + 2000] *= 50
+    for algorithm in (0, 1):
+        h = B.EF21(n, d, k, 0.05)
+        h.set_variant(variant)
+        h.set_topk_algorithm(algorithm)
+        h.init_grads(None, B.INIT_ZERO)
+        for v in V:
+            h.step_grads(v, 2)
+        assert h.poll() == 0
+        states.append(h.get_state())
+    for a, b in zip(*states):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
