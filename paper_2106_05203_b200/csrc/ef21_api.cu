@@ -125,7 +125,7 @@ TopkLayout topk_layout(i64 batch, i64 d, i64 k) {
         L.samples = std::max<i64>(512 * d / k, d / 64);
         L.samples = std::min<i64>(std::max<i64>(L.samples, 65536), std::max<i64>(65536, std::min<i64>(262144, 4194304 / batch)));
         L.samples = std::min<i64>(L.samples, d / 4);
-        L.samples = L.samples >= 262144 ? 262144 : (L.samples >= 131072 ? 131072 : 65536);
+        L.samples = L.samples >= 262144 ? 262144 : (L.samples >= 131072 ? 131072 : (L.samples >= 65536 ? 65536 : 32768));
         // Records per region: the expected candidates (the message plus the bracket's upper half) and six standard deviations
         // of a region's count; where more than a tenth of the entries are wanted a region is cheaper to read again.
         const double rank = (double)k * (double)L.samples / (double)d;
@@ -351,7 +351,8 @@ struct TcShape { int C, slice, threads; };
 // Blocks per vector: as few as hold the vector in shared memory, then more while all clusters still run at once and a
 // block keeps at least 8,192 entries (a shorter sweep per block; below that the two cluster barriers cost more than they
 // save).  False where the vector is too long, or so long and the batch so large that the clusters would run in several
-// waves of one-block-per-SM: the streaming kernels read such a batch at HBM speed.
+// waves of one-block-per-SM: the streaming kernels read such a batch at HBM speed (rounds with k = d / 100: 20 x 204,979 68 us in two waves,
+// 48 streamed, 40 x 135,000 62 and 44, 100 x 131,072 122 and 74; k = d / 10 109 and 68, 95 and 63, 181 and 120).
 bool tc_shape(i64 batch, i64 d, TcShape& S) {
     constexpr i64 SMS = 148;
     i64 C = 1;
@@ -425,10 +426,11 @@ StArgs stream_args(const float* a, i64 pitch_a, const float* b, i64 pitch_b, flo
 template <int MODE>
 ef21_status enqueue_stream_sample(cudaStream_t st, const StArgs& p, int batch, const TopkLayout& L, i64* launches) {
     const double rank = (double)p.k * (double)L.samples / (double)p.d;
-    const int C = batch <= 37 ? 8 : (batch <= 74 ? 4 : 2);
+    const int most = batch <= 37 ? 8 : (batch <= 74 ? 4 : 2);
+    const int C = most == 8 && L.samples < 65536 ? 4 : most;         // (eight samples per thread at least)
     const i64 per_thread = L.samples / (ST_SAMPLE_THREADS * C);
-    auto kern = C == 2 ? st_sample_kernel<MODE, 2, 32>
-                       : (C == 4 ? st_sample_kernel<MODE, 4, 16>
+    auto kern = C == 2 ? (per_thread >= 32 ? st_sample_kernel<MODE, 2, 32> : st_sample_kernel<MODE, 2, 16>)
+                       : (C == 4 ? (per_thread >= 16 ? st_sample_kernel<MODE, 4, 16> : st_sample_kernel<MODE, 4, 8>)
                                  : (per_thread >= 32 ? st_sample_kernel<MODE, 8, 32>
                                                      : (per_thread >= 16 ? st_sample_kernel<MODE, 8, 16> : st_sample_kernel<MODE, 8, 8>)));
     CU(launch(kern, dim3((unsigned)(batch * C)), ST_SAMPLE_THREADS, 0, st, (unsigned)C, p, (float)rank, (float)st_margin(rank)));

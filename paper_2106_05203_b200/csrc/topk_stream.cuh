@@ -38,7 +38,7 @@ constexpr int ST_OPEN_BINS = 2048;
 constexpr int ST_OPEN_STAGE = 8192;     // open entries of the deciding step that are ranked in shared memory
 constexpr int ST_BLOCK_OPEN = 2048;     // open entries a block of the streaming pass gathers before they go to the list
 constexpr int ST_GATHER = 160;          // a warp's buffer for candidates: emptied from 32 on, after at most 128 more
-constexpr i64 ST_MIN_D = 262144;        // shorter vectors always fit into a cluster
+constexpr i64 ST_MIN_D = 131072;        // shorter vectors go to a cluster each, however many there are
 
 // Per vector: the bracket, the counters of the streaming pass, the exact cut.
 struct StCtl {

@@ -22,7 +22,9 @@ def _vectors(n, d, crowd):
 
 @pytest.mark.parametrize("variant", [0, 2])
 @pytest.mark.parametrize("n,d,k,crowd", [(20, 262144, 2621, 256), (20, 262147, 2621, 257), (19, 263169, 30000, 1024), (20, 263168, 50000, 1023),
-                                         (20, 300001, 150000, 512), (20, 300004, 300, 1024)])
+                                         (20, 300001, 150000, 512), (20, 300004, 300, 1024),
+                                         # the shortest vectors of the pass, with smaller samples (clusters of them would run in turn)
+                                         (38, 131072, 131, 129), (40, 135001, 1350, 1024), (75, 131073, 20000, 300), (19, 262143, 60000, 512)])
 def test_rounds_and_topk(n, d, k, crowd, variant):
     from paper_2106_05203_b200 import binding as B
     V = _vectors(n, d, crowd)
