@@ -9,9 +9,11 @@ typedef long long i64;
 
 // Programmatic dependent launch.  Launched the plain way, a kernel that follows another one in a stream starts 2-4 us after
 // its predecessor's end (in steps of about 1 us; measured with spinning kernels of 0.3-10 us); launched as a programmatic
-// dependent it starts after 0.5 us.  Every kernel of the library calls pdl_wait() before it touches global memory (it
-// returns when the preceding kernels of the stream have completed and their writes are visible) and pdl_trigger() early (the
-// staged aggregation only where that pays, see apply.cuh), so that the kernel behind it can be placed on the device meanwhile.
+// dependent it starts after 0.5 us.  Every kernel of the library calls pdl_wait() before it touches global memory that a kernel may
+// have written since the shards were loaded (it returns when the preceding kernels of the stream have completed and their writes are
+// visible) and pdl_trigger() early (the staged aggregation only where that pays, see apply.cuh), so that the kernel behind it can
+// be placed on the device meanwhile.  Rows, labels and tables of the shards may be read in front of the wait: grad_wide_kernel, the
+// selection behind it and the persistent kernels do, see there.
 // The kernel's pointers go through pdl_wait so that no load through them -- a read-only one (const __restrict__, __ldg, __ldcs) is
 // otherwise free to move -- is placed in front of the wait.  Where they come in a struct, the local pointer that such loads
 // start from is made by pdl_ptr, behind the wait; or the loads are plain ones, which the wait's memory clobber keeps behind it

@@ -30,6 +30,12 @@
 // dense mean; whole-block body only), the original EF (Algorithm 4: the leader compresses e_i + gamma grad_i, the
 // messages move x directly) and the exchange skeleton (a measuring aid).  This header holds what they share.
 //
+// A launch loads its rows (and the shards' offsets and labels) before it waits for the kernel in front of it, as a rule the one that
+// forms the initial g.  They are complete by then whatever that kernel is: loading shards ends with copies of the offsets, which are no
+// programmatic dependents and have none, so that every kernel behind them starts after they, and the kernel that wrote the rows,
+// have ended.  The state and the lists of sampled rows are read behind the wait.  (1 to 3 us of a call: 20 x 2,487 x 300, 50 iterations,
+// 557 -> 549 us, 20 x 406 x 112, 100 iterations, 272 -> 270.)
+//
 // All summation orders are fixed by the launch shape, so two runs give identical bits.  A wait
 // that exceeds its spin limit records EF21_ERR_TIMEOUT in the status word; from then on every
 // block skips work but keeps arriving at the cluster barriers, so the kernel always terminates.
