@@ -159,12 +159,13 @@ GradPlan grad_plan(i64 ld) {
                                             : (slots == 2 ? grad_stream_kernel<2, 8> : (slots == 3 ? grad_stream_kernel<3, 4> : grad_stream_kernel<4, 4>));
         return {k, GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * ld * 4, 0, 0};
     }
-    // rows of up to 8,192 columns: 256 threads hold 1,024 columns, 512 threads 2,048 a chunk
-    static const GradTileKernel kernels[5] = {grad_wide_kernel<1, 256>, grad_wide_kernel<1, 512>, grad_wide_kernel<2, 512>, grad_wide_kernel<3, 512>,
-                                              grad_wide_kernel<4, 512>};
+    // rows of up to 2,048 columns: two groups of 256 threads that hold 1,024 columns a chunk; up to 8,192: 512 threads, 2,048 columns a chunk
+    static const GradTileKernel kernels[5] = {grad_wide_kernel<1, 256, 2>, grad_wide_kernel<2, 256, 2>, grad_wide_kernel<2, 512, 1>,
+                                              grad_wide_kernel<3, 512, 1>, grad_wide_kernel<4, 512, 1>};
     if (ld <= 8192) {
-        const int nc = (int)ceil_div(ld, 2048), rows = grad_wide_rows(nc);
-        return {kernels[ld <= 1024 ? 0 : nc], ld <= 1024 ? 256u : 512u, (size_t)grad_wide_stages(rows, (int)ld) * rows * ld * 4, 1, rows};
+        const int at = ld <= 1024 ? 0 : (ld <= 2048 ? 1 : (int)ceil_div(ld, 2048));
+        const int groups = at < 2 ? 2 : 1, rows = grad_wide_rows(at < 2 ? at + 1 : at);
+        return {kernels[at], 512u, (size_t)groups * grad_wide_stages(groups, rows, (int)ld) * rows * ld * 4, 1, rows};
     }
     return {grad_tiles_kernel, GRAD_BLOCK, 0, 0, 0};
 }

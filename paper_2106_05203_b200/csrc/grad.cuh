@@ -226,22 +226,25 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
 // through shared memory, one barrier), every warp forms the residuals, and rho_r a_r is added from the registers.  A block goes
 // through a long tile, so that few partials are written, and its rows arrive through a ring in shared memory: bulk copies, a row
 // each, that refill a stage as soon as the barrier shows that it has been taken into registers.
+// GROUPS groups of THREADS threads share a tile, batch by batch in turn, each with its own ring and barriers: on rows of up to 2,048 columns a
+// batch is a chain of latencies with little in it, and two of them overlap (50 x 930 x 1,038, 193 MB: a call of 17 iterations 1,433 us with
+// one group of 512 threads, 1,217 with two of 256; two blocks per SM with a second register buffer 1,252).
 // early: the rows (and labels, tile table and sampled row numbers) were complete before an earlier gradient kernel of the same call
 // passed its wait, so the ring is filled before this kernel waits for the one in front of it, while that selects and aggregates: up
 // to 160 KB per SM, 24 MB in all, arrive in time in which HBM and L2 would idle.  The first kernel of a call (early == 0) waits first,
 // and lets nothing behind it start before.
 // 20 x 300 x 5,001 (120 MB, more than stays in L2): 26.2 us with the next rows in a second register buffer, 24.2 through the ring,
-// 19.6 with the early start, of which HBM takes 15; 20 x 285 x 2,625: 13.2, 11.1; 20 x 208 x 1,463: 8.4, 6.0 (latencies: x, two to four
+// 19.6 with the early start, of which HBM takes 15; 20 x 285 x 2,625: 13.2, 11.1; 20 x 208 x 1,463: 8.4, 6.0 (one group; latencies: x, two to four
 // batches of 0.5 us, launch).
 constexpr int GRAD_WIDE_SMEM = 160 * 1024, GRAD_WIDE_MAX_STAGES = 8, GRAD_WIDE_SPINS = 1 << 22;
 __host__ __device__ constexpr int grad_wide_rows(int nc) { return nc == 1 ? 8 : (nc <= 3 ? 4 : 2); }
-__host__ __device__ inline int grad_wide_stages(int rows, int ld) {
-    const int fit = GRAD_WIDE_SMEM / (rows * ld * 4);
+__host__ __device__ inline int grad_wide_stages(int groups, int rows, int ld) {          // of a group
+    const int fit = GRAD_WIDE_SMEM / (groups * rows * ld * 4);
     return fit < GRAD_WIDE_MAX_STAGES ? fit : GRAD_WIDE_MAX_STAGES;
 }
 
-template <int NC, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1)
+template <int NC, int THREADS, int GROUPS>
+__global__ void __launch_bounds__(THREADS * GROUPS, 1)
 grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
                  const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                  double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
@@ -249,11 +252,12 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
     constexpr int RB = grad_wide_rows(NC), WARPS = THREADS / 32;
     constexpr int LOG_GROUP = RB == 8 ? 2 : (RB == 4 ? 3 : 4);                  // log2(32 / RB): lanes that end up with one row
     extern __shared__ __align__(128) unsigned char grad_smem[];
-    __shared__ float red[2][WARPS][RB];
-    __shared__ unsigned long long bars[GRAD_WIDE_MAX_STAGES];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ float red_sh[GROUPS][2][WARPS][RB];
+    __shared__ unsigned long long bars_sh[GROUPS][GRAD_WIDE_MAX_STAGES];
+    __shared__ double loss_sh[GROUPS];
+    const int group = threadIdx.x / THREADS, tid = threadIdx.x - group * THREADS, lane = tid & 31, warp = tid >> 5;       // within the group
     if (tid < GRAD_WIDE_MAX_STAGES)
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(bars + tid)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&bars_sh[group][tid])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -264,7 +268,10 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         pdl_trigger();
     }
     const RowTile t = tiles[blockIdx.x];
-    const int chunks = ld >> 2, batches = (t.rows + RB - 1) / RB, stages = grad_wide_stages(RB, ld);
+    const int chunks = ld >> 2, stages = grad_wide_stages(GROUPS, RB, ld);
+    const int batches = ((t.rows + RB - 1) / RB - group + GROUPS - 1) / GROUPS;             // of this group: `group`, `group` + GROUPS, ...
+    unsigned char* ring = grad_smem + (size_t)group * stages * RB * ld * 4;
+    unsigned long long* bars = bars_sh[group];
     const i64 lo = gather ? row_off[t.worker] : 0, m = gather ? row_off[t.worker + 1] - lo : 0;
     auto row_id = [&](int r) -> i64 {
         if (!gather) return t.row0 + r;
@@ -274,13 +281,13 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
     };
     // the first warp fetches batch b into `stage`, a lane per row
     auto fetch = [&](int b, int stage) {
-        const int r = b * RB + lane, bytes = ld * 4;
+        const int r0 = (b * GROUPS + group) * RB, r = r0 + lane, bytes = ld * 4;
         const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage);
-        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(min(RB, t.rows - b * RB) * bytes) : "memory");
+        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(min(RB, t.rows - r0) * bytes) : "memory");
         __syncwarp();
         if (lane < RB && r < t.rows)
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"((unsigned)__cvta_generic_to_shared(grad_smem) + (unsigned)((stage * RB + lane) * bytes)), "l"(A + row_id(r) * (i64)ld),
+                         ::"r"((unsigned)__cvta_generic_to_shared(ring) + (unsigned)((stage * RB + lane) * bytes)), "l"(A + row_id(r) * (i64)ld),
                            "r"(bytes), "r"(bar) : "memory");
     };
     if (warp == 0) for (int b = 0; b < min(stages, batches); ++b) fetch(b, b);
@@ -294,7 +301,7 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
     }
     double loss_acc = 0.0;
     // label of the row whose margin this lane ends up with, a batch ahead
-    auto label_of = [&](int b) { const int r = b * RB + (lane >> LOG_GROUP); return r < t.rows ? __ldg(y + row_id(r)) : 0.f; };
+    auto label_of = [&](int b) { const int r = (b * GROUPS + group) * RB + (lane >> LOG_GROUP); return r < t.rows ? __ldg(y + row_id(r)) : 0.f; };
     float next_label = label_of(0);
     int stage = 0;
     unsigned parity = 0u;
@@ -308,8 +315,8 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
             asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                          : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
         if (!ok) record_error(status, 5u /* EF21_ERR_TIMEOUT */);
-        const float4* rows = reinterpret_cast<const float4*>(grad_smem) + stage * RB * chunks;
-        const int left = t.rows - b * RB;
+        const float4* rows = reinterpret_cast<const float4*>(ring) + stage * RB * chunks;
+        const int left = t.rows - (b * GROUPS + group) * RB;
         float4 a[RB][NC];
         float pd[RB];
 #pragma unroll
@@ -329,8 +336,9 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         }
         const float zw = reduce_rows<RB>(pd, lane);             // this warp's part of the margin of row lane >> LOG_GROUP
         const int half = b & 1;
+        float (&red)[2][WARPS][RB] = red_sh[group];
         if ((lane & ((1 << LOG_GROUP) - 1)) == 0) red[half][warp][lane >> LOG_GROUP] = zw;
-        __syncthreads();
+        if (GROUPS == 1) __syncthreads(); else asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(THREADS) : "memory");
         if (warp == 0 && b + stages < batches) fetch(b + stages, stage);        // the rows are in registers
         float z = red[half][0][lane >> LOG_GROUP];
 #pragma unroll
@@ -353,15 +361,45 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         }
         if (++stage == stages) { stage = 0; parity ^= 1u; }
     }
+    if (loss_partial && warp == 0) {
+        loss_acc = warp_sum(loss_acc);
+        if (lane == 0) loss_sh[group] = loss_acc;
+    }
+    // the groups' sums in ascending order
+    if (GROUPS > 1) {
+        __syncthreads();                                        // nothing is in flight, and the rings are read
+        float4* sums = reinterpret_cast<float4*>(grad_smem);
+        for (int g = 1; g < GROUPS; ++g) {
+            if (group == g) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) { const int at = tid + c * THREADS; if (at < chunks) sums[at] = acc[c]; }
+            }
+            __syncthreads();
+            if (group == 0) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const int at = tid + c * THREADS;
+                    if (at < chunks) {
+                        const float4 o = sums[at];
+                        acc[c].x = __fadd_rn(acc[c].x, o.x); acc[c].y = __fadd_rn(acc[c].y, o.y);
+                        acc[c].z = __fadd_rn(acc[c].z, o.z); acc[c].w = __fadd_rn(acc[c].w, o.w);
+                    }
+                }
+            }
+            if (g + 1 < GROUPS) __syncthreads();
+        }
+    }
+    if (group != 0) return;
     float4* __restrict__ out = reinterpret_cast<float4*>(partial + (i64)blockIdx.x * ld);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         const int at = tid + c * THREADS;
         if (at < chunks) out[at] = acc[c];
     }
-    if (loss_partial && warp == 0) {
-        loss_acc = warp_sum(loss_acc);
-        if (lane == 0) loss_partial[blockIdx.x] = loss_acc;
+    if (loss_partial && tid == 0) {
+        double sum = 0.0;
+        for (int g = 0; g < GROUPS; ++g) sum += loss_sh[g];
+        loss_partial[blockIdx.x] = sum;
     }
 }
 
