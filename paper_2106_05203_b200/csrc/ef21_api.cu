@@ -98,11 +98,11 @@ double st_margin(double rank) { return 4.5 * std::sqrt(rank) + 4.0; }
 
 // The three sections every Top-k call needs (selection state, histogram, per-chunk counts); the
 // one-pass sections are absent.
-TopkLayout topk_layout_general(i64 batch, i64 d) {
+TopkLayout topk_layout_general(i64 batch, i64 d, bool counted = false) {
     TopkLayout L{};
     L.nchunks = (int)ceil_div(d, TK_CHUNK);
     size_t o = 0;
-    L.slow_count = o; o += align_up(4);                    // (in the same place for every batch: a handle's count runs on)
+    if (counted) { L.slow_count = o; o += align_up(4); }   // (in the same place for every batch: a handle's count runs on)
     L.state = o; o += align_up((size_t)batch * sizeof(TkState));
     L.hist = o; o += align_up((size_t)batch * TK_BINS * sizeof(unsigned));
     L.chunks = o; o += align_up((size_t)batch * (size_t)L.nchunks * sizeof(uint2));
@@ -112,7 +112,7 @@ TopkLayout topk_layout_general(i64 batch, i64 d) {
 }
 
 TopkLayout topk_layout(i64 batch, i64 d, i64 k) {
-    TopkLayout L = topk_layout_general(batch, d);
+    TopkLayout L = topk_layout_general(batch, d, fast_topk_eligible(d, k));
     size_t o = L.total;
     L.fast = fast_topk_eligible(d, k);
     if (L.fast) {
@@ -210,7 +210,7 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.gi = take((size_t)n * L.ld * 4);
     L.msg_idx = take((size_t)n * k * 4);
     L.msg_val = take((size_t)n * k * 4);
-    L.topk = take(std::max(L.tk.total, L.tk2.total));
+    L.topk = take(L.tk2.fast ? std::max(L.tk.total, L.tk2.total) : L.tk.total);
     L.agg_off = take((size_t)n * (L.agg_tiles + 1) * 4);
     L.eval_out = take(256);
     L.slots = take((size_t)2 * n * k * 8);
@@ -750,7 +750,7 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmo
     float* val_b = c->at<float>(c->L.msg2_val);
     unsigned long long* cuts = c->at<unsigned long long>(c->L.plus_cuts);       // [2][n]: Markov, plain
     PlusSums sums = {};
-    if (long_topk(c) && c->L.tk2.cap > 0) {
+    if (long_topk(c) && c->L.tk2.cap > 0 && 2 * c->n <= 65535) {            // (a batch of 2 n as one dimension of a grid)
         EF(enqueue_plus_select(c, a, pitch_a, cuts, sums));
     } else if (long_topk(c)) {
         const StOut om = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status(), cuts};

@@ -341,10 +341,11 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
 
     const int j0 = (int)min((i64)rank * p.slice, (i64)p.d), len = min(p.slice, p.d - j0);
     const bool few = C == 1 && !STREAM && p.k <= THREADS / 4 && p.d <= THREADS * tc_few_values(THREADS);
-    // (sixteen blocks: a share of a few dozen entries makes an uneven floor, and every exchange goes to sixteen: 4 x 452,034, Top-452, 29.2
-    // against 30.0 us a round)
+    // (Many blocks with a few entries each: their floors are uneven, the bisection in their tails is long, and a share of some ten entries per
+    // thread is counted quickly.  Rounds, us, with the histogram / this way: 4 x 452,034 Top-452 in sixteen blocks 29.2 / 30.0, 16 x 79,311
+    // Top-79 in eight 29.3 / 31.5; 20 x 116,750 Top-116 in four 24.9 / 22.9, 1 x 81,822 Top-818 in eight 16.2 / 14.0.)
     constexpr bool MAY_FEW = C > 1 && C <= 8 && !STREAM;
-    const bool few_cluster = MAY_FEW && p.k <= TC_FEW_OWN && (p.k + C - 1) / C <= THREADS / 5;
+    const bool few_cluster = MAY_FEW && p.k <= TC_FEW_OWN && (p.k + C - 1) / C <= THREADS / 5 && (C <= 4 || p.k >= 64 * C);
     unsigned largest = 0u;
     auto clear = [&]() {
 #pragma unroll 1
