@@ -21,6 +21,7 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include "bisect.cuh"
 #include "common.cuh"
 #include "grad.cuh"
 
@@ -124,14 +125,7 @@ __device__ __forceinline__ bool tc_few(const TcArgs& p, int vec, const unsigned*
     __syncthreads();
     unsigned floor = __reduce_min_sync(0xffffffffu, wmin[lane < WARPS ? lane : 0]);
     unsigned top = __reduce_max_sync(0xffffffffu, wmax[lane < WARPS ? lane : 0]);            // largest: of floor k or more are at or above it, of top + 1 none
-#pragma unroll 1
-    while (floor < top) {
-        const unsigned mid = floor + (top - floor + 1u) / 2u;
-        const int n = __syncthreads_count(largest >= mid);
-        if (n >= k) { floor = mid; if (n <= k + k / 4 + 4) break; }
-        else top = mid - 1u;
-    }
-    floor &= ~1u;                                                               // both signs of a magnitude
+    floor = bisect_floor(floor, top, k, [&](unsigned key) { return __syncthreads_count(largest >= key); }) & ~1u;      // both signs of a magnitude
     unsigned n = 0u;
 #pragma unroll
     for (int u = 0; u < NV; ++u) n += w[u] >= floor && tid + u * THREADS < p.d ? 1u : 0u;
@@ -210,13 +204,7 @@ __device__ __forceinline__ bool tc_few_cluster(const TcArgs& p, int vec, int ran
     unsigned floor = __reduce_min_sync(0xffffffffu, wmin[lane]), top = __reduce_max_sync(0xffffffffu, wmax[lane]);
     static_assert(WARPS == 32, "a lane per warp");
     if (tid == 0) top_sh = top;
-#pragma unroll 1
-    while (floor < top) {
-        const unsigned mid = floor + (top - floor + 1u) / 2u;
-        const int n = __syncthreads_count(largest >= mid);
-        if (n >= share) { floor = mid; if (n <= share + share / 4 + 4) break; }
-        else top = mid - 1u;
-    }
+    floor = bisect_floor(floor, top, share, [&](unsigned key) { return __syncthreads_count(largest >= key); });
     if (tid == 0) floor_sh = floor & ~1u;                                       // both signs of a magnitude
     cluster.sync();
     floor = 0xffffffffu; top = 0u;
