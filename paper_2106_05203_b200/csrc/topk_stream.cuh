@@ -105,7 +105,7 @@ st_sample_kernel(const __grid_constant__ StArgs p, float rank, float margin) {
 #pragma unroll
     for (int s = 0; s < PT; ++s) {
         const i64 j = ((i64)s * warps + w) * stride + lane;
-        key[s] = mag_key(st_value<MODE>(av[j], MODE == TC_PLAIN || second ? 0.f : bv[j], p.gamma));
+        key[s] = mag_key(second ? av[j] : st_value<MODE>(av[j], MODE == TC_PLAIN ? 0.f : bv[j], p.gamma));
     }
     // open histogram of this vector, for the streaming pass
     for (int q = rk * ST_SAMPLE_THREADS + tid; q < ST_OPEN_BINS; q += C * ST_SAMPLE_THREADS) p.open_hist[(i64)vec * ST_OPEN_BINS + q] = 0u;
@@ -495,7 +495,8 @@ st_collect_pair_kernel(const __grid_constant__ StArgs p, const __grid_constant__
             int4* out = p.cand + ((i64)vecs[s] * p.nreg + region) * p.cap;
 #pragma unroll 1
             for (unsigned e = lane; e < held[s]; e += 32u) {
-                const float a = sh.a[s][warp][e], g = s == 0 ? sh.g[warp][e] : 0.f, v = __fsub_rn(a, g);
+                const float a = sh.a[s][warp][e], g = s == 0 ? sh.g[warp][e] : 0.f;
+                const float v = s == 0 ? __fsub_rn(a, g) : a;                   // (a - 0 would change the bits, and so the order, of a NaN)
                 const int j = (int)base + sh.at[s][warp][e];
                 const unsigned key = mag_key(v);
                 if (done[s] + e < (unsigned)p.cap) out[done[s] + e] = make_int4(j, __float_as_int(v), __float_as_int(g), __float_as_int(a));
@@ -864,7 +865,7 @@ st_compact_kernel(const __grid_constant__ StArgs p, const StOut o) {
 }
 
 // The messages of EF21+ and the candidates' terms of the distortions; grid = (ceil(nreg / 32), 2 n), 256 threads, eight lanes per region.
-// A Markov record is (index, v, g, a), a plain one (index, a, g, a).
+// A Markov record is (index, v, g, a), a plain one (index, a, 0, a).
 __global__ void __launch_bounds__(256)
 st_compact_pair_kernel(const __grid_constant__ StArgs p, const __grid_constant__ PlusSums sums, int* idx_m, float* val_m, int* idx_b, float* val_b,
                        unsigned long long* cut_out, unsigned* status) {

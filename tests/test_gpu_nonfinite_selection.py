@@ -78,7 +78,7 @@ def test_initial_messages(n, d, k, kind, oracle32):
 
 
 @pytest.mark.parametrize("kind", KINDS)
-@pytest.mark.parametrize("n,d,k", [(3, 200, 2), (20, 70001, 700)])
+@pytest.mark.parametrize("n,d,k", [(3, 200, 2), (20, 70001, 700), (20, 262147, 2621), (19, 263168, 263)])
 def test_plus(n, d, k, kind):
     """EF21+, whose plain selection takes the gradients unchanged: one step behind two finite ones, against the multi-pass selection."""
     from paper_2106_05203_b200 import binding as B
