@@ -151,6 +151,12 @@ typedef void (*GradTileKernel)(const float*, const float*, const float*, const R
 // through a long tile, `resident` blocks per SM and `rows` rows at a time (0: short tiles, several per SM).
 struct GradPlan { GradTileKernel kernel; unsigned threads; size_t smem; int resident, rows; };
 
+template <int I>
+constexpr GradTileKernel wide_kernel() {
+    constexpr WideShape S = GRAD_WIDE_SHAPES[I];
+    return grad_wide_kernel<S.columns, S.threads, S.groups, S.rows>;
+}
+
 GradPlan grad_plan(i64 ld) {
     const i64 slots = (ld / 4 + 31) / 32;
     if (slots <= 4) {
@@ -159,13 +165,11 @@ GradPlan grad_plan(i64 ld) {
                                             : (slots == 2 ? grad_stream_kernel<2, 8> : (slots == 3 ? grad_stream_kernel<3, 4> : grad_stream_kernel<4, 4>));
         return {k, GRAD_STREAM_BLOCK, (size_t)(GRAD_STREAM_BLOCK / 32) * ld * 4, 0, 0};
     }
-    // rows of up to 2,048 columns: two groups of 256 threads that hold 1,024 columns a chunk; up to 8,192: 512 threads, 2,048 columns a chunk
-    static const GradTileKernel kernels[5] = {grad_wide_kernel<1, 256, 2>, grad_wide_kernel<2, 256, 2>, grad_wide_kernel<2, 512, 1>,
-                                              grad_wide_kernel<3, 512, 1>, grad_wide_kernel<4, 512, 1>};
     if (ld <= 8192) {
-        const int at = ld <= 1024 ? 0 : (ld <= 2048 ? 1 : (int)ceil_div(ld, 2048));
-        const int groups = at < 2 ? 2 : 1, rows = grad_wide_rows(at < 2 ? at + 1 : at);
-        return {kernels[at], 512u, (size_t)groups * grad_wide_stages(groups, rows, (int)ld) * rows * ld * 4, 1, rows};
+        static const GradTileKernel kernels[5] = {wide_kernel<0>(), wide_kernel<1>(), wide_kernel<2>(), wide_kernel<3>(), wide_kernel<4>()};
+        const int at = grad_wide_shape((int)ld);
+        const WideShape S = GRAD_WIDE_SHAPES[at];
+        return {kernels[at], (unsigned)(S.threads * S.groups), (size_t)S.groups * grad_wide_stages(S.groups, S.rows, (int)ld) * S.rows * ld * 4, 1, S.rows};
     }
     return {grad_tiles_kernel, GRAD_BLOCK, 0, 0, 0};
 }

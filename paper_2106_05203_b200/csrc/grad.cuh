@@ -15,6 +15,7 @@
 // are reproducible.
 #pragma once
 #include "common.cuh"
+#include "wide_ring.cuh"
 
 namespace ef21 {
 
@@ -236,20 +237,15 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
 // 20 x 300 x 5,001 (120 MB, more than stays in L2): 26.2 us with the next rows in a second register buffer, 24.2 through the ring,
 // 19.6 with the early start, of which HBM takes 15; 20 x 285 x 2,625: 13.2, 11.1; 20 x 208 x 1,463: 8.4, 6.0 (one group; latencies: x, two to four
 // batches of 0.5 us, launch).
-constexpr int GRAD_WIDE_SMEM = 160 * 1024, GRAD_WIDE_MAX_STAGES = 8, GRAD_WIDE_SPINS = 1 << 22;
-__host__ __device__ constexpr int grad_wide_rows(int nc) { return nc == 1 ? 8 : (nc <= 3 ? 4 : 2); }
-__host__ __device__ inline int grad_wide_stages(int groups, int rows, int ld) {          // of a group
-    const int fit = GRAD_WIDE_SMEM / (groups * rows * ld * 4);
-    return fit < GRAD_WIDE_MAX_STAGES ? fit : GRAD_WIDE_MAX_STAGES;
-}
+constexpr int GRAD_WIDE_SPINS = 1 << 22;
 
-template <int NC, int THREADS, int GROUPS>
+template <int NC, int THREADS, int GROUPS, int RB>
 __global__ void __launch_bounds__(THREADS * GROUPS, 1)
 grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
                  const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                  double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
                  const i64* __restrict__ row_off, unsigned* __restrict__ status, int early) {
-    constexpr int RB = grad_wide_rows(NC), WARPS = THREADS / 32;
+    constexpr int WARPS = THREADS / 32;
     constexpr int LOG_GROUP = RB == 8 ? 2 : (RB == 4 ? 3 : 4);                  // log2(32 / RB): lanes that end up with one row
     extern __shared__ __align__(128) unsigned char grad_smem[];
     __shared__ float red_sh[GROUPS][2][WARPS][RB];

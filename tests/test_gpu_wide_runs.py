@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 # d, n, rows, k: clusters of 8, 4, 2 and 1 forming blocks; k up to and beyond a quarter of 512 threads; tiles from one row on; up to 40
 # tiles per worker and more
 SHAPES = [(513, 3, 40, 5), (700, 2, 900, 7), (1025, 37, 500, 20), (2047, 75, 300, 128), (2048, 75, 160, 129), (2049, 9, 70, 1), (4100, 4, 700, 41),
-          (5001, 20, 900, 50), (6145, 40, 300, 60), (8192, 5, 333, 128)]
+          (5001, 20, 900, 50), (5121, 20, 900, 51), (6144, 9, 1500, 61), (6145, 40, 300, 60), (8192, 5, 333, 128)]
 
 
 def _workload(d, n, rows, k):
