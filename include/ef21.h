@@ -231,7 +231,8 @@ ef21_status ef21_eval(ef21_ctx* ctx, double* f, double* grad_norm2, double* G);
  *     ef21_set_state and call ef21_clear_status.  The standalone ef21_topk has no status word and does
  *     not check.
  *   EF21_ERR_TIMEOUT: a bounded wait of the persistent kernel expired (its clusters were not all
- *     running at once, e.g. another kernel of the process held SMs).  The blocks leave the iteration
+ *     running at once, e.g. another kernel of the process held SMs), or one of the gradient kernel of
+ *     rows of 513 to 8,192 columns for rows under way.  The blocks leave the iteration
  *     loop at different iterations, so the state (x, g, g_i, last messages) is unspecified afterwards:
  *     restore it with ef21_set_state, call ef21_clear_status, and use EF21_PATH_LAUNCHES if the
  *     device stays shared.
@@ -285,7 +286,8 @@ ef21_status ef21_clear_status(ef21_ctx* ctx);
 
 /* Self-check of the bounded device-side wait used by the persistent path: one thread spins
  * at most spin_limit (1 .. 2^24) times on a word that nothing writes, then records
- * EF21_ERR_TIMEOUT, which the next ef21_poll returns.  The device and the context stay usable. */
+ * EF21_ERR_TIMEOUT, which the next ef21_poll returns.  On a handle whose rows have 513 to 8,192 columns, one pass
+ * of its gradient kernel that gives up at its first wait goes with it.  The device and the context stay usable. */
 ef21_status ef21_selftest_bounded_wait(ef21_ctx* ctx, uint32_t spin_limit);
 
 /* Measuring aid: `steps` iterations of the persistent path's exchange skeleton for this handle's shape -- the

@@ -169,7 +169,7 @@ GradPlan grad_plan(i64 ld) {
         static const GradTileKernel kernels[5] = {wide_kernel<0>(), wide_kernel<1>(), wide_kernel<2>(), wide_kernel<3>(), wide_kernel<4>()};
         const int at = grad_wide_shape((int)ld);
         const WideShape S = GRAD_WIDE_SHAPES[at];
-        return {kernels[at], (unsigned)(S.threads * S.groups), (size_t)S.groups * grad_wide_stages(S.groups, S.rows, (int)ld) * S.rows * ld * 4, 1, S.rows};
+        return {kernels[at], (unsigned)(S.threads * S.groups), (size_t)grad_wide_smem_bytes(S, (int)ld), 1, S.rows};
     }
     return {grad_tiles_kernel, GRAD_BLOCK, 0, 0, 0};
 }
@@ -546,13 +546,13 @@ struct GradSource { int num_tiles, worker_tiles; size_t tiles, tile_begin; const
 
 GradSource full_source(const ef21_ctx* c) { return {c->num_tiles, c->worker_tiles, c->L.tiles, c->L.tile_begin, nullptr, 0}; }
 
-ef21_status launch_grad_tiles(ef21_ctx* c, const GradSource& G, bool with_loss, bool early = false) {
+ef21_status launch_grad_tiles(ef21_ctx* c, const GradSource& G, bool with_loss, bool early = false, bool stopped = false) {
     if (G.num_tiles == 0) return EF21_OK;
     const GradPlan P = grad_plan(c->L.ld);
-    if (P.resident) EF(allow_smem(reinterpret_cast<const void*>(P.kernel), GRAD_WIDE_SMEM));
+    if (P.resident) EF(allow_smem(reinterpret_cast<const void*>(P.kernel), GRAD_WIDE_SMEM + GRAD_WIDE_SUMS));
     CU(launch(P.kernel, dim3((unsigned)G.num_tiles), P.threads, P.smem, c->stream, 1, c->at<float>(c->L.A), c->at<float>(c->L.y), c->x(),
               c->at<RowTile>(G.tiles), (int)c->L.ld, c->objective, c->at<float>(c->L.partial),
-              with_loss ? c->at<double>(c->L.loss_partial) : nullptr, G.batch_dev, G.tau, c->at<i64>(c->L.row_off), c->status(), early ? 1 : 0));
+              with_loss ? c->at<double>(c->L.loss_partial) : nullptr, G.batch_dev, G.tau, c->at<i64>(c->L.row_off), c->status(), (early ? GRAD_WIDE_EARLY : 0) | (stopped ? GRAD_WIDE_STOPPED : 0)));
     c->launches += 1;
     return EF21_OK;
 }
@@ -1735,6 +1735,8 @@ ef21_status ef21_selftest_bounded_wait(ef21_ctx* c, uint32_t spin_limit) {
     CU(cudaMemsetAsync(c->at<unsigned long long>(c->L.slots), 0, 8, c->stream));
     CU(launch(bounded_wait_selftest_kernel, dim3(1), 1, 0, c->stream, 1, c->at<unsigned long long>(c->L.slots), c->status(), spin_limit));
     c->launches += 1;
+    // the gradient kernel of wide rows, as if its first wait had run out, with copies of rows under way (its partials are scratch)
+    if (c->shards_loaded && grad_plan(c->L.ld).resident) EF(launch_grad_tiles(c, full_source(c), false, false, true));
     CU(cudaGetLastError());
     return EF21_OK;
 }

@@ -237,20 +237,33 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
 // 20 x 300 x 5,001 (120 MB, more than stays in L2): 26.2 us with the next rows in a second register buffer, 24.2 through the ring,
 // 19.6 with the early start, of which HBM takes 15; 20 x 285 x 2,625: 13.2, 11.1; 20 x 208 x 1,463: 8.4, 6.0 (one group; latencies: x, two to four
 // batches of 0.5 us, launch).
+// A wait for rows that runs out is remembered: the group fetches and waits for nothing more, goes through its barriers, waits for what it has
+// under way and marks the block's partial by NaN.  stopped: as if the first one had.
 constexpr int GRAD_WIDE_SPINS = 1 << 22;
+enum { GRAD_WIDE_EARLY = 1, GRAD_WIDE_STOPPED = 2 };            // bits of `how`
+
+__device__ __forceinline__ void grad_wide_wait(unsigned long long* bar, unsigned parity, unsigned& ok) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(bar);
+    for (int spins = 0; spins < GRAD_WIDE_SPINS && !ok; ++spins)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(at), "r"(parity) : "memory");
+}
 
 template <int NC, int THREADS, int GROUPS, int RB>
 __global__ void __launch_bounds__(THREADS * GROUPS, 1)
 grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const float* __restrict__ x,
                  const RowTile* __restrict__ tiles, int ld, int objective, float* __restrict__ partial,
                  double* __restrict__ loss_partial, const int* __restrict__ gather, int gather_pitch,
-                 const i64* __restrict__ row_off, unsigned* __restrict__ status, int early) {
+                 const i64* __restrict__ row_off, unsigned* __restrict__ status, int how) {
     constexpr int WARPS = THREADS / 32;
     constexpr int LOG_GROUP = RB == 8 ? 2 : (RB == 4 ? 3 : 4);                  // log2(32 / RB): lanes that end up with one row
     extern __shared__ __align__(128) unsigned char grad_smem[];
     __shared__ float red_sh[GROUPS][2][WARPS][RB];
     __shared__ unsigned long long bars_sh[GROUPS][GRAD_WIDE_MAX_STAGES];
     __shared__ double loss_sh[GROUPS];
+    constexpr int RUNNING = 0x7fffffff;
+    const bool early = (how & GRAD_WIDE_EARLY) != 0;
+    int stop = (how & GRAD_WIDE_STOPPED) != 0 ? 0 : RUNNING;    // the batch whose rows this thread has not seen come
     const int group = threadIdx.x / THREADS, tid = threadIdx.x - group * THREADS, lane = tid & 31, warp = tid >> 5;       // within the group
     if (tid < GRAD_WIDE_MAX_STAGES)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&bars_sh[group][tid])) : "memory");
@@ -275,13 +288,14 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         if (pick < 0 || pick >= m) { record_error(status, 1u /* EF21_ERR_INVALID_ARG */); pick = 0; }
         return lo + pick;
     };
-    // the first warp fetches batch b into `stage`, a lane per row
+    // the first warp fetches batch b into `stage`, a lane per row; not behind a stop (settled below)
     auto fetch = [&](int b, int stage) {
         const int r0 = (b * GROUPS + group) * RB, r = r0 + lane, bytes = ld * 4;
         const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage);
-        if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(min(RB, t.rows - r0) * bytes) : "memory");
+        const bool go = b < stages || __all_sync(0xffffffffu, stop == RUNNING);
+        if (lane == 0 && go) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(min(RB, t.rows - r0) * bytes) : "memory");
         __syncwarp();
-        if (lane < RB && r < t.rows)
+        if (lane < RB && r < t.rows && go)
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"((unsigned)__cvta_generic_to_shared(ring) + (unsigned)((stage * RB + lane) * bytes)), "l"(A + row_id(r) * (i64)ld),
                            "r"(bytes), "r"(bar) : "memory");
@@ -305,12 +319,9 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
     for (int b = 0; b < batches; ++b) {
         const float label = next_label;
         next_label = label_of(b + 1);
-        const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage);
-        unsigned ok = 0u;
-        for (int spins = 0; spins < GRAD_WIDE_SPINS && !ok; ++spins)
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (!ok) record_error(status, 5u /* EF21_ERR_TIMEOUT */);
+        unsigned ok = stop != RUNNING;
+        grad_wide_wait(bars + stage, parity, ok);
+        if (!ok) stop = b;
         const float4* rows = reinterpret_cast<const float4*>(ring) + stage * RB * chunks;
         const int left = t.rows - (b * GROUPS + group) * RB;
         float4 a[RB][NC];
@@ -357,14 +368,24 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         }
         if (++stage == stages) { stage = 0; parity ^= 1u; }
     }
+    if (stop != RUNNING) {
+        record_error(status, 5u /* EF21_ERR_TIMEOUT */);
+        const float nan = __uint_as_float(0x7fffffffu);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[c] = make_float4(nan, nan, nan, nan);
+        loss_acc = (double)nan;
+    }
+    if (warp == 0 && __any_sync(0xffffffffu, stop != RUNNING)) {                // the refill of batch `stop` was the first to be left out
+        const int issued = min(batches, __reduce_min_sync(0xffffffffu, stop) + stages);
+        grad_wide_settle(issued, stages, [&](int at, unsigned of) { unsigned ok = 0u; grad_wide_wait(bars + at, of, ok); });
+    }
     if (loss_partial && warp == 0) {
         loss_acc = warp_sum(loss_acc);
         if (lane == 0) loss_sh[group] = loss_acc;
     }
     // the groups' sums in ascending order
     if (GROUPS > 1) {
-        __syncthreads();                                        // nothing is in flight, and the rings are read
-        float4* sums = reinterpret_cast<float4*>(grad_smem);
+        float4* sums = reinterpret_cast<float4*>(grad_smem + (size_t)GROUPS * stages * RB * ld * 4);
         for (int g = 1; g < GROUPS; ++g) {
             if (group == g) {
 #pragma unroll

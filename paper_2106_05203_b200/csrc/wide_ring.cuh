@@ -11,6 +11,7 @@
 namespace ef21 {
 
 constexpr int GRAD_WIDE_SMEM = 192 * 1024, GRAD_WIDE_MAX_STAGES = 8;      // of the rings, at most
+constexpr int GRAD_WIDE_SUMS = 8192;                                    // at most, of a second group
 
 // Threads per group, float4 columns per thread, groups of threads per block, rows a group takes at a time.
 struct WideShape { int threads, columns, groups, rows; };
@@ -26,6 +27,17 @@ EF21_WIDE_FN int grad_wide_shape(int ld) { return ld <= 1024 ? 0 : (ld <= 2048 ?
 EF21_WIDE_FN int grad_wide_stages(int groups, int rows, int ld) {
     const int batch = groups * rows * ld * 4, usual = 160 * 1024, fit = (2 * batch > usual ? GRAD_WIDE_SMEM : usual) / batch;
     return fit < GRAD_WIDE_MAX_STAGES ? fit : GRAD_WIDE_MAX_STAGES;
+}
+
+// Dynamic shared memory of a block: the rings, and behind them the sums of the groups other than the first (no copy of rows lands there).
+EF21_WIDE_FN int grad_wide_ring_bytes(const WideShape& s, int ld) { return s.groups * grad_wide_stages(s.groups, s.rows, ld) * s.rows * ld * 4; }
+EF21_WIDE_FN int grad_wide_smem_bytes(const WideShape& s, int ld) { return grad_wide_ring_bytes(s, ld) + (s.groups - 1) * ld * 4; }
+
+// A group that stops early must not leave copies on their way into shared memory that others get: wait(stage, parity) for the last batch of
+// every stage, of `issued` batches that went to the stages in turn.  (A wait for one that has been taken returns at once.)
+template <typename Wait>
+EF21_WIDE_FN void grad_wide_settle(int issued, int stages, Wait wait) {
+    for (int b = issued > stages ? issued - stages : 0; b < issued; ++b) wait(b % stages, (unsigned)(b / stages) & 1u);
 }
 
 }  // namespace ef21

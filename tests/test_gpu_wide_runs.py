@@ -49,6 +49,26 @@ def test_one_call_gives_the_bits_of_many(d, n, rows, k, variant):
         assert torch.equal(a.view(torch.int32), b.view(torch.int32))
 
 
+@pytest.mark.parametrize("d,n,rows,k", [SHAPES[1], SHAPES[4], (2049, 9, 7000, 1), (5001, 20, 9000, 50), (5121, 20, 9000, 51), (6145, 40, 3000, 60)])
+def test_a_gradient_kernel_that_gives_up_leaves_nothing_behind(d, n, rows, k, oracle32):
+    # its first copies of rows are under way when it stops; the kernels behind it get its shared memory
+    from paper_2106_05203_b200 import binding as B
+    w = _workload(d, n, rows, k)
+    h = make_gpu(w)
+    st = make_oracle_state(oracle32, w)
+    h.init(B.INIT_COMPRESSED)
+    st.init(0)
+    saved = h.get_state()[:3]
+    for _ in range(3):
+        h.selftest_bounded_wait(1)
+        h.step(1)
+    assert h.poll() == 5
+    h.set_state(*saved)
+    h.clear_status()
+    lockstep(h, st, oracle32, w, 2)
+    assert h.poll() == 0
+
+
 # blocks of 256, 512 and 1,024 threads: k at a quarter of them and one more, lengths at the values a thread holds
 @pytest.mark.parametrize("kind", ["gauss", "ties", "signs", "few nonzero", "zeros", "spread"])
 @pytest.mark.parametrize("batch,d,k", [(3, 7, 7), (3, 257, 64), (5, 2048, 64), (5, 2048, 65), (3, 2049, 128), (3, 8192, 128), (3, 8192, 129), (150, 8193, 256),
