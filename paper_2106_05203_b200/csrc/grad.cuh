@@ -289,10 +289,9 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         return lo + pick;
     };
     // the first warp fetches batch b into `stage`, a lane per row; not behind a stop (settled below)
-    auto fetch = [&](int b, int stage) {
+    auto fetch = [&](int b, int stage, bool go) {
         const int r0 = (b * GROUPS + group) * RB, r = r0 + lane, bytes = ld * 4;
         const unsigned bar = (unsigned)__cvta_generic_to_shared(bars + stage);
-        const bool go = b < stages || __all_sync(0xffffffffu, stop == RUNNING);
         if (lane == 0 && go) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(min(RB, t.rows - r0) * bytes) : "memory");
         __syncwarp();
         if (lane < RB && r < t.rows && go)
@@ -300,7 +299,7 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
                          ::"r"((unsigned)__cvta_generic_to_shared(ring) + (unsigned)((stage * RB + lane) * bytes)), "l"(A + row_id(r) * (i64)ld),
                            "r"(bytes), "r"(bar) : "memory");
     };
-    if (warp == 0) for (int b = 0; b < min(stages, batches); ++b) fetch(b, b);
+    if (warp == 0) for (int b = 0; b < min(stages, batches); ++b) fetch(b, b, true);
     if (early) pdl_wait(x, partial, loss_partial);
     float4 xr[NC], acc[NC];
 #pragma unroll
@@ -322,6 +321,7 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         unsigned ok = stop != RUNNING;
         grad_wide_wait(bars + stage, parity, ok);
         if (!ok) stop = b;
+        const bool go = __all_sync(0xffffffffu, stop == RUNNING);
         const float4* rows = reinterpret_cast<const float4*>(ring) + stage * RB * chunks;
         const int left = t.rows - (b * GROUPS + group) * RB;
         float4 a[RB][NC];
@@ -346,7 +346,7 @@ grad_wide_kernel(const float* __restrict__ A, const float* __restrict__ y, const
         float (&red)[2][WARPS][RB] = red_sh[group];
         if ((lane & ((1 << LOG_GROUP) - 1)) == 0) red[half][warp][lane >> LOG_GROUP] = zw;
         if (GROUPS == 1) __syncthreads(); else asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(THREADS) : "memory");
-        if (warp == 0 && b + stages < batches) fetch(b + stages, stage);        // the rows are in registers
+        if (warp == 0 && b + stages < batches) fetch(b + stages, stage, go);    // the rows are in registers
         float z = red[half][0][lane >> LOG_GROUP];
 #pragma unroll
         for (int w = 1; w < WARPS; ++w) z += red[half][w][lane >> LOG_GROUP];
