@@ -30,11 +30,14 @@
 // dense mean; whole-block body only), the original EF (Algorithm 4: the leader compresses e_i + gamma grad_i, the
 // messages move x directly) and the exchange skeleton (a measuring aid).  This header holds what they share.
 //
-// A launch loads its rows (and the shards' offsets and labels) before it waits for the kernel in front of it, as a rule the one that
-// forms the initial g.  They are complete by then whatever that kernel is: loading shards ends with copies of the offsets, which are no
+// Rows (and the shards' offsets and labels) may be loaded in front of the wait for the kernel before, as a rule the one that forms the
+// initial g.  They are complete by then whatever that kernel is: loading shards ends with copies of the offsets, which are no
 // programmatic dependents and have none, so that every kernel behind them starts after they, and the kernel that wrote the rows,
-// have ended.  The state and the lists of sampled rows are read behind the wait.  (1 to 3 us of a call: 20 x 2,487 x 300, 50 iterations,
-// 557 -> 549 us, 20 x 406 x 112, 100 iterations, 272 -> 270.)
+// have ended.  The state and the lists of sampled rows are read behind the wait.  Which comes first, by measurement (us a call, state first and
+// rows first): one cluster, rows first (4 x 50 x 64, 100 iterations, 229.2, 225.8; a ring is filled behind the state); many
+// clusters, rows to shared memory first (100 x 200 x 200, 50 iterations, 308.4, 304.7), rows to registers last and the wait in front of
+// everything: the loop behind it comes out slower otherwise (20 x 406 x 112, 100 iterations, 277.7, 283.4; 20 x 1,628 x 123 Top-16,
+// 50 iterations, 250.6, 253.5, Algorithm 4 229.6, 233.6), though the shortest calls lose by it (5 x 616 x 211, 12 iterations, 64.3, 61.9).
 //
 // All summation orders are fixed by the launch shape, so two runs give identical bits.  A wait
 // that exceeds its spin limit records EF21_ERR_TIMEOUT in the status word; from then on every
