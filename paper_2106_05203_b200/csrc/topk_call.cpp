@@ -20,6 +20,12 @@ WorkspaceBytes workspace_bytes = nullptr;
 Topk topk_entry = nullptr;
 constexpr size_t ALIGN = 256;
 
+// Allocation and launch can wait for the device (a full launch queue, memory given back to the driver): not with the interpreter held.
+struct Released {
+    PyThreadState* state = PyEval_SaveThread();
+    ~Released() { PyEval_RestoreThread(state); }
+};
+
 // topk(v, k) -> (idx, val), the library's status where it refuses, or None where the call is not one of the usual ones.
 PyObject* topk(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     HANDLE_TH_ERRORS
@@ -32,17 +38,25 @@ PyObject* topk(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
     int overflow = 0;
     const long long k = PyLong_AsLongLongAndOverflow(args[1], &overflow);
     if (overflow || k < 1 || k > d || k > INT32_MAX || batch < 1 || batch > 65535) Py_RETURN_NONE;
-    const size_t bytes = workspace_bytes((int32_t)batch, d, (int32_t)k);
-    if (bytes == 0) Py_RETURN_NONE;
-    const at::TensorOptions here = at::TensorOptions().device(v.device());
-    at::Tensor idx = at::empty({batch, k}, here.dtype(at::kInt)), val = at::empty({batch, k}, here.dtype(at::kFloat)), ws;
-    void* scratch = idx.data_ptr();                     // up to ALIGN bytes: checked, not used
-    if (bytes > ALIGN || reinterpret_cast<uintptr_t>(scratch) % ALIGN != 0) {
-        ws = at::empty({(int64_t)(bytes + ALIGN)}, here.dtype(at::kByte));
-        scratch = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws.data_ptr()) + ALIGN - 1) / ALIGN * ALIGN);
+    at::Tensor idx, val;
+    int status = 0;
+    {
+        const Released released;
+        const size_t bytes = workspace_bytes((int32_t)batch, d, (int32_t)k);
+        if (bytes != 0) {
+            const at::TensorOptions here = at::TensorOptions().device(v.device());
+            idx = at::empty({batch, k}, here.dtype(at::kInt)); val = at::empty({batch, k}, here.dtype(at::kFloat));
+            at::Tensor ws;
+            void* scratch = idx.data_ptr();                 // up to ALIGN bytes: checked, not used
+            if (bytes > ALIGN || reinterpret_cast<uintptr_t>(scratch) % ALIGN != 0) {
+                ws = at::empty({(int64_t)(bytes + ALIGN)}, here.dtype(at::kByte));
+                scratch = reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws.data_ptr()) + ALIGN - 1) / ALIGN * ALIGN);
+            }
+            status = topk_entry(static_cast<const float*>(v.data_ptr()), (int32_t)batch, d, (int32_t)k, static_cast<int32_t*>(idx.data_ptr()),
+                                static_cast<float*>(val.data_ptr()), scratch, bytes, c10::cuda::getCurrentCUDAStream(v.get_device()).stream());
+        }
     }
-    const int status = topk_entry(static_cast<const float*>(v.data_ptr()), (int32_t)batch, d, (int32_t)k, static_cast<int32_t*>(idx.data_ptr()),
-                                  static_cast<float*>(val.data_ptr()), scratch, bytes, c10::cuda::getCurrentCUDAStream(v.get_device()).stream());
+    if (!idx.defined()) Py_RETURN_NONE;
     if (status != 0) return PyLong_FromLong(status);
     PyObject* out = PyTuple_New(2);
     if (!out) return nullptr;

@@ -1,4 +1,11 @@
 """topk() by its native call and by the general one: the same results and the same refusals."""
+import ctypes
+import importlib.util
+import os
+import shutil
+import subprocess
+import threading
+
 import pytest
 import torch
 
@@ -53,3 +60,42 @@ def test_refusals(B):
     batched = torch.func.vmap(lambda r: B.topk(r, 3)[1])
     with pytest.raises(RuntimeError):
         batched(v)
+
+
+# an entry that comes back when another thread has set `seen`, with an error after two seconds
+WAITING_ENTRY = """
+#include <stddef.h>
+#include <stdint.h>
+#include <unistd.h>
+extern "C" { volatile int entered = 0, seen = 0; }
+extern "C" size_t bytes(int32_t, int64_t, int32_t) { return 64; }
+extern "C" int entry(const float*, int32_t, int64_t, int32_t, int32_t*, float*, void*, size_t, void*) {
+    entered = 1;
+    for (int ms = 0; ms < 2000 && !seen; ++ms) usleep(1000);
+    return seen ? 0 : 4;
+}
+"""
+
+
+def test_other_threads_run_while_the_call_waits(B, tmp_path):
+    (tmp_path / "entry.cpp").write_text(WAITING_ENTRY)
+    subprocess.run([os.environ.get("CXX", "g++"), "-shared", "-fPIC", str(tmp_path / "entry.cpp"), "-o", str(tmp_path / "entry.so")], check=True)
+    lib = ctypes.CDLL(str(tmp_path / "entry.so"))
+    path = str(tmp_path / "_topk_call.so")                  # a copy, whose entry points are its own
+    shutil.copy(os.path.join(os.path.dirname(B.__file__), "_topk_call.so"), path)
+    spec = importlib.util.spec_from_file_location("_topk_call", path)
+    module = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(module)
+    module.set_entry(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.bytes, lib.entry)))
+    entered, seen = ctypes.c_int.in_dll(lib, "entered"), ctypes.c_int.in_dll(lib, "seen")
+
+    def other():
+        while not entered.value:
+            pass
+        seen.value = 1
+
+    thread = threading.Thread(target=other)
+    thread.start()
+    out = module.topk(torch.randn(2, 100, device="cuda"), 3)
+    thread.join()
+    assert type(out) is tuple
