@@ -11,13 +11,17 @@ import ctypes
 import functools
 import importlib.util
 import os
+import warnings
 from typing import Optional, Tuple
 
 import numpy as np
 import torch
 
+from .build import call_built_for
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libef21.so")
+CALL_PATH = os.path.join(_HERE, "_topk_call.so")
 
 EF21_OK = 0
 STATUS_NAMES = {0: "EF21_OK", 1: "EF21_ERR_INVALID_ARG", 2: "EF21_ERR_STATE", 3: "EF21_ERR_WORKSPACE",
@@ -93,14 +97,18 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     return lib
 
 
-def _load_call():
-    """The native form of topk() for the usual arguments (csrc/topk_call.cpp)."""
-    path = os.path.join(_HERE, "_topk_call.so")
-    if not os.path.exists(path):
-        raise ImportError(f"{path} is missing: build it with `python -m paper_2106_05203_b200.build`")
-    spec = importlib.util.spec_from_file_location("_topk_call", path)
-    module = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(module)
+def _load_call(path: str = CALL_PATH):
+    """The native form of topk() for the usual arguments (csrc/topk_call.cpp).  Where it is missing or does not fit this torch, every
+    call of topk() is the general one, 4 us slower on short vectors."""
+    try:
+        spec = importlib.util.spec_from_file_location("_topk_call", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        if module.built_for != call_built_for():
+            raise ImportError(f"{path} was built for {module.built_for}, this is {call_built_for()}")
+    except (ImportError, OSError, AttributeError) as e:
+        warnings.warn(f"topk() without its native call ({e}): build it with `python -m paper_2106_05203_b200.build`", RuntimeWarning, stacklevel=2)
+        return lambda v, k: None
     module.set_entry(*(ctypes.cast(f, _vp).value for f in (_lib.ef21_topk_workspace_bytes, _lib.ef21_topk)))
     return module.topk
 

@@ -31,8 +31,22 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+def call_built_for() -> str:
+    """What _topk_call.so depends on beside its source; the module carries it as `built_for`."""
+    import sysconfig
+    import torch
+    return f"torch {torch.__version__}, {sysconfig.get_config_var('SOABI')}"
+
+
+def _call_is_current() -> bool:
+    if not os.path.exists(CALL) or os.path.getmtime(CALL) < os.path.getmtime(CALL_SOURCE):
+        return False
+    with open(CALL, "rb") as f:
+        return call_built_for().encode() + b"\0" in f.read()
+
+
 def build_call(force: bool = False) -> str:
-    if not force and os.path.exists(CALL) and os.path.getmtime(CALL) >= os.path.getmtime(CALL_SOURCE):
+    if not force and _call_is_current():
         return CALL
     import sysconfig
     import torch
@@ -40,7 +54,7 @@ def build_call(force: bool = False) -> str:
     cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc_path())), "include")
     include = [sysconfig.get_paths()["include"], *cpp_extension.include_paths(), cuda]
     tmp = CALL + f".tmp{os.getpid()}"
-    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f'-DEF21_BUILT_FOR="{call_built_for()}"',
                     f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{i}" for i in include), CALL_SOURCE,
                     *(f"-L{p}" for p in cpp_extension.library_paths()), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
                     "-o", tmp], check=True)         # (found by name at run time: the import of torch has loaded them)

@@ -81,4 +81,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_topk_call", nullptr, -1, methods,
 
 }  // namespace
 
-extern "C" __attribute__((visibility("default"))) PyObject* PyInit__topk_call() { return PyModule_Create(&module); }
+// EF21_BUILT_FOR: the torch and the interpreter that this was compiled against (build.py), which are looked at before the module is used
+extern "C" __attribute__((visibility("default"))) PyObject* PyInit__topk_call() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", EF21_BUILT_FOR) != 0) { Py_DECREF(m); return nullptr; }
+    return m;
+}
