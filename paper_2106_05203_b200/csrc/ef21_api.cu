@@ -198,7 +198,10 @@ struct Layout {
     size_t A, y, row_off, tile_begin, tiles, partial, loss_partial, grad, mb_tile_begin, mb_tiles;
     size_t total;
     TopkLayout tk, tk2;                   // of n vectors; of the 2 n vectors of EF21+ (the same memory)
+    bool pair;                            // EF21+ selects from 2 n vectors in one pass; else tk2 takes no part
 };
+
+bool fits_clusters(i64 batch, i64 d);     // (tc_shape)
 
 Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     Layout L;
@@ -206,6 +209,7 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.agg_tiles = (int)ceil_div(d, AGG_TILE);
     L.tk = topk_layout(n, d, k);
     L.tk2 = topk_layout(2 * n, d, k);
+    L.pair = L.tk2.fast && L.tk2.cap > 0 && 2 * n <= 65535 && !fits_clusters(n, d);          // (a batch of 2 n as one dimension of a grid)
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o += align_up(bytes); return at; };
     L.status = take(256);
@@ -214,7 +218,7 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.gi = take((size_t)n * L.ld * 4);
     L.msg_idx = take((size_t)n * k * 4);
     L.msg_val = take((size_t)n * k * 4);
-    L.topk = take(L.tk2.fast ? std::max(L.tk.total, L.tk2.total) : L.tk.total);
+    L.topk = take(L.pair ? std::max(L.tk.total, L.tk2.total) : L.tk.total);
     L.agg_off = take((size_t)n * (L.agg_tiles + 1) * 4);
     L.eval_out = take(256);
     L.slots = take((size_t)2 * n * k * 8);
@@ -224,9 +228,9 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.plus_choice = take((size_t)n * 4);
     L.plus_parts = take((size_t)n * PLUS_MAX_PARTS * sizeof(double2));
     L.plus_pitch = (int)std::max<i64>(1, 148 * 4 / n);         // blocks per worker: four per SM in one wave
-    L.plus_low = take(L.tk2.fast ? (size_t)n * L.plus_pitch * sizeof(double2) : 0);
-    L.plus_nonzero = take(L.tk2.fast ? (size_t)n * L.plus_pitch * 4 : 0);
-    L.plus_cand = take(L.tk2.fast ? (size_t)2 * n * ceil_div(L.tk2.nreg, 32) * 8 : 0);
+    L.plus_low = take(L.pair ? (size_t)n * L.plus_pitch * sizeof(double2) : 0);
+    L.plus_nonzero = take(L.pair ? (size_t)n * L.plus_pitch * 4 : 0);
+    L.plus_cand = take(L.pair ? (size_t)2 * n * ceil_div(L.tk2.nreg, 32) * 8 : 0);
     L.tile_rows = 0; L.max_tiles = 0;
     L.A = L.y = L.row_off = L.tile_begin = L.tiles = L.partial = L.loss_partial = L.grad = L.mb_tile_begin = L.mb_tiles = 0;
     if (N > 0) {
@@ -369,6 +373,8 @@ bool tc_shape(i64 batch, i64 d, TcShape& S) {
     S.threads = C == 1 && d <= 2048 ? 256 : (C == 1 && d <= 8192 ? 512 : 1024);
     return true;
 }
+
+bool fits_clusters(i64 batch, i64 d) { TcShape S; return tc_shape(batch, d, S); }
 
 typedef void (*TcKernel)(const TcArgs);
 template <int MODE>
@@ -754,7 +760,7 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmo
     float* val_b = c->at<float>(c->L.msg2_val);
     unsigned long long* cuts = c->at<unsigned long long>(c->L.plus_cuts);       // [2][n]: Markov, plain
     PlusSums sums = {};
-    if (long_topk(c) && c->L.tk2.cap > 0 && 2 * c->n <= 65535) {            // (a batch of 2 n as one dimension of a grid)
+    if (long_topk(c) && c->L.pair) {
         EF(enqueue_plus_select(c, a, pitch_a, cuts, sums));
     } else if (long_topk(c)) {
         const StOut om = {c->msg_idx(), c->msg_val(), nullptr, 0, nullptr, 0, c->status(), cuts};

@@ -71,3 +71,12 @@ def test_host_side_argument_checks(lib):
     assert h.value is None
     lib.ef21_destroy.argtypes = [ctypes.c_void_p]
     lib.ef21_destroy(None)
+
+
+@pytest.mark.parametrize("n,d,k,mib", [(40, 200000, 90000, 197), (64, 1000003, 300000, 977), (40, 200000, 25000, 84), (16, 300000, 300, 26), (37, 131072, 1310, 32)])
+def test_no_memory_for_a_route_that_is_not_taken(lib, n, d, k, mib):
+    # EF21+ selects from 2 n vectors in one pass only where n vectors do not fit into clusters and at most a tenth of the entries is wanted;
+    # elsewhere the sections of the one-pass selection are those of n vectors (of 2 n: 251, 1,115, 105, 31 and 42 MiB)
+    lib.ef21_workspace_bytes.restype = ctypes.c_size_t
+    lib.ef21_workspace_bytes.argtypes = [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32, ctypes.c_int64]
+    assert lib.ef21_workspace_bytes(n, d, k, 0) <= mib << 20
