@@ -38,7 +38,9 @@ constexpr int TC_MAX_SLICE = 47104;         // floats per block (184 KB)
 // first half of the batch is a - b, the second half the same a once more.
 enum { TC_PLAIN = 0, TC_DIFF = 1, TC_EF = 2, TC_SENT = 3, TC_PAIR = 4 };
 
-template <bool V> struct TcFlag { static constexpr bool value = V; };
+// What a sweep does with an entry beside keeping it: count it, take the thread's largest, nothing.
+enum { TC_COUNT = 0, TC_LARGEST = 1, TC_KEEP = 2 };
+template <int V> struct TcUse { static constexpr int value = V; };
 
 struct TcArgs {
     const float* a; i64 pitch_a;
@@ -97,7 +99,7 @@ __device__ __noinline__ void tc_find_bin(const unsigned* hist, unsigned need, un
     __syncthreads();
 }
 
-// Few entries (k <= THREADS / 4) of a vector that one block holds, NV per thread: at least k threads have an entry at or above the k-th
+// Few entries (few_limit: a quarter of the threads at most) of a vector that one block holds, NV per thread: at least k threads have an entry at or above the k-th
 // largest of the threads' largest ones.  A floor with k to 5/4 k + 4 of these above it is found by bisection (a barrier that counts per
 // step, six to eight steps between the smallest and the greatest of them); the message is among the entries from the floor on, about 5/4 k
 // again as a rule, which are ranked one against the other, two to eight lanes per entry.  No histogram, no sweep for the compaction.
@@ -328,12 +330,14 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     auto sync_all = [&]() { if (C > 1) cluster.sync(); else __syncthreads(); };
 
     const int j0 = (int)min((i64)rank * p.slice, (i64)p.d), len = min(p.slice, p.d - j0);
-    const bool few = C == 1 && !STREAM && p.k <= THREADS / 4 && p.d <= THREADS * tc_few_values(THREADS);
+    const bool few = C == 1 && !STREAM && p.d <= THREADS * tc_few_values(THREADS) &&
+                     p.k <= few_limit(THREADS, p.d, gridDim.x <= 148u * (GRAD > 1 ? GRAD : 1), GRAD > 0);
     // (Many blocks with a few entries each: their floors are uneven, the bisection in their tails is long, and a share of some ten entries per
     // thread is counted quickly.  Rounds, us, with the histogram / this way: 4 x 452,034 Top-452 in sixteen blocks 29.2 / 30.0, 16 x 79,311
-    // Top-79 in eight 29.3 / 31.5; 20 x 116,750 Top-116 in four 24.9 / 22.9, 1 x 81,822 Top-818 in eight 16.2 / 14.0.)
+    // Top-79 in eight 29.3 / 31.5; 20 x 116,750 Top-116 in four 24.9 / 22.9, 1 x 81,822 Top-818 in eight 16.2 / 14.0.  Eight rounds: 37 x 60,000 in four
+    // Top-10 210 / 226, Top-60 241 / 243, Top-200 323 / 300; 70 x 30,000 in two Top-8 150 / 158, Top-30 169 / 172, Top-100 301 / 294.)
     constexpr bool MAY_FEW = C > 1 && C <= 8 && !STREAM;
-    const bool few_cluster = MAY_FEW && p.k <= TC_FEW_OWN && (p.k + C - 1) / C <= THREADS / 5 && (C <= 4 || p.k >= 64 * C);
+    const bool few_cluster = MAY_FEW && p.k <= TC_FEW_OWN && (p.k + C - 1) / C <= THREADS / 5 && p.k >= (C <= 4 ? 20 : 64) * C;
     unsigned largest = 0u;
     auto clear = [&]() {
 #pragma unroll 1
@@ -357,8 +361,8 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     float* bv = MODE == TC_PLAIN ? nullptr : p.b + (i64)vec * p.pitch_b + j0;
     float* dense = MODE == TC_PLAIN && !STREAM && p.apply ? p.apply + (i64)vec * p.pitch_apply + j0 : nullptr;
     // entries of bin 0 (zeros and the smallest magnitudes) are not counted: what the other bins leave over is theirs
-    auto count = [&](unsigned w) { if (!few && (w >> 21)) atomicAdd(&hist[w >> 21], 1u); };
-    auto take = [&](int j, float a, float b, auto only_largest) {
+    auto count = [&](unsigned w) { if (w >> 21) atomicAdd(&hist[w >> 21], 1u); };
+    auto take = [&](int j, float a, float b, auto use) {
         float v = a;
         if (MODE == TC_DIFF) v = __fsub_rn(a, b);
         if (MODE == TC_EF) { v = __fadd_rn(b, __fmul_rn(p.gamma, a)); bv[j] = v; }
@@ -367,10 +371,9 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         if (MODE == TC_PLAIN && dense) dense[j] = 0.f;
         if (GRAD > 1) { cluster.map_shared_rank(ws, 0)[j] = w; return; }
         if (!STREAM) ws[j] = w;
-        if (decltype(only_largest)::value) largest = max(largest, w);
-        else count(w);
+        if (decltype(use)::value == TC_LARGEST) largest = max(largest, w);
+        if (decltype(use)::value == TC_COUNT) count(w);
     };
-    const TcFlag<false> all_counted;
     if (GRAD > 0) {
         const i64 m = p.batch_rows > 0 ? (i64)p.batch_rows : m_all;
         const int share = GRAD > 1 ? (len + GRAD - 1) / GRAD : len;
@@ -419,8 +422,8 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
                 for (int q = 1; q < Q; ++q) acc[u][0] = __fadd_rn(acc[u][0], acc[u][q]);
                 g[u] = __fadd_rn(m > 0 ? __fdiv_rn(acc[u][0], (float)m) : 0.f, regulariser_grad(p.lambda, xj[u]));
             }
-            take(js[0], g[0], b[0], all_counted);
-            if (jj + THREADS < c1) take(js[1], g[1], b[1], all_counted);
+            auto both = [&](auto use) { take(js[0], g[0], b[0], use); if (jj + THREADS < c1) take(js[1], g[1], b[1], use); };
+            if (few) both(TcUse<TC_KEEP>()); else both(TcUse<TC_COUNT>());
         }
         // Behind the aggregation waits grad_wide_kernel, which fetches rows as soon as it is placed: not before this kernel's own
         // loads are through (20 x 5,001: 38.4 us an iteration instead of 39.4).
@@ -432,7 +435,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         }
     } else {
         constexpr int U = THREADS == 1024 ? 8 : 4;
-        auto sweep = [&](auto only_largest) {
+        auto sweep = [&](auto use) {
             int j = tid;
 #pragma unroll 1
             for (; j + (U - 1) * THREADS < len; j += U * THREADS) {
@@ -440,12 +443,14 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) { a[u] = MODE == TC_SENT ? 0.f : av[j + u * THREADS]; b[u] = MODE == TC_PLAIN ? 0.f : bv[j + u * THREADS]; }
 #pragma unroll
-                for (int u = 0; u < U; ++u) take(j + u * THREADS, a[u], b[u], only_largest);
+                for (int u = 0; u < U; ++u) take(j + u * THREADS, a[u], b[u], use);
             }
 #pragma unroll 1
-            for (; j < len; j += THREADS) take(j, MODE == TC_SENT ? 0.f : av[j], MODE == TC_PLAIN ? 0.f : bv[j], only_largest);
+            for (; j < len; j += THREADS) take(j, MODE == TC_SENT ? 0.f : av[j], MODE == TC_PLAIN ? 0.f : bv[j], use);
         };
-        if (MAY_FEW && few_cluster) sweep(TcFlag<MAY_FEW>()); else sweep(all_counted);
+        if (MAY_FEW && few_cluster) sweep(TcUse<MAY_FEW ? TC_LARGEST : TC_COUNT>());
+        else if (C == 1 && few) sweep(TcUse<C == 1 ? TC_KEEP : TC_COUNT>());
+        else sweep(TcUse<TC_COUNT>());
     }
     constexpr int OWN = TC_BINS / C;                                // bins summed by one block
     auto sum_histograms = [&]() {                                   // hist of all blocks -> hsum
@@ -709,8 +714,9 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     }
 }
 
+// (512 threads: left alone the compiler takes 40 registers; ten rounds of 20 x 8,192 Top-128 158.7 us with these, 149.5 with 56.)
 template <int MODE, int C, int THREADS, bool STREAM = false, int GRAD = 0>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, THREADS == 512 && GRAD == 0 ? 2 : 0)
 tc_topk_kernel(const __grid_constant__ TcArgs p) {
     if (STREAM) {
         // a few clusters look through the flags: as a rule there is nothing to do

@@ -24,6 +24,7 @@ extern "C" int search(const unsigned* keys, int n, int need, unsigned floor, uns
     } catch (Endless) { return -1; }
     return counts;
 }
+extern "C" int limit(int threads, int d, int alone, int grad) { return ef21::few_limit(threads, d, alone, grad); }
 extern "C" unsigned middle(unsigned floor, unsigned top) { return ef21::bisect_middle(floor, top); }
 """
 
@@ -85,3 +86,16 @@ def test_search_ends_and_its_floor_holds(lib, kind, top_key):
             assert reach >= need, (n, need)
             if reach > need + need // 4 + 4:              # ties: nothing above has enough
                 assert out.value == 0xffffffff or int((keys > np.uint32(out.value)).sum()) < need, (n, need)
+
+
+@pytest.mark.parametrize("threads,first,last", [(256, 1, 2048), (512, 2049, 8192), (512, 513, 8192), (1024, 8193, 16384)])
+def test_limit_of_few_entries(lib, threads, first, last):
+    """Never more than a quarter of the threads (more of them need not have an entry to count), and not where a histogram was measured to be
+    faster: many vectors, us with it and without, in bisect.cuh."""
+    for d in range(first, last + 1):
+        for grad in (0, 1):
+            crowded, alone = lib.limit(threads, d, 0, grad), lib.limit(threads, d, 1, grad)
+            assert 1 <= crowded <= alone <= threads // 4
+    for slower in ((1024, 16384, 0, 0, 192), (1024, 9000, 0, 0, 128), (512, 8192, 0, 0, 112), (512, 2100, 0, 0, 64), (256, 2048, 0, 0, 64), (256, 300, 0, 0, 32),
+                   (1024, 9000, 1, 0, 192), (512, 8192, 1, 0, 128), (512, 4000, 1, 0, 96), (256, 1000, 1, 0, 64), (512, 1500, 1, 1, 128)):
+        assert lib.limit(*slower[:4]) < slower[4]

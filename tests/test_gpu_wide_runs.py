@@ -72,7 +72,8 @@ def test_a_gradient_kernel_that_gives_up_leaves_nothing_behind(d, n, rows, k, or
 # blocks of 256, 512 and 1,024 threads: k at a quarter of them and one more, lengths at the values a thread holds
 @pytest.mark.parametrize("kind", ["gauss", "ties", "signs", "few nonzero", "zeros", "spread"])
 @pytest.mark.parametrize("batch,d,k", [(3, 7, 7), (3, 257, 64), (5, 2048, 64), (5, 2048, 65), (3, 2049, 128), (3, 8192, 128), (3, 8192, 129), (150, 8193, 256),
-                                       (150, 16384, 256), (150, 16384, 257), (150, 16385, 20), (2, 5000, 1)])
+                                       (150, 16384, 256), (150, 16384, 257), (150, 16385, 20), (2, 5000, 1), (3, 8192, 118), (3, 8192, 119),
+                                       (150, 16384, 155), (150, 16384, 156), (3, 300, 32), (3, 300, 33)])
 def test_few_entries_of_short_vectors(batch, d, k, kind, oracle32):
     from paper_2106_05203_b200 import binding as B
     rng = np.random.default_rng(d + k)
@@ -98,6 +99,7 @@ def test_few_entries_of_short_vectors(batch, d, k, kind, oracle32):
 # share (more candidates than it lists), ties at the cut in several blocks
 @pytest.mark.parametrize("kind", ["gauss", "ties", "signs", "layers", "bf16", "few nonzero"])
 @pytest.mark.parametrize("batch,d,k", [(1, 16384, 1), (40, 16385, 408), (3, 65537, 700), (20, 70001, 816), (20, 70001, 817), (2, 94209, 1024), (2, 376833, 1024),
+                                       (70, 30000, 39), (70, 30000, 40), (37, 60000, 79), (37, 60000, 80),
                                        (1, 376833, 1025), (1, 753664, 753)])
 def test_few_entries_in_a_cluster(batch, d, k, kind, oracle32):
     from paper_2106_05203_b200 import binding as B
