@@ -201,7 +201,7 @@ struct Layout {
     bool pair;                            // EF21+ selects from 2 n vectors in one pass; else tk2 takes no part
 };
 
-bool fits_clusters(i64 batch, i64 d);     // (tc_shape)
+bool fits_clusters(i64 batch, i64 d, i64 k);     // (tc_shape)
 
 Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     Layout L;
@@ -209,7 +209,7 @@ Layout make_layout(i64 n, i64 d, i64 k, i64 N) {
     L.agg_tiles = (int)ceil_div(d, AGG_TILE);
     L.tk = topk_layout(n, d, k);
     L.tk2 = topk_layout(2 * n, d, k);
-    L.pair = L.tk2.fast && L.tk2.cap > 0 && 2 * n <= 65535 && !fits_clusters(n, d);          // (a batch of 2 n as one dimension of a grid)
+    L.pair = L.tk2.fast && L.tk2.cap > 0 && 2 * n <= 65535 && !fits_clusters(n, d, k);          // (a batch of 2 n as one dimension of a grid)
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o += align_up(bytes); return at; };
     L.status = take(256);
@@ -362,11 +362,14 @@ struct TcShape { int C, slice, threads; };
 // save).  False where the vector is too long, or so long and the batch so large that the clusters would run in several
 // waves of one-block-per-SM: the streaming kernels read such a batch at HBM speed (rounds with k = d / 100: 20 x 204,979 68 us in two waves,
 // 48 streamed, 40 x 135,000 62 and 44, 100 x 131,072 122 and 74; k = d / 10 109 and 68, 95 and 63, 181 and 120).
-bool tc_shape(i64 batch, i64 d, TcShape& S) {
+// streamed: whether they would take it (fast_topk_eligible, and the caller has their scratch).  Where not, the limit is twice as long, and above it
+// the multi-pass select follows (multi-pass / clusters in waves: 150 x 131,072 with 0.51 d 213 / 184 us, with 0.9 d 211 / 166; a round of
+// 100 x 140,000 with 0.6 d 611 / 562).
+bool tc_shape(i64 batch, i64 d, bool streamed, TcShape& S) {
     constexpr i64 SMS = 148;
     i64 C = 1;
     while (C <= TC_MAX_CLUSTER && ceil_div(d, C) > TC_MAX_SLICE) C *= 2;
-    if (C > TC_MAX_CLUSTER || (d >= ST_MIN_D && batch * C > SMS)) return false;
+    if (C > TC_MAX_CLUSTER || (d >= (streamed ? ST_MIN_D : 2 * ST_MIN_D) && batch * C > SMS)) return false;
     while (C < 8 && batch * C * 2 <= SMS && d / (2 * C) >= 8192) C *= 2;
     S.C = (int)C;
     S.slice = (int)((ceil_div(d, C) + 127) / 128 * 128);
@@ -374,7 +377,7 @@ bool tc_shape(i64 batch, i64 d, TcShape& S) {
     return true;
 }
 
-bool fits_clusters(i64 batch, i64 d) { TcShape S; return tc_shape(batch, d, S); }
+bool fits_clusters(i64 batch, i64 d, i64 k) { TcShape S; return tc_shape(batch, d, fast_topk_eligible(d, k), S); }
 
 typedef void (*TcKernel)(const TcArgs);
 template <int MODE>
@@ -509,7 +512,7 @@ ef21_status enqueue_topk_general(cudaStream_t st, const float* a, i64 pitch_a, c
                                  i64 pitch_apply = 0, bool* applied = nullptr, unsigned long long* cut_out = nullptr) {
     if (applied) *applied = false;
     TcShape S;
-    if (tc_shape(batch, d, S)) {
+    if (tc_shape(batch, d, false, S)) {
         // the whole selection in one launch (no scratch), which also adds the messages to apply_to if the caller asks for it
         if (applied) *applied = apply_to != nullptr;
         return enqueue_topk_cluster(st, b ? TC_DIFF : TC_PLAIN, S, a, pitch_a, b, pitch_b, 0.f, batch, d, k, idx_out, val_out, apply_to,
@@ -577,7 +580,7 @@ ef21_status launch_grad_finish(ef21_ctx* c, const GradSource& G) {
 // than SMs, since they are placed as the blocks of the gradient kernel end (20 x 5,001: 32.7 us an iteration with clusters of four, 35.0 of
 // eight, 39.0 of two; 10 x 4,180: 16.1 with eight, 17.1 with four; two kernels 36.5 and 21.3).
 bool select_can_form_grads(const ef21_ctx* c, const GradSource& G, TcShape& S) {
-    if (c->d <= 512) return tc_shape(c->n, c->d, S) && S.threads == 256 && G.worker_tiles <= 4 * GRAD_FINISH_LANES;
+    if (c->d <= 512) return tc_shape(c->n, c->d, false, S) && S.threads == 256 && G.worker_tiles <= 4 * GRAD_FINISH_LANES;
     if (c->d > 8192 || G.worker_tiles > 5 * GRAD_FINISH_LANES) return false;
     i64 C = 1;
     while (C < 8 && c->n * C * 2 <= 148 && c->d / (2 * C) >= 128) C *= 2;
@@ -637,7 +640,7 @@ ef21_status minibatch_source(ef21_ctx* c, const int* batch_dev, int tau, GradSou
 // Whether the handle's rounds take the one-pass Top-k of long vectors.
 bool long_topk(const ef21_ctx* c) {
     TcShape S;
-    return c->L.tk.fast && !c->force_general_topk && !tc_shape(c->n, c->d, S);
+    return c->L.tk.fast && !c->force_general_topk && !tc_shape(c->n, c->d, true, S);
 }
 
 // Selection half of a message round: c_i = C(a_i - g_i) and g_i += c_i.  sampled: the threshold
@@ -796,7 +799,7 @@ ef21_status enqueue_ef_round(ef21_ctx* c, const float* a, i64 pitch_a) {
     TopkBuffers B = topk_buffers(c->ws + c->L.topk, c->L.tk);
     TcShape S;
     c->agg_off_ready = false;
-    if (tc_shape(c->n, c->d, S)) {
+    if (tc_shape(c->n, c->d, c->L.tk.fast && !c->force_general_topk, S)) {
         // the kernel that selects also forms p_i (kept as the new error) and clears the sent coordinates
         EF(enqueue_topk_cluster(c->stream, TC_EF, S, a, pitch_a, c->gi(), c->L.ld, c->gamma, c->n, c->d, c->k, c->msg_idx(), c->msg_val(),
                                 c->gi(), c->L.ld, &c->launches, c->status(), slow_counter(B)));
@@ -1511,7 +1514,7 @@ ef21_status ef21_local_grads(ef21_ctx* c, float* grads_out_dev) {
 size_t ef21_topk_workspace_bytes(int32_t batch, int64_t d, int32_t k) {
     if (batch < 1 || batch > 65535 || !valid_shape(1, d, k, 0)) return 0;
     TcShape S;
-    if (tc_shape(batch, d, S)) return ALIGN;         // one launch, no scratch
+    if (tc_shape(batch, d, fast_topk_eligible(d, k), S)) return ALIGN;         // one launch, no scratch
     return topk_layout(batch, d, k).total;
 }
 
@@ -1521,7 +1524,7 @@ ef21_status ef21_topk(const float* v_dev, int32_t batch, int64_t d, int32_t k, i
         return EF21_ERR_INVALID_ARG;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
     TcShape S;
-    const bool one_launch = tc_shape(batch, d, S);
+    const bool one_launch = tc_shape(batch, d, fast_topk_eligible(d, k), S);
     TopkLayout L{};
     if (one_launch) L.total = ALIGN; else L = topk_layout(batch, d, k);
     if (!workspace_dev || workspace_bytes < L.total || (reinterpret_cast<uintptr_t>(workspace_dev) % ALIGN) != 0)
