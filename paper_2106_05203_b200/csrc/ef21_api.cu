@@ -779,9 +779,9 @@ ef21_status enqueue_plus_round(ef21_ctx* c, const float* a, i64 pitch_a, int xmo
     // four blocks per SM over all workers, parts of at least 4,096 coordinates
     const i64 parts = std::max<i64>(1, std::min<i64>(std::min<i64>(PLUS_MAX_PARTS, 148 * 4 / c->n), c->d / 4096));
     double2* part = c->at<double2>(c->L.plus_parts);
-    CU(launch(plus_distortion_kernel, dim3((unsigned)parts, (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, a, pitch_a, c->gi(), c->L.ld, c->d,
+    CU(launch(sums.low ? plus_distortion_kernel<true> : plus_distortion_kernel<false>, dim3((unsigned)parts, (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, a, pitch_a, c->gi(), c->L.ld, c->d,
               ceil_div(c->d, parts), cuts, part, sums));
-    CU(launch(plus_choose_kernel, dim3((unsigned)ceil_div(c->k, PLUS_BLOCK), (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, part, (int)parts, c->gi(),
+    CU(launch(sums.low ? plus_choose_kernel<true> : plus_choose_kernel<false>, dim3((unsigned)ceil_div(c->k, PLUS_BLOCK), (unsigned)c->n), PLUS_BLOCK, 0, c->stream, 1, part, (int)parts, c->gi(),
               c->L.ld, c->k, c->msg_idx(), c->msg_val(), idx_b, val_b, c->at<int>(c->L.plus_choice), sums));
     const unsigned blocks = (unsigned)std::min<i64>(ceil_div(c->d, 1024), 148 * 8);
     auto mean = xmode == AGG_X_KEEP ? plus_mean_kernel<AGG_X_KEEP>

@@ -37,7 +37,6 @@ __device__ __forceinline__ double block_sum_f64(double v, double* scratch /* [PL
 // sums below, where M and B are bit-identical whenever the candidates coincide.  (g_i = 0, the state of the first round: they coincide
 // term by term, and a tie goes to the Markov compressor.)
 __device__ __forceinline__ int plus_decision(const PlusSums& s, int i, int n) {
-    if (s.low == nullptr) return 2;
     const int lane = threadIdx.x & 31;
     double M = 0.0, B = 0.0;
     bool nonzero = false;
@@ -57,6 +56,8 @@ __device__ __forceinline__ int plus_decision(const PlusSums& s, int i, int n) {
 // The ordered sums.  grid = (parts, n); part p of worker i covers the coordinates [p * len, (p + 1) * len).  part_out[i][p] = (M, B) of the part.  M and B
 // are summed over the same coordinates in the same order, so that they are bit-identical whenever the two candidates coincide
 // (e.g. g_i = 0).
+// SUMS: the selecting kernels have left sums that decide as a rule.
+template <bool SUMS>
 __global__ void __launch_bounds__(PLUS_BLOCK)
 plus_distortion_kernel(const float* __restrict__ a, i64 pitch_a, const float* __restrict__ gi, i64 ld, i64 d, i64 len,
                        const unsigned long long* __restrict__ cuts /* [2][n]: Markov, plain */, double2* __restrict__ part_out, const __grid_constant__ PlusSums sums) {
@@ -64,7 +65,7 @@ plus_distortion_kernel(const float* __restrict__ a, i64 pitch_a, const float* __
     pdl_wait(a, gi, cuts, part_out);
     __shared__ double scratch[PLUS_BLOCK / 32];
     const int i = blockIdx.y, n = gridDim.y;
-    if (plus_decision(sums, i, n) != 2) return;                      // as a rule
+    if (SUMS && plus_decision(sums, i, n) != 2) return;                      // as a rule
     const unsigned long long cut_m = cuts[i], cut_b = cuts[n + i];
     const unsigned km = (unsigned)(cut_m >> 32), jm = 0xffffffffu - (unsigned)cut_m, kb = (unsigned)(cut_b >> 32), jb = 0xffffffffu - (unsigned)cut_b;
     const float* __restrict__ grad = a + (i64)i * pitch_a;
@@ -96,6 +97,7 @@ plus_distortion_kernel(const float* __restrict__ a, i64 pitch_a, const float* __
 
 // grid = (ceil(k / 256), n).  Every block adds up the parts of its worker in the same fixed order; a Markov worker's entries are
 // added to g_i, a plain worker's message takes the place of the Markov one (the rows are rewritten by plus_mean_kernel).
+template <bool SUMS>
 __global__ void __launch_bounds__(PLUS_BLOCK)
 plus_choose_kernel(const double2* __restrict__ parts_in, int parts, float* __restrict__ gi, i64 ld, int k,
                    int* __restrict__ idx_m, float* __restrict__ val_m, const int* __restrict__ idx_b, const float* __restrict__ val_b,
@@ -103,7 +105,7 @@ plus_choose_kernel(const double2* __restrict__ parts_in, int parts, float* __res
     pdl_trigger();
     pdl_wait(parts_in, gi, idx_m, val_m, idx_b, val_b, choice);
     const int i = blockIdx.y, lane = threadIdx.x & 31;
-    int plain = plus_decision(sums, i, gridDim.y);
+    int plain = SUMS ? plus_decision(sums, i, gridDim.y) : 2;
     if (plain == 2) {
         double M = 0.0, B = 0.0;
         for (int q = lane; q < parts; q += 32) { const double2 s = parts_in[(i64)i * PLUS_MAX_PARTS + q]; M += s.x; B += s.y; }
