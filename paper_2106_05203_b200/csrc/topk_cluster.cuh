@@ -55,7 +55,7 @@ struct TcArgs {
     // GRAD only: a is the mean of worker i's tile partials plus the regulariser term at x (the sums of grad_finish_kernel)
     const float* partial; const int* tile_begin; const i64* row_off; const float* x;
     float lambda; int ld, batch_rows;
-    // STREAM only: vectors whose flag (one word every flag_pitch words) is zero are left alone; tile_off (may be null):
+    // REDO only: vectors whose flag (one word every flag_pitch words) is zero are left alone; tile_off (may be null):
     // [batch][ntiles + 1] first message position of every `tile` coordinates
     const unsigned* flag; int flag_pitch, batch;
     int* tile_off; int ntiles, tile;
@@ -305,9 +305,10 @@ __device__ __forceinline__ bool tc_few_cluster(const TcArgs& p, int vec, int ran
 }
 
 // STREAM: the vector is longer than the cluster's shared memory; it stays in global memory and every sweep reads it again.
+// REDO: of vectors that are flagged, one after the other.
 // GRAD > 0: the local gradients are formed from the tile partials on the way in (no kernel and no array for them), by a cluster of GRAD
 // blocks that each take a share of the columns and leave v in the first one's shared memory; that one selects alone (C = 1).
-template <int MODE, int C, int THREADS, bool STREAM, int GRAD>
+template <int MODE, int C, int THREADS, bool STREAM, int GRAD, bool REDO = STREAM>
 __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     namespace cg = cooperative_groups;
     constexpr int WARPS = THREADS / 32;
@@ -336,7 +337,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
     // thread is counted quickly.  Rounds, us, with the histogram / this way: 4 x 452,034 Top-452 in sixteen blocks 29.2 / 30.0, 16 x 79,311
     // Top-79 in eight 29.3 / 31.5; 20 x 116,750 Top-116 in four 24.9 / 22.9, 1 x 81,822 Top-818 in eight 16.2 / 14.0.  Eight rounds: 37 x 60,000 in four
     // Top-10 210 / 226, Top-60 241 / 243, Top-200 323 / 300; 70 x 30,000 in two Top-8 150 / 158, Top-30 169 / 172, Top-100 301 / 294.)
-    constexpr bool MAY_FEW = C > 1 && C <= 8 && !STREAM;
+    constexpr bool MAY_FEW = C > 1 && C <= 8 && !STREAM && !REDO;
     const bool few_cluster = MAY_FEW && p.k <= TC_FEW_OWN && (p.k + C - 1) / C <= THREADS / 5 && p.k >= (C <= 4 ? 20 : 64) * C;
     unsigned largest = 0u;
     auto clear = [&]() {
@@ -698,7 +699,7 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
         }
     }
     if (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (STREAM && p.tile_off) {
+    if (REDO && p.tile_off) {
         cluster.sync();                                              // the message is complete and visible to the cluster
         int* off = p.tile_off + (i64)vec * (p.ntiles + 1);
         const int* io = pdl_ptr(p.idx_out + (i64)vec * p.k);
@@ -715,16 +716,16 @@ __device__ __forceinline__ void tc_vector(const TcArgs& p, int vec) {
 }
 
 // (512 threads: left alone the compiler takes 40 registers; ten rounds of 20 x 8,192 Top-128 158.7 us with these, 149.5 with 56.)
-template <int MODE, int C, int THREADS, bool STREAM = false, int GRAD = 0>
+template <int MODE, int C, int THREADS, bool STREAM = false, int GRAD = 0, bool REDO = STREAM>
 __global__ void __launch_bounds__(THREADS, THREADS == 512 && GRAD == 0 ? 2 : 0)
 tc_topk_kernel(const __grid_constant__ TcArgs p) {
-    if (STREAM) {
+    if (REDO) {
         // a few clusters look through the flags: as a rule there is nothing to do
         pdl_trigger();
         pdl_wait();
         for (int vec = (int)(blockIdx.x / (unsigned)C); vec < p.batch; vec += (int)(gridDim.x / (unsigned)C))
             if (p.flag[(i64)vec * p.flag_pitch] != 0u) {
-                tc_vector<MODE, C, THREADS, STREAM, GRAD>(p, vec);
+                tc_vector<MODE, C, THREADS, STREAM, GRAD, REDO>(p, vec);
                 cooperative_groups::this_cluster().sync();
             }
     } else {

@@ -43,3 +43,34 @@ def test_rounds_and_topk(n, d, k, crowd, variant):
     for i in (0, 1, n - 1):
         order = torch.sort(V[i].abs(), descending=True, stable=True).indices[:k].sort().values
         assert torch.equal(idx[i].long(), order) and torch.equal(val[i], V[i][order])
+
+
+# vectors that are redone: clusters of eight with the vector in shared memory up to 376,832 entries, above it from global memory
+@pytest.mark.parametrize("kind", ["zeros", "few nonzero", "signs", "one vector"])
+@pytest.mark.parametrize("variant", [0, 2])
+@pytest.mark.parametrize("n,d,k", [(38, 131072, 1310), (38, 131073, 20000), (19, 262143, 262), (19, 376832, 3768), (19, 376833, 3768)])
+def test_redone_vectors(n, d, k, variant, kind):
+    from paper_2106_05203_b200 import binding as B
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    V = torch.randn(2, n, d, device="cuda", generator=gen)
+    if kind == "zeros":
+        V[1].zero_()
+    elif kind == "few nonzero":
+        V *= torch.rand(2, n, d, device="cuda", generator=gen) < 0.5 * k / d
+    elif kind == "signs":
+        V = V.sign()
+    else:
+        V[:, n // 2] = 1.0
+    states = []
+    for algorithm in (0, 1):
+        h = B.EF21(n, d, k, 0.05)
+        h.set_variant(variant)
+        h.set_topk_algorithm(algorithm)
+        h.init_grads(None, B.INIT_ZERO)
+        for v in V:
+            h.step_grads(v, 2)
+        assert h.poll() == 0
+        states.append(h.get_state())
+    for a, b in zip(*states):
+        assert torch.equal(a.view(torch.int32), b.view(torch.int32))
