@@ -277,7 +277,7 @@ ef21_status ef21_get_plus_choice(ef21_ctx* ctx, int32_t* choice_host);
  * candidates; messages of more than half of a long vector take the multi-pass radix select), 1 = no one-pass
  * path.  All give the same bits. */
 ef21_status ef21_set_topk_algorithm(ef21_ctx* ctx, int32_t algorithm);
-/* Number of vectors of d >= 2^18 entries, since creation, whose selection had to be repeated over the whole
+/* Number of vectors of d >= 2^17 entries, since creation, whose selection had to be repeated over the whole
  * vector (the sampled bracket missed, or too many ties); synchronises. */
 ef21_status ef21_fallback_count(ef21_ctx* ctx, int64_t* count);
 

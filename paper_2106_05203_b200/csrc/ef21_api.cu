@@ -41,7 +41,8 @@ namespace {
 constexpr size_t ALIGN = 256;
 // Launch-path iterations up to this dimension are replayed as a CUDA graph.  Wider ones are launched one by one: a graph per iteration is
 // a full stop between iterations, across which the gradient kernel could not fetch its first rows (20 x 300 x 5,001: 41.2 us an
-// iteration without the graph, 43.1 with it; three launches take the host about 7 us).
+// iteration without the graph, 43.1 with it; three launches take the host about 7 us).  EF21+, seven launches, 20 iterations one by one / replayed:
+// 20 x 600 x 700 554 / 597, 4 x 60 x 3,000 494 / 527, 20 x 200 x 5,001 800 / 831; 4 x 50 x 600 398 / 389, 2 x 30 x 513 400 / 398.
 constexpr i64 GRAPH_MAX_D = 512;
 inline size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 inline i64 ceil_div(i64 a, i64 b) { return (a + b - 1) / b; }
