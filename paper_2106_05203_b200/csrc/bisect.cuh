@@ -34,9 +34,10 @@ EF21_BISECT_FN unsigned bisect_floor(unsigned floor, unsigned top, int need, Cou
 // 24.6 / 23.1, Top-128 26.4 / 30.9; 888 x 8,192 Top-80 24.2 / 20.4, Top-112 25.1 / 28.7, 888 x 2,100 Top-32 14.1 / 14.1, Top-64 14.8 / 16.8;
 // 3,000 x 2,048 Top-48 26.7 / 23.7, Top-64 27.3 / 29.3, 3,000 x 300 Top-32 18.0 / 18.2.  Ten rounds of 20 workers: 9,000 Top-128 140.8 / 137.7, Top-192
 // 149 / 194; 8,192 Top-96 131.8 / 121.3, Top-128 146.8 / 153.2; 4,000 Top-64 104.6 / 98.9, Top-96 108.3 / 111.4; 2,048 Top-64 99.7 / 90.5; 300 Top-32
-// 76.6 / 77.2.  20 iterations on 10 x 100 rows: 8,000 columns Top-128 464 / 418, 5,001 Top-128 399 / 378, 1,500 Top-64 258 / 254, Top-128 279 / 314.
+// 76.6 / 77.2.  20 iterations on 10 x 100 rows: 8,000 columns Top-128 464 / 418, 5,001 Top-128 399 / 378, 1,500 Top-64 258 / 254, Top-128 279 / 314,
+// 600 Top-64 247 / 235, Top-128 251 / 282.
 EF21_BISECT_FN int few_limit(int threads, int d, bool alone, bool grad) {
-    const int line = threads == 256 ? d / 48 + 16 : (threads == 512 ? d / (grad ? 60 : 112) + 18 : d / 133 + 32);
+    const int line = threads == 256 ? d / 48 + 16 : (threads == 512 ? (grad ? d / 60 + 36 : d / 112 + 18) : d / 133 + 32);
     const int more = !alone ? 0 : (threads == 256 ? 10 : (threads == 512 ? 30 : 32));
     return line + more < threads / 4 ? line + more : threads / 4;
 }
