@@ -232,7 +232,7 @@ grad_stream_kernel(const float* __restrict__ A, const float* __restrict__ y, con
 // one group of 512 threads, 1,217 with two of 256; two blocks per SM with a second register buffer 1,252).
 // early: the rows (and labels, tile table and sampled row numbers) were complete before an earlier gradient kernel of the same call
 // passed its wait, so the ring is filled before this kernel waits for the one in front of it, while that selects and aggregates: up
-// to 160 KB per SM, 24 MB in all, arrive in time in which HBM and L2 would idle.  The first kernel of a call (early == 0) waits first,
+// to 192 KB per SM, 28 MB in all, arrive in time in which HBM and L2 would idle.  The first kernel of a call (early == 0) waits first,
 // and lets nothing behind it start before.
 // 20 x 300 x 5,001 (120 MB, more than stays in L2): 26.2 us with the next rows in a second register buffer, 24.2 through the ring,
 // 19.6 with the early start, of which HBM takes 15; 20 x 285 x 2,625: 13.2, 11.1; 20 x 208 x 1,463: 8.4, 6.0 (one group; latencies: x, two to four
